@@ -589,7 +589,7 @@ def _exact_net(case, u, seed):
     for w, g in zip(weights, grads):                     # Adam's first step on real and imaginary parts
         r = torch.view_as_real(g)
         new.append(w.detach() - torch.view_as_complex(1e-2 * r / (r.abs() + 1e-8)))
-    return {"out": out, "loss": float(loss), "grads": grads, "weights": new}
+    return {"out": out, "loss": float(loss.detach()), "grads": grads, "weights": new}
 
 
 def exact(case, seed):
