@@ -21,17 +21,75 @@ template <> struct RealOf<float2> { typedef float R; };
 constexpr int kChunk = 16;
 template <class T2> struct Ptrs8 { const T2* p[kChunk]; };
 
-// CTAs per right-hand side of a reduction: at least 8 elements per thread, and
-// R * CTAs within the partial buffer.
-static int reduce_ctas(size_t n, int R) {
-  const size_t per = std::max<size_t>(1, (size_t)kMaxReduceCta / (size_t)std::max(R, 1));
-  return (int)std::max<size_t>(1, std::min<size_t>((n + 2047) / 2048, per));
+// CTAs per right-hand side of a reduction over n elements, slots double2 of
+// partial sums each: 8 elements a thread, R * CTAs within the partial buffer.
+// A vector too short to give every SM a CTA that way (152 over all right-hand
+// sides) is cut finer, down to one element a thread: there the pass takes the
+// latency of one thread's loads and not bandwidth (the 20480-entry coarse
+// vectors of 16^3 x 32: a 12-vector dot pass 24.9 us on 5 CTAs).
+static int reduce_ctas(size_t n, int R, size_t slots = kChunk) {
+  const size_t r = (size_t)std::max(R, 1);
+  const size_t per = std::max<size_t>(1, kPartialSums / slots / r);
+  const size_t fill = std::min<size_t>((n + 255) / 256, (152 + r - 1) / r);
+  return (int)std::max<size_t>(1, std::min<size_t>(std::max((n + 2047) / 2048, fill), per));
+}
+
+// Reductions end inside the kernel that forms the partial sums: the CTA of a
+// right-hand side that arrives last (a counter per right-hand side behind the
+// partial sums; atomicInc wraps it back to 0) adds the CTAs' parts in their
+// fixed order, so the result does not depend on which CTA that is.  A separate
+// one-CTA kernel for it cost a launch and 7.8 us (12 sums one after the other).
+__device__ __forceinline__ bool last_cta(double2* partial, int r) {
+  __shared__ int last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0)
+    last = atomicInc(reinterpret_cast<unsigned*>(partial + kPartialSums) + r, gridDim.x - 1) == gridDim.x - 1;
+  __syncthreads();
+  if (last) __threadfence();
+  return last != 0;
+}
+
+// The calling warp's sum of slot j over the CTAs' partial sums of right-hand side r.
+__device__ __forceinline__ double2 sum_slot(const double2* partial, int r, int slots, int j) {
+  double a = 0, b = 0;
+#pragma unroll 4
+  for (int c = threadIdx.x & 31; c < (int)gridDim.x; c += 32) {
+    const double2 v = __ldcg(partial + ((size_t)r * gridDim.x + c) * slots + j);
+    a += v.x;
+    b += v.y;
+  }
+  return make_double2(warp_sum(a), warp_sum(b));
+}
+
+// where the K sums of a dot pass go: out[r*ldo + j] = (mode 1: out +) the sum,
+// out2[r*ldo + j] = the sum if out2 != nullptr
+struct DotOut {
+  double2* out;
+  double2* out2;
+  int ldo, mode;
+};
+template <int K>
+__device__ __forceinline__ void finish_dots(double2* partial, const DotOut& d) {
+  const int r = blockIdx.y;
+  if (!last_cta(partial, r)) return;
+  for (int j = threadIdx.x >> 5; j < K; j += 8) {
+    const double2 t = sum_slot(partial, r, kChunk, j);
+    if ((threadIdx.x & 31) == 0) {
+      if (d.out) {
+        double2* o = d.out + (size_t)r * d.ldo + j;
+        if (d.mode == 1) { o->x += t.x; o->y += t.y; }
+        else *o = t;
+      }
+      if (d.out2) d.out2[(size_t)r * d.ldo + j] = t;
+    }
+  }
 }
 
 template <class T2, int K>
 __global__ void __launch_bounds__(256) multidot_partial(Ptrs8<T2> v, const T2* __restrict__ w, size_t n,
                                                         size_t vstride, size_t wstride,
-                                                        double2* __restrict__ partial) {
+                                                        double2* __restrict__ partial, DotOut dout) {
   typedef typename RealOf<T2>::R R;
   const int r = blockIdx.y;
   const T2* wr = w + r * wstride;
@@ -65,13 +123,14 @@ __global__ void __launch_bounds__(256) multidot_partial(Ptrs8<T2> v, const T2* _
     for (int q = 0; q < 8; ++q) { s += red[q][2 * threadIdx.x]; m += red[q][2 * threadIdx.x + 1]; }
     partial[((size_t)r * gridDim.x + blockIdx.x) * kChunk + threadIdx.x] = make_double2(s, m);
   }
+  finish_dots<K>(partial, dout);
 }
 
 // FP32 vectors with an even length: two complex numbers per 16-byte load.
 template <int K>
 __global__ void __launch_bounds__(256) multidot_partial_f4(Ptrs8<float2> v, const float2* __restrict__ w, size_t n,
                                                            size_t vstride, size_t wstride,
-                                                           double2* __restrict__ partial) {
+                                                           double2* __restrict__ partial, DotOut dout) {
   const int r = blockIdx.y;
   const float4* wr = reinterpret_cast<const float4*>(w + r * wstride);
   const size_t n4 = n / 2;
@@ -103,55 +162,25 @@ __global__ void __launch_bounds__(256) multidot_partial_f4(Ptrs8<float2> v, cons
     for (int q = 0; q < 8; ++q) { s += red[q][2 * threadIdx.x]; m += red[q][2 * threadIdx.x + 1]; }
     partial[((size_t)r * gridDim.x + blockIdx.x) * kChunk + threadIdx.x] = make_double2(s, m);
   }
-}
-
-// out[r*ldo + j] = (mode 1: out +) sum over CTAs; out2[r*ldo + j] = the sum if out2 != nullptr.
-__global__ void multidot_finalize(const double2* __restrict__ partial, int ncta, int k, double2* out, int ldo,
-                                  int mode, double2* out2) {
-  __shared__ double red[8][2];
-  const int r = blockIdx.x;
-  for (int j = 0; j < k; ++j) {
-    double s = 0, m = 0;
-    for (int c = threadIdx.x; c < ncta; c += blockDim.x) {
-      const double2 v = partial[((size_t)r * ncta + c) * kChunk + j];
-      s += v.x;
-      m += v.y;
-    }
-    s = warp_sum(s);
-    m = warp_sum(m);
-    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (lane == 0) { red[wid][0] = s; red[wid][1] = m; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double ss = 0, sm = 0;
-      for (int q = 0; q < 8; ++q) { ss += red[q][0]; sm += red[q][1]; }
-      if (out) {
-        double2* o = out + (size_t)r * ldo + j;
-        if (mode == 1) { o->x += ss; o->y += sm; }
-        else *o = make_double2(ss, sm);
-      }
-      if (out2) out2[(size_t)r * ldo + j] = make_double2(ss, sm);
-    }
-    __syncthreads();
-  }
+  finish_dots<K>(partial, dout);
 }
 
 template <class T2, int K>
 static void md_launch(dim3 grid, const Ptrs8<T2>& p, const T2* w, size_t n, size_t vs, size_t ws, double2* part,
-                      cudaStream_t s) {
-  multidot_partial<T2, K><<<grid, 256, 0, s>>>(p, w, n, vs, ws, part); count_launches(1);
+                      const DotOut& d, cudaStream_t s) {
+  multidot_partial<T2, K><<<grid, 256, 0, s>>>(p, w, n, vs, ws, part, d); count_launches(1);
 }
 
 template <class T2, int K>
 static void md_launch_any(bool vec4, dim3 grid, const Ptrs8<T2>& p, const T2* w, size_t n, size_t vs, size_t ws,
-                          double2* part, cudaStream_t s) {
+                          double2* part, const DotOut& d, cudaStream_t s) {
   if constexpr (std::is_same<T2, float2>::value) {
     if (vec4) {
-      multidot_partial_f4<K><<<grid, 256, 0, s>>>(p, w, n, vs, ws, part); count_launches(1);
+      multidot_partial_f4<K><<<grid, 256, 0, s>>>(p, w, n, vs, ws, part, d); count_launches(1);
       return;
     }
   }
-  md_launch<T2, K>(grid, p, w, n, vs, ws, part, s);
+  md_launch<T2, K>(grid, p, w, n, vs, ws, part, d, s);
 }
 
 template <class T2>
@@ -168,15 +197,14 @@ static int multidot_t(const BVec& b, const void* const* v, int k, const void* w,
     Ptrs8<T2> p;
     for (int j = 0; j < kChunk; ++j) p.p[j] = (const T2*)v[j0 + std::min(j, kk - 1)];
     const T2* wp = (const T2*)w;
-#define SAPMG_MD(K) case K: md_launch_any<T2, K>(vec4, grid, p, wp, b.n, b.vstride, b.wstride, partial, s); break;
+    const DotOut d{out ? out + j0 : nullptr, out2 ? out2 + j0 : nullptr, ldo, mode};
+#define SAPMG_MD(K) case K: md_launch_any<T2, K>(vec4, grid, p, wp, b.n, b.vstride, b.wstride, partial, d, s); break;
     switch (kk) {
       SAPMG_MD(1) SAPMG_MD(2) SAPMG_MD(3) SAPMG_MD(4) SAPMG_MD(5) SAPMG_MD(6) SAPMG_MD(7) SAPMG_MD(8)
       SAPMG_MD(9) SAPMG_MD(10) SAPMG_MD(11) SAPMG_MD(12) SAPMG_MD(13) SAPMG_MD(14) SAPMG_MD(15)
-      default: md_launch_any<T2, 16>(vec4, grid, p, wp, b.n, b.vstride, b.wstride, partial, s); break;
+      default: md_launch_any<T2, 16>(vec4, grid, p, wp, b.n, b.vstride, b.wstride, partial, d, s); break;
     }
 #undef SAPMG_MD
-    multidot_finalize<<<b.R, 256, 0, s>>>(partial, ncta, kk, out ? out + j0 : nullptr, ldo, mode,
-                                          out2 ? out2 + j0 : nullptr); count_launches(1);
   }
   SAPMG_CUDA_TRY(cudaGetLastError());
   return MG_OK;
@@ -191,13 +219,13 @@ int blas_multidot(int type, const BVec& b, const void* const* v, int k, const vo
   return MG_ERR_ARG;
 }
 
-// w[r] += sign * sum_j coeff[r*ldc + j] v_j[r]; with partial != nullptr the
-// CTA also writes its part of ||w_new||^2 (finished by multidot_finalize).
+// w[r] += sign * sum_j coeff[r*ldc + j] v_j[r]; with partial != nullptr also
+// nrm[r*ldn] = ||w_new||^2.
 template <class T2, int K>
 __global__ void __launch_bounds__(256) multiaxpy_kernel(T2* __restrict__ w, Ptrs8<T2> v,
                                                         const double2* __restrict__ coeff, int ldc, double sign,
                                                         size_t n, size_t vstride, size_t wstride,
-                                                        double2* __restrict__ partial) {
+                                                        double2* __restrict__ partial, DotOut dout) {
   typedef typename RealOf<T2>::R R;
   const int r = blockIdx.y;
   R cr[K], ci[K];
@@ -231,19 +259,25 @@ __global__ void __launch_bounds__(256) multiaxpy_kernel(T2* __restrict__ w, Ptrs
       for (int q = 0; q < 8; ++q) sum += red[q];
       partial[((size_t)r * gridDim.x + blockIdx.x) * kChunk] = make_double2(sum, 0.0);
     }
+      finish_dots<1>(partial, dout);
   }
 }
 
-// Streaming kernels: about 8 CTAs of 256 threads per SM over all right-hand sides.
+// Streaming kernels: about 8 CTAs of 256 threads per SM over all right-hand
+// sides, 4 elements a thread; a short vector one element a thread until every
+// SM has a CTA (as reduce_ctas).
 static dim3 stream_grid(size_t n, int R) {
-  const size_t per = std::max<size_t>(16, (size_t)152 * 8 / (size_t)std::max(R, 1));
-  return dim3((unsigned)std::max<size_t>(1, std::min<size_t>((n + 1023) / 1024, per)), R);
+  const size_t r = (size_t)std::max(R, 1);
+  const size_t per = std::max<size_t>(16, (size_t)152 * 8 / r);
+  const size_t fill = std::min<size_t>((n + 255) / 256, (152 + r - 1) / r);
+  return dim3((unsigned)std::max<size_t>(1, std::min<size_t>(std::max((n + 1023) / 1024, fill), per)), R);
 }
 
 template <class T2, int K>
 static void ma_launch(dim3 g, T2* w, const Ptrs8<T2>& p, const double2* c, int ldc, double sign, const BVec& b,
-                      double2* partial, cudaStream_t s) {
-  multiaxpy_kernel<T2, K><<<g, 256, 0, s>>>(w, p, c, ldc, sign, b.n, b.vstride, b.wstride, partial); count_launches(1);
+                      double2* partial, const DotOut& d, cudaStream_t s) {
+  multiaxpy_kernel<T2, K><<<g, 256, 0, s>>>(w, p, c, ldc, sign, b.n, b.vstride, b.wstride, partial, d);
+  count_launches(1);
 }
 
 template <class T2>
@@ -257,16 +291,14 @@ static int multiaxpy_t(const BVec& b, void* w, const void* const* v, int k, cons
     for (int j = 0; j < kChunk; ++j) p.p[j] = (const T2*)v[j0 + std::min(j, kk - 1)];
     const double2* c = coeff + j0;
     double2* part = (last && nrm2) ? partial : nullptr;
-#define SAPMG_MA(K) case K: ma_launch<T2, K>(g, (T2*)w, p, c, ldc, sign, b, part, s); break;
+    const DotOut d{nrm2, nullptr, ldn, 0};
+#define SAPMG_MA(K) case K: ma_launch<T2, K>(g, (T2*)w, p, c, ldc, sign, b, part, d, s); break;
     switch (kk) {
       SAPMG_MA(1) SAPMG_MA(2) SAPMG_MA(3) SAPMG_MA(4) SAPMG_MA(5) SAPMG_MA(6) SAPMG_MA(7) SAPMG_MA(8)
       SAPMG_MA(9) SAPMG_MA(10) SAPMG_MA(11) SAPMG_MA(12) SAPMG_MA(13) SAPMG_MA(14) SAPMG_MA(15)
-      default: ma_launch<T2, 16>(g, (T2*)w, p, c, ldc, sign, b, part, s); break;
+      default: ma_launch<T2, 16>(g, (T2*)w, p, c, ldc, sign, b, part, d, s); break;
     }
 #undef SAPMG_MA
-  }
-  if (nrm2) {
-    multidot_finalize<<<b.R, 256, 0, s>>>(partial, (int)g.x, 1, nrm2, ldn, 0, nullptr); count_launches(1);
   }
   SAPMG_CUDA_TRY(cudaGetLastError());
   return MG_OK;
@@ -366,87 +398,101 @@ int blas_normalize(int type, const BVec& b, const void* x, void* out, const doub
 }
 
 // Least-squares solve of the (m+1) x m Hessenberg system min ||beta e1 - H y||
-// of fixed-step GMRES, one warp per right-hand side: H in shared memory, each
-// Givens rotation computed by every lane (same values) and applied to the
-// columns in parallel, back substitution with warp-reduced row sums.  H for
+// of fixed-step GMRES, one warp per right-hand side: H in shared memory, column
+// k on lane k; step j's rotation [conj a, conj b; -b, a] / sqrt(|a|^2 + |b|^2)
+// is formed by every lane from the pivot column and applied to the lane's own,
+// then the back substitution takes y_i out of all rows above at once.  H for
 // RHS r at H + r*ldr, column-major with leading dimension ldh; beta2[r].x =
-// ||b_r||^2; y[r*ldy + j].  Columns after a zero subdiagonal entry are
-// unused.  m <= 32.
+// ||b_r||^2; y[r*ldy + j].  scale != nullptr: basis vector j has the norm
+// scale[r*ldr + j].x (j = 0: 1) and y is divided by it.  Columns after a zero
+// subdiagonal entry are unused.  m <= 32.
+// Latency-bound (one reciprocal square root a step; every load and every
+// division is issued for all columns at once): 12 steps on one vector 73 us
+// with two square roots and divisions a step and serial loads, about 12 now.
 __global__ void __launch_bounds__(32) hessenberg_solve_kernel(const double2* __restrict__ Hall, int ldh, int ldr,
                                                               int m, const double2* __restrict__ beta2,
+                                                              const double2* __restrict__ scale,
                                                               double2* __restrict__ yall, int ldy) {
   __shared__ double hr[33 * 32], hi[33 * 32];
-  __shared__ double gr[33], gi[33], yr[32], yi[32];
   const int r = blockIdx.x, lane = threadIdx.x;
   const double2* Hin = Hall + (size_t)r * ldr;
   double2* y = yall + (size_t)r * ldy;
   const double beta = sqrt(fmax(beta2[r].x, 0.0));
   if (beta == 0.0) {
-    for (int j = lane; j < m; j += 32) y[j] = make_double2(0, 0);
+    if (lane < m) y[lane] = make_double2(0, 0);
     return;
   }
-  int mm = m;
-  for (int j = 0; j < m; ++j)
-    if (Hin[(j + 1) + j * ldh].x == 0.0) { mm = j + 1; break; }
-  for (int idx = lane; idx < 33 * mm; idx += 32) {
-    const int k = idx / 33, i = idx % 33;
-    const bool in = i <= k + 1;
-    hr[idx] = in ? Hin[i + k * ldh].x : 0.0;
-    hi[idx] = in ? Hin[i + k * ldh].y : 0.0;
+  const double sub = lane < m ? Hin[lane + 1 + lane * ldh].x : 1.0;
+  double inv_s = 1.0;
+  if (scale && lane > 0 && lane < m) {
+    const double t = scale[(size_t)r * ldr + lane].x;
+    inv_s = t > 0.0 ? 1.0 / t : 0.0;
   }
-  for (int i = lane; i <= mm; i += 32) { gr[i] = i == 0 ? beta : 0.0; gi[i] = 0.0; }
+  const unsigned zero = __ballot_sync(0xffffffffu, sub == 0.0);
+  const int mm = zero ? __ffs(zero) : m;                 // columns up to the first zero subdiagonal entry
+  for (int k = 0; k < mm; ++k) {                         // lane = row; the last row by lane 0
+    const double2 v = lane <= k + 1 && lane <= mm ? Hin[lane + k * ldh] : make_double2(0, 0);
+    hr[lane + k * 33] = v.x;
+    hi[lane + k * 33] = v.y;
+  }
+  if (lane == 0 && mm == 32) {
+    for (int k = 0; k < 31; ++k) hr[32 + k * 33] = hi[32 + k * 33] = 0.0;
+    const double2 v = Hin[32 + 31 * ldh];
+    hr[32 + 31 * 33] = v.x;
+    hi[32 + 31 * 33] = v.y;
+  }
+  double gr = lane == 0 ? beta : 0.0, gi = 0.0;          // g_lane; g_32 only closes the residual
   __syncwarp();
   for (int j = 0; j < mm; ++j) {
     const double ar = hr[j + j * 33], ai = hi[j + j * 33];
     const double br = hr[j + 1 + j * 33], bi = hi[j + 1 + j * 33];
-    const double na = sqrt(ar * ar + ai * ai), nb = sqrt(br * br + bi * bi);
-    const double den = sqrt(na * na + nb * nb);
-    double c, sr, si;
-    if (den == 0.0) { c = 1; sr = si = 0; }
-    else if (na == 0.0) { c = 0; sr = 1; si = 0; }
-    else {
-      c = na / den;
-      const double pr = ar / na, pi = ai / na;    // s = (a/|a|) conj(b) / den
-      sr = (pr * br + pi * bi) / den;
-      si = (pi * br - pr * bi) / den;
+    const double d2 = ar * ar + ai * ai + br * br + bi * bi;
+    const double inv = rsqrt(d2);
+    // a vanishing pivot column is left as it is (the identity rotation)
+    const double cr = d2 > 0.0 ? ar * inv : 1.0, ci = d2 > 0.0 ? ai * inv : 0.0;
+    const double sr = d2 > 0.0 ? br * inv : 0.0, si = d2 > 0.0 ? bi * inv : 0.0;
+    __syncwarp();                                         // every lane has read column j
+    if (lane >= j && lane < mm) {
+      const double xr = hr[j + lane * 33], xi = hi[j + lane * 33];
+      const double zr = hr[j + 1 + lane * 33], zi = hi[j + 1 + lane * 33];
+      hr[j + lane * 33] = cr * xr + ci * xi + sr * zr + si * zi;
+      hi[j + lane * 33] = cr * xi - ci * xr + sr * zi - si * zr;
+      hr[j + 1 + lane * 33] = cr * zr - ci * zi - sr * xr + si * xi;
+      hi[j + 1 + lane * 33] = cr * zi + ci * zr - sr * xi - si * xr;
     }
-    __syncwarp();                                   // every lane has read column j
-    for (int k = j + lane; k < mm; k += 32) {       // rotate rows j, j+1 of column k
-      const double xr = hr[j + k * 33], xi = hi[j + k * 33];
-      const double zr = hr[j + 1 + k * 33], zi = hi[j + 1 + k * 33];
-      hr[j + k * 33] = c * xr + (sr * zr - si * zi);
-      hi[j + k * 33] = c * xi + (sr * zi + si * zr);
-      hr[j + 1 + k * 33] = -(sr * xr + si * xi) + c * zr;
-      hi[j + 1 + k * 33] = -(sr * xi - si * xr) + c * zi;
-    }
-    if (lane == 0) {
-      const double xr = gr[j], xi = gi[j];
-      gr[j] = c * xr;
-      gi[j] = c * xi;
-      gr[j + 1] = -(sr * xr + si * xi);
-      gi[j + 1] = -(sr * xi - si * xr);
+    const double xr = __shfl_sync(0xffffffffu, gr, j), xi = __shfl_sync(0xffffffffu, gi, j);
+    if (lane == j) {                                      // g_{j+1} was 0
+      gr = cr * xr + ci * xi;
+      gi = cr * xi - ci * xr;
+    } else if (lane == j + 1) {
+      gr = -(sr * xr - si * xi);
+      gi = -(sr * xi + si * xr);
     }
     __syncwarp();
   }
+  // the reciprocals of the diagonal, one a lane; a zero entry gives y_i = 0
+  double wr = 0.0, wi = 0.0;
+  if (lane < mm) {
+    const double dr = hr[lane + lane * 33], di = hi[lane + lane * 33];
+    const double d2 = dr * dr + di * di;
+    if (d2 > 0.0) {
+      const double q = 1.0 / d2;
+      wr = dr * q;
+      wi = -di * q;
+    }
+  }
+  double yr = 0.0, yi = 0.0;
   for (int i = mm - 1; i >= 0; --i) {
-    double sr = 0, si = 0;
-    for (int k = i + 1 + lane; k < mm; k += 32) {
-      const double hr_ = hr[i + k * 33], hi_ = hi[i + k * 33];
-      sr += hr_ * yr[k] - hi_ * yi[k];
-      si += hr_ * yi[k] + hi_ * yr[k];
+    const double tr = gr * wr - gi * wi, ti = gr * wi + gi * wr;
+    const double sr = __shfl_sync(0xffffffffu, tr, i), si = __shfl_sync(0xffffffffu, ti, i);
+    if (lane == i) { yr = sr; yi = si; }
+    if (lane < i) {
+      const double ur = hr[lane + i * 33], ui = hi[lane + i * 33];
+      gr -= ur * sr - ui * si;
+      gi -= ur * si + ui * sr;
     }
-    sr = warp_sum(sr);
-    si = warp_sum(si);
-    if (lane == 0) {
-      const double tr = gr[i] - sr, ti = gi[i] - si;
-      const double dr = hr[i + i * 33], di = hi[i + i * 33];
-      const double d2 = dr * dr + di * di;
-      yr[i] = d2 > 0 ? (tr * dr + ti * di) / d2 : 0.0;
-      yi[i] = d2 > 0 ? (ti * dr - tr * di) / d2 : 0.0;
-    }
-    __syncwarp();
   }
-  for (int j = lane; j < m; j += 32) y[j] = j < mm ? make_double2(yr[j], yi[j]) : make_double2(0, 0);
+  if (lane < m) y[lane] = make_double2(yr * inv_s, yi * inv_s);
 }
 
 // ------------------------------------------------------------ delayed reorthogonalisation
@@ -493,12 +539,81 @@ constexpr int kDots2Max = 12;      // basis vectors per pass-1 launch
 constexpr int kDots2Slots = 32;    // partial slots per (right-hand side, CTA)
 template <class V> struct PtrsV { const V* p[16]; };
 
+// What ends a pass 1: the sums go to A[r*ld + j0 + i], B[r*ld + j0 + i] (i < K)
+// and X[r*4 + e]; the pass's last chunk (last) then forms, in one thread,
+// beta, h_j and the pass-2 coefficients for the vector list
+// [u, w, v_0 .. v_{j-1}]: c1 makes v_j, c2 makes the new w; hcol[0..j] =
+// (B_0 .. B_{j-1}, h_j); acol[0..j] = (A_0 .. A_{j-1}, beta).  A vanishing beta
+// (u in the span of the basis: a zero or invariant direction) gives zero
+// coefficients.
+struct Dcgs2Out {
+  double2 *A, *B, *X, *c1, *c2, *hcol, *acol;
+  int ld, j0, j, last;
+};
+__device__ inline void dcgs2_coeff(const Dcgs2Out& d, int r) {
+  const int j = d.j;
+  const double2* a = d.A + (size_t)r * d.ld;
+  const double2* b = d.B + (size_t)r * d.ld;
+  const double2* x = d.X + (size_t)r * 4;
+  double2* o1 = d.c1 + (size_t)r * d.ld;
+  double2* o2 = d.c2 + (size_t)r * d.ld;
+  double2* hc = d.hcol + (size_t)r * d.ld;
+  double2* ac = d.acol + (size_t)r * d.ld;
+  double na = 0;
+  for (int i = 0; i < j; ++i) na += a[i].x * a[i].x + a[i].y * a[i].y;
+  const double dd = x[0].x;
+  const double beta2 = dd - na;
+  if (!(beta2 > 1e-24 * dd) || !(dd > 0)) {
+    for (int i = 0; i < j + 2; ++i) { o1[i] = make_double2(0, 0); o2[i] = make_double2(0, 0); }
+    for (int i = 0; i <= j; ++i) { hc[i] = make_double2(0, 0); ac[i] = make_double2(0, 0); }
+    return;
+  }
+  const double beta = sqrt(beta2), ib = 1.0 / beta;
+  double sr = x[1].x, si = x[1].y;                          // c - sum conj(a_i) b_i
+  for (int i = 0; i < j; ++i) {
+    sr -= a[i].x * b[i].x + a[i].y * b[i].y;
+    si -= a[i].x * b[i].y - a[i].y * b[i].x;
+  }
+  const double hr = sr * ib, hi = si * ib;                  // h_j
+  const double gr = hr * ib, gi = hi * ib;                  // h_j / beta
+  o1[0] = make_double2(ib, 0);
+  o1[1] = make_double2(0, 0);
+  o2[0] = make_double2(-gr, -gi);
+  o2[1] = make_double2(1, 0);
+  for (int i = 0; i < j; ++i) {
+    o1[2 + i] = make_double2(-a[i].x * ib, -a[i].y * ib);
+    // -(b_i - (h_j / beta) a_i)
+    o2[2 + i] = make_double2(-(b[i].x - (gr * a[i].x - gi * a[i].y)), -(b[i].y - (gr * a[i].y + gi * a[i].x)));
+    hc[i] = b[i];
+    ac[i] = a[i];
+  }
+  hc[j] = make_double2(hr, hi);
+  ac[j] = make_double2(beta, 0);
+}
+template <int K, bool EXTRA>
+__device__ __forceinline__ void finish_dots2(double2* partial, const Dcgs2Out& d) {
+  const int r = blockIdx.y;
+  if (!last_cta(partial, r)) return;
+  constexpr int NS = 2 * K + (EXTRA ? 3 : 0);
+  for (int q = threadIdx.x >> 5; q < NS; q += 8) {
+    const double2 t = sum_slot(partial, r, kDots2Slots, q);
+    if ((threadIdx.x & 31) == 0) {
+      if (q < K) d.A[(size_t)r * d.ld + d.j0 + q] = t;
+      else if (q < 2 * K) d.B[(size_t)r * d.ld + d.j0 + q - K] = t;
+      else d.X[(size_t)r * 4 + q - 2 * K] = t;
+    }
+  }
+  if (!d.last) return;
+  __syncthreads();
+  if (threadIdx.x == 0) dcgs2_coeff(d, r);
+}
+
 // slots: [i] = <v_i, u>, [K + i] = <v_i, w>, [2K + 0..2] = <u,u>, <u,w>, <w,w> (EXTRA only)
 template <class T2, int K, bool EXTRA>
 __global__ void __launch_bounds__(256) dots2_partial(PtrsV<typename Unit<T2>::V> v,
                                                      const typename Unit<T2>::V* __restrict__ u,
                                                      const typename Unit<T2>::V* __restrict__ w, size_t nu,
-                                                     size_t stride, double2* __restrict__ partial) {
+                                                     size_t stride, double2* __restrict__ partial, Dcgs2Out dout) {
   typedef typename Unit<T2>::V V;
   typedef typename Unit<T2>::R R;
   constexpr int NS = 2 * K + (EXTRA ? 3 : 0);
@@ -539,85 +654,7 @@ __global__ void __launch_bounds__(256) dots2_partial(PtrsV<typename Unit<T2>::V>
     for (int q = 0; q < 8; ++q) { s += red[q][2 * threadIdx.x]; m += red[q][2 * threadIdx.x + 1]; }
     partial[((size_t)r * gridDim.x + blockIdx.x) * kDots2Slots + threadIdx.x] = make_double2(s, m);
   }
-}
-
-// Sums the CTAs' slots: A[r*ld + j0 + i], B[r*ld + j0 + i] (i < K), X[r*4 + e].
-__global__ void dots2_finalize(const double2* __restrict__ partial, int ncta, int K, bool extra, double2* A,
-                               double2* B, double2* X, int ld, int j0) {
-  __shared__ double red[8][2];
-  const int r = blockIdx.x;
-  const int ns = 2 * K + (extra ? 3 : 0);
-  for (int q = 0; q < ns; ++q) {
-    double s = 0, m = 0;
-    for (int c = threadIdx.x; c < ncta; c += blockDim.x) {
-      const double2 v = partial[((size_t)r * ncta + c) * kDots2Slots + q];
-      s += v.x;
-      m += v.y;
-    }
-    s = warp_sum(s);
-    m = warp_sum(m);
-    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (lane == 0) { red[wid][0] = s; red[wid][1] = m; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double ss = 0, sm = 0;
-      for (int k = 0; k < 8; ++k) { ss += red[k][0]; sm += red[k][1]; }
-      const double2 o = make_double2(ss, sm);
-      if (q < K) A[(size_t)r * ld + j0 + q] = o;
-      else if (q < 2 * K) B[(size_t)r * ld + j0 + q - K] = o;
-      else X[(size_t)r * 4 + q - 2 * K] = o;
-    }
-    __syncthreads();
-  }
-}
-
-// Per right-hand side (one thread): beta, h_j and the pass-2 coefficients for
-// the vector list [u, w, v_0 .. v_{j-1}]: c1 makes v_j, c2 makes the new w.
-// hcol[0..j] = (B_0 .. B_{j-1}, h_j); acol[0..j] = (A_0 .. A_{j-1}, beta).  A
-// vanishing beta (u in the span of the basis: a zero or invariant direction)
-// gives zero coefficients.
-__global__ void dcgs2_coeff_kernel(int j, const double2* __restrict__ A, const double2* __restrict__ B,
-                                   const double2* __restrict__ X, int ld, double2* c1, double2* c2, int ldc,
-                                   double2* hcol, double2* acol) {
-  if (threadIdx.x != 0) return;
-  const int r = blockIdx.x;
-  const double2* a = A + (size_t)r * ld;
-  const double2* b = B + (size_t)r * ld;
-  const double2* x = X + (size_t)r * 4;
-  double2* o1 = c1 + (size_t)r * ldc;
-  double2* o2 = c2 + (size_t)r * ldc;
-  double2* hc = hcol + (size_t)r * ld;
-  double2* ac = acol + (size_t)r * ld;
-  double na = 0;
-  for (int i = 0; i < j; ++i) na += a[i].x * a[i].x + a[i].y * a[i].y;
-  const double d = x[0].x;
-  const double beta2 = d - na;
-  if (!(beta2 > 1e-24 * d) || !(d > 0)) {
-    for (int i = 0; i < j + 2; ++i) { o1[i] = make_double2(0, 0); o2[i] = make_double2(0, 0); }
-    for (int i = 0; i <= j; ++i) { hc[i] = make_double2(0, 0); ac[i] = make_double2(0, 0); }
-    return;
-  }
-  const double beta = sqrt(beta2), ib = 1.0 / beta;
-  double sr = x[1].x, si = x[1].y;                          // c - sum conj(a_i) b_i
-  for (int i = 0; i < j; ++i) {
-    sr -= a[i].x * b[i].x + a[i].y * b[i].y;
-    si -= a[i].x * b[i].y - a[i].y * b[i].x;
-  }
-  const double hr = sr * ib, hi = si * ib;                  // h_j
-  const double gr = hr * ib, gi = hi * ib;                  // h_j / beta
-  o1[0] = make_double2(ib, 0);
-  o1[1] = make_double2(0, 0);
-  o2[0] = make_double2(-gr, -gi);
-  o2[1] = make_double2(1, 0);
-  for (int i = 0; i < j; ++i) {
-    o1[2 + i] = make_double2(-a[i].x * ib, -a[i].y * ib);
-    // -(b_i - (h_j / beta) a_i)
-    o2[2 + i] = make_double2(-(b[i].x - (gr * a[i].x - gi * a[i].y)), -(b[i].y - (gr * a[i].y + gi * a[i].x)));
-    hc[i] = b[i];
-    ac[i] = a[i];
-  }
-  hc[j] = make_double2(hr, hi);
-  ac[j] = make_double2(beta, 0);
+  finish_dots2<K, EXTRA>(partial, dout);
 }
 
 // y1 = (acc ? y1 : 0) + sum c1_q v_q, y2 likewise; y1 and y2 may be v_0, v_1
@@ -627,7 +664,8 @@ template <class T2, int K>
 __global__ void __launch_bounds__(256) axpy2_kernel(PtrsV<typename Unit<T2>::V> v, const double2* __restrict__ c1,
                                                     const double2* __restrict__ c2, int ldc, int j0,
                                                     typename Unit<T2>::V* y1, typename Unit<T2>::V* y2, size_t nu,
-                                                    size_t stride, int acc, double2* __restrict__ partial) {
+                                                    size_t stride, int acc, double2* __restrict__ partial,
+                                                    DotOut dout) {
   typedef typename Unit<T2>::V V;
   typedef typename Unit<T2>::R R;
   __shared__ R cf[4][16];
@@ -670,6 +708,7 @@ __global__ void __launch_bounds__(256) axpy2_kernel(PtrsV<typename Unit<T2>::V> 
       for (int q = 0; q < 8; ++q) sum += red[q][threadIdx.x];
       partial[((size_t)r * gridDim.x + blockIdx.x) * kChunk + threadIdx.x] = make_double2(sum, 0.0);
     }
+      finish_dots<2>(partial, dout);
   }
 }
 
@@ -681,18 +720,19 @@ static int dcgs2_step_t(const BVec& b, const void* const* v, int j, void* u, voi
   const size_t nu = b.n / C, stride = b.vstride / C;
   const int R = b.R;
   // pass 1: dots of u and w with the basis (chunks of kDots2Max) and with each other
-  const int ncta1 = std::max(1, std::min(reduce_ctas(nu, R), (int)(kPartialDouble2 / kDots2Slots / (size_t)R)));
+  const int ncta1 = reduce_ctas(nu, R, kDots2Slots);
   const dim3 g1(ncta1, R);
   int j0 = 0;
   do {
     const int kk = std::min(kDots2Max, j - j0);
     const bool extra = (j0 == 0);
+    const Dcgs2Out d{ws.A, ws.B, ws.X, ws.c1, ws.c2, ws.hcol, ws.acol, ws.ld, j0, j, j0 + kk >= j};
     PtrsV<V> p;
     for (int q = 0; q < 16; ++q) p.p[q] = j > 0 ? (const V*)v[std::max(0, std::min(j0 + q, j - 1))] : (const V*)u;
 #define SAPMG_D2(K)                                                                                          \
   case K:                                                                                                    \
-    if (extra) { dots2_partial<T2, K, true><<<g1, 256, 0, s>>>(p, (const V*)u, (const V*)w, nu, stride, ws.partial); } \
-    else { dots2_partial<T2, K, false><<<g1, 256, 0, s>>>(p, (const V*)u, (const V*)w, nu, stride, ws.partial); } \
+    if (extra) { dots2_partial<T2, K, true><<<g1, 256, 0, s>>>(p, (const V*)u, (const V*)w, nu, stride, ws.partial, d); } \
+    else { dots2_partial<T2, K, false><<<g1, 256, 0, s>>>(p, (const V*)u, (const V*)w, nu, stride, ws.partial, d); } \
     count_launches(1);                                                                                       \
     break;
     switch (kk) {
@@ -701,13 +741,11 @@ static int dcgs2_step_t(const BVec& b, const void* const* v, int j, void* u, voi
       default: return MG_ERR_ARG;
     }
 #undef SAPMG_D2
-    dots2_finalize<<<R, 256, 0, s>>>(ws.partial, ncta1, kk, extra, ws.A, ws.B, ws.X, ws.ld, j0); count_launches(1);
     j0 += kk;
   } while (j0 < j);
-  dcgs2_coeff_kernel<<<R, 32, 0, s>>>(j, ws.A, ws.B, ws.X, ws.ld, ws.c1, ws.c2, ws.ld, ws.hcol, ws.acol);
-  count_launches(1);
   // pass 2 over the list [u, w, v_0 .. v_{j-1}] in chunks of 16
   const dim3 g2(reduce_ctas(nu, R), R);
+  const DotOut dn{ws.nrm, nullptr, ws.ld, 0};
   const int total = j + 2;
   for (int q0 = 0; q0 < total; q0 += 16) {
     const int kk = std::min(16, total - q0);
@@ -721,7 +759,7 @@ static int dcgs2_step_t(const BVec& b, const void* const* v, int j, void* u, voi
     const int acc = q0 > 0;
 #define SAPMG_A2(K)                                                                                            \
   case K:                                                                                                      \
-    axpy2_kernel<T2, K><<<g2, 256, 0, s>>>(p, ws.c1, ws.c2, ws.ld, q0, (V*)u, (V*)w, nu, stride, acc, part); \
+    axpy2_kernel<T2, K><<<g2, 256, 0, s>>>(p, ws.c1, ws.c2, ws.ld, q0, (V*)u, (V*)w, nu, stride, acc, part, dn); \
     count_launches(1);                                                                                         \
     break;
     switch (kk) {
@@ -731,7 +769,6 @@ static int dcgs2_step_t(const BVec& b, const void* const* v, int j, void* u, voi
     }
 #undef SAPMG_A2
   }
-  multidot_finalize<<<R, 256, 0, s>>>(ws.partial, (int)g2.x, 2, ws.nrm, ws.ld, 0, nullptr); count_launches(1);
   SAPMG_CUDA_TRY(cudaGetLastError());
   return MG_OK;
 }
@@ -782,7 +819,7 @@ __device__ __forceinline__ uint2 f4_to_h4(float4 v) {
 template <int K, bool EXTRA>
 __global__ void __launch_bounds__(256) dots2h_partial(PtrsV<uint2> v, const float4* __restrict__ u,
                                                       const float4* __restrict__ w, size_t nu, size_t stride,
-                                                      double2* __restrict__ partial) {
+                                                      double2* __restrict__ partial, Dcgs2Out dout) {
   constexpr int NS = 2 * K + (EXTRA ? 3 : 0);
   const int r = blockIdx.y;
   const float4* ur = u + r * stride;
@@ -822,6 +859,7 @@ __global__ void __launch_bounds__(256) dots2h_partial(PtrsV<uint2> v, const floa
     for (int q = 0; q < 8; ++q) { a += red[q][2 * threadIdx.x]; b += red[q][2 * threadIdx.x + 1]; }
     partial[((size_t)r * gridDim.x + blockIdx.x) * kDots2Slots + threadIdx.x] = make_double2(a, b);
   }
+  finish_dots2<K, EXTRA>(partial, dout);
 }
 
 // pass 2 with an FP16 basis.  Coefficient q of c1/c2 belongs to [u, w, v_0, ...].
@@ -832,7 +870,7 @@ template <int K>
 __global__ void __launch_bounds__(256) axpy2h_kernel(PtrsV<uint2> v, const double2* __restrict__ c1,
                                                      const double2* __restrict__ c2, int ldc, int q0, float4* u,
                                                      float4* w, uint2* __restrict__ vout, size_t nu, size_t stride,
-                                                     int first, int keep_u, double2* __restrict__ partial) {
+                                                     int first, double2* __restrict__ partial, DotOut dout) {
   __shared__ float cf[4][18];
   const int r = blockIdx.y;
   if ((int)threadIdx.x < K + 2) {
@@ -872,7 +910,7 @@ __global__ void __launch_bounds__(256) axpy2h_kernel(PtrsV<uint2> v, const doubl
       caxpy(cf[0][2 + q], cf[1][2 + q], av, s1);
       caxpy(cf[2][2 + q], cf[3][2 + q], av, s2);
     }
-    if (!ov || keep_u) o1[i] = s1;
+    if (!ov) o1[i] = s1;
     o2[i] = s2;
     if (ov) ov[i] = f4_to_h4(s1);
     n1 += nrm_of(s1);
@@ -889,6 +927,7 @@ __global__ void __launch_bounds__(256) axpy2h_kernel(PtrsV<uint2> v, const doubl
       for (int q = 0; q < 8; ++q) sum += red[q][threadIdx.x];
       partial[((size_t)r * gridDim.x + blockIdx.x) * kChunk + threadIdx.x] = make_double2(sum, 0.0);
     }
+      finish_dots<2>(partial, dout);
   }
 }
 
@@ -905,7 +944,7 @@ int blas_dcgs2_step_h(const BVec& b, const void* const* vh, int j, void* u, void
   count_bytes(((double)2 * j * 4 + 5 * 8 + 4) * b.n * b.R);
   const size_t nu = b.n / 2, stride = b.vstride / 2;
   const int R = b.R;
-  const int ncta1 = std::max(1, std::min(reduce_ctas(nu, R), (int)(kPartialDouble2 / kDots2Slots / (size_t)R)));
+  const int ncta1 = reduce_ctas(nu, R, kDots2Slots);
   const dim3 g1(ncta1, R);
   const float4* uf = (const float4*)u;
   const float4* wf = (const float4*)w;
@@ -913,12 +952,13 @@ int blas_dcgs2_step_h(const BVec& b, const void* const* vh, int j, void* u, void
   do {
     const int kk = std::min(kDots2Max, j - j0);
     const bool extra = (j0 == 0);
+    const Dcgs2Out d{ws.A, ws.B, ws.X, ws.c1, ws.c2, ws.hcol, ws.acol, ws.ld, j0, j, j0 + kk >= j};
     PtrsV<uint2> p;
     for (int q = 0; q < 16; ++q) p.p[q] = j > 0 ? (const uint2*)vh[std::max(0, std::min(j0 + q, j - 1))] : (const uint2*)vout;
 #define SAPMG_D2H(K)                                                                                              \
   case K:                                                                                                         \
-    if (extra) { dots2h_partial<K, true><<<g1, 256, 0, s>>>(p, uf, wf, nu, stride, ws.partial); }                \
-    else { dots2h_partial<K, false><<<g1, 256, 0, s>>>(p, uf, wf, nu, stride, ws.partial); }                     \
+    if (extra) { dots2h_partial<K, true><<<g1, 256, 0, s>>>(p, uf, wf, nu, stride, ws.partial, d); }                \
+    else { dots2h_partial<K, false><<<g1, 256, 0, s>>>(p, uf, wf, nu, stride, ws.partial, d); }                     \
     count_launches(1);                                                                                            \
     break;
     switch (kk) {
@@ -927,12 +967,10 @@ int blas_dcgs2_step_h(const BVec& b, const void* const* vh, int j, void* u, void
       default: return MG_ERR_ARG;
     }
 #undef SAPMG_D2H
-    dots2_finalize<<<R, 256, 0, s>>>(ws.partial, ncta1, kk, extra, ws.A, ws.B, ws.X, ws.ld, j0); count_launches(1);
     j0 += kk;
   } while (j0 < j);
-  dcgs2_coeff_kernel<<<R, 32, 0, s>>>(j, ws.A, ws.B, ws.X, ws.ld, ws.c1, ws.c2, ws.ld, ws.hcol, ws.acol);
-  count_launches(1);
   const dim3 g2(reduce_ctas(nu, R), R);
+  const DotOut dn{ws.nrm, nullptr, ws.ld, 0};
   int q0 = 0;
   bool first = true;
   do {
@@ -945,7 +983,7 @@ int blas_dcgs2_step_h(const BVec& b, const void* const* vh, int j, void* u, void
 #define SAPMG_A2H(K)                                                                                                \
   case K:                                                                                                           \
     axpy2h_kernel<K><<<g2, 256, 0, s>>>(p, ws.c1, ws.c2, ws.ld, q0, (float4*)u, (float4*)w, vo, nu, stride, first, \
-                                        0, part);                                                                   \
+                                        part, dn);                                                                  \
     count_launches(1);                                                                                              \
     break;
     switch (kk) {
@@ -958,82 +996,8 @@ int blas_dcgs2_step_h(const BVec& b, const void* const* vh, int j, void* u, void
     q0 += kk;
     first = false;
   } while (q0 < j);
-  multidot_finalize<<<R, 256, 0, s>>>(ws.partial, (int)g2.x, 2, ws.nrm, ws.ld, 0, nullptr); count_launches(1);
   SAPMG_CUDA_TRY(cudaGetLastError());
   return MG_OK;
-}
-
-// The coarse-level GMRES with an FP16 basis (same format): <v_j, w> for a list
-// of FP16 vectors, w += sign sum c_j v_j (FP32 w, optional norm), and
-// out = x / ||x|| written in FP16.
-template <int K>
-__global__ void __launch_bounds__(256) multidot_h_partial(PtrsV<uint2> v, const float4* __restrict__ w, size_t nu,
-                                                          size_t stride, double2* __restrict__ partial) {
-  const int r = blockIdx.y;
-  const float4* wr = w + r * stride;
-  float re[K], im[K];
-#pragma unroll
-  for (int q = 0; q < K; ++q) re[q] = im[q] = 0.f;
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < nu; i += (size_t)gridDim.x * blockDim.x) {
-    uint2 a[K];
-#pragma unroll
-    for (int q = 0; q < K; ++q) a[q] = __ldg(v.p[q] + r * stride + i);
-    const float4 x = __ldg(wr + i);
-#pragma unroll
-    for (int q = 0; q < K; ++q) cdot_acc(h4_to_f4(a[q]), x, re[q], im[q]);
-  }
-  __shared__ double red[8][2 * K];
-  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-#pragma unroll
-  for (int q = 0; q < K; ++q) {
-    const float a = warp_sum(re[q]);
-    const float b = warp_sum(im[q]);
-    if (lane == 0) { red[wid][2 * q] = (double)a; red[wid][2 * q + 1] = (double)b; }
-  }
-  __syncthreads();
-  if ((int)threadIdx.x < K) {
-    double a = 0, b = 0;
-    for (int q = 0; q < 8; ++q) { a += red[q][2 * threadIdx.x]; b += red[q][2 * threadIdx.x + 1]; }
-    partial[((size_t)r * gridDim.x + blockIdx.x) * kChunk + threadIdx.x] = make_double2(a, b);
-  }
-}
-
-template <int K>
-__global__ void __launch_bounds__(256) multiaxpy_h_kernel(float4* __restrict__ w, PtrsV<uint2> v,
-                                                          const double2* __restrict__ coeff, int ldc, double sign,
-                                                          size_t nu, size_t stride, double2* __restrict__ partial) {
-  __shared__ float cf[2][16];
-  const int r = blockIdx.y;
-  if ((int)threadIdx.x < K) {
-    const double2 c = coeff[(size_t)r * ldc + threadIdx.x];
-    cf[0][threadIdx.x] = (float)(sign * c.x);
-    cf[1][threadIdx.x] = (float)(sign * c.y);
-  }
-  __syncthreads();
-  float4* wr = w + r * stride;
-  float nn = 0.f;
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < nu; i += (size_t)gridDim.x * blockDim.x) {
-    uint2 a[K];
-#pragma unroll
-    for (int q = 0; q < K; ++q) a[q] = __ldg(v.p[q] + r * stride + i);
-    float4 x = wr[i];
-#pragma unroll
-    for (int q = 0; q < K; ++q) caxpy(cf[0][q], cf[1][q], h4_to_f4(a[q]), x);
-    wr[i] = x;
-    nn += nrm_of(x);
-  }
-  if (partial) {
-    __shared__ double red[8];
-    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const float t = warp_sum(nn);
-    if (lane == 0) red[wid] = (double)t;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double sum = 0;
-      for (int q = 0; q < 8; ++q) sum += red[q];
-      partial[((size_t)r * gridDim.x + blockIdx.x) * kChunk] = make_double2(sum, 0.0);
-    }
-  }
 }
 
 __global__ void normalize_h_kernel(const float4* __restrict__ x, uint2* __restrict__ out,
@@ -1055,66 +1019,6 @@ __global__ void normalize_h_kernel(const float4* __restrict__ x, uint2* __restri
   }
 }
 
-static bool half_ok(const BVec& b, const void* w, const void* const* v, int k) {
-  bool al = (b.n % 2 == 0) && (b.vstride == b.n) && ((reinterpret_cast<uintptr_t>(w) & 15) == 0);
-  for (int q = 0; q < k; ++q) al = al && ((reinterpret_cast<uintptr_t>(v[q]) & 7) == 0);
-  return al;
-}
-
-int blas_multidot_h(const BVec& b, const void* const* v, int k, const void* w, double2* out, int ldo,
-                    double2* partial, cudaStream_t s) {
-  if (k <= 0 || b.R <= 0) return MG_OK;
-  if (!half_ok(b, w, v, k)) return MG_ERR_ARG;
-  count_bytes(((double)k * 4 + 8) * b.n * b.R);
-  const size_t nu = b.n / 2, stride = b.vstride / 2;
-  const int ncta = reduce_ctas(nu, b.R);
-  const dim3 grid(ncta, b.R);
-  for (int j0 = 0; j0 < k; j0 += kChunk) {
-    const int kk = std::min(kChunk, k - j0);
-    PtrsV<uint2> p;
-    for (int q = 0; q < 16; ++q) p.p[q] = (const uint2*)v[j0 + std::min(q, kk - 1)];
-#define SAPMG_MDH(K) case K: multidot_h_partial<K><<<grid, 256, 0, s>>>(p, (const float4*)w, nu, stride, partial); count_launches(1); break;
-    switch (kk) {
-      SAPMG_MDH(1) SAPMG_MDH(2) SAPMG_MDH(3) SAPMG_MDH(4) SAPMG_MDH(5) SAPMG_MDH(6) SAPMG_MDH(7) SAPMG_MDH(8)
-      SAPMG_MDH(9) SAPMG_MDH(10) SAPMG_MDH(11) SAPMG_MDH(12) SAPMG_MDH(13) SAPMG_MDH(14) SAPMG_MDH(15)
-      default: multidot_h_partial<16><<<grid, 256, 0, s>>>(p, (const float4*)w, nu, stride, partial); count_launches(1); break;
-    }
-#undef SAPMG_MDH
-    multidot_finalize<<<b.R, 256, 0, s>>>(partial, ncta, kk, out + j0, ldo, 0, nullptr); count_launches(1);
-  }
-  SAPMG_CUDA_TRY(cudaGetLastError());
-  return MG_OK;
-}
-
-int blas_multiaxpy_h(const BVec& b, void* w, const void* const* v, int k, const double2* coeff, int ldc, double sign,
-                     double2* nrm2, int ldn, double2* partial, cudaStream_t s) {
-  if (k <= 0 || b.R <= 0) return MG_OK;
-  if (!half_ok(b, w, v, k)) return MG_ERR_ARG;
-  count_bytes(((double)k * 4 + 16) * b.n * b.R);
-  const size_t nu = b.n / 2, stride = b.vstride / 2;
-  const dim3 g = nrm2 ? dim3(reduce_ctas(nu, b.R), b.R) : stream_grid(nu, b.R);
-  for (int j0 = 0; j0 < k; j0 += kChunk) {
-    const int kk = std::min(kChunk, k - j0);
-    const bool last = j0 + kChunk >= k;
-    PtrsV<uint2> p;
-    for (int q = 0; q < 16; ++q) p.p[q] = (const uint2*)v[j0 + std::min(q, kk - 1)];
-    double2* part = (last && nrm2) ? partial : nullptr;
-    const double2* c = coeff + j0;
-#define SAPMG_MAH(K) case K: multiaxpy_h_kernel<K><<<g, 256, 0, s>>>((float4*)w, p, c, ldc, sign, nu, stride, part); count_launches(1); break;
-    switch (kk) {
-      SAPMG_MAH(1) SAPMG_MAH(2) SAPMG_MAH(3) SAPMG_MAH(4) SAPMG_MAH(5) SAPMG_MAH(6) SAPMG_MAH(7) SAPMG_MAH(8)
-      SAPMG_MAH(9) SAPMG_MAH(10) SAPMG_MAH(11) SAPMG_MAH(12) SAPMG_MAH(13) SAPMG_MAH(14) SAPMG_MAH(15)
-      default: multiaxpy_h_kernel<16><<<g, 256, 0, s>>>((float4*)w, p, c, ldc, sign, nu, stride, part); count_launches(1); break;
-    }
-#undef SAPMG_MAH
-  }
-  if (nrm2) {
-    multidot_finalize<<<b.R, 256, 0, s>>>(partial, (int)g.x, 1, nrm2, ldn, 0, nullptr); count_launches(1);
-  }
-  SAPMG_CUDA_TRY(cudaGetLastError());
-  return MG_OK;
-}
-
 int blas_normalize_h(const BVec& b, const void* x, void* out, const double2* nrm2, int ldn, double2* store, int lds,
                      cudaStream_t s) {
   if (b.n % 2 != 0 || b.wstride != b.n) return MG_ERR_ARG;
@@ -1127,11 +1031,351 @@ int blas_normalize_h(const BVec& b, const void* x, void* out, const double2* nrm
   return MG_OK;
 }
 
+// ------------------------------------------------------------ one Arnoldi step of the coarse levels
+// Two kernels a step of fixed-step (flexible) GMRES, w = A v_j given:
+//   dots    <v_i, w> (i <= j) and <w, w> in one pass; the last CTA of a
+//           right-hand side turns them into column j of H, the update's
+//           coefficients and beta^2 = <w, w> - sum |<v_i, w>|^2 / |v_i|^2;
+//   update  x = w - sum (<v_i, w> / |v_i|^2) v_i, v_{j+1} = x / beta, and ||x||
+//           itself, which is H_{j+1,j}.
+// beta (formed before x exists) only has to be near ||x||: v_{j+1} has the norm
+// s_{j+1} = ||x|| / beta, which is kept, and H and y are those of the unit
+// vectors v_i / s_i, so a beta that cancellation has made inexact costs no
+// accuracy; a floor under it (kFloor <w, w>) bounds s_{j+1}.  Against a norm pass
+// before a separate normalisation this reads and writes w once less and takes
+// two launches a step instead of five.  Bound by L2/HBM bandwidth for 12 right-hand
+// sides, by latency for one.
+struct HalfBasis {          // FP16 basis scaled by kBasisScale, FP32 w
+  typedef uint2 V;
+  typedef float4 W;
+  typedef float R;
+  static constexpr int C = 2, CH = 32;
+  // 2^10 |v_{j+1}| has to stay below 65504 where the basis has lost its
+  // orthogonality and beta^2 comes out too small: beta >= ||w|| / 8
+  static constexpr double kFloor = 1.0 / 64;
+  static __device__ __forceinline__ W get(V a) { return h4_to_f4(a); }
+  static __device__ __forceinline__ V put(W x, R f) { return f4_to_h4(make_float4(x.x * f, x.y * f, x.z * f, x.w * f)); }
+};
+struct SingleBasis {
+  typedef float4 V;
+  typedef float4 W;
+  typedef float R;
+  static constexpr int C = 2, CH = 32;
+  static constexpr double kFloor = 1e-6;
+  static __device__ __forceinline__ W get(V a) { return a; }
+  static __device__ __forceinline__ V put(W x, R f) { return make_float4(x.x * f, x.y * f, x.z * f, x.w * f); }
+};
+struct DoubleBasis {
+  typedef double2 V;
+  typedef double2 W;
+  typedef double R;
+  static constexpr int C = 1, CH = 16;
+  static constexpr double kFloor = 1e-14;
+  static __device__ __forceinline__ W get(V a) { return a; }
+  static __device__ __forceinline__ V put(W x, R f) { return make_double2(x.x * f, x.y * f); }
+};
+template <class V> struct PtrsK { const V* p[32]; };
+
+// Scalars of a step (per right-hand side, stride ldr): H (33 x 33 column-major);
+// t[0..32] raw dots of earlier chunks, then the coefficients; t[40] = (1/beta, beta);
+// t[64 + i].x = s_i for i >= 1.
+struct ArnoldiOut {
+  double2 *H, *t;
+  int ldr, j, i0, last;    // the step, the chunk's first vector, the chunk that ends the pass
+};
+__device__ __forceinline__ double inv_scale(const double2* t, int i) {
+  if (i == 0) return 1.0;
+  const double s = t[64 + i].x;
+  return s > 0.0 ? 1.0 / s : 0.0;
+}
+
+// v[0..N) summed over the warp, N a power of two up to 32: halving the values a
+// lane holds with every exchange, N - 1 + (5 - log2 N) shuffles instead of 5 N.
+// Lane l gets value l / (32 / N).
+template <int N, class R>
+__device__ __forceinline__ R warp_sums(R (&v)[N]) {
+  const int lane = threadIdx.x & 31;
+  int mask = 16;
+#pragma unroll
+  for (int n = N / 2; n >= 1; n /= 2, mask /= 2) {
+    const bool up = (lane & mask) != 0;
+#pragma unroll
+    for (int i = 0; i < n; ++i) {
+      const R send = up ? v[i] : v[i + n];
+      const R keep = up ? v[i + n] : v[i];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, mask);
+    }
+  }
+  for (; mask >= 1; mask /= 2) v[0] += __shfl_xor_sync(0xffffffffu, v[0], mask);
+  return v[0];
+}
+
+template <class B, int KM>
+__global__ void __launch_bounds__(256) arnoldi_dots_kernel(PtrsK<typename B::V> v, int k,
+                                                           const typename B::W* __restrict__ w, size_t nu,
+                                                           size_t stride, double2* __restrict__ partial,
+                                                           ArnoldiOut o) {
+  typedef typename B::R R;
+  typedef typename B::V V;
+  const int r = blockIdx.y, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const typename B::W* wr = w + r * stride;
+  R acc[KM][2], ww = 0;
+#pragma unroll
+  for (int q = 0; q < KM; ++q) acc[q][0] = acc[q][1] = 0;
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < nu; i += (size_t)gridDim.x * blockDim.x) {
+    const typename B::W x = wr[i];
+#pragma unroll
+    for (int g = 0; g < KM; g += 8) {                    // up to eight loads in flight
+      constexpr int G = KM < 8 ? KM : 8;
+      V a[G];
+#pragma unroll
+      for (int q = 0; q < G; ++q)
+        if (g + q < k) a[q] = __ldg(v.p[g + q] + r * stride + i);
+#pragma unroll
+      for (int q = 0; q < G; ++q)
+        if (g + q < k) cdot_acc(B::get(a[q]), x, acc[g + q][0], acc[g + q][1]);
+    }
+    ww += nrm_of(x);
+  }
+  constexpr int NV = 2 * KM < 32 ? 2 * KM : 32, NG = 2 * KM / NV;
+  __shared__ double red[8][2 * KM + 1];
+#pragma unroll
+  for (int g = 0; g < NG; ++g) {
+    R u[NV];
+#pragma unroll
+    for (int q = 0; q < NV; ++q) u[q] = acc[(g * NV + q) >> 1][q & 1];
+    const R t = warp_sums<NV>(u);
+    if (lane % (32 / NV) == 0) red[wid][g * NV + lane / (32 / NV)] = (double)t;
+  }
+  ww = warp_sum(ww);
+  if (lane == 0) red[wid][2 * KM] = (double)ww;
+  __syncthreads();
+  double* part = reinterpret_cast<double*>(partial + ((size_t)r * gridDim.x + blockIdx.x) * (KM + 1));
+  if ((int)threadIdx.x <= 2 * KM) {
+    double t = 0;
+    for (int q = 0; q < 8; ++q) t += red[q][threadIdx.x];
+    part[threadIdx.x] = t;
+    if ((int)threadIdx.x == 2 * KM) part[2 * KM + 1] = 0.0;
+  }
+  if (!last_cta(partial, r)) return;
+  __shared__ double2 raw[KM + 1];
+  for (int q = wid; q <= KM; q += 8) {
+    if (q < k || q == KM) {
+      const double2 t = sum_slot(partial, r, KM + 1, q);
+      if (lane == 0) raw[q] = t;
+    }
+  }
+  __syncthreads();
+  if (wid > 0) return;
+  double2* t = o.t + (size_t)r * o.ldr;
+  if (!o.last) {
+    if (lane < k) t[o.i0 + lane] = raw[lane];
+    return;
+  }
+  // lane = basis vector i <= j
+  const bool on = lane <= o.j;
+  const double2 d = !on ? make_double2(0, 0) : (lane < o.i0 ? t[lane] : raw[lane - o.i0]);
+  const double is = on ? inv_scale(t, lane) : 0.0, isj = inv_scale(t, o.j);
+  double e = (d.x * d.x + d.y * d.y) * is * is;
+  e = warp_sum(e);
+  if (on) {
+    o.H[(size_t)r * o.ldr + lane + 33 * o.j] = make_double2(d.x * is * isj, d.y * is * isj);
+    t[lane] = make_double2(d.x * is * is, d.y * is * is);
+  }
+  if (lane == 0) {
+    const double n2 = raw[KM].x, b = sqrt(fmax(n2 - e, B::kFloor * n2));
+    t[40] = make_double2(b > 0.0 ? 1.0 / b : 0.0, b);
+  }
+}
+
+// x = w - sum t_i v_i over the chunk's vectors (written back to w unless the chunk
+// ends the pass); last: vnext = x / beta if vnext != nullptr, ||x|| and s_{j+1}.
+template <class B, int KM>
+__global__ void __launch_bounds__(256) arnoldi_update_kernel(PtrsK<typename B::V> v, int k, typename B::W* w,
+                                                             typename B::V* __restrict__ vnext, size_t nu,
+                                                             size_t stride, double2* __restrict__ partial,
+                                                             ArnoldiOut o) {
+  typedef typename B::R R;
+  typedef typename B::V V;
+  __shared__ R cf[2][KM];
+  __shared__ double red[8];
+  const int r = blockIdx.y, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  double2* t = o.t + (size_t)r * o.ldr;
+  if ((int)threadIdx.x < k) {
+    const double2 c = t[o.i0 + threadIdx.x];
+    cf[0][threadIdx.x] = (R)-c.x;
+    cf[1][threadIdx.x] = (R)-c.y;
+  }
+  const R invb = (R)t[40].x;
+  __syncthreads();
+  typename B::W* wr = w + r * stride;
+  R nn = 0;
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < nu; i += (size_t)gridDim.x * blockDim.x) {
+    typename B::W x = wr[i];
+#pragma unroll
+    for (int g = 0; g < KM; g += 8) {
+      constexpr int G = KM < 8 ? KM : 8;
+      V a[G];
+#pragma unroll
+      for (int q = 0; q < G; ++q)
+        if (g + q < k) a[q] = __ldg(v.p[g + q] + r * stride + i);
+#pragma unroll
+      for (int q = 0; q < G; ++q)
+        if (g + q < k) caxpy(cf[0][g + q], cf[1][g + q], B::get(a[q]), x);
+    }
+    if (!o.last) wr[i] = x;
+    else if (vnext) vnext[r * stride + i] = B::put(x, invb);
+    nn += nrm_of(x);
+  }
+  if (!o.last) return;
+  nn = warp_sum(nn);
+  if (lane == 0) red[wid] = (double)nn;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double sum = 0;
+    for (int q = 0; q < 8; ++q) sum += red[q];
+    partial[(size_t)r * gridDim.x + blockIdx.x] = make_double2(sum, 0.0);
+  }
+  if (!last_cta(partial, r)) return;
+  if (wid > 0) return;
+  const double2 sum = sum_slot(partial, r, 1, 0);
+  if (lane == 0) {
+    const double nrm = sqrt(fmax(sum.x, 0.0));
+    o.H[(size_t)r * o.ldr + o.j + 1 + 33 * o.j] = make_double2(nrm * inv_scale(t, o.j), 0.0);
+    t[64 + o.j + 1] = make_double2(nrm * (double)invb, 0.0);
+  }
+}
+
+// out = sum y_i v_i (acc: added to what out holds)
+template <class B, int KM>
+__global__ void __launch_bounds__(256) combine_kernel(PtrsK<typename B::V> v, int k, const double2* __restrict__ y,
+                                                      int ldy, typename B::W* __restrict__ out, size_t nu,
+                                                      size_t stride, int acc) {
+  typedef typename B::R R;
+  typedef typename B::V V;
+  __shared__ R cf[2][KM];
+  const int r = blockIdx.y;
+  if ((int)threadIdx.x < k) {
+    const double2 c = y[(size_t)r * ldy + threadIdx.x];
+    cf[0][threadIdx.x] = (R)c.x;
+    cf[1][threadIdx.x] = (R)c.y;
+  }
+  __syncthreads();
+  typename B::W* o = out + r * stride;
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < nu; i += (size_t)gridDim.x * blockDim.x) {
+    typename B::W x = acc ? o[i] : vzero<typename B::W>();
+#pragma unroll
+    for (int g = 0; g < KM; g += 8) {
+      constexpr int G = KM < 8 ? KM : 8;
+      V a[G];
+#pragma unroll
+      for (int q = 0; q < G; ++q)
+        if (g + q < k) a[q] = __ldg(v.p[g + q] + r * stride + i);
+#pragma unroll
+      for (int q = 0; q < G; ++q)
+        if (g + q < k) caxpy(cf[0][g + q], cf[1][g + q], B::get(a[q]), x);
+    }
+    o[i] = x;
+  }
+}
+
+// Vectors per kernel: the smallest of 4, 8, 16, 32 (FP64: 16, longer lists in
+// chunks of 16) that holds the list.
+#define SAPMG_KM(KERNEL, kk, ...)                                                                          \
+  if ((kk) <= 4) { KERNEL<B, 4><<<grid, 256, 0, s>>>(__VA_ARGS__); }                                       \
+  else if ((kk) <= 8) { KERNEL<B, 8><<<grid, 256, 0, s>>>(__VA_ARGS__); }                                  \
+  else if ((kk) <= 16) { KERNEL<B, 16><<<grid, 256, 0, s>>>(__VA_ARGS__); }                                \
+  else { KERNEL<B, B::CH><<<grid, 256, 0, s>>>(__VA_ARGS__); }                                             \
+  count_launches(1);
+
+template <class B>
+static PtrsK<typename B::V> ptrs_k(const void* const* v, int i0, int kk) {
+  PtrsK<typename B::V> p;
+  for (int q = 0; q < 32; ++q) p.p[q] = (const typename B::V*)v[i0 + std::min(q, kk - 1)];
+  return p;
+}
+
+template <class B>
+static int arnoldi_step_t(const BVec& b, const void* const* v, int j, void* w, void* vnext, const ArnoldiWork& a,
+                          cudaStream_t s) {
+  typedef typename B::V V;
+  typedef typename B::W W;
+  const size_t nu = b.n / B::C, stride = b.vstride / B::C;
+  for (int i0 = 0; i0 <= j; i0 += B::CH) {
+    const int kk = std::min(B::CH, j + 1 - i0);
+    const ArnoldiOut o{a.H, a.t, a.ldr, j, i0, i0 + kk > j};
+    const dim3 grid(reduce_ctas(nu, b.R, 33), b.R);
+    SAPMG_KM(arnoldi_dots_kernel, kk, ptrs_k<B>(v, i0, kk), kk, (const W*)w, nu, stride, a.partial, o)
+  }
+  for (int i0 = 0; i0 <= j; i0 += B::CH) {
+    const int kk = std::min(B::CH, j + 1 - i0);
+    const ArnoldiOut o{a.H, a.t, a.ldr, j, i0, i0 + kk > j};
+    const dim3 grid(reduce_ctas(nu, b.R), b.R);
+    SAPMG_KM(arnoldi_update_kernel, kk, ptrs_k<B>(v, i0, kk), kk, (W*)w, (V*)vnext, nu, stride, a.partial, o)
+  }
+  SAPMG_CUDA_TRY(cudaGetLastError());
+  return MG_OK;
+}
+
+template <class B>
+static int combine_t(const BVec& b, const void* const* v, int k, const double2* y, int ldy, void* out,
+                     cudaStream_t s) {
+  typedef typename B::W W;
+  const size_t nu = b.n / B::C, stride = b.vstride / B::C;
+  const dim3 grid = stream_grid(nu, b.R);
+  for (int i0 = 0; i0 < k; i0 += B::CH) {
+    const int kk = std::min(B::CH, k - i0);
+    SAPMG_KM(combine_kernel, kk, ptrs_k<B>(v, i0, kk), kk, y + i0, ldy, (W*)out, nu, stride, i0 > 0)
+  }
+  SAPMG_CUDA_TRY(cudaGetLastError());
+  return MG_OK;
+}
+#undef SAPMG_KM
+
+// FP32 units are pairs of complex numbers: an even length, 16-byte aligned
+// (FP16 basis vectors 8-byte aligned) and contiguous systems.
+static bool units_ok(int basis, const BVec& b, const void* const* v, int k, const void* w) {
+  if (b.vstride != b.n || b.wstride != b.n) return false;
+  if (basis == P64) return true;
+  bool al = b.n % 2 == 0 && (reinterpret_cast<uintptr_t>(w) & 15) == 0;
+  const uintptr_t m = basis == P16 ? 7 : 15;
+  for (int q = 0; q < k; ++q) al = al && (reinterpret_cast<uintptr_t>(v[q]) & m) == 0;
+  return al;
+}
+
+int blas_arnoldi_step(int basis, const BVec& b, const void* const* v, int j, void* w, void* vnext,
+                      const ArnoldiWork& a, cudaStream_t s) {
+  if (b.R <= 0) return MG_OK;
+  if (j < 0 || j > 31 || b.R > 32 || !units_ok(basis, b, v, j + 1, w)) return MG_ERR_ARG;
+  const double vb = basis == P64 ? 16 : (basis == P16 ? 4 : 8), wb = basis == P64 ? 16 : 8;
+  // both passes read the basis and w; v_{j+1} written
+  count_bytes((2.0 * (j + 1) * vb + 2 * wb + (vnext ? vb : 0)) * b.n * b.R);
+  switch (basis) {
+    case P16: return arnoldi_step_t<HalfBasis>(b, v, j, w, vnext, a, s);
+    case P32: return arnoldi_step_t<SingleBasis>(b, v, j, w, vnext, a, s);
+    case P64: return arnoldi_step_t<DoubleBasis>(b, v, j, w, vnext, a, s);
+    default: return MG_ERR_ARG;
+  }
+}
+
+int blas_combine(int basis, const BVec& b, const void* const* v, int k, const double2* y, int ldy, void* out,
+                 cudaStream_t s) {
+  if (k <= 0 || b.R <= 0) return MG_OK;
+  if (b.R > 32 || !units_ok(basis, b, v, k, out)) return MG_ERR_ARG;
+  const double vb = basis == P64 ? 16 : (basis == P16 ? 4 : 8), wb = basis == P64 ? 16 : 8;
+  count_bytes((k * vb + wb) * b.n * b.R);
+  switch (basis) {
+    case P16: return combine_t<HalfBasis>(b, v, k, y, ldy, out, s);
+    case P32: return combine_t<SingleBasis>(b, v, k, y, ldy, out, s);
+    case P64: return combine_t<DoubleBasis>(b, v, k, y, ldy, out, s);
+    default: return MG_ERR_ARG;
+  }
+}
 
 int blas_hessenberg_solve(const double2* H, int ldh, int ldr, int m, const double2* beta2, double2* y, int ldy,
-                          int R, cudaStream_t s) {
+                          int R, cudaStream_t s, const double2* scale) {
   if (m > 32) return MG_ERR_ARG;
-  hessenberg_solve_kernel<<<R, 32, 0, s>>>(H, ldh, ldr, m, beta2, y, ldy); count_launches(1);
+  hessenberg_solve_kernel<<<R, 32, 0, s>>>(H, ldh, ldr, m, beta2, scale, y, ldy); count_launches(1);
   SAPMG_CUDA_TRY(cudaGetLastError());
   return MG_OK;
 }

@@ -4,10 +4,11 @@
 
 namespace sapmg {
 
-// Upper bound on the CTAs of one reduction over all right-hand sides; the
-// partial buffer holds kMaxReduceCta * 16 double2.
-constexpr int kMaxReduceCta = 4096;
-constexpr size_t kPartialDouble2 = (size_t)kMaxReduceCta * 16;
+// The buffer of a reduction's partial sums: kPartialSums double2 of sums, then
+// one arrival counter (unsigned) per right-hand side, zero between kernels
+// (whoever allocates the buffer clears it from kPartialSums on).
+constexpr size_t kPartialDouble2 = 65536;
+constexpr size_t kPartialSums = kPartialDouble2 - 256;
 
 // Geometry of a batched vector operation: R systems, n elements each; the
 // vector v_j of system r is at v_j + r*vstride, w of system r at w + r*wstride.
@@ -57,17 +58,28 @@ int blas_dcgs2_step(int type, const BVec& b, const void* const* v, int j, void* 
 // normalised.
 int blas_dcgs2_step_h(const BVec& b, const void* const* vh, int j, void* u, void* w, void* vout, const DcgsWork& ws,
                       cudaStream_t s);
-// Kernels on FP16 basis vectors (scaled by 2^10, as blas_dcgs2_step_h stores
-// them) with FP32 w / x: <v_j, w>; w += sign sum c_j v_j (and ||w_new||^2 when
-// nrm2 != nullptr); out = x / ||x|| stored in the FP16 format.
-int blas_multidot_h(const BVec& b, const void* const* v, int k, const void* w, double2* out, int ldo,
-                    double2* partial, cudaStream_t s);
-int blas_multiaxpy_h(const BVec& b, void* w, const void* const* v, int k, const double2* coeff, int ldc, double sign,
-                     double2* nrm2, int ldn, double2* partial, cudaStream_t s);
+// out = x / ||x|| stored as an FP16 basis vector (scaled by 2^10).
 int blas_normalize_h(const BVec& b, const void* x, void* out, const double2* nrm2, int ldn, double2* store, int lds,
                      cudaStream_t s);
-// y[r] = argmin || sqrt(beta2[r]) e1 - H_r y || for (m+1) x m Hessenberg H_r (column-major, ldh; H_r at H + r*ldr).
+// Scalars of fixed-step GMRES on a coarse level, per right-hand side at stride
+// ldr >= 33 * 33: H (column-major, leading dimension 33) and scratch t (33 * 33),
+// whose entries 64 + i hold the norms s_i of the basis vectors.
+struct ArnoldiWork {
+  double2 *H, *t;
+  int ldr;
+  double2* partial;
+};
+// Step j < 32 of the Arnoldi process on w = A v_j (contents undefined
+// afterwards): column j of H and, unless vnext is null, v_{j+1}, whose norm s_{j+1} is near 1.
+// basis: P16 (FP16 vectors as blas_normalize_h stores them, FP32 w), P32 or P64.
+int blas_arnoldi_step(int basis, const BVec& b, const void* const* v, int j, void* w, void* vnext,
+                      const ArnoldiWork& a, cudaStream_t s);
+// out[r] = sum_i y[r*ldy + i] v_i[r] (basis as above; out in the precision of w).
+int blas_combine(int basis, const BVec& b, const void* const* v, int k, const double2* y, int ldy, void* out,
+                 cudaStream_t s);
+// y[r] = argmin || sqrt(beta2[r]) e1 - H_r y || for (m+1) x m Hessenberg H_r (column-major, ldh; H_r at H + r*ldr);
+// scale: divide y_i by the norm scale[r*ldr + i] of basis vector i >= 1.
 int blas_hessenberg_solve(const double2* H, int ldh, int ldr, int m, const double2* beta2, double2* y, int ldy,
-                          int R, cudaStream_t s);
+                          int R, cudaStream_t s, const double2* scale = nullptr);
 
 }  // namespace sapmg

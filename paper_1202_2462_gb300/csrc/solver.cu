@@ -403,25 +403,25 @@ static int coarse_gmres(mg_ctx* c, CoarseLevel& L, int k, int R) {
   CBLAS(dot_to(c, vt, bv, L.b, L.b, L.beta2, 1));
   CBLAS(blas_normalize(vt, bv, L.b, Vj(0), L.beta2, 1, nullptr, 0, c->s));
   std::vector<const void*> vl;
+  const ArnoldiWork aw{L.H, L.tmp, 33 * 33, c->partial};
   for (int j = 0; j < k; ++j) {
     TRY(coarse_apply(c, L, Vj(j), L.w, R));
     vl.push_back(Vj(j));
-    double2* hcol = L.H + (size_t)j * 33;
-    CBLAS(blas_multidot(vt, bv, vl.data(), j + 1, L.w, hcol, 33 * 33, 0, nullptr, c->partial, c->s));
     if (c->coarse_reorth) {
+      double2* hcol = L.H + (size_t)j * 33;
+      CBLAS(blas_multidot(vt, bv, vl.data(), j + 1, L.w, hcol, 33 * 33, 0, nullptr, c->partial, c->s));
       CBLAS(blas_multiaxpy(vt, bv, L.w, vl.data(), j + 1, hcol, 33 * 33, -1.0, c->s));
       CBLAS(blas_multidot(vt, bv, vl.data(), j + 1, L.w, hcol, 33 * 33, 1, L.tmp, c->partial, c->s));
       CBLAS(blas_multiaxpy_norm(vt, bv, L.w, vl.data(), j + 1, L.tmp, 33 * 33, -1.0, L.tmp + 40, 33 * 33, c->partial,
                               c->s));
+      CBLAS(blas_normalize(vt, bv, L.w, Vj(j + 1), L.tmp + 40, 33 * 33, hcol + j + 1, 33 * 33, c->s));
     } else {
-      CBLAS(blas_multiaxpy_norm(vt, bv, L.w, vl.data(), j + 1, hcol, 33 * 33, -1.0, L.tmp + 40, 33 * 33, c->partial,
-                              c->s));
+      CBLAS(blas_arnoldi_step(vt, bv, vl.data(), j, L.w, j + 1 < k ? Vj(j + 1) : nullptr, aw, c->s));
     }
-    CBLAS(blas_normalize(vt, bv, L.w, Vj(j + 1), L.tmp + 40, 33 * 33, hcol + j + 1, 33 * 33, c->s));
   }
-  CBLAS(blas_hessenberg_solve(L.H, 33, 33 * 33, k, L.beta2, L.y, 33, R, c->s));
-  SAPMG_CUDA_TRY(cudaMemsetAsync(L.x, 0, (size_t)R * n * eb, c->s));
-  CBLAS(blas_multiaxpy(vt, bv, L.x, vl.data(), k, L.y, 33, 1.0, c->s));
+  CBLAS(blas_hessenberg_solve(L.H, 33, 33 * 33, k, L.beta2, L.y, 33, R, c->s,
+                              c->coarse_reorth ? nullptr : L.tmp + 64));
+  CBLAS(blas_combine(vt, bv, vl.data(), k, L.y, 33, L.x, c->s));
   return MG_OK;
 }
 
@@ -435,17 +435,14 @@ static int coarse_gmres_h(mg_ctx* c, CoarseLevel& L, int k, int R) {
   CBLAS(dot_to(c, P32, bv, L.b, L.b, L.beta2, 1));
   CBLAS(blas_normalize_h(bv, L.b, Vj(0), L.beta2, 1, nullptr, 0, c->s));
   std::vector<const void*> vl;
+  const ArnoldiWork aw{L.H, L.tmp, 33 * 33, c->partial};
   for (int j = 0; j < k; ++j) {
     TRY(coarse_apply(c, L, Vj(j), L.w, R, true));
     vl.push_back(Vj(j));
-    double2* hcol = L.H + (size_t)j * 33;
-    CBLAS(blas_multidot_h(bv, vl.data(), j + 1, L.w, hcol, 33 * 33, c->partial, c->s));
-    CBLAS(blas_multiaxpy_h(bv, L.w, vl.data(), j + 1, hcol, 33 * 33, -1.0, L.tmp + 40, 33 * 33, c->partial, c->s));
-    CBLAS(blas_normalize_h(bv, L.w, Vj(j + 1), L.tmp + 40, 33 * 33, hcol + j + 1, 33 * 33, c->s));
+    CBLAS(blas_arnoldi_step(P16, bv, vl.data(), j, L.w, j + 1 < k ? Vj(j + 1) : nullptr, aw, c->s));
   }
-  CBLAS(blas_hessenberg_solve(L.H, 33, 33 * 33, k, L.beta2, L.y, 33, R, c->s));
-  SAPMG_CUDA_TRY(cudaMemsetAsync(L.x, 0, (size_t)R * n * 8, c->s));
-  CBLAS(blas_multiaxpy_h(bv, L.x, vl.data(), k, L.y, 33, 1.0, nullptr, 0, c->partial, c->s));
+  CBLAS(blas_hessenberg_solve(L.H, 33, 33 * 33, k, L.beta2, L.y, 33, R, c->s, L.tmp + 64));
+  CBLAS(blas_combine(P16, bv, vl.data(), k, L.y, 33, L.x, c->s));
   return MG_OK;
 }
 
@@ -465,31 +462,31 @@ static int fgmres_fixed1(mg_ctx* c, int k, int R) {
   CBLAS(dot_to(c, vt, bv, L.b, L.b, c->f1beta2, 1));
   CBLAS(blas_normalize(vt, bv, L.b, Vj(0), c->f1beta2, 1, nullptr, 0, c->s));
   std::vector<const void*> vl, zl;
+  const ArnoldiWork aw{c->f1H, c->f1tmp, 33 * 33, c->partial};
   for (int j = 0; j < k; ++j) {
     TRY(cycle1(c, Vj(j), Zj(j), R));
     TRY(coarse_apply(c, L, Zj(j), c->f1w, R));
     vl.push_back(Vj(j));
     zl.push_back(Zj(j));
-    double2* hcol = c->f1H + (size_t)j * 33;
-    CBLAS(blas_multidot(vt, bv, vl.data(), j + 1, c->f1w, hcol, 33 * 33, 0, nullptr, c->partial, c->s));
     if (c->coarse_reorth) {
+      double2* hcol = c->f1H + (size_t)j * 33;
+      CBLAS(blas_multidot(vt, bv, vl.data(), j + 1, c->f1w, hcol, 33 * 33, 0, nullptr, c->partial, c->s));
       CBLAS(blas_multiaxpy(vt, bv, c->f1w, vl.data(), j + 1, hcol, 33 * 33, -1.0, c->s));
       CBLAS(blas_multidot(vt, bv, vl.data(), j + 1, c->f1w, hcol, 33 * 33, 1, c->f1tmp, c->partial, c->s));
       CBLAS(blas_multiaxpy_norm(vt, bv, c->f1w, vl.data(), j + 1, c->f1tmp, 33 * 33, -1.0, c->f1tmp + 40, 33 * 33,
                               c->partial, c->s));
+      CBLAS(blas_normalize(vt, bv, c->f1w, Vj(j + 1), c->f1tmp + 40, 33 * 33, hcol + j + 1, 33 * 33, c->s));
     } else {
-      CBLAS(blas_multiaxpy_norm(vt, bv, c->f1w, vl.data(), j + 1, hcol, 33 * 33, -1.0, c->f1tmp + 40, 33 * 33,
-                              c->partial, c->s));
+      CBLAS(blas_arnoldi_step(vt, bv, vl.data(), j, c->f1w, j + 1 < k ? Vj(j + 1) : nullptr, aw, c->s));
     }
-    CBLAS(blas_normalize(vt, bv, c->f1w, Vj(j + 1), c->f1tmp + 40, 33 * 33, hcol + j + 1, 33 * 33, c->s));
   }
-  CBLAS(blas_hessenberg_solve(c->f1H, 33, 33 * 33, k, c->f1beta2, c->f1y, 33, R, c->s));
-  SAPMG_CUDA_TRY(cudaMemsetAsync(L.x, 0, (size_t)R * n * eb, c->s));
-  CBLAS(blas_multiaxpy(vt, bv, L.x, zl.data(), k, c->f1y, 33, 1.0, c->s));
+  CBLAS(blas_hessenberg_solve(c->f1H, 33, 33 * 33, k, c->f1beta2, c->f1y, 33, R, c->s,
+                              c->coarse_reorth ? nullptr : c->f1tmp + 64));
+  CBLAS(blas_combine(vt, bv, zl.data(), k, c->f1y, 33, L.x, c->s));
   return MG_OK;
 }
 
-// The FP16-basis coarse GMRES as a CUDA graph: its ~4k+3 launches use fixed
+// The FP16-basis coarse GMRES as a CUDA graph: its ~3k+4 launches use fixed
 // buffers and no host synchronisation, so after one run with plain launches
 // (which also sets every kernel attribute) the sequence is captured once per
 // (level, R) on a stream of the context's own and replayed on the context's
@@ -1701,7 +1698,8 @@ static int do_setup(mg_ctx* c, const double* U) {
   const int R = p.nrhs_max;
   c->partial = (double2*)c->alloc(sizeof(double2) * kPartialDouble2);
   c->dev_err = (int*)c->alloc(2 * sizeof(int));
-  if (!c->dev_err) return fail(MG_ERR_OOM, "workspace");
+  if (!c->dev_err || !c->partial) return fail(MG_ERR_OOM, "workspace");
+  SAPMG_CUDA_TRY(cudaMemsetAsync(c->partial + kPartialSums, 0, sizeof(double2) * (kPartialDouble2 - kPartialSums), c->s));
   {
     const int init[2] = {0, kMaxSpins};
     SAPMG_CUDA_TRY(cudaMemcpyAsync(c->dev_err, init, sizeof(init), cudaMemcpyHostToDevice, c->s));

@@ -1,0 +1,69 @@
+"""The launch forms for few blocks (one-warp CTAs of D, a cluster of CTAs per
+Schwarz block, the coarse kernels of a short vector) against the forms that the
+same call takes for many: the same fields once alone and once in a batch that
+is large enough for the other form."""
+
+import numpy as np
+import pytest
+
+import synth
+from tests.gpu_util import torch_cuda, dev, host, rel
+
+pytestmark = pytest.mark.gpu
+
+DIMS = (8, 8, 8, 8)      # 16 blocks, 8 of a colour
+
+
+def _solver(prec, **kw):
+    torch = torch_cuda()
+    import paper_1202_2462_gb300 as G
+    u = dev(torch, synth.random_gauge_field(DIMS, 0.4, 301))
+    return torch, G, G.Solver(u, 1.0, -0.1, precision=prec, **kw)
+
+
+@pytest.mark.parametrize("prec,tol", [("fp64", 1e-13), ("fp32", 1e-3), ("fp16", 1e-3)])
+@pytest.mark.parametrize("iters", [1, 4, 5, 16, 17, 32])
+def test_coarse_gmres_minimises(prec, tol, iters):
+    """The fixed-step coarse solve against the least-squares minimiser over the
+    Krylov space, at the step counts where its kernels change size: the norms
+    of the two residuals, relative to the source's (the mixed form applies an
+    FP16 operator, entries rounded by up to 5e-4, so its residual under the FP64
+    operator is off by that much; 1e-13 is FP64 rounding times 256 terms).  The
+    longest runs go on after the Krylov space is exhausted."""
+    torch, G, s = _solver(prec, n_levels=2, n_vec=(8,), setup_iters=2, coarse_iters=iters, seed=3)
+    nb, n2 = 16, 16
+    m = torch.empty((nb, 9, n2, n2), dtype=torch.complex128, device="cuda")
+    G.mg_get_coarse_op(s.ctx, 1, m)
+    mh = host(m)
+    nbr = np.zeros((nb, 9), dtype=int)
+    for a in range(nb):
+        x = [(a >> q) & 1 for q in range(4)]
+        nbr[a, 0] = a
+        for mu in range(4):
+            nbr[a, 1 + 2 * mu] = nbr[a, 2 + 2 * mu] = a ^ (1 << mu)
+        assert sum(v << q for q, v in enumerate(x)) == a
+    dense = np.zeros((nb * n2, nb * n2), dtype=complex)
+    for a in range(nb):
+        for d in range(9):
+            dense[a * n2:(a + 1) * n2, nbr[a, d] * n2:(nbr[a, d] + 1) * n2] += mh[a, d]
+    rng = np.random.default_rng(5)
+    b = rng.normal(size=nb * n2) + 1j * rng.normal(size=nb * n2)
+    dt = torch.complex128 if prec == "fp64" else torch.complex64
+    bd = dev(torch, b, dt)
+    x = torch.empty_like(bd)
+    G.mg_coarse_solve(s.ctx, 1, bd, x, s.prec)
+    q = [b / np.linalg.norm(b)]
+    for _ in range(iters - 1):
+        w = dense @ q[-1]
+        for _ in range(2):
+            for v in q:
+                w = w - np.vdot(v, w) * v
+        q.append(w / np.linalg.norm(w))
+    aq = dense @ np.array(q).T
+    y = np.linalg.lstsq(aq, b, rcond=None)[0]
+    want = np.linalg.norm(b - aq @ y)
+    got = np.linalg.norm(b - dense @ host(x).reshape(-1))
+    assert abs(got - want) <= tol * np.linalg.norm(b)
+    G.mg_coarse_solve(s.ctx, 1, torch.zeros_like(bd), x, s.prec)
+    assert torch.count_nonzero(x) == 0
+    s.close()
