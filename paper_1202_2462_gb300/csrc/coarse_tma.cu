@@ -331,14 +331,20 @@ __device__ __forceinline__ uint32_t pack16(float2 v) {
   return *reinterpret_cast<const uint32_t*>(&h);
 }
 
-template <int RB, int N2, int ST, bool XH>
+// The depth st_n of the staging ring is a launch parameter.  With more sites
+// than resident CTAs two stages are the fastest (more CTAs an SM); with fewer,
+// the deepest ring that keeps every site resident (up to all nine blocks in
+// flight at once) shortens the serial chain of nine copies a site: 512 sites,
+// one right-hand side, 12.0 us with 2 stages.
+constexpr int kMaxRing = 9;
+template <int RB, int N2, bool XH>
 __global__ void __launch_bounds__(256) coarse_apply_mma16_kernel(const __half2* __restrict__ M,
                                                                  const void* __restrict__ xv,
                                                                  float2* __restrict__ out, CGeom c, int r0, int nr,
-                                                                 int* __restrict__ err) {
+                                                                 int st_n, int* __restrict__ err) {
   extern __shared__ __align__(128) unsigned char smem[];
   const int spins = wait_spins(err);
-  __shared__ __align__(8) uint64_t bar[ST];
+  __shared__ __align__(8) uint64_t bar[kMaxRing];
   const int n2 = N2 > 0 ? N2 : c.n2;                         // N2 > 0: block size fixed at compile time
   const int xst = n2 + 4;                                     // padded row stride (conflict-free fragment loads)
   const int tile = n2 * n2;
@@ -347,7 +353,8 @@ __global__ void __launch_bounds__(256) coarse_apply_mma16_kernel(const __half2* 
   // half2 and used as B fragments directly; otherwise FP32, packed per fragment
   constexpr int xb = XH ? 4 : 8;                              // bytes per staged complex entry
   const uint32_t row_bytes = (uint32_t)n2 * xb;
-  const size_t stage_bytes = tile_bytes + (size_t)16 * xst * xb;
+  constexpr int kRows = RB <= 8 ? 8 : 16;                     // vector rows staged (fragment columns in use)
+  const size_t stage_bytes = tile_bytes + (size_t)kRows * xst * xb;
   auto stage_tile = [&](int st) { return reinterpret_cast<const uint32_t*>(smem + st * stage_bytes); };
   auto stage_x = [&](int st) { return reinterpret_cast<float2*>(smem + st * stage_bytes + tile_bytes); };
   auto stage_xh = [&](int st) { return reinterpret_cast<uint32_t*>(smem + st * stage_bytes + tile_bytes); };
@@ -358,12 +365,12 @@ __global__ void __launch_bounds__(256) coarse_apply_mma16_kernel(const __half2* 
   const int nsite_cta = (c.nsites - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
   const int T = 9 * nsite_cta;
   if (T <= 0) return;
-  for (int st = 0; st < ST; ++st) {
+  for (int st = 0; st < st_n; ++st) {
     uint32_t* z = reinterpret_cast<uint32_t*>(smem + st * stage_bytes + tile_bytes + (size_t)nr * xst * xb);
-    for (int e = tid; e < (16 - nr) * xst * xb / 4; e += blockDim.x) z[e] = 0u;
+    for (int e = tid; e < (kRows - nr) * xst * xb / 4; e += blockDim.x) z[e] = 0u;
   }
   if (tid == 0) {
-    for (int st = 0; st < ST; ++st) mbar_init(&bar[st], 1);
+    for (int st = 0; st < st_n; ++st) mbar_init(&bar[st], 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
@@ -376,8 +383,7 @@ __global__ void __launch_bounds__(256) coarse_apply_mma16_kernel(const __half2* 
     const int xc = (site / stride) % c.L[mu];
     return site + (((xc + step + c.L[mu]) % c.L[mu]) - xc) * stride;
   };
-  auto issue = [&](int t) {
-    const int st = t % ST;
+  auto issue = [&](int t, int st) {
     const int site = MG_CLAMP(kCoarseSite, site_of(t), c.nsites), d = t % 9;
     uint64_t* b = &bar[st];
     mbar_expect_tx(b, tile_bytes + nr * row_bytes);
@@ -389,12 +395,13 @@ __global__ void __launch_bounds__(256) coarse_apply_mma16_kernel(const __half2* 
   };
   if (tid == 0) {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    for (int t = 0; t < ST - 1 && t < T; ++t) issue(t);
+    for (int t = 0; t < st_n - 1 && t < T; ++t) issue(t, t);
   }
   const int m0 = warp * 16;
   const int i0 = (m0 >> 1) + (g >> 1), a = g & 1;            // output rows i0 (fragment row g) and i0 + 4 (g + 8)
   float acc[2][4];
   int tfail = -1;
+  int st = 0, phase = 0;                                      // t % st_n, (t / st_n) & 1
   for (int t = 0; t < T; ++t) {
     const int d = t % 9;
     const int site = MG_CLAMP(kCoarseSite, site_of(t), c.nsites);
@@ -402,12 +409,11 @@ __global__ void __launch_bounds__(256) coarse_apply_mma16_kernel(const __half2* 
 #pragma unroll
       for (int q = 0; q < 2; ++q) acc[q][0] = acc[q][1] = acc[q][2] = acc[q][3] = 0.f;
     }
-    if (tid == 0 && t + ST - 1 < T) {
+    if (tid == 0 && t + st_n - 1 < T) {
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      issue(t + ST - 1);
+      issue(t + st_n - 1, st == 0 ? st_n - 1 : st - 1);
     }
-    const int st = t % ST;
-    const bool waited = mbar_wait(&bar[st], (uint32_t)((t / ST) & 1), spins);
+    const bool waited = mbar_wait(&bar[st], (uint32_t)phase, spins);
     if (__syncthreads_or(!waited)) {
       tfail = t;
       break;
@@ -447,46 +453,48 @@ __global__ void __launch_bounds__(256) coarse_apply_mma16_kernel(const __half2* 
       }
     }
     __syncthreads();
+    if (++st == st_n) { st = 0; phase ^= 1; }
   }
   if (tfail >= 0) {
     if (tid == 0) {
       atomicExch(err, 1);
-      // stages tfail .. tfail + ST - 1 were issued (the copy of t + ST - 1 goes out
-      // before the wait of t): let every one of them land
-      for (int u = tfail; u < T && u < tfail + ST; ++u) mbar_wait(&bar[u % ST], (uint32_t)((u / ST) & 1));
+      // blocks tfail .. tfail + st_n - 1 were issued (the copy of t + st_n - 1 goes
+      // out before the wait of t): let every one of them land
+      for (int u = tfail; u < T && u < tfail + st_n; ++u) mbar_wait(&bar[u % st_n], (uint32_t)((u / st_n) & 1));
     }
     __syncthreads();
   }
 }
 
-template <int RB, int N2, int ST, bool XH>
+template <int RB, int N2, bool XH>
 static void launch_mma16_t(const CGeom& c, const __half2* M, const void* x, float2* out, int r0, int nr, int* err,
-                           int ctas, cudaStream_t s) {
-  const size_t stage = (size_t)c.n2 * c.n2 * sizeof(__half2) + (size_t)16 * (c.n2 + 4) * (XH ? 4 : 8);
-  const size_t smem = ST * stage;
+                           const CoarseTune& t, cudaStream_t s) {
+  const size_t stage = (size_t)c.n2 * c.n2 * sizeof(__half2) + (size_t)(RB <= 8 ? 8 : 16) * (c.n2 + 4) * (XH ? 4 : 8);
   static bool attr = false;
   if (!attr) {
-    cudaFuncSetAttribute(coarse_apply_mma16_kernel<RB, N2, ST, XH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaFuncSetAttribute(coarse_apply_mma16_kernel<RB, N2, XH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          200 * 1024);
     attr = true;
   }
   const int threads = 32 * (c.n2 / 8);
-  int per_sm = (int)std::max<size_t>(1, std::min<size_t>(16, (220 * 1024) / (smem + 1024)));
-  if (ctas > 0) per_sm = std::min(per_sm, ctas);
-  const int grid = std::min(c.nsites, 152 * per_sm);
-  coarse_apply_mma16_kernel<RB, N2, ST, XH><<<grid, threads, smem, s>>>(M, x, out, c, r0, nr, err); count_launches(1);
+  auto per_sm = [&](int st) {
+    const int k = (int)std::max<size_t>(1, std::min<size_t>(16, (220 * 1024) / (st * stage + 1024)));
+    return t.ctas > 0 ? std::min(k, t.ctas) : k;
+  };
+  int st = c.n2 == 40 && t.stages == 3 ? 3 : 2;
+  for (int d = kMaxRing; d > st; --d)
+    if (d * stage <= 200 * 1024 && c.nsites <= 152 * per_sm(d)) { st = d; break; }
+  const int grid = std::min(c.nsites, 152 * per_sm(st));
+  coarse_apply_mma16_kernel<RB, N2, XH><<<grid, threads, st * stage, s>>>(M, x, out, c, r0, nr, st, err);
+  count_launches(1);
 }
 
-// Two stages (one block in flight while the previous is multiplied) keep the
-// shared memory per CTA small enough for eight CTAs per SM, which measured
-// faster than deeper rings with fewer CTAs; 2N = 40 has a specialised
-// instance with the k loop unrolled.
+// 2N = 40 has a specialised instance with the k loop unrolled.
 template <int RB, bool XH>
 static void launch_mma16(const CGeom& c, const __half2* M, const void* x, float2* out, int r0, int nr, int* err,
                          const CoarseTune& t, cudaStream_t s) {
-  if (c.n2 == 40 && t.stages == 3) launch_mma16_t<RB, 40, 3, XH>(c, M, x, out, r0, nr, err, t.ctas, s);
-  else if (c.n2 == 40) launch_mma16_t<RB, 40, 2, XH>(c, M, x, out, r0, nr, err, t.ctas, s);
-  else launch_mma16_t<RB, 0, 2, XH>(c, M, x, out, r0, nr, err, t.ctas, s);
+  if (c.n2 == 40) launch_mma16_t<RB, 40, XH>(c, M, x, out, r0, nr, err, t, s);
+  else launch_mma16_t<RB, 0, XH>(c, M, x, out, r0, nr, err, t, s);
 }
 
 template <int RB, class TM>
