@@ -72,6 +72,12 @@ int launch_coarse_apply_mma(const CGeom& c, int store, const void* M, const void
 // results with the same operator.
 int launch_coarse_sap_mrhs(const CGeom& c, const Box4& bx, const void* M, bool m16, void* z, const void* b,
                            int colour, int n_mr, int nrhs, cudaStream_t s);
+// The same pass from the FP16 operator copy on clusters of eight CTAs per box (any
+// nrhs), where the box and its operator rows fit (coarse_sap_cluster_ok: sites a
+// multiple of eight, 2N even; 16 sites up to 2N = 48); the same results bit for bit.
+bool coarse_sap_cluster_ok(const CGeom& c, const Box4& bx);
+int launch_coarse_sap_cluster(const CGeom& c, const Box4& bx, const void* M16, void* z, const void* b, int colour,
+                              int n_mr, int nrhs, int* err, cudaStream_t s);
 int launch_coarse_sap(int prec, const CGeom& c, const Box4& bx, const void* M, void* z, const void* b, int colour,
                       int n_mr, int nrhs, cudaStream_t s, bool m16 = false);
 int launch_transfer1(bool restrict_, int prec, const CGeom& c, const Box4& ag, const void* in, void* out,

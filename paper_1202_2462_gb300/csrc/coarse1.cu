@@ -6,6 +6,7 @@
 // level-2 aggregates are boxes of coarse sites (Box4).  Level-1 test vectors
 // are vector-major [k][site][n2]; the level-2 operator uses the stencil layout
 // M[site][d][j][i] of every coarse level.
+#include "async.cuh"
 #include "internal.h"
 #include "coarse.h"
 
@@ -150,7 +151,9 @@ __global__ void __launch_bounds__(1024) coarse_sap_kernel(const TM* __restrict__
         }
         const TM* m = M + (((size_t)site * 9 + d) * n2) * n2 + i;
         const Cplx<R>* rn = rs + ln * n2;
-        for (int j = 0; j < n2; ++j) cfma(p, Io<R, TM>::ld(m + (size_t)j * n2), rn[j]);
+        Cplx<R> t = cmk<R>(0, 0);                  // each direction summed on its own, as the cluster form does
+        for (int j = 0; j < n2; ++j) cfma(t, Io<R, TM>::ld(m + (size_t)j * n2), rn[j]);
+        p = p + t;
       }
       mr_dots(p, rs[tid], v);
     }
@@ -268,6 +271,9 @@ __global__ void __launch_bounds__(MAXT) coarse_sap_mrhs_kernel(const TM* __restr
         }
         const TM* m = M + (((size_t)site * 9 + d) * n2) * n2 + i;
         const float4* rn = reinterpret_cast<const float4*>(rs + (size_t)ln * n2 * NR);
+        float2 tre[NR / 2], tim[NR / 2];
+#pragma unroll
+        for (int q = 0; q < NR / 2; ++q) tre[q] = tim[q] = make_float2(0.f, 0.f);
         for (int j = 0; j < n2; ++j) {
           const Cplx<float> mv = Io<float, TM>::ld(m + (size_t)j * n2);
           const float2 mr = make_float2(mv.re, mv.re), mi = make_float2(mv.im, mv.im);
@@ -276,11 +282,16 @@ __global__ void __launch_bounds__(MAXT) coarse_sap_mrhs_kernel(const TM* __restr
           for (int q = 0; q < NR / 2; ++q) {
             const float4 x = rn[j * (NR / 2) + q];                // (re_r, im_r, re_r+1, im_r+1)
             const float2 xre = make_float2(x.x, x.z), xim = make_float2(x.y, x.w);
-            pre[q] = __ffma2_rn(mr, xre, pre[q]);
-            pre[q] = __ffma2_rn(nmi, xim, pre[q]);
-            pim[q] = __ffma2_rn(mr, xim, pim[q]);
-            pim[q] = __ffma2_rn(mi, xre, pim[q]);
+            tre[q] = __ffma2_rn(mr, xre, tre[q]);
+            tre[q] = __ffma2_rn(nmi, xim, tre[q]);
+            tim[q] = __ffma2_rn(mr, xim, tim[q]);
+            tim[q] = __ffma2_rn(mi, xre, tim[q]);
           }
+        }
+#pragma unroll
+        for (int q = 0; q < NR / 2; ++q) {
+          pre[q] = __fadd2_rn(pre[q], tre[q]);
+          pim[q] = __fadd2_rn(pim[q], tim[q]);
         }
       }
     }
@@ -369,6 +380,231 @@ int launch_coarse_sap_mrhs(const CGeom& c, const Box4& bx, const void* M, bool m
                            int colour, int n_mr, int nrhs, cudaStream_t s) {
   return m16 ? coarse_sap_mrhs_any<__half2>(c, bx, M, z, b, colour, n_mr, nrhs, s)
              : coarse_sap_mrhs_any<float2>(c, bx, M, z, b, colour, n_mr, nrhs, s);
+}
+
+// ------------------------------------------------------------ the colour pass on clusters (FP16 operator)
+// One box on a cluster of eight CTAs, each holding the operator rows of its
+// sites / 8 box sites in shared memory: copied there once (bulk copies, one
+// mbarrier), used by the residual and by every MR step of every right-hand
+// side.  The kernels above read a box's operator (0.9 MB for 16 sites, 2N = 40)
+// from L2 once per MR step through the one SM that holds the box, which bounds
+// them by that SM's L2 port: 130 us for one right-hand side on 16 boxes.
+// Here a product's (site, direction, row) terms are one thread each; the row
+// sums p (in direction order) go to all eight CTAs by distributed shared
+// memory, and every CTA then forms the box's scalar products and updates rho
+// itself, in the order of the kernels above, so that one cluster barrier per MR
+// step is the only exchange and the results are the same bit for bit.
+constexpr int kBoxCluster = 8;
+
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t cluster_addr(const void* p, int rank) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+  return a;
+}
+__device__ __forceinline__ void cluster_store(void* p, int rank, Cplx<float> v) {
+  asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(cluster_addr(p, rank)), "f"(v.re), "f"(v.im)
+               : "memory");
+}
+__device__ __forceinline__ void cluster_store(int* p, int rank, int v) {
+  asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(cluster_addr(p, rank)), "r"(v) : "memory");
+}
+
+// shared memory of the cluster form: operator rows, staged neighbour vectors,
+// direction terms, rho and p (two buffers each), reduction words
+static size_t box_cluster_smem(int sites, int n2) {
+  const size_t spc = (size_t)sites / kBoxCluster, elems = (size_t)sites * n2;
+  return spc * 9 * n2 * n2 * 4 + 2 * spc * 9 * n2 * 8 + 4 * elems * 8 + 32 * 16 + 64;
+}
+
+__global__ void __launch_bounds__(1024) coarse_sap_cluster_kernel(const __half2* __restrict__ M, float2* z,
+                                                                  const float2* __restrict__ b, CGeom c, Box4 bx,
+                                                                  int colour, int n_mr, int nrhs,
+                                                                  int* __restrict__ err) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  const int n2 = c.n2, bs = bx.sites, spc = bs / kBoxCluster, elems = bs * n2, rows = spc * n2;
+  const int rank = (int)cluster_rank();
+  const size_t mbytes = (size_t)9 * n2 * n2 * 4;                 // one site's operator rows
+  const uint32_t* Ms = reinterpret_cast<const uint32_t*>(smem_raw);
+  Cplx<float>* xs = reinterpret_cast<Cplx<float>*>(smem_raw + spc * mbytes);       // [spc * 9][n2]
+  Cplx<float>* ts = xs + spc * 9 * n2;                                             // [spc * 9][n2]
+  Cplx<float>* rho = ts + spc * 9 * n2;                                            // [2][elems]
+  Cplx<float>* pb = rho + 2 * elems;                                               // [2][elems]
+  float (*red)[4] = reinterpret_cast<float (*)[4]>(pb + 2 * elems);                // [32][4]
+  int* flag = reinterpret_cast<int*>(red + 32);                                    // [kBoxCluster]
+  uint64_t* bar = reinterpret_cast<uint64_t*>(flag + kBoxCluster);
+  int bc[4];
+  colour_box(bx, blockIdx.x / kBoxCluster, colour, bc);
+  const size_t fs = (size_t)c.nsites * n2;
+  const int tid = threadIdx.x, nt = blockDim.x;
+  const bool act = tid < elems;
+  const int s = act ? tid / n2 : 0, i = act ? tid % n2 : 0;      // this thread's element of the box
+  const bool own = act && s / spc == rank;
+  int lc[4];
+  const int site = box_site(c, bx, bc, s, lc);
+  if (tid == 0) {
+    mbar_init(bar, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    mbar_expect_tx(bar, (uint32_t)(spc * mbytes));
+    for (int k = 0; k < spc; ++k) {
+      int l2[4];
+      const int st = box_site(c, bx, bc, rank * spc + k, l2);
+      bulk_copy_g2s(smem_raw + k * mbytes, M + (size_t)st * 9 * n2 * n2, (uint32_t)mbytes, bar);
+    }
+  }
+  const int spins = wait_spins(err);
+  cluster_barrier();                                             // every CTA of the cluster runs, the barrier is set up
+  const bool waited = mbar_wait(bar, 0, spins);
+  const int failed = __syncthreads_or(!waited);
+  if (tid < kBoxCluster) cluster_store(flag + rank, tid, failed);
+  int pbuf = 0;
+  for (int r = 0; r < nrhs; ++r) {
+    float2* zr = z + r * fs;
+    const float2* br = b + r * fs;
+    Cplx<float>* rs = rho + (r & 1) * elems;
+    if (!failed) {
+      // residual: the nine terms of every own row, then b minus them in direction order
+      for (int e = tid; e < spc * 9 * n2; e += nt) {
+        const int j = e % n2, q = e / n2, k = q / 9, d = q % 9;
+        int l2[4];
+        const int st = box_site(c, bx, bc, rank * spc + k, l2);
+        xs[e] = Io<float, float2>::ldc(zr + (size_t)stencil_nb(c, st, d) * n2 + j);
+      }
+      __syncthreads();
+      for (int e = tid; e < spc * 9 * n2; e += nt) {
+        const int q = e / n2, row = e % n2;
+        const uint32_t* m = Ms + (size_t)q * n2 * n2 + row;
+        const Cplx<float>* x = xs + q * n2;
+        Cplx<float> t = cmk(0.f, 0.f);
+#pragma unroll 8
+        for (int j = 0; j < n2; ++j) {
+          const float2 v = half2_bits_to_float2(m[(size_t)j * n2]);
+          cfma(t, cmk(v.x, v.y), x[j]);
+        }
+        ts[e] = t;
+      }
+      __syncthreads();
+      for (int e = tid; e < rows; e += nt) {
+        const int k = e / n2, row = e % n2;
+        int l2[4];
+        const int st = box_site(c, bx, bc, rank * spc + k, l2);
+        Cplx<float> acc = Io<float, float2>::ldc(br + (size_t)st * n2 + row);
+        for (int d = 0; d < 9; ++d) acc = acc - ts[(k * 9 + d) * n2 + row];
+#pragma unroll
+        for (int q = 0; q < kBoxCluster; ++q) cluster_store(rs + rank * rows + e, q, acc);
+      }
+    }
+    cluster_barrier();                                           // rho of the box complete in every CTA
+    if (r == 0) {
+      int any = 0;
+      for (int q = 0; q < kBoxCluster; ++q) any |= flag[q];
+      if (any) {                                                 // the same decision in all eight CTAs
+        if (tid == 0) {
+          if (failed) atomicExch(err, 1);
+          mbar_wait(bar, 0);                                     // let the copies in flight land
+        }
+        __syncthreads();
+        return;
+      }
+    }
+    Cplx<float> e_own = cmk(0.f, 0.f);
+    for (int it = 0; it < n_mr; ++it) {
+      Cplx<float>* pc = pb + pbuf * elems;
+      pbuf ^= 1;
+      for (int e = tid; e < spc * 9 * n2; e += nt) {
+        const int q = e / n2, row = e % n2, k = q / 9, d = q % 9, ls = rank * spc + k;
+        int ln = ls;
+        if (d > 0) {
+          const int mu = (d - 1) >> 1, step = (d & 1) ? 1 : -1;
+          int stride = 1;
+          for (int m = 0; m < mu; ++m) stride *= bx.b[m];
+          const int l2 = (ls / stride) % bx.b[mu] + step;
+          if (l2 < 0 || l2 >= bx.b[mu]) continue;                // coupling leaves the box
+          ln = ls + step * stride;
+        }
+        const uint32_t* m = Ms + (size_t)q * n2 * n2 + row;
+        const Cplx<float>* x = rs + ln * n2;
+        Cplx<float> t = cmk(0.f, 0.f);
+#pragma unroll 8
+        for (int j = 0; j < n2; ++j) {
+          const float2 v = half2_bits_to_float2(m[(size_t)j * n2]);
+          cfma(t, cmk(v.x, v.y), x[j]);
+        }
+        ts[e] = t;
+      }
+      __syncthreads();
+      for (int e = tid; e < rows; e += nt) {
+        const int k = e / n2, row = e % n2, ls = rank * spc + k;
+        Cplx<float> p = cmk(0.f, 0.f);
+        int rest = ls;
+        p = p + ts[(k * 9) * n2 + row];
+        for (int mu = 0; mu < 4; ++mu) {
+          const int l = rest % bx.b[mu];
+          rest /= bx.b[mu];
+          if (l + 1 < bx.b[mu]) p = p + ts[(k * 9 + 1 + 2 * mu) * n2 + row];
+          if (l > 0) p = p + ts[(k * 9 + 2 + 2 * mu) * n2 + row];
+        }
+#pragma unroll
+        for (int q = 0; q < kBoxCluster; ++q) cluster_store(pc + rank * rows + e, q, p);
+      }
+      cluster_barrier();                                         // p of the box complete in every CTA
+      const Cplx<float> p = act ? pc[tid] : cmk(0.f, 0.f);
+      Cplx<float> ro = act ? rs[tid] : cmk(0.f, 0.f);
+      float v[3] = {0.f, 0.f, 0.f};
+      if (act) mr_dots(p, ro, v);
+      block_reduce_n(v, red);
+      Cplx<float> alpha = cmk(0.f, 0.f);
+      if (v[2] > 0.f) alpha = cmk(v[0] / v[2], v[1] / v[2]);
+      if (act) {
+        mr_update(alpha, p, e_own, ro);
+        rs[tid] = ro;
+      }
+      __syncthreads();                                           // rho updated; red reused by the next reduction
+    }
+    if (own) {
+      float2* zq = zr + (size_t)site * n2 + i;
+      Io<float, float2>::st(zq, Io<float, float2>::ldc(zq) + e_own);
+    }
+  }
+}
+
+bool coarse_sap_cluster_ok(const CGeom& c, const Box4& bx) {
+  return bx.sites % kBoxCluster == 0 && c.n2 % 2 == 0 && bx.sites * c.n2 <= 1024 &&
+         box_cluster_smem(bx.sites, c.n2) <= 227 * 1024;
+}
+
+int launch_coarse_sap_cluster(const CGeom& c, const Box4& bx, const void* M16, void* z, const void* b, int colour,
+                              int n_mr, int nrhs, int* err, cudaStream_t s) {
+  if (!coarse_sap_cluster_ok(c, bx)) return MG_ERR_ARG;
+  static bool attr = false;
+  if (!attr) {
+    SAPMG_CUDA_TRY(cudaFuncSetAttribute(coarse_sap_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        227 * 1024));
+    attr = true;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(bx.nboxes / 2 * kBoxCluster));
+  cfg.blockDim = dim3((unsigned)((bx.sites * c.n2 + 31) / 32 * 32));
+  cfg.dynamicSmemBytes = box_cluster_smem(bx.sites, c.n2);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = kBoxCluster;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  SAPMG_CUDA_TRY(cudaLaunchKernelEx(&cfg, coarse_sap_cluster_kernel, (const __half2*)M16, (float2*)z,
+                                    (const float2*)b, c, bx, colour, n_mr, nrhs, err));
+  count_launches(1);
+  return MG_OK;
 }
 
 int launch_coarse_sap(int prec, const CGeom& c, const Box4& bx, const void* M, void* z, const void* b, int colour,

@@ -540,21 +540,24 @@ static int coarse_solve(mg_ctx* c, int level, int R) {
 }
 
 // Schwarz sweeps on level 1 (boxes of coarse sites, red-black as on the fine level).
-// Mixed form: all right-hand sides in one CTA per box (each operator entry
-// loaded once for all of them), unless SAPMG_COARSE_SAP_MRHS=0, reading the
-// FP16 copy of the level-1 operator that the level-1 Krylov operator already
-// uses (the pass reads the box's operator once per MR step: half the bytes),
-// unless SAPMG_COARSE_SAP_FP16=0.
+// Mixed form: the FP16 copy of the level-1 operator that the level-1 Krylov
+// operator already uses, unless SAPMG_COARSE_SAP_FP16=0, held in the shared
+// memory of a cluster of CTAs per box where it fits; else all right-hand sides in
+// one CTA per box (each operator entry loaded once for all of them).
+// SAPMG_COARSE_SAP_MRHS=0: one right-hand side per CTA.
 static int smoother_sweeps1(mg_ctx* c, const void* b, void* z, int n_sweeps, int R) {
   const bool mrhs = c->coarse_sap_mrhs && c->c1.store == P32 && R >= 2 && R <= 12;
   const bool m16 = c->coarse_sap_fp16 && c->c1.store == P32 && c->c1.Mh != nullptr;
   const void* M = m16 ? c->c1.Mh : c->c1.M;
+  const bool cluster = m16 && c->coarse_sap_mrhs && coarse_sap_cluster_ok(c->c1.cg, c->sap1);
   for (int it = 0; it < n_sweeps; ++it)
     for (int col = 0; col < 2; ++col) {
       ProfScope ps(c->prof, FAM_SAP1, c->s);
       count_bytes((double)c->c1.cg.nsites / 2 * 9.0 * c->c1.cg.n2 * c->c1.cg.n2 *
-                  complex_bytes(m16 ? P16 : c->c1.store) * (mrhs ? 1.0 : R) * (c->p.n_mr + 1));
-      if (mrhs) TRY(launch_coarse_sap_mrhs(c->c1.cg, c->sap1, M, m16, z, b, col, c->p.n_mr, R, c->s));
+                  complex_bytes(m16 ? P16 : c->c1.store) *
+                  (cluster ? 1.0 : (mrhs ? 1.0 : R) * (c->p.n_mr + 1)));
+      if (cluster) TRY(launch_coarse_sap_cluster(c->c1.cg, c->sap1, M, z, b, col, c->p.n_mr, R, c->dev_err, c->s));
+      else if (mrhs) TRY(launch_coarse_sap_mrhs(c->c1.cg, c->sap1, M, m16, z, b, col, c->p.n_mr, R, c->s));
       else TRY(launch_coarse_sap(c->c1.store == P64 ? P64 : P32, c->c1.cg, c->sap1, M, z, b, col, c->p.n_mr, R, c->s,
                                  m16));
     }

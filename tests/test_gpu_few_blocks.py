@@ -21,6 +21,26 @@ def _solver(prec, **kw):
     return torch, G, G.Solver(u, 1.0, -0.1, precision=prec, **kw)
 
 
+@pytest.mark.parametrize("n_vec,nrhs", [(4, 1), (20, 1), (20, 3), (24, 12)])
+def test_level1_schwarz_cluster_matches_one_cta_per_box(n_vec, nrhs, monkeypatch):
+    """Level-1 boxes of 2^4 sites: the cluster form gives the one-CTA-per-box solve bit for bit."""
+    torch = torch_cuda()
+    import paper_1202_2462_gb300 as G
+    dims = (16, 16, 16, 16)
+    u = dev(torch, synth.random_gauge_field(dims, 0.4, 191))
+    b = dev(torch, synth.random_spinor(dims, 192, nvec=nrhs))
+    out = {}
+    for flag in ("0", "1"):
+        monkeypatch.setenv("SAPMG_COARSE_SAP_MRHS", flag)
+        s = G.Solver(u, 1.0, -0.1, n_levels=3, n_vec=(n_vec, 4), setup_iters=2, precision="bf16", nrhs_max=nrhs,
+                     seed=7, coarse_iters=8, fgmres_m=10, inner_iters=3)
+        z, info, code = s.solve(b)
+        s.close()
+        assert code == 0
+        out[flag] = (z, info.iterations)
+    assert torch.equal(out["0"][0], out["1"][0]) and out["0"][1] == out["1"][1]
+
+
 @pytest.mark.parametrize("prec,tol", [("fp64", 1e-13), ("fp32", 1e-3), ("fp16", 1e-3)])
 @pytest.mark.parametrize("iters", [1, 4, 5, 16, 17, 32])
 def test_coarse_gmres_minimises(prec, tol, iters):
