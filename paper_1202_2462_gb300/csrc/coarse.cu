@@ -795,6 +795,42 @@ __global__ void __launch_bounds__(256) coarse_apply_kernel(const TM* __restrict_
   for (int r = 0; r < RB; ++r) Io<R, TX>::st(out + (size_t)(r0 + r) * fs + t, acc[r]);
 }
 
+// The same for a lattice too small to give every SM a CTA of the kernel above: one
+// CTA per site, thread (direction, row) sums the n2 terms of its block's row and
+// the nine directions' sums are added in direction order.  Latency-bound: the
+// chain of 9 n2 terms a thread becomes one of n2 (16 sites, 2N = 16, FP64: 45 us
+// with the kernel above, whose 256 threads fill one CTA).
+template <class R, class TM, class TX, int RB>
+__global__ void __launch_bounds__(576) coarse_apply_site_kernel(const TM* __restrict__ M, const TX* __restrict__ x,
+                                                                TX* __restrict__ out, CGeom c, int r0) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  Cplx<R>* t = reinterpret_cast<Cplx<R>*>(smem_raw);            // [RB][9][n2]
+  const int n2 = c.n2, site = MG_CLAMP(kCoarseSite, blockIdx.x, c.nsites);
+  const int d = threadIdx.x / n2, i = threadIdx.x % n2;
+  const size_t fs = (size_t)c.nsites * n2;
+  const TX* xr = x + (size_t)r0 * fs;
+  Cplx<R> acc[RB];
+#pragma unroll
+  for (int r = 0; r < RB; ++r) acc[r] = cmk<R>(0, 0);
+  const TM* m = M + (((size_t)site * 9 + d) * n2) * n2 + i;
+  const TX* xn = xr + (size_t)cg_neighbour(c, site, d) * n2;
+#pragma unroll 8
+  for (int j = 0; j < n2; ++j) {
+    const Cplx<R> mv = Io<R, TM>::ld(m + (size_t)j * n2);
+#pragma unroll
+    for (int r = 0; r < RB; ++r) cfma(acc[r], mv, Io<R, TX>::ld(xn + r * fs + j));
+  }
+#pragma unroll
+  for (int r = 0; r < RB; ++r) t[r * 9 * n2 + threadIdx.x] = acc[r];
+  __syncthreads();
+  for (int e = threadIdx.x; e < RB * n2; e += blockDim.x) {
+    const int r = e / n2, row = e % n2;
+    Cplx<R> sum = t[r * 9 * n2 + row];
+    for (int q = 1; q < 9; ++q) sum = sum + t[(r * 9 + q) * n2 + row];
+    Io<R, TX>::st(out + (size_t)(r0 + r) * fs + (size_t)site * n2 + row, sum);
+  }
+}
+
 template <class R, class TM, class TX>
 static void coarse_apply_t(const CGeom& c, const void* M, const void* x, void* out, int nrhs, cudaStream_t s) {
   const long long n = (long long)c.nsites * c.n2;
@@ -804,6 +840,15 @@ static void coarse_apply_t(const CGeom& c, const void* M, const void* x, void* o
     const TM* m = (const TM*)M;
     const TX* xi = (const TX*)x;
     TX* o = (TX*)out;
+    if (grid < 152 && c.n2 <= 64) {
+      const int nt = 9 * c.n2, rb = left >= 2 ? 2 : 1;
+      const size_t smem = sizeof(Cplx<R>) * nt * rb;
+      if (rb == 2) coarse_apply_site_kernel<R, TM, TX, 2><<<(unsigned)c.nsites, nt, smem, s>>>(m, xi, o, c, r0);
+      else coarse_apply_site_kernel<R, TM, TX, 1><<<(unsigned)c.nsites, nt, smem, s>>>(m, xi, o, c, r0);
+      count_launches(1);
+      r0 += rb;
+      continue;
+    }
     if (left >= 12) { coarse_apply_kernel<R, TM, TX, 12><<<grid, 256, 0, s>>>(m, xi, o, c, r0); count_launches(1); r0 += 12; }
     else if (left >= 4) { coarse_apply_kernel<R, TM, TX, 4><<<grid, 256, 0, s>>>(m, xi, o, c, r0); count_launches(1); r0 += 4; }
     else if (left >= 2) { coarse_apply_kernel<R, TM, TX, 2><<<grid, 256, 0, s>>>(m, xi, o, c, r0); count_launches(1); r0 += 2; }

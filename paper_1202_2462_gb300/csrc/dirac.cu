@@ -14,16 +14,19 @@ namespace sapmg {
 // DAG: apply D^dagger = gamma5 D gamma5 instead (the operator of the normal
 // equations).  NORM: also write the CTA's share of ||out||^2 to
 // part[blockIdx.x] (CTA index = block * nrhs + right-hand side), reduced in a
-// fixed order so that the result does not depend on scheduling.
-template <class R, class TS, class TG, bool DAG, bool NORM>
-__global__ void __launch_bounds__(256, (sizeof(R) == 4 ? 3 : 1)) dirac_kernel(TS* __restrict__ out, const TS* __restrict__ in,
+// fixed order so that the result does not depend on scheduling.  TPB: sites per
+// CTA, 256 or (not with NORM) 32, eight CTAs to a block (see parts_of).
+template <class R, class TS, class TG, bool DAG, bool NORM, int TPB>
+__global__ void __launch_bounds__(TPB, TPB < 256 ? 1 : (sizeof(R) == 4 ? 3 : 1)) dirac_kernel(TS* __restrict__ out, const TS* __restrict__ in,
                                                     const TG* __restrict__ U, const TG* __restrict__ A, Geom g,
                                                     int nrhs, double* __restrict__ part) {
   // right-hand side fastest in the grid: the CTAs of one block run back to
   // back and share its links and clover through L2
-  const int blk = MG_CLAMP(kBlock, blockIdx.x / nrhs, g.nblocks);
-  const int loc = threadIdx.x;
-  const size_t off = (size_t)(blockIdx.x % nrhs) * g.V * 12;
+  constexpr int kParts = 256 / TPB;
+  const int id = blockIdx.x / kParts;
+  const int blk = MG_CLAMP(kBlock, id / nrhs, g.nblocks);
+  const int loc = threadIdx.x + TPB * (blockIdx.x % kParts);
+  const size_t off = (size_t)(id % nrhs) * g.V * 12;
   in += off;
   out += off;
   // acc = -2 A psi + sum of hops, so D psi = -acc / 2
@@ -58,11 +61,31 @@ __global__ void __launch_bounds__(256, (sizeof(R) == 4 ? 3 : 1)) dirac_kernel(TS
   }
 }
 
+// CTAs a block is cut into.  With few blocks a CTA per block leaves SMs idle:
+// the FP64 units of one SM take 58 us for a block's 1848 x 256 flops whatever the
+// number of warps, so 16 blocks (8^4) took 87 us on 16 SMs and CTAs of one warp
+// spread them over 128.  FP64 is cut up to eight blocks an SM, where the last
+// wave of whole blocks would still leave a tenth of the SMs' time unused; FP32,
+// which needs the warps of a block to hide latency, below one block an SM.
+template <class R>
+static int parts_of(const Geom& g, int nrhs) {
+  return (long long)g.nblocks * nrhs < 152 * (sizeof(R) == 8 ? 8 : 1) ? 8 : 1;
+}
+
 template <class R, class TS, class TG, bool DAG, bool NORM>
 static void run(const Geom& g, void* out, const void* in, const void* U, const void* A, int nrhs, double* part,
                 cudaStream_t s) {
-  dirac_kernel<R, TS, TG, DAG, NORM><<<(unsigned)(g.nblocks * nrhs), 256, 0, s>>>(
-      (TS*)out, (const TS*)in, (const TG*)U, (const TG*)A, g, nrhs, part);
+  const unsigned ctas = (unsigned)(g.nblocks * nrhs);
+  if constexpr (!NORM) {
+    if (parts_of<R>(g, nrhs) == 8) {
+      dirac_kernel<R, TS, TG, DAG, false, 32><<<ctas * 8, 32, 0, s>>>((TS*)out, (const TS*)in, (const TG*)U,
+                                                                      (const TG*)A, g, nrhs, nullptr);
+      count_launches(1);
+      return;
+    }
+  }
+  dirac_kernel<R, TS, TG, DAG, NORM, 256><<<ctas, 256, 0, s>>>((TS*)out, (const TS*)in, (const TG*)U, (const TG*)A, g,
+                                                               nrhs, part);
   count_launches(1);
 }
 

@@ -11,6 +11,7 @@
 // memory for the neighbour accesses of D_i, and so does the correction e; the
 // block-wide dots are warp shuffles plus one shared-memory exchange.  The two
 // colours are two launches in stream order.
+#include "async.cuh"
 #include "internal.h"
 #include "stencil.cuh"
 
@@ -148,9 +149,183 @@ __global__ void __launch_bounds__(256, (sizeof(R) == 4 ? 2 : 1))
   for (int c = 0; c < 12; ++c) Io<R, TS>::st(zq + c * 256, Io<R, TS>::ldc(zq + c * 256) + es[c * 256 + loc]);
 }
 
+// The same pass with a block on a cluster of eight one-warp CTAs (warp w of the
+// kernel above is CTA w), for few blocks: a block's MR steps then run on eight
+// SMs instead of one.  FP64 is bound by the SM's FP64 units (two FMAs a clock: 58
+// us for a block's MR step on one SM), so the 8 blocks of a colour of 8^4 took
+// 514 us a pass on 8 SMs.  rho stays in the shared memory of the CTA that owns
+// the site and its neighbours read it through distributed shared memory; the
+// block sums add the eight warps' parts in the order of the kernel above, so
+// the results are the same bit for bit.
+__device__ __forceinline__ void sap_cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t sap_cluster_addr(uint32_t addr, int rank) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(addr), "r"(rank));
+  return a;
+}
+__device__ __forceinline__ Cplx<double> ld_cluster(uint32_t a, double) {
+  Cplx<double> v;
+  asm volatile("ld.shared::cluster.v2.f64 {%0, %1}, [%2];" : "=d"(v.re), "=d"(v.im) : "r"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ Cplx<float> ld_cluster(uint32_t a, float) {
+  Cplx<float> v;
+  asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.re), "=f"(v.im) : "r"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_cluster(uint32_t a, double v) {
+  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
+}
+__device__ __forceinline__ void st_cluster(uint32_t a, float v) {
+  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
+}
+
+// Sum of the hops of D_i at loc, rho in the CTAs' shared memory (rs: its address, [12][32] per CTA)
+template <int MU, class R, class TG>
+__device__ __forceinline__ void cluster_hops_dir(const TG* __restrict__ U, uint32_t rs, int blk, int loc,
+                                                 Cplx<R> (&acc)[12]) {
+  const int ls = 1 << (2 * MU);
+  const int c = (loc >> (2 * MU)) & 3;
+  Cplx<R> h[6], gg[6], u[9];
+  auto at = [&](int l) { return sap_cluster_addr(rs + (uint32_t)((l & 31) * sizeof(Cplx<R>)), l >> 5); };
+  if (c < 3) {
+    const uint32_t q = at(loc + ls);
+    spin_project_ld<MU, -1, R>([&](int k) { return ld_cluster(q + (uint32_t)(k * 32 * sizeof(Cplx<R>)), R(0)); }, h);
+    load_link<R>(U, blk, MU, loc, u);
+    su3_mul(u, h, gg);
+    spin_reconstruct_add<MU, -1>(gg, acc);
+  }
+  if (c > 0) {
+    const uint32_t q = at(loc - ls);
+    spin_project_ld<MU, 1, R>([&](int k) { return ld_cluster(q + (uint32_t)(k * 32 * sizeof(Cplx<R>)), R(0)); }, h);
+    load_link<R>(U, blk, MU, loc - ls, u);
+    su3_dag_mul(u, h, gg);
+    spin_reconstruct_add<MU, 1>(gg, acc);
+  }
+}
+
+template <class R, class TS, class TG>
+__global__ void __launch_bounds__(32) sap_cluster_kernel(TS* __restrict__ z, const TS* __restrict__ b,
+                                                         const TG* __restrict__ U, const TG* __restrict__ A, Geom g,
+                                                         int colour, int n_mr, int nrhs) {
+  __shared__ __align__(16) unsigned char rs_raw[sizeof(Cplx<R>) * 12 * 32];
+  __shared__ R red[2][8][4];                             // two buffers: a step's sums are read while the next arrive
+  Cplx<R>* rs = reinterpret_cast<Cplx<R>*>(rs_raw);      // rho of the warp's sites [12][32]
+  const uint32_t rsa = smem_u32(rs);
+  const int rank = (int)(blockIdx.x & 7), lane = threadIdx.x, loc = rank * 32 + lane;
+  const int id = blockIdx.x >> 3;
+  const size_t off = (size_t)(id % nrhs) * g.V * 12;
+  z += off;
+  b += off;
+  const int blk = colour_block(g, id / nrhs, colour);
+  {
+    Cplx<R> acc[12];
+    {
+      Cplx<R> zz[12];
+      load_spinor<R>(z, blk, loc, zz);
+      clover_apply<R>(A, blk, loc, zz, acc);
+    }
+#pragma unroll
+    for (int c = 0; c < 12; ++c) acc[c] = (R)(-2) * acc[c];
+    hops_global_dir<0>(g, z, U, blk, loc, acc);
+    asm volatile("" ::: "memory");
+    hops_global_dir<1>(g, z, U, blk, loc, acc);
+    asm volatile("" ::: "memory");
+    hops_global_dir<2>(g, z, U, blk, loc, acc);
+    asm volatile("" ::: "memory");
+    hops_global_dir<3>(g, z, U, blk, loc, acc);
+    const TS* bq = b + (size_t)blk * 12 * 256 + loc;
+#pragma unroll
+    for (int c = 0; c < 12; ++c) rs[c * 32 + lane] = Io<R, TS>::ldc(bq + c * 256) + (R)0.5 * acc[c];
+  }
+  Cplx<R> e[12];
+#pragma unroll
+  for (int c = 0; c < 12; ++c) e[c] = cmk<R>(0, 0);
+  for (int it = 0; it < n_mr; ++it) {
+    sap_cluster_barrier();                               // rho of every site written
+    Cplx<R> p[12];
+    {
+      Cplx<R> ro[12];
+#pragma unroll
+      for (int c = 0; c < 12; ++c) ro[c] = rs[c * 32 + lane];
+      clover_apply<R>(A, blk, loc, ro, p);
+    }
+#pragma unroll
+    for (int c = 0; c < 12; ++c) p[c] = (R)(-2) * p[c];
+    cluster_hops_dir<0>(U, rsa, blk, loc, p);
+    asm volatile("" ::: "memory");
+    cluster_hops_dir<1>(U, rsa, blk, loc, p);
+    asm volatile("" ::: "memory");
+    cluster_hops_dir<2>(U, rsa, blk, loc, p);
+    asm volatile("" ::: "memory");
+    cluster_hops_dir<3>(U, rsa, blk, loc, p);
+    R v[3] = {0, 0, 0};
+#pragma unroll
+    for (int c = 0; c < 12; ++c) {
+      p[c] = (R)(-0.5) * p[c];
+      const Cplx<R> ro = rs[c * 32 + lane];
+      v[0] += p[c].re * ro.re + p[c].im * ro.im;
+      v[1] += p[c].re * ro.im - p[c].im * ro.re;
+      v[2] += p[c].re * p[c].re + p[c].im * p[c].im;
+    }
+#pragma unroll
+    for (int q = 0; q < 3; ++q) v[q] = warp_sum(v[q]);
+    if (lane < 8) {                                      // lane q: this warp's sums to CTA q
+      const uint32_t a = sap_cluster_addr(smem_u32(&red[it & 1][rank][0]), lane);
+#pragma unroll
+      for (int q = 0; q < 3; ++q) st_cluster(a + (uint32_t)(q * sizeof(R)), v[q]);
+    }
+    sap_cluster_barrier();                               // the sums arrived; every neighbour read of rho done
+    R pr_re = 0, pr_im = 0, pp = 0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) { pr_re += red[it & 1][k][0]; pr_im += red[it & 1][k][1]; pp += red[it & 1][k][2]; }
+    Cplx<R> alpha = cmk<R>(0, 0);
+    if (pp > (R)0) alpha = cmk(pr_re / pp, pr_im / pp);
+#pragma unroll
+    for (int c = 0; c < 12; ++c) {
+      const Cplx<R> ro = rs[c * 32 + lane];
+      e[c] = e[c] + alpha * ro;
+      rs[c * 32 + lane] = ro - alpha * p[c];
+    }
+  }
+  sap_cluster_barrier();                                 // the residuals' reads of z (n_mr = 0) and rho are over
+  TS* zq = z + (size_t)blk * 12 * 256 + loc;
+#pragma unroll
+  for (int c = 0; c < 12; ++c) Io<R, TS>::st(zq + c * 256, Io<R, TS>::ldc(zq + c * 256) + e[c]);
+}
+
+// A cluster per block where whole blocks leave SMs idle: FP64, which is bound by
+// the SMs' FP64 units, up to four blocks an SM; FP32 below one block an SM.
+template <class R>
+static bool cluster_wins(const Geom& g, int nrhs) {
+  return (long long)(g.nblocks / 2) * nrhs < 152 * (sizeof(R) == 8 ? 4 : 1);
+}
+
+template <class R, class TS, class TG>
+static int run_cluster(const Geom& g, void* z, const void* b, const void* U, const void* A, int colour, int n_mr,
+                       int nrhs, cudaStream_t s) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(g.nblocks / 2 * nrhs * 8));
+  cfg.blockDim = dim3(32);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = 8;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  SAPMG_CUDA_TRY(cudaLaunchKernelEx(&cfg, sap_cluster_kernel<R, TS, TG>, (TS*)z, (const TS*)b, (const TG*)U,
+                                    (const TG*)A, g, colour, n_mr, nrhs));
+  count_launches(1);
+  return MG_OK;
+}
+
 template <class R, class TS, class TG>
 static int run(const Geom& g, void* z, const void* b, const void* U, const void* A, int colour, int n_mr, int nrhs,
                cudaStream_t s) {
+  if (cluster_wins<R>(g, nrhs)) return run_cluster<R, TS, TG>(g, z, b, U, A, colour, n_mr, nrhs, s);
   const size_t smem = sizeof(Cplx<R>) * 24 * 256 + sizeof(R) * 8 * 4;
   static bool attr = false;
   if (!attr) {

@@ -21,6 +21,44 @@ def _solver(prec, **kw):
     return torch, G, G.Solver(u, 1.0, -0.1, precision=prec, **kw)
 
 
+# 1216 / 16 = 76 fields (FP64) and 10 fields (FP32) reach the whole-block form of D; 608 / 8 = 76 and 19 that of
+# the Schwarz pass (an odd count: an even one of FP32 fields goes to the paired kernel).  The two forms run the
+# same operations: they may differ by what the compiler contracts, a few roundings of sums of about 100 terms.
+@pytest.mark.parametrize("prec,many,tol", [("fp64", 77, 1e-15), ("fp32", 11, 5e-7), ("bf16", 11, 5e-7)])
+def test_dirac_one_warp_ctas(prec, many, tol):
+    torch, G, s = _solver(prec, n_levels=1, fgmres_m=1)
+    dt = torch.complex128 if prec == "fp64" else torch.complex64
+    x = torch.randn((many, 16, 12, 256), dtype=dt, device="cuda", generator=torch.Generator("cuda").manual_seed(1))
+    for flag in (0, G.MG_DAGGER) if prec != "bf16" else (0,):
+        a, one = torch.empty_like(x), torch.empty_like(x[:1])
+        G.dirac_apply(s.ctx, x, a, s.prec | G.MG_BLOCKED | flag, many)
+        for k in (0, many - 1):
+            G.dirac_apply(s.ctx, x[k:k + 1].contiguous(), one, s.prec | G.MG_BLOCKED | flag, 1)
+            assert rel(host(a[k]), host(one[0])) < tol
+    s.close()
+
+
+@pytest.mark.parametrize("prec,many,tol", [("fp64", 77, 1e-14), ("fp32", 19, 5e-6), ("bf16", 19, 5e-6)])
+@pytest.mark.parametrize("n_mr", [0, 1, 4])
+def test_schwarz_cluster(prec, many, tol, n_mr):
+    torch, G, s = _solver(prec, n_levels=1, fgmres_m=1, n_mr=n_mr)
+    dt = torch.complex128 if prec == "fp64" else torch.complex64
+    gen = torch.Generator("cuda").manual_seed(2)
+    b = torch.randn((many, 16, 12, 256), dtype=dt, device="cuda", generator=gen)
+    z = torch.randn((many, 16, 12, 256), dtype=dt, device="cuda", generator=gen)
+    b[1], z[1] = 0, 0                                    # a zero system
+    a = z.clone()
+    G.sap_smooth(s.ctx, b, a, 2, s.prec | G.MG_BLOCKED, many)
+    for k in (0, 1, many - 1):
+        one = z[k:k + 1].clone()
+        G.sap_smooth(s.ctx, b[k:k + 1].contiguous(), one, 2, s.prec | G.MG_BLOCKED, 1)
+        if k == 1:
+            assert torch.count_nonzero(one) == 0 and torch.count_nonzero(a[1]) == 0
+        else:
+            assert rel(host(a[k]), host(one[0])) < tol
+    s.close()
+
+
 @pytest.mark.parametrize("n_vec,nrhs", [(4, 1), (20, 1), (20, 3), (24, 12)])
 def test_level1_schwarz_cluster_matches_one_cta_per_box(n_vec, nrhs, monkeypatch):
     """Level-1 boxes of 2^4 sites: the cluster form gives the one-CTA-per-box solve bit for bit."""
