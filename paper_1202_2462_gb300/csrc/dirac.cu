@@ -8,25 +8,23 @@
 #include "internal.h"
 #include "stencil.cuh"
 #include "dfloat.cuh"
+#include "quad.cuh"
 
 namespace sapmg {
 
 // DAG: apply D^dagger = gamma5 D gamma5 instead (the operator of the normal
 // equations).  NORM: also write the CTA's share of ||out||^2 to
 // part[blockIdx.x] (CTA index = block * nrhs + right-hand side), reduced in a
-// fixed order so that the result does not depend on scheduling.  TPB: sites per
-// CTA, 256 or (not with NORM) 32, eight CTAs to a block (see parts_of).
-template <class R, class TS, class TG, bool DAG, bool NORM, int TPB>
-__global__ void __launch_bounds__(TPB, TPB < 256 ? 1 : (sizeof(R) == 4 ? 3 : 1)) dirac_kernel(TS* __restrict__ out, const TS* __restrict__ in,
+// fixed order so that the result does not depend on scheduling.
+template <class R, class TS, class TG, bool DAG, bool NORM>
+__global__ void __launch_bounds__(256, (sizeof(R) == 4 ? 3 : 1)) dirac_kernel(TS* __restrict__ out, const TS* __restrict__ in,
                                                     const TG* __restrict__ U, const TG* __restrict__ A, Geom g,
                                                     int nrhs, double* __restrict__ part) {
   // right-hand side fastest in the grid: the CTAs of one block run back to
   // back and share its links and clover through L2
-  constexpr int kParts = 256 / TPB;
-  const int id = blockIdx.x / kParts;
-  const int blk = MG_CLAMP(kBlock, id / nrhs, g.nblocks);
-  const int loc = threadIdx.x + TPB * (blockIdx.x % kParts);
-  const size_t off = (size_t)(id % nrhs) * g.V * 12;
+  const int blk = MG_CLAMP(kBlock, blockIdx.x / nrhs, g.nblocks);
+  const int loc = threadIdx.x;
+  const size_t off = (size_t)(blockIdx.x % nrhs) * g.V * 12;
   in += off;
   out += off;
   // acc = -2 A psi + sum of hops, so D psi = -acc / 2
@@ -61,15 +59,37 @@ __global__ void __launch_bounds__(TPB, TPB < 256 ? 1 : (sizeof(R) == 4 ? 3 : 1))
   }
 }
 
-// CTAs a block is cut into.  With few blocks a CTA per block leaves SMs idle:
-// the FP64 units of one SM take 58 us for a block's 1848 x 256 flops whatever the
-// number of warps, so 16 blocks (8^4) took 87 us on 16 SMs and CTAs of one warp
-// spread them over 128.  FP64 is cut up to eight blocks an SM, where the last
-// wave of whole blocks would still leave a tenth of the SMs' time unused; FP32,
-// which needs the warps of a block to hide latency, below one block an SM.
+// The same for few blocks: eight CTAs of 32 sites a block, four threads a site (quad.cuh).
+template <class R, class TS, class TG, bool DAG>
+__global__ void __launch_bounds__(128) dirac_quad_kernel(TS* __restrict__ out, const TS* __restrict__ in,
+                                                         const TG* __restrict__ U, const TG* __restrict__ A, Geom g,
+                                                         int nrhs) {
+  __shared__ __align__(16) unsigned char part_raw[sizeof(Cplx<R>) * 4 * 12 * 32];
+  Cplx<R>* part = reinterpret_cast<Cplx<R>*>(part_raw);
+  const int id = blockIdx.x >> 3, blk = MG_CLAMP(kBlock, id / nrhs, g.nblocks);
+  const int m = threadIdx.x >> 5, lane = threadIdx.x & 31, loc = (blockIdx.x & 7) * 32 + lane;
+  const size_t off = (size_t)(id % nrhs) * g.V * 12;
+  in += off;
+  out += off;
+  Cplx<R> o[3];
+  switch (m) {
+    case 0: quad_dirac<0, R, TS, TG, DAG>(g, in, U, A, blk, loc, lane, part, o); break;
+    case 1: quad_dirac<1, R, TS, TG, DAG>(g, in, U, A, blk, loc, lane, part, o); break;
+    case 2: quad_dirac<2, R, TS, TG, DAG>(g, in, U, A, blk, loc, lane, part, o); break;
+    default: quad_dirac<3, R, TS, TG, DAG>(g, in, U, A, blk, loc, lane, part, o); break;
+  }
+  TS* q = out + (size_t)blk * 12 * 256 + loc;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) Io<R, TS>::st(q + (3 * m + k) * 256, o[k]);
+}
+
+// Few blocks: FP64 below eight blocks an SM, where the last wave of whole blocks
+// leaves a tenth or more of the FP64 units' time unused (16 blocks, 8^4: 87 us
+// with a CTA per block on 16 SMs, 46 us with a warp per 32 sites); FP32, which
+// needs the warps of a block to hide latency, below one block an SM.
 template <class R>
-static int parts_of(const Geom& g, int nrhs) {
-  return (long long)g.nblocks * nrhs < 152 * (sizeof(R) == 8 ? 8 : 1) ? 8 : 1;
+static bool few_blocks(const Geom& g, int nrhs) {
+  return (long long)g.nblocks * nrhs < 152 * (sizeof(R) == 8 ? 8 : 1);
 }
 
 template <class R, class TS, class TG, bool DAG, bool NORM>
@@ -77,15 +97,15 @@ static void run(const Geom& g, void* out, const void* in, const void* U, const v
                 cudaStream_t s) {
   const unsigned ctas = (unsigned)(g.nblocks * nrhs);
   if constexpr (!NORM) {
-    if (parts_of<R>(g, nrhs) == 8) {
-      dirac_kernel<R, TS, TG, DAG, false, 32><<<ctas * 8, 32, 0, s>>>((TS*)out, (const TS*)in, (const TG*)U,
-                                                                      (const TG*)A, g, nrhs, nullptr);
+    if (few_blocks<R>(g, nrhs)) {
+      dirac_quad_kernel<R, TS, TG, DAG><<<ctas * 8, 128, 0, s>>>((TS*)out, (const TS*)in, (const TG*)U, (const TG*)A,
+                                                                 g, nrhs);
       count_launches(1);
       return;
     }
   }
-  dirac_kernel<R, TS, TG, DAG, NORM, 256><<<ctas, 256, 0, s>>>((TS*)out, (const TS*)in, (const TG*)U, (const TG*)A, g,
-                                                               nrhs, part);
+  dirac_kernel<R, TS, TG, DAG, NORM><<<ctas, 256, 0, s>>>((TS*)out, (const TS*)in, (const TG*)U, (const TG*)A, g, nrhs,
+                                                          part);
   count_launches(1);
 }
 

@@ -13,6 +13,7 @@
 // colours are two launches in stream order.
 #include "async.cuh"
 #include "internal.h"
+#include "quad.cuh"
 #include "stencil.cuh"
 
 namespace sapmg {
@@ -149,14 +150,13 @@ __global__ void __launch_bounds__(256, (sizeof(R) == 4 ? 2 : 1))
   for (int c = 0; c < 12; ++c) Io<R, TS>::st(zq + c * 256, Io<R, TS>::ldc(zq + c * 256) + es[c * 256 + loc]);
 }
 
-// The same pass with a block on a cluster of eight one-warp CTAs (warp w of the
-// kernel above is CTA w), for few blocks: a block's MR steps then run on eight
-// SMs instead of one.  FP64 is bound by the SM's FP64 units (two FMAs a clock: 58
-// us for a block's MR step on one SM), so the 8 blocks of a colour of 8^4 took
-// 514 us a pass on 8 SMs.  rho stays in the shared memory of the CTA that owns
-// the site and its neighbours read it through distributed shared memory; the
-// block sums add the eight warps' parts in the order of the kernel above, so
-// the results are the same bit for bit.
+// The same pass with a block on a cluster of eight CTAs of 32 sites, four threads
+// a site (quad.cuh), for few blocks: a block's MR steps then run on eight SMs
+// instead of one.  FP64 is bound by the SMs' FP64 units, so the 8 blocks of a
+// colour of 8^4 took 514 us a pass on 8 SMs (262 us with one thread a site on
+// clusters of eight warps).  rho stays in the shared memory of the CTA that owns
+// the site, its neighbours read it through distributed shared memory; e, p and
+// the update of a component belong to one thread.
 __device__ __forceinline__ void sap_cluster_barrier() {
   asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
 }
@@ -182,118 +182,90 @@ __device__ __forceinline__ void st_cluster(uint32_t a, float v) {
   asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
 }
 
-// Sum of the hops of D_i at loc, rho in the CTAs' shared memory (rs: its address, [12][32] per CTA)
-template <int MU, class R, class TG>
-__device__ __forceinline__ void cluster_hops_dir(const TG* __restrict__ U, uint32_t rs, int blk, int loc,
-                                                 Cplx<R> (&acc)[12]) {
-  const int ls = 1 << (2 * MU);
-  const int c = (loc >> (2 * MU)) & 3;
-  Cplx<R> h[6], gg[6], u[9];
-  auto at = [&](int l) { return sap_cluster_addr(rs + (uint32_t)((l & 31) * sizeof(Cplx<R>)), l >> 5); };
-  if (c < 3) {
-    const uint32_t q = at(loc + ls);
-    spin_project_ld<MU, -1, R>([&](int k) { return ld_cluster(q + (uint32_t)(k * 32 * sizeof(Cplx<R>)), R(0)); }, h);
-    load_link<R>(U, blk, MU, loc, u);
-    su3_mul(u, h, gg);
-    spin_reconstruct_add<MU, -1>(gg, acc);
-  }
-  if (c > 0) {
-    const uint32_t q = at(loc - ls);
-    spin_project_ld<MU, 1, R>([&](int k) { return ld_cluster(q + (uint32_t)(k * 32 * sizeof(Cplx<R>)), R(0)); }, h);
-    load_link<R>(U, blk, MU, loc - ls, u);
-    su3_dag_mul(u, h, gg);
-    spin_reconstruct_add<MU, 1>(gg, acc);
-  }
+// Rows 3 M .. 3 M + 2 of D_i rho at the warp's sites (rsa: the address of the CTAs' rho, [12][32])
+template <int M, class R, class TG>
+__device__ __forceinline__ void quad_block(const Geom& g, const TG* __restrict__ U, const TG* __restrict__ A,
+                                           const Cplx<R>* rs, uint32_t rsa, int blk, int loc, Cplx<R>* part,
+                                           Cplx<R> (&out)[3]) {
+  const int ls = 1 << (2 * M), cm = (loc >> (2 * M)) & 3, lane = loc & 31;
+  auto at = [&](int l) { return sap_cluster_addr(rsa + (uint32_t)((l & 31) * sizeof(Cplx<R>)), l >> 5); };
+  const uint32_t q0 = at(cm < 3 ? loc + ls : loc), q1 = at(cm > 0 ? loc - ls : loc);
+  Cplx<R> acc[12];
+  quad_hops<M, R, TG, false>(
+      g, U, blk, loc,
+      [&](int step, int c) { return ld_cluster((step > 0 ? q0 : q1) + (uint32_t)(c * 32 * sizeof(Cplx<R>)), R(0)); },
+      [&](int step) { return step > 0 ? cm < 3 : cm > 0; }, acc);
+  quad_clover<M, R>(A, blk, loc, [&](int c) { return rs[c * 32 + lane]; }, out);
+  quad_swap<M>(part, lane, acc, out);
 }
 
 template <class R, class TS, class TG>
-__global__ void __launch_bounds__(32) sap_cluster_kernel(TS* __restrict__ z, const TS* __restrict__ b,
-                                                         const TG* __restrict__ U, const TG* __restrict__ A, Geom g,
-                                                         int colour, int n_mr, int nrhs) {
-  __shared__ __align__(16) unsigned char rs_raw[sizeof(Cplx<R>) * 12 * 32];
-  __shared__ R red[2][8][4];                             // two buffers: a step's sums are read while the next arrive
-  Cplx<R>* rs = reinterpret_cast<Cplx<R>*>(rs_raw);      // rho of the warp's sites [12][32]
+__global__ void __launch_bounds__(128) sap_cluster_kernel(TS* __restrict__ z, const TS* __restrict__ b,
+                                                          const TG* __restrict__ U, const TG* __restrict__ A, Geom g,
+                                                          int colour, int n_mr, int nrhs) {
+  __shared__ __align__(16) unsigned char smem_raw[sizeof(Cplx<R>) * 5 * 12 * 32];
+  __shared__ R red[2][32][4];                            // two buffers: a step's sums are read while the next arrive
+  Cplx<R>* rs = reinterpret_cast<Cplx<R>*>(smem_raw);    // rho of the CTA's sites [12][32]
+  Cplx<R>* part = rs + 12 * 32;                          // [4][12][32]
   const uint32_t rsa = smem_u32(rs);
-  const int rank = (int)(blockIdx.x & 7), lane = threadIdx.x, loc = rank * 32 + lane;
+  const int rank = (int)(blockIdx.x & 7), m = threadIdx.x >> 5, lane = threadIdx.x & 31, loc = rank * 32 + lane;
   const int id = blockIdx.x >> 3;
   const size_t off = (size_t)(id % nrhs) * g.V * 12;
   z += off;
   b += off;
   const int blk = colour_block(g, id / nrhs, colour);
-  {
-    Cplx<R> acc[12];
-    {
-      Cplx<R> zz[12];
-      load_spinor<R>(z, blk, loc, zz);
-      clover_apply<R>(A, blk, loc, zz, acc);
-    }
-#pragma unroll
-    for (int c = 0; c < 12; ++c) acc[c] = (R)(-2) * acc[c];
-    hops_global_dir<0>(g, z, U, blk, loc, acc);
-    asm volatile("" ::: "memory");
-    hops_global_dir<1>(g, z, U, blk, loc, acc);
-    asm volatile("" ::: "memory");
-    hops_global_dir<2>(g, z, U, blk, loc, acc);
-    asm volatile("" ::: "memory");
-    hops_global_dir<3>(g, z, U, blk, loc, acc);
-    const TS* bq = b + (size_t)blk * 12 * 256 + loc;
-#pragma unroll
-    for (int c = 0; c < 12; ++c) rs[c * 32 + lane] = Io<R, TS>::ldc(bq + c * 256) + (R)0.5 * acc[c];
+  const size_t own = ((size_t)blk * 12 + 3 * m) * 256 + loc;   // this thread's components 3 m .. 3 m + 2
+  Cplx<R> ro[3], e[3], p[3];
+  switch (m) {
+    case 0: quad_dirac<0, R, TS, TG, false>(g, z, U, A, blk, loc, lane, part, p); break;
+    case 1: quad_dirac<1, R, TS, TG, false>(g, z, U, A, blk, loc, lane, part, p); break;
+    case 2: quad_dirac<2, R, TS, TG, false>(g, z, U, A, blk, loc, lane, part, p); break;
+    default: quad_dirac<3, R, TS, TG, false>(g, z, U, A, blk, loc, lane, part, p); break;
   }
-  Cplx<R> e[12];
 #pragma unroll
-  for (int c = 0; c < 12; ++c) e[c] = cmk<R>(0, 0);
+  for (int k = 0; k < 3; ++k) {
+    ro[k] = Io<R, TS>::ldc(b + own + k * 256) - p[k];
+    rs[(3 * m + k) * 32 + lane] = ro[k];
+    e[k] = cmk<R>(0, 0);
+  }
   for (int it = 0; it < n_mr; ++it) {
-    sap_cluster_barrier();                               // rho of every site written
-    Cplx<R> p[12];
-    {
-      Cplx<R> ro[12];
-#pragma unroll
-      for (int c = 0; c < 12; ++c) ro[c] = rs[c * 32 + lane];
-      clover_apply<R>(A, blk, loc, ro, p);
+    sap_cluster_barrier();                               // rho of every site written, part free again
+    switch (m) {
+      case 0: quad_block<0, R, TG>(g, U, A, rs, rsa, blk, loc, part, p); break;
+      case 1: quad_block<1, R, TG>(g, U, A, rs, rsa, blk, loc, part, p); break;
+      case 2: quad_block<2, R, TG>(g, U, A, rs, rsa, blk, loc, part, p); break;
+      default: quad_block<3, R, TG>(g, U, A, rs, rsa, blk, loc, part, p); break;
     }
-#pragma unroll
-    for (int c = 0; c < 12; ++c) p[c] = (R)(-2) * p[c];
-    cluster_hops_dir<0>(U, rsa, blk, loc, p);
-    asm volatile("" ::: "memory");
-    cluster_hops_dir<1>(U, rsa, blk, loc, p);
-    asm volatile("" ::: "memory");
-    cluster_hops_dir<2>(U, rsa, blk, loc, p);
-    asm volatile("" ::: "memory");
-    cluster_hops_dir<3>(U, rsa, blk, loc, p);
     R v[3] = {0, 0, 0};
 #pragma unroll
-    for (int c = 0; c < 12; ++c) {
-      p[c] = (R)(-0.5) * p[c];
-      const Cplx<R> ro = rs[c * 32 + lane];
-      v[0] += p[c].re * ro.re + p[c].im * ro.im;
-      v[1] += p[c].re * ro.im - p[c].im * ro.re;
-      v[2] += p[c].re * p[c].re + p[c].im * p[c].im;
+    for (int k = 0; k < 3; ++k) {
+      v[0] += p[k].re * ro[k].re + p[k].im * ro[k].im;
+      v[1] += p[k].re * ro[k].im - p[k].im * ro[k].re;
+      v[2] += p[k].re * p[k].re + p[k].im * p[k].im;
     }
 #pragma unroll
     for (int q = 0; q < 3; ++q) v[q] = warp_sum(v[q]);
     if (lane < 8) {                                      // lane q: this warp's sums to CTA q
-      const uint32_t a = sap_cluster_addr(smem_u32(&red[it & 1][rank][0]), lane);
+      const uint32_t a = sap_cluster_addr(smem_u32(&red[it & 1][rank * 4 + m][0]), lane);
 #pragma unroll
       for (int q = 0; q < 3; ++q) st_cluster(a + (uint32_t)(q * sizeof(R)), v[q]);
     }
     sap_cluster_barrier();                               // the sums arrived; every neighbour read of rho done
-    R pr_re = 0, pr_im = 0, pp = 0;
+    // the 32 warps' sums, one a lane
 #pragma unroll
-    for (int k = 0; k < 8; ++k) { pr_re += red[it & 1][k][0]; pr_im += red[it & 1][k][1]; pp += red[it & 1][k][2]; }
+    for (int q = 0; q < 3; ++q) v[q] = warp_sum(red[it & 1][lane][q]);
     Cplx<R> alpha = cmk<R>(0, 0);
-    if (pp > (R)0) alpha = cmk(pr_re / pp, pr_im / pp);
+    if (v[2] > (R)0) alpha = cmk(v[0] / v[2], v[1] / v[2]);
 #pragma unroll
-    for (int c = 0; c < 12; ++c) {
-      const Cplx<R> ro = rs[c * 32 + lane];
-      e[c] = e[c] + alpha * ro;
-      rs[c * 32 + lane] = ro - alpha * p[c];
+    for (int k = 0; k < 3; ++k) {
+      e[k] = e[k] + alpha * ro[k];
+      ro[k] = ro[k] - alpha * p[k];
+      rs[(3 * m + k) * 32 + lane] = ro[k];
     }
   }
-  sap_cluster_barrier();                                 // the residuals' reads of z (n_mr = 0) and rho are over
-  TS* zq = z + (size_t)blk * 12 * 256 + loc;
+  sap_cluster_barrier();                                 // n_mr = 0: the residuals' reads of z are over
 #pragma unroll
-  for (int c = 0; c < 12; ++c) Io<R, TS>::st(zq + c * 256, Io<R, TS>::ldc(zq + c * 256) + e[c]);
+  for (int k = 0; k < 3; ++k) Io<R, TS>::st(z + own + k * 256, Io<R, TS>::ldc(z + own + k * 256) + e[k]);
 }
 
 // A cluster per block where whole blocks leave SMs idle: FP64, which is bound by
@@ -308,7 +280,7 @@ static int run_cluster(const Geom& g, void* z, const void* b, const void* U, con
                        int nrhs, cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(g.nblocks / 2 * nrhs * 8));
-  cfg.blockDim = dim3(32);
+  cfg.blockDim = dim3(128);
   cfg.stream = s;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;

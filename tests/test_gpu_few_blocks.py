@@ -22,10 +22,10 @@ def _solver(prec, **kw):
 
 
 # 1216 / 16 = 76 fields (FP64) and 10 fields (FP32) reach the whole-block form of D; 608 / 8 = 76 and 19 that of
-# the Schwarz pass (an odd count: an even one of FP32 fields goes to the paired kernel).  The two forms run the
-# same operations: they may differ by what the compiler contracts, a few roundings of sums of about 100 terms.
+# the Schwarz pass (an odd count: an even one of FP32 fields goes to the paired kernel).  The two forms add the
+# same terms in another order: a few roundings of sums of about 100 terms.
 @pytest.mark.parametrize("prec,many,tol", [("fp64", 77, 1e-15), ("fp32", 11, 5e-7), ("bf16", 11, 5e-7)])
-def test_dirac_one_warp_ctas(prec, many, tol):
+def test_dirac_four_threads_a_site(prec, many, tol):
     torch, G, s = _solver(prec, n_levels=1, fgmres_m=1)
     dt = torch.complex128 if prec == "fp64" else torch.complex64
     x = torch.randn((many, 16, 12, 256), dtype=dt, device="cuda", generator=torch.Generator("cuda").manual_seed(1))
