@@ -8,6 +8,7 @@
 // sums use the vector's own precision; CTA-level and final sums use FP64.
 #include "internal.h"
 #include "blas.h"
+#include "hessenberg.cuh"
 
 #include <type_traits>
 
@@ -398,17 +399,15 @@ int blas_normalize(int type, const BVec& b, const void* x, void* out, const doub
 }
 
 // Least-squares solve of the (m+1) x m Hessenberg system min ||beta e1 - H y||
-// of fixed-step GMRES, one warp per right-hand side: H in shared memory, column
-// k on lane k; step j's rotation [conj a, conj b; -b, a] / sqrt(|a|^2 + |b|^2)
-// is formed by every lane from the pivot column and applied to the lane's own,
-// then the back substitution takes y_i out of all rows above at once.  H for
+// of fixed-step GMRES, one warp per right-hand side (hessenberg.cuh).  H for
 // RHS r at H + r*ldr, column-major with leading dimension ldh; beta2[r].x =
 // ||b_r||^2; y[r*ldy + j].  scale != nullptr: basis vector j has the norm
 // scale[r*ldr + j].x (j = 0: 1) and y is divided by it.  Columns after a zero
 // subdiagonal entry are unused.  m <= 32.
-// Latency-bound (one reciprocal square root a step; every load and every
-// division is issued for all columns at once): 12 steps on one vector 73 us
-// with two square roots and divisions a step and serial loads, about 12 now.
+// Latency-bound (an FP64 instruction of a warp takes 64 cycles of its
+// sub-partition): 12 steps on one vector 73 us with two square roots and
+// divisions a step and serial loads, 27 us with one reciprocal square root a
+// step and every load and division issued for all columns at once.
 __global__ void __launch_bounds__(32) hessenberg_solve_kernel(const double2* __restrict__ Hall, int ldh, int ldr,
                                                               int m, const double2* __restrict__ beta2,
                                                               const double2* __restrict__ scale,
@@ -441,58 +440,8 @@ __global__ void __launch_bounds__(32) hessenberg_solve_kernel(const double2* __r
     hr[32 + 31 * 33] = v.x;
     hi[32 + 31 * 33] = v.y;
   }
-  double gr = lane == 0 ? beta : 0.0, gi = 0.0;          // g_lane; g_32 only closes the residual
-  __syncwarp();
-  for (int j = 0; j < mm; ++j) {
-    const double ar = hr[j + j * 33], ai = hi[j + j * 33];
-    const double br = hr[j + 1 + j * 33], bi = hi[j + 1 + j * 33];
-    const double d2 = ar * ar + ai * ai + br * br + bi * bi;
-    const double inv = rsqrt(d2);
-    // a vanishing pivot column is left as it is (the identity rotation)
-    const double cr = d2 > 0.0 ? ar * inv : 1.0, ci = d2 > 0.0 ? ai * inv : 0.0;
-    const double sr = d2 > 0.0 ? br * inv : 0.0, si = d2 > 0.0 ? bi * inv : 0.0;
-    __syncwarp();                                         // every lane has read column j
-    if (lane >= j && lane < mm) {
-      const double xr = hr[j + lane * 33], xi = hi[j + lane * 33];
-      const double zr = hr[j + 1 + lane * 33], zi = hi[j + 1 + lane * 33];
-      hr[j + lane * 33] = cr * xr + ci * xi + sr * zr + si * zi;
-      hi[j + lane * 33] = cr * xi - ci * xr + sr * zi - si * zr;
-      hr[j + 1 + lane * 33] = cr * zr - ci * zi - sr * xr + si * xi;
-      hi[j + 1 + lane * 33] = cr * zi + ci * zr - sr * xi - si * xr;
-    }
-    const double xr = __shfl_sync(0xffffffffu, gr, j), xi = __shfl_sync(0xffffffffu, gi, j);
-    if (lane == j) {                                      // g_{j+1} was 0
-      gr = cr * xr + ci * xi;
-      gi = cr * xi - ci * xr;
-    } else if (lane == j + 1) {
-      gr = -(sr * xr - si * xi);
-      gi = -(sr * xi + si * xr);
-    }
-    __syncwarp();
-  }
-  // the reciprocals of the diagonal, one a lane; a zero entry gives y_i = 0
-  double wr = 0.0, wi = 0.0;
-  if (lane < mm) {
-    const double dr = hr[lane + lane * 33], di = hi[lane + lane * 33];
-    const double d2 = dr * dr + di * di;
-    if (d2 > 0.0) {
-      const double q = 1.0 / d2;
-      wr = dr * q;
-      wi = -di * q;
-    }
-  }
-  double yr = 0.0, yi = 0.0;
-  for (int i = mm - 1; i >= 0; --i) {
-    const double tr = gr * wr - gi * wi, ti = gr * wi + gi * wr;
-    const double sr = __shfl_sync(0xffffffffu, tr, i), si = __shfl_sync(0xffffffffu, ti, i);
-    if (lane == i) { yr = sr; yi = si; }
-    if (lane < i) {
-      const double ur = hr[lane + i * 33], ui = hi[lane + i * 33];
-      gr -= ur * sr - ui * si;
-      gi -= ur * si + ui * sr;
-    }
-  }
-  if (lane < m) y[lane] = make_double2(yr * inv_s, yi * inv_s);
+  const Cplx<double> v = hessenberg_warp(hr, hi, mm, beta);
+  if (lane < m) y[lane] = make_double2(v.re * inv_s, v.im * inv_s);
 }
 
 // ------------------------------------------------------------ delayed reorthogonalisation

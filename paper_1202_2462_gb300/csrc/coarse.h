@@ -65,6 +65,14 @@ struct CoarseTune {
 int launch_coarse_apply_mma(const CGeom& c, int store, const void* M, const void* x, void* out, int nrhs, int* err,
                             bool x_half, cudaStream_t s, const CoarseTune& t = CoarseTune());
 
+// Fixed-step GMRES of k steps from zero on a small lattice, b -> x for R systems, in
+// one kernel (coarse_gmres.cu): operator in FP16 (store P16, FP32 vectors) or FP64
+// (P64), 2N even; coarse_gmres_cluster_ok: whether its rows, the basis and the
+// scalars fit a cluster's shared memory (FP16, 2N = 40: up to 48 sites).
+bool coarse_gmres_cluster_ok(int store, const CGeom& c, int k);
+int launch_coarse_gmres_cluster(int store, const CGeom& c, const void* M, const void* b, void* x, int k, int R,
+                                int* err, cudaStream_t s);
+
 // Intermediate level of a three-level hierarchy (coarse1.cu).
 // The colour pass of launch_coarse_sap for 1 <= nrhs <= 12 right-hand sides in one
 // CTA per box (FP32 vectors; FP32 operator, or its FP16 copy with m16; each

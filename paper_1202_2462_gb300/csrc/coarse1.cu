@@ -6,7 +6,7 @@
 // level-2 aggregates are boxes of coarse sites (Box4).  Level-1 test vectors
 // are vector-major [k][site][n2]; the level-2 operator uses the stencil layout
 // M[site][d][j][i] of every coarse level.
-#include "async.cuh"
+#include "cluster.cuh"
 #include "internal.h"
 #include "coarse.h"
 
@@ -383,12 +383,16 @@ int launch_coarse_sap_mrhs(const CGeom& c, const Box4& bx, const void* M, bool m
 }
 
 // ------------------------------------------------------------ the colour pass on clusters (FP16 operator)
-// One box on a cluster of eight CTAs, each holding the operator rows of its
-// sites / 8 box sites in shared memory: copied there once (bulk copies, one
-// mbarrier), used by the residual and by every MR step of every right-hand
-// side.  The kernels above read a box's operator (0.9 MB for 16 sites, 2N = 40)
-// from L2 once per MR step through the one SM that holds the box, which bounds
-// them by that SM's L2 port: 130 us for one right-hand side on 16 boxes.
+// One box on a cluster of eight CTAs, each holding the in-box operator blocks of
+// its sites / 8 box sites in shared memory (five of a site's nine for boxes of
+// 2^4): copied there once (bulk copies, one mbarrier), used by the residual and
+// by every MR step of every right-hand side; the blocks that couple to other
+// boxes are read once per right-hand side, by the residual alone.  The kernels
+// above read a box's operator (0.9 MB for 16 sites, 2N = 40) from L2 once per MR
+// step through the one SM that holds the box, which bounds them by that SM's L2
+// port: 130 us for one right-hand side on 16 boxes.  Two CTAs an SM, so that
+// the 16 clusters of a colour of an 8 x 4^3 lattice run at once (with all nine
+// blocks, one CTA an SM, only 15 of them do: 58 us).
 // Here a product's (site, direction, row) terms are one thread each; the row
 // sums p (in direction order) go to all eight CTAs by distributed shared
 // memory, and every CTA then forms the box's scalar products and updates rho
@@ -396,75 +400,101 @@ int launch_coarse_sap_mrhs(const CGeom& c, const Box4& bx, const void* M, bool m
 // step is the only exchange and the results are the same bit for bit.
 constexpr int kBoxCluster = 8;
 
-__device__ __forceinline__ uint32_t cluster_rank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
+// in-box blocks of a site, at most: itself and per direction one neighbour (two from extent 3 on)
+static int box_blocks(const Box4& bx) {
+  int n = 1;
+  for (int mu = 0; mu < 4; ++mu) n += std::min(bx.b[mu] - 1, 2);
+  return n;
 }
-__device__ __forceinline__ void cluster_barrier() {
-  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
-}
-__device__ __forceinline__ uint32_t cluster_addr(const void* p, int rank) {
-  uint32_t a;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
-  return a;
-}
-__device__ __forceinline__ void cluster_store(void* p, int rank, Cplx<float> v) {
-  asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(cluster_addr(p, rank)), "f"(v.re), "f"(v.im)
-               : "memory");
-}
-__device__ __forceinline__ void cluster_store(int* p, int rank, int v) {
-  asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(cluster_addr(p, rank)), "r"(v) : "memory");
+// shared memory: in-box operator blocks, staged neighbour vectors, direction terms,
+// rho and p (two buffers each), reduction words, tables
+static size_t box_cluster_smem(const Box4& bx, int n2) {
+  const size_t spc = (size_t)bx.sites / kBoxCluster, elems = (size_t)bx.sites * n2;
+  return spc * box_blocks(bx) * n2 * n2 * 4 + 2 * spc * 9 * n2 * 8 + 4 * elems * 8 + (32 * 4 + 4) * 4 +
+         (3 * spc * 9 + spc * box_blocks(bx) + kBoxCluster + 2) * 4 + 16;
 }
 
-// shared memory of the cluster form: operator rows, staged neighbour vectors,
-// direction terms, rho and p (two buffers each), reduction words
-static size_t box_cluster_smem(int sites, int n2) {
-  const size_t spc = (size_t)sites / kBoxCluster, elems = (size_t)sites * n2;
-  return spc * 9 * n2 * n2 * 4 + 2 * spc * 9 * n2 * 8 + 4 * elems * 8 + 32 * 16 + 64;
+// row sum over j of M[j][row] x[j], j in order (M in shared or global memory)
+template <class LD>
+__device__ __forceinline__ Cplx<float> row_sum(LD m, const Cplx<float>* x, int n2) {
+  Cplx<float> t = cmk(0.f, 0.f);
+#pragma unroll 8
+  for (int j = 0; j < n2; ++j) {
+    const float2 v = half2_bits_to_float2(m(j));
+    cfma(t, cmk(v.x, v.y), x[j]);
+  }
+  return t;
 }
 
-__global__ void __launch_bounds__(1024) coarse_sap_cluster_kernel(const __half2* __restrict__ M, float2* z,
-                                                                  const float2* __restrict__ b, CGeom c, Box4 bx,
-                                                                  int colour, int n_mr, int nrhs,
-                                                                  int* __restrict__ err) {
+template <int MAXT, int MINB>
+__global__ void __launch_bounds__(MAXT, MINB) coarse_sap_cluster_kernel(const __half2* __restrict__ M, float2* z,
+                                                                        const float2* __restrict__ b, CGeom c,
+                                                                        Box4 bx, int nblk, int colour, int n_mr,
+                                                                        int nrhs, int* __restrict__ err) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  const int n2 = c.n2, bs = bx.sites, spc = bs / kBoxCluster, elems = bs * n2, rows = spc * n2;
-  const int rank = (int)cluster_rank();
-  const size_t mbytes = (size_t)9 * n2 * n2 * 4;                 // one site's operator rows
-  const uint32_t* Ms = reinterpret_cast<const uint32_t*>(smem_raw);
-  Cplx<float>* xs = reinterpret_cast<Cplx<float>*>(smem_raw + spc * mbytes);       // [spc * 9][n2]
+  const int n2 = c.n2, tile = n2 * n2, spc = bx.sites / kBoxCluster, elems = bx.sites * n2, rows = spc * n2;
+  const int rank = cluster_rank();
+  uint32_t* Ms = reinterpret_cast<uint32_t*>(smem_raw);                            // [spc * nblk][n2][n2]
+  Cplx<float>* xs = reinterpret_cast<Cplx<float>*>(Ms + (size_t)spc * nblk * tile);  // [spc * 9][n2]
   Cplx<float>* ts = xs + spc * 9 * n2;                                             // [spc * 9][n2]
   Cplx<float>* rho = ts + spc * 9 * n2;                                            // [2][elems]
   Cplx<float>* pb = rho + 2 * elems;                                               // [2][elems]
-  float (*red)[4] = reinterpret_cast<float (*)[4]>(pb + 2 * elems);                // [32][4]
-  int* flag = reinterpret_cast<int*>(red + 32);                                    // [kBoxCluster]
-  uint64_t* bar = reinterpret_cast<uint64_t*>(flag + kBoxCluster);
+  float (*red)[4] = reinterpret_cast<float (*)[4]>(pb + 2 * elems);                // [32][4], then the sums
+  int* tab_site = reinterpret_cast<int*>(red + 33);                                // per (own site, direction):
+  int* tab_loc = tab_site + spc * 9;       // global site of the neighbour; its box site, or -1 outside;
+  int* tab_slot = tab_loc + spc * 9;       // its block in Ms
+  int* tab_term = tab_slot + spc * 9;      // the (own site, direction) of a block of Ms, or -1
+  int* flag = tab_term + spc * nblk;                                               // [kBoxCluster]
+  uint64_t* bar = reinterpret_cast<uint64_t*>((reinterpret_cast<uintptr_t>(flag + kBoxCluster) + 7) & ~(uintptr_t)7);
   int bc[4];
   colour_box(bx, blockIdx.x / kBoxCluster, colour, bc);
   const size_t fs = (size_t)c.nsites * n2;
   const int tid = threadIdx.x, nt = blockDim.x;
-  const bool act = tid < elems;
-  const int s = act ? tid / n2 : 0, i = act ? tid % n2 : 0;      // this thread's element of the box
-  const bool own = act && s / spc == rank;
-  int lc[4];
-  const int site = box_site(c, bx, bc, s, lc);
+  for (int q = tid; q < spc * nblk; q += nt) tab_term[q] = -1;
+  __syncthreads();
+  for (int q = tid; q < spc * 9; q += nt) {
+    const int k = q / 9, d = q % 9, ls = rank * spc + k;
+    int lc[4], ln = ls, slot = k * nblk;
+    const int st = box_site(c, bx, bc, ls, lc);
+    int stride = 1, at = 1;
+#pragma unroll
+    for (int mu = 0; mu < 4; ++mu) {
+      const bool up = lc[mu] + 1 < bx.b[mu], dn = lc[mu] > 0;
+      if (d == 1 + 2 * mu) { ln = up ? ls + stride : -1; slot += up ? at : 0; }
+      at += up;
+      if (d == 2 + 2 * mu) { ln = dn ? ls - stride : -1; slot += dn ? at : 0; }
+      at += dn;
+      stride *= bx.b[mu];
+    }
+    tab_site[q] = stencil_nb(c, st, d);
+    tab_loc[q] = ln;
+    tab_slot[q] = slot;
+    if (ln >= 0) tab_term[slot] = q;
+  }
   if (tid == 0) {
     mbar_init(bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    mbar_expect_tx(bar, (uint32_t)(spc * mbytes));
-    for (int k = 0; k < spc; ++k) {
-      int l2[4];
-      const int st = box_site(c, bx, bc, rank * spc + k, l2);
-      bulk_copy_g2s(smem_raw + k * mbytes, M + (size_t)st * 9 * n2 * n2, (uint32_t)mbytes, bar);
-    }
+  }
+  __syncthreads();
+  if (tid == 0) {
+    int n = 0;
+    for (int q = 0; q < spc * 9; ++q) n += tab_loc[q] >= 0;
+    mbar_expect_tx(bar, (uint32_t)n * tile * 4);
+    for (int q = 0; q < spc * 9; ++q)
+      if (tab_loc[q] >= 0)
+        bulk_copy_g2s(Ms + (size_t)tab_slot[q] * tile, M + ((size_t)tab_site[q / 9 * 9] * 9 + q % 9) * tile,
+                      (uint32_t)tile * 4, bar);
   }
   const int spins = wait_spins(err);
-  cluster_barrier();                                             // every CTA of the cluster runs, the barrier is set up
+  cluster_barrier();                                             // every CTA of the cluster runs
   const bool waited = mbar_wait(bar, 0, spins);
   const int failed = __syncthreads_or(!waited);
-  if (tid < kBoxCluster) cluster_store(flag + rank, tid, failed);
+  if (tid < kBoxCluster) cluster_st(cluster_addr(smem_u32(flag + rank), tid), failed);
+  // this thread's term (own site and direction q, row) of the products, its own box element
+  const int q0 = tid / n2, r0 = tid - q0 * n2;
+  const bool act = tid < elems, own = act && tid / rows == rank;
+  const uint32_t rs_a = smem_u32(rho), pb_a = smem_u32(pb);
   int pbuf = 0;
   for (int r = 0; r < nrhs; ++r) {
     float2* zr = z + r * fs;
@@ -472,34 +502,28 @@ __global__ void __launch_bounds__(1024) coarse_sap_cluster_kernel(const __half2*
     Cplx<float>* rs = rho + (r & 1) * elems;
     if (!failed) {
       // residual: the nine terms of every own row, then b minus them in direction order
-      for (int e = tid; e < spc * 9 * n2; e += nt) {
-        const int j = e % n2, q = e / n2, k = q / 9, d = q % 9;
-        int l2[4];
-        const int st = box_site(c, bx, bc, rank * spc + k, l2);
-        xs[e] = Io<float, float2>::ldc(zr + (size_t)stencil_nb(c, st, d) * n2 + j);
-      }
+      for (int e = tid, q = q0, row = r0; e < spc * 9 * n2; e += nt, q = e / n2, row = e - q * n2)
+        xs[e] = Io<float, float2>::ldc(zr + (size_t)tab_site[q] * n2 + row);
       __syncthreads();
-      for (int e = tid; e < spc * 9 * n2; e += nt) {
-        const int q = e / n2, row = e % n2;
-        const uint32_t* m = Ms + (size_t)q * n2 * n2 + row;
+      for (int e = tid, q = q0, row = r0; e < spc * 9 * n2; e += nt, q = e / n2, row = e - q * n2) {
         const Cplx<float>* x = xs + q * n2;
-        Cplx<float> t = cmk(0.f, 0.f);
-#pragma unroll 8
-        for (int j = 0; j < n2; ++j) {
-          const float2 v = half2_bits_to_float2(m[(size_t)j * n2]);
-          cfma(t, cmk(v.x, v.y), x[j]);
+        if (tab_loc[q] >= 0) {
+          const uint32_t* m = Ms + (size_t)tab_slot[q] * tile + row;
+          ts[e] = row_sum([&](int j) { return m[j * n2]; }, x, n2);
+        } else {
+          const unsigned* m = reinterpret_cast<const unsigned*>(M) +
+                              ((size_t)tab_site[q / 9 * 9] * 9 + q % 9) * tile + row;
+          ts[e] = row_sum([&](int j) { return __ldg(m + j * n2); }, x, n2);
         }
-        ts[e] = t;
       }
       __syncthreads();
-      for (int e = tid; e < rows; e += nt) {
-        const int k = e / n2, row = e % n2;
-        int l2[4];
-        const int st = box_site(c, bx, bc, rank * spc + k, l2);
-        Cplx<float> acc = Io<float, float2>::ldc(br + (size_t)st * n2 + row);
-        for (int d = 0; d < 9; ++d) acc = acc - ts[(k * 9 + d) * n2 + row];
+      if (tid < rows) {
+        const int k = q0;
+        Cplx<float> acc = Io<float, float2>::ldc(br + (size_t)tab_site[k * 9] * n2 + r0);
+        for (int d = 0; d < 9; ++d) acc = acc - ts[(k * 9 + d) * n2 + r0];
+        const uint32_t a = rs_a + (uint32_t)(((r & 1) * elems + rank * rows + tid) * 8);
 #pragma unroll
-        for (int q = 0; q < kBoxCluster; ++q) cluster_store(rs + rank * rows + e, q, acc);
+        for (int q = 0; q < kBoxCluster; ++q) cluster_st(cluster_addr(a, q), acc);
       }
     }
     cluster_barrier();                                           // rho of the box complete in every CTA
@@ -517,52 +541,44 @@ __global__ void __launch_bounds__(1024) coarse_sap_cluster_kernel(const __half2*
     }
     Cplx<float> e_own = cmk(0.f, 0.f);
     for (int it = 0; it < n_mr; ++it) {
-      Cplx<float>* pc = pb + pbuf * elems;
+      const int pc = pbuf * elems;
       pbuf ^= 1;
-      for (int e = tid; e < spc * 9 * n2; e += nt) {
-        const int q = e / n2, row = e % n2, k = q / 9, d = q % 9, ls = rank * spc + k;
-        int ln = ls;
-        if (d > 0) {
-          const int mu = (d - 1) >> 1, step = (d & 1) ? 1 : -1;
-          int stride = 1;
-          for (int m = 0; m < mu; ++m) stride *= bx.b[m];
-          const int l2 = (ls / stride) % bx.b[mu] + step;
-          if (l2 < 0 || l2 >= bx.b[mu]) continue;                // coupling leaves the box
-          ln = ls + step * stride;
+      for (int e = tid, sl = q0, row = r0; e < spc * nblk * n2; e += nt, sl = e / n2, row = e - sl * n2) {
+        const int q = tab_term[sl];
+        if (q >= 0) {
+          const uint32_t* m = Ms + (size_t)sl * tile + row;
+          ts[q * n2 + row] = row_sum([&](int j) { return m[j * n2]; }, rs + tab_loc[q] * n2, n2);
         }
-        const uint32_t* m = Ms + (size_t)q * n2 * n2 + row;
-        const Cplx<float>* x = rs + ln * n2;
-        Cplx<float> t = cmk(0.f, 0.f);
-#pragma unroll 8
-        for (int j = 0; j < n2; ++j) {
-          const float2 v = half2_bits_to_float2(m[(size_t)j * n2]);
-          cfma(t, cmk(v.x, v.y), x[j]);
-        }
-        ts[e] = t;
       }
       __syncthreads();
-      for (int e = tid; e < rows; e += nt) {
-        const int k = e / n2, row = e % n2, ls = rank * spc + k;
+      if (tid < rows) {
         Cplx<float> p = cmk(0.f, 0.f);
-        int rest = ls;
-        p = p + ts[(k * 9) * n2 + row];
-        for (int mu = 0; mu < 4; ++mu) {
-          const int l = rest % bx.b[mu];
-          rest /= bx.b[mu];
-          if (l + 1 < bx.b[mu]) p = p + ts[(k * 9 + 1 + 2 * mu) * n2 + row];
-          if (l > 0) p = p + ts[(k * 9 + 2 + 2 * mu) * n2 + row];
-        }
 #pragma unroll
-        for (int q = 0; q < kBoxCluster; ++q) cluster_store(pc + rank * rows + e, q, p);
+        for (int d = 0; d < 9; ++d)
+          if (tab_loc[q0 * 9 + d] >= 0) p = p + ts[(q0 * 9 + d) * n2 + r0];
+        const uint32_t a = pb_a + (uint32_t)((pc + rank * rows + tid) * 8);
+#pragma unroll
+        for (int q = 0; q < kBoxCluster; ++q) cluster_st(cluster_addr(a, q), p);
       }
       cluster_barrier();                                         // p of the box complete in every CTA
-      const Cplx<float> p = act ? pc[tid] : cmk(0.f, 0.f);
+      const Cplx<float> p = act ? pb[pc + tid] : cmk(0.f, 0.f);
       Cplx<float> ro = act ? rs[tid] : cmk(0.f, 0.f);
       float v[3] = {0.f, 0.f, 0.f};
       if (act) mr_dots(p, ro, v);
-      block_reduce_n(v, red);
+      // the sums of block_reduce_n, added by three threads
+#pragma unroll
+      for (int q = 0; q < 3; ++q) v[q] = warp_sum(v[q]);
+      if ((tid & 31) == 0) { red[tid >> 5][0] = v[0]; red[tid >> 5][1] = v[1]; red[tid >> 5][2] = v[2]; }
+      __syncthreads();
+      if (tid < 3) {
+        float s = 0.f;
+        for (int k = 0; k < (nt >> 5); ++k) s += red[k][tid];
+        red[32][tid] = s;
+      }
+      __syncthreads();
+      const float pp = red[32][2];
       Cplx<float> alpha = cmk(0.f, 0.f);
-      if (v[2] > 0.f) alpha = cmk(v[0] / v[2], v[1] / v[2]);
+      if (pp > 0.f) alpha = cmk(red[32][0] / pp, red[32][1] / pp);
       if (act) {
         mr_update(alpha, p, e_own, ro);
         rs[tid] = ro;
@@ -570,7 +586,7 @@ __global__ void __launch_bounds__(1024) coarse_sap_cluster_kernel(const __half2*
       __syncthreads();                                           // rho updated; red reused by the next reduction
     }
     if (own) {
-      float2* zq = zr + (size_t)site * n2 + i;
+      float2* zq = zr + (size_t)tab_site[(tid - rank * rows) / n2 * 9] * n2 + (tid - rank * rows) % n2;
       Io<float, float2>::st(zq, Io<float, float2>::ldc(zq) + e_own);
     }
   }
@@ -578,33 +594,31 @@ __global__ void __launch_bounds__(1024) coarse_sap_cluster_kernel(const __half2*
 
 bool coarse_sap_cluster_ok(const CGeom& c, const Box4& bx) {
   return bx.sites % kBoxCluster == 0 && c.n2 % 2 == 0 && bx.sites * c.n2 <= 1024 &&
-         box_cluster_smem(bx.sites, c.n2) <= 227 * 1024;
+         box_cluster_smem(bx, c.n2) <= 227 * 1024;
+}
+
+template <int MAXT, int MINB>
+static int coarse_sap_cluster_run(const CGeom& c, const Box4& bx, const void* M16, void* z, const void* b, int colour,
+                                  int n_mr, int nrhs, int* err, unsigned threads, cudaStream_t s) {
+  static bool attr = false;
+  if (!attr) {
+    SAPMG_CUDA_TRY(cudaFuncSetAttribute(coarse_sap_cluster_kernel<MAXT, MINB>,
+                                        cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+    attr = true;
+  }
+  ClusterLaunch l((unsigned)(bx.nboxes / 2 * kBoxCluster), threads, box_cluster_smem(bx, c.n2), kBoxCluster, s);
+  SAPMG_CUDA_TRY(cudaLaunchKernelEx(&l.cfg, coarse_sap_cluster_kernel<MAXT, MINB>, (const __half2*)M16, (float2*)z,
+                                    (const float2*)b, c, bx, box_blocks(bx), colour, n_mr, nrhs, err));
+  count_launches(1);
+  return MG_OK;
 }
 
 int launch_coarse_sap_cluster(const CGeom& c, const Box4& bx, const void* M16, void* z, const void* b, int colour,
                               int n_mr, int nrhs, int* err, cudaStream_t s) {
   if (!coarse_sap_cluster_ok(c, bx)) return MG_ERR_ARG;
-  static bool attr = false;
-  if (!attr) {
-    SAPMG_CUDA_TRY(cudaFuncSetAttribute(coarse_sap_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        227 * 1024));
-    attr = true;
-  }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(bx.nboxes / 2 * kBoxCluster));
-  cfg.blockDim = dim3((unsigned)((bx.sites * c.n2 + 31) / 32 * 32));
-  cfg.dynamicSmemBytes = box_cluster_smem(bx.sites, c.n2);
-  cfg.stream = s;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = kBoxCluster;
-  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  SAPMG_CUDA_TRY(cudaLaunchKernelEx(&cfg, coarse_sap_cluster_kernel, (const __half2*)M16, (float2*)z,
-                                    (const float2*)b, c, bx, colour, n_mr, nrhs, err));
-  count_launches(1);
-  return MG_OK;
+  const unsigned threads = (unsigned)((bx.sites * c.n2 + 31) / 32 * 32);
+  if (threads <= 640) return coarse_sap_cluster_run<640, 2>(c, bx, M16, z, b, colour, n_mr, nrhs, err, threads, s);
+  return coarse_sap_cluster_run<1024, 1>(c, bx, M16, z, b, colour, n_mr, nrhs, err, threads, s);
 }
 
 int launch_coarse_sap(int prec, const CGeom& c, const Box4& bx, const void* M, void* z, const void* b, int colour,

@@ -530,12 +530,23 @@ static int coarse_gmres_h_graph(mg_ctx* c, int level, CoarseLevel& L, int k, int
   return MG_OK;
 }
 
+// The coarsest level's fixed-step GMRES, b -> x of L for R systems: one kernel on a
+// small lattice, the FP16-basis form (as a graph), or the general one.
+static int coarsest_solve(mg_ctx* c, int level, CoarseLevel& L, int R) {
+  const int k = c->p.coarse_iters, store = c->vt == P64 ? P64 : P16;
+  if (!c->coarse_reorth && !c->generic_coarse && (store == P64 || L.Vh) && coarse_gmres_cluster_ok(store, L.cg, k)) {
+    ProfScope ps(c->prof, FAM_CBLAS, c->s);
+    count_bytes((double)L.n() * (9.0 * L.cg.n2 * complex_bytes(store) + 2.0 * R * complex_bytes(c->vt)));
+    return launch_coarse_gmres_cluster(store, L.cg, store == P64 ? L.M : L.Mh, L.b, L.x, k, R, c->dev_err, c->s);
+  }
+  if (L.Vh) return coarse_gmres_h_graph(c, level, L, k, R);
+  return coarse_gmres(c, L, k, R);
+}
+
 static int coarse_solve(mg_ctx* c, int level, int R) {
-  if (level == 1 && c->p.n_levels == 2 && c->c1.Vh) return coarse_gmres_h_graph(c, 1, c->c1, c->p.coarse_iters, R);
-  if (level == 1 && c->p.n_levels == 2) return coarse_gmres(c, c->c1, c->p.coarse_iters, R);
+  if (level == 1 && c->p.n_levels == 2) return coarsest_solve(c, 1, c->c1, R);
   if (level == 1 && c->p.n_levels == 3) return fgmres_fixed1(c, c->p.inner_iters, R);
-  if (level == 2 && c->p.n_levels == 3 && c->c2.Vh) return coarse_gmres_h_graph(c, 2, c->c2, c->p.coarse_iters, R);
-  if (level == 2 && c->p.n_levels == 3) return coarse_gmres(c, c->c2, c->p.coarse_iters, R);
+  if (level == 2 && c->p.n_levels == 3) return coarsest_solve(c, 2, c->c2, R);
   return fail(MG_ERR_ARG, "coarse level out of range");
 }
 
