@@ -559,38 +559,59 @@ int launch_transfer0(bool restrict_, int prec, const Geom& g, const void* in, vo
 // K7: modified Gram-Schmidt of the N vectors on every (block, chirality),
 // vectors k = 0..N-1 in order, each normalised to a positive real norm.
 // V: FP64 vector-major blocked fields [k][blk][12][256].
+// Bound by the FP64 units (64 cycles an instruction of a warp): 48 instructions a
+// site for a projection, so its block sum counts.  The two halves of a warp
+// reduce the real and the imaginary part (5 additions instead of 10) and sixteen
+// lanes add the eight warps' words (3 instead of 16 in every thread).
 __device__ __forceinline__ double2 block_sum2(double a, double b, double (*red)[2]) {
-  a = warp_sum(a);
-  b = warp_sum(b);
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (lane == 0) { red[w][0] = a; red[w][1] = b; }
+  double v = (lane & 16) ? b : a;
+  v += __shfl_xor_sync(0xffffffffu, (lane & 16) ? a : b, 16);
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if ((lane & 15) == 0) red[w][lane >> 4] = v;
   __syncthreads();
-  double sa = 0, sb = 0;
-  for (int q = 0; q < (int)(blockDim.x >> 5); ++q) { sa += red[q][0]; sb += red[q][1]; }
-  __syncthreads();
-  return make_double2(sa, sb);
+  double t = red[lane & 7][(lane >> 3) & 1];
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  return make_double2(__shfl_sync(0xffffffffu, t, 0), __shfl_sync(0xffffffffu, t, 8));
 }
 
 __global__ void __launch_bounds__(256) block_gs0_kernel(double2* __restrict__ V, int N, long long fstride) {
-  __shared__ double red[8][2];
+  __shared__ double red[2][8][2];                      // two buffers: one barrier per sum
   const int blk = blockIdx.x, chi = blockIdx.y, loc = threadIdx.x;
   const size_t base = ((size_t)blk * 12 + 6 * chi) * 256 + loc;
+  int buf = 0;
   for (int k = 0; k < N; ++k) {
     double2* vk = V + k * fstride + base;
-    Cplx<double> x[6];
+    Cplx<double> x[6], q[6];
+#pragma unroll
     for (int c = 0; c < 6; ++c) { double2 t = vk[c * 256]; x[c] = cmk(t.x, t.y); }
+    if (k > 0)
+#pragma unroll
+      for (int c = 0; c < 6; ++c) { double2 t = V[base + c * 256]; q[c] = cmk(t.x, t.y); }
     for (int j = 0; j < k; ++j) {
-      const double2* vj = V + j * fstride + base;
-      Cplx<double> q[6], d = cmk(0.0, 0.0);
-      for (int c = 0; c < 6; ++c) { double2 t = vj[c * 256]; q[c] = cmk(t.x, t.y); cfma_conj(d, q[c], x[c]); }
-      const double2 s = block_sum2(d.re, d.im, red);
-      const Cplx<double> cs = cmk(s.x, s.y);
-      for (int c = 0; c < 6; ++c) x[c] = x[c] - cs * q[c];
+      Cplx<double> d = cmk(0.0, 0.0), qn[6];
+#pragma unroll
+      for (int c = 0; c < 6; ++c) cfma_conj(d, q[c], x[c]);
+      if (j + 1 < k) {                                 // the next vector's loads fly during the sum
+        const double2* vj = V + (j + 1) * fstride + base;
+#pragma unroll
+        for (int c = 0; c < 6; ++c) { double2 t = vj[c * 256]; qn[c] = cmk(t.x, t.y); }
+      }
+      const double2 s = block_sum2(d.re, d.im, red[buf ^= 1]);
+#pragma unroll
+      for (int c = 0; c < 6; ++c) cfma(x[c], cmk(-s.x, -s.y), q[c]);
+      if (j + 1 < k)
+#pragma unroll
+        for (int c = 0; c < 6; ++c) q[c] = qn[c];
     }
     double nn = 0;
+#pragma unroll
     for (int c = 0; c < 6; ++c) nn += x[c].re * x[c].re + x[c].im * x[c].im;
-    const double2 s = block_sum2(nn, 0.0, red);
+    const double2 s = block_sum2(nn, 0.0, red[buf ^= 1]);
     const double inv = s.x > 0 ? 1.0 / sqrt(s.x) : 0.0;
+#pragma unroll
     for (int c = 0; c < 6; ++c) vk[c * 256] = make_double2(x[c].re * inv, x[c].im * inv);
   }
 }
@@ -666,10 +687,10 @@ __device__ __forceinline__ void assemble_dir(const Geom& g, const T2* U, const T
   }
 }
 
-// R = double with FP64 vectors and fields (the plain form, exact to rounding);
-// R = float with FP32 copies (the mixed form, whose coarse operator is stored
-// in FP32 and FP16: FP64 arithmetic is scarce on this GPU).  The entries are
-// written in FP64 either way.
+// FP64 vectors and fields (the plain form, exact to rounding).  The mixed form, whose
+// coarse operator is stored in FP32 and FP16, assembles it from FP32 copies
+// (assemble0_tiled_kernel): FP64 arithmetic is scarce on this GPU.  The entries
+// are written in FP64 either way.
 template <class R, class T2>
 __global__ void __launch_bounds__(256) assemble0_kernel(const T2* __restrict__ V, const T2* __restrict__ U,
                                                         const T2* __restrict__ A, double2* __restrict__ M,
@@ -729,6 +750,179 @@ __global__ void __launch_bounds__(256) assemble0_kernel(const T2* __restrict__ V
   }
 }
 
+// The FP32 form: CTA (block a, direction d).  The images of all 2N columns at
+// sixteen sites at a time are formed in shared memory (both chirality halves of
+// a vector from the same link products: with X the lower-to-upper spin block of
+// gamma, U acts on colour alone, so the half psi_u gives (U psi_u, S X^+ U psi_u) and
+// psi_l gives (S X U psi_l, U psi_l)), and the 2N x 2N block of products with the
+// vectors at those sites is a register-tiled matrix product: 4 x 4 entries a
+// thread, groups of threads sharing out the 96 terms of a chirality.  The kernel
+// above, one column a CTA, re-reads the N vectors for each of 2N columns and
+// reduces every product over its warps by shuffles: 14.4 ms at 16^3 x 32, N = 20.
+// The sums of a chunk are added to the totals per chunk, and the groups' totals
+// in FP64.
+constexpr int kAsmSites = 16;
+
+// w0, w1: the images of the upper and of the lower half at the site, -1/2 (1 + S gamma_MU) W u
+template <int MU, int S>
+__device__ __forceinline__ void assemble_half_hops(const float2* __restrict__ un, const Cplx<float> (&l)[9],
+                                                   Cplx<float> (&w0)[12], Cplx<float> (&w1)[12]) {
+  Cplx<float> h[6], gu[6], gl[6];
+#pragma unroll
+  for (int c = 0; c < 6; ++c) h[c] = Io<float, float2>::ldc(un + c * 256);
+  if (S < 0) su3_mul(l, h, gu);
+  else su3_dag_mul(l, h, gu);
+#pragma unroll
+  for (int c = 0; c < 6; ++c) h[c] = Io<float, float2>::ldc(un + (6 + c) * 256);
+  if (S < 0) su3_mul(l, h, gl);
+  else su3_dag_mul(l, h, gl);
+#pragma unroll
+  for (int c = 0; c < 6; ++c) { gu[c] = -0.5f * gu[c]; gl[c] = -0.5f * gl[c]; }
+  spin_reconstruct_add<MU, S>(gu, w0);                 // upper: gu, lower: S X^+ gu
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const Cplx<float> l0 = gl[c], l1 = gl[3 + c];
+    Cplx<float> x0, x1;                                // X (l0, l1), as spin_project
+    if (MU == 0) { x0 = mul_mi(l1); x1 = mul_mi(l0); }
+    else if (MU == 1) { x0 = cmk(-l1.re, -l1.im); x1 = l0; }
+    else if (MU == 2) { x0 = mul_mi(l0); x1 = mul_i(l1); }
+    else { x0 = l0; x1 = l1; }
+    w1[c] = S > 0 ? w1[c] + x0 : w1[c] - x0;
+    w1[3 + c] = S > 0 ? w1[3 + c] + x1 : w1[3 + c] - x1;
+    w1[6 + c] = w1[6 + c] + l0;
+    w1[9 + c] = w1[9 + c] + l1;
+  }
+}
+
+// the hop of direction MU, sign STEP, if it stays in the block (inside) or leaves it
+template <int MU, int STEP>
+__device__ __forceinline__ void assemble_image_hop(const Geom& g, const float2* __restrict__ vk,
+                                                   const float2* __restrict__ U, int blk, int loc, bool inside,
+                                                   Cplx<float> (&w0)[12], Cplx<float> (&w1)[12]) {
+  int nb, nl;
+  neighbour(g, blk, loc, MU, STEP, nb, nl);
+  const int cm = (loc >> (2 * MU)) & 3;
+  if ((STEP > 0 ? cm < 3 : cm > 0) != inside) return;
+  Cplx<float> l[9];
+  if (STEP > 0) load_link<float>(U, blk, MU, loc, l);
+  else load_link<float>(U, nb, MU, nl, l);
+  assemble_half_hops<MU, -STEP>(vk + (size_t)nb * 12 * 256 + nl, l, w0, w1);
+}
+
+__global__ void __launch_bounds__(256) assemble0_tiled_kernel(const float2* __restrict__ V,
+                                                              const float2* __restrict__ U,
+                                                              const float2* __restrict__ A,
+                                                              double2* __restrict__ M, Geom g, int N) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int blk = MG_CLAMP(kAggregate, blockIdx.x, g.nblocks), d = blockIdx.y;
+  const int Np = (N + 3) & ~3, ldw = 2 * Np + 2, ldv = Np + 2, n2 = 2 * N;
+  constexpr int KC = 12 * kAsmSites, KH = 6 * kAsmSites;
+  float2* W = reinterpret_cast<float2*>(smem_raw);              // [component * 16 + site][2 Np + 2]
+  float2* Vs = W + KC * ldw;                                    // [component * 16 + site][Np + 2]
+  const int tid = threadIdx.x;
+  const long long fs = g.V * 12;
+  const int T = Np / 2, G = min(16, 256 / (T * T));             // 4 x 4 tiles a side, groups over the terms
+  const int tile = tid % (T * T), grp = tid / (T * T), ti = tile % T, tj = tile / T;
+  const int chi = ti / (Np / 4), i0 = 4 * (ti % (Np / 4));
+  for (int e = tid; e < KC * (ldw + ldv); e += 256) W[e] = make_float2(0.f, 0.f);   // padding columns stay zero
+  const int mu = (d - 1) >> 1, nsites = d == 0 ? 256 : 64;
+  Cplx<float> tot[4][4];
+#pragma unroll
+  for (int p = 0; p < 4; ++p)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) tot[p][q] = cmk(0.f, 0.f);
+  for (int s0 = 0; s0 < nsites; s0 += kAsmSites) {
+    __syncthreads();
+    const int s = tid & (kAsmSites - 1);
+    int loc = s0 + s;
+    if (d > 0) {                                                // the face towards direction d
+      const int f = loc, low = f & ((1 << (2 * mu)) - 1);
+      loc = low | (((d & 1) ? 3 : 0) << (2 * mu)) | ((f >> (2 * mu)) << (2 * mu + 2));
+    }
+    for (int k = tid / kAsmSites; k < N; k += 256 / kAsmSites) {
+      const float2* vk = V + k * fs;
+      Cplx<float> w0[12], w1[12];
+      {
+        Cplx<float> u[12];
+        load_spinor<float>(vk, blk, loc, u);
+#pragma unroll
+        for (int c = 0; c < 12; ++c) Vs[(c * kAsmSites + s) * ldv + k] = make_float2(u[c].re, u[c].im);
+        if (d == 0) {
+          clover_apply<float>(A, blk, loc, u, w0);
+#pragma unroll
+          for (int c = 0; c < 6; ++c) {
+            w1[c] = cmk(0.f, 0.f);
+            w1[6 + c] = w0[6 + c];
+            w0[6 + c] = cmk(0.f, 0.f);
+          }
+        } else {
+#pragma unroll
+          for (int c = 0; c < 12; ++c) w0[c] = w1[c] = cmk(0.f, 0.f);
+        }
+      }
+      if (d == 0 || d == 1) assemble_image_hop<0, 1>(g, vk, U, blk, loc, d == 0, w0, w1);
+      if (d == 0 || d == 2) assemble_image_hop<0, -1>(g, vk, U, blk, loc, d == 0, w0, w1);
+      if (d == 0 || d == 3) assemble_image_hop<1, 1>(g, vk, U, blk, loc, d == 0, w0, w1);
+      if (d == 0 || d == 4) assemble_image_hop<1, -1>(g, vk, U, blk, loc, d == 0, w0, w1);
+      if (d == 0 || d == 5) assemble_image_hop<2, 1>(g, vk, U, blk, loc, d == 0, w0, w1);
+      if (d == 0 || d == 6) assemble_image_hop<2, -1>(g, vk, U, blk, loc, d == 0, w0, w1);
+      if (d == 0 || d == 7) assemble_image_hop<3, 1>(g, vk, U, blk, loc, d == 0, w0, w1);
+      if (d == 0 || d == 8) assemble_image_hop<3, -1>(g, vk, U, blk, loc, d == 0, w0, w1);
+#pragma unroll
+      for (int c = 0; c < 12; ++c) {
+        float2* q = W + (c * kAsmSites + s) * ldw + k;
+        q[0] = make_float2(w0[c].re, w0[c].im);
+        q[Np] = make_float2(w1[c].re, w1[c].im);
+      }
+    }
+    __syncthreads();
+    if (grp < G) {
+      Cplx<float> acc[4][4];
+#pragma unroll
+      for (int p = 0; p < 4; ++p)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[p][q] = cmk(0.f, 0.f);
+      for (int kk = chi * KH + grp; kk < (chi + 1) * KH; kk += G) {
+        const float4* xa = reinterpret_cast<const float4*>(Vs + kk * ldv + i0);
+        const float4* xb = reinterpret_cast<const float4*>(W + kk * ldw + 4 * tj);
+        const float4 a0 = xa[0], a1 = xa[1], b0 = xb[0], b1 = xb[1];
+        const Cplx<float> a[4] = {cmk(a0.x, a0.y), cmk(a0.z, a0.w), cmk(a1.x, a1.y), cmk(a1.z, a1.w)};
+        const Cplx<float> b[4] = {cmk(b0.x, b0.y), cmk(b0.z, b0.w), cmk(b1.x, b1.y), cmk(b1.z, b1.w)};
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) cfma_conj(acc[p][q], a[p], b[q]);
+      }
+#pragma unroll
+      for (int p = 0; p < 4; ++p)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) tot[p][q] = tot[p][q] + acc[p][q];
+    }
+  }
+  __syncthreads();
+  float2* red = W;                                              // [G][column][row], 2 Np x 2 Np
+  const int m2 = 2 * Np;
+  if (grp < G)
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int p = 0; p < 4; ++p)
+        red[(grp * m2 + 4 * tj + q) * m2 + 4 * ti + p] = make_float2(tot[p][q].re, tot[p][q].im);
+  __syncthreads();
+  double2* out = M + (size_t)(blk * 9 + d) * n2 * n2;
+  for (int e = tid; e < n2 * n2; e += 256) {
+    const int j = e / n2, i = e % n2;
+    const int jp = (j / N) * Np + j % N, ip = (i / N) * Np + i % N;
+    double a = 0, b = 0;
+    for (int q = 0; q < G; ++q) {
+      const float2 v = red[(q * m2 + jp) * m2 + ip];
+      a += v.x;
+      b += v.y;
+    }
+    out[e] = make_double2(a, b);
+  }
+}
+
 int launch_assemble0(const Geom& g, int prec, const void* V, const void* U, const void* A, void* M64, int N,
                      cudaStream_t s) {
   dim3 grid(g.nblocks, 2 * N);
@@ -736,11 +930,20 @@ int launch_assemble0(const Geom& g, int prec, const void* V, const void* U, cons
   if (prec == P64)
     assemble0_kernel<double, double2><<<grid, 256, smem, s>>>((const double2*)V, (const double2*)U,
                                                               (const double2*)A, (double2*)M64, g, N);
-  else if (prec == P32)
-    assemble0_kernel<float, float2><<<grid, 256, smem, s>>>((const float2*)V, (const float2*)U, (const float2*)A,
-                                                            (double2*)M64, g, N);
-  else
+  else if (prec == P32) {
+    const int Np = (N + 3) & ~3;
+    const size_t tiled = sizeof(float2) * 12 * kAsmSites * (3 * Np + 4);      // holds the groups' totals too
+    static bool attr = false;
+    if (!attr) {
+      SAPMG_CUDA_TRY(cudaFuncSetAttribute(assemble0_tiled_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          (int)(sizeof(float2) * 12 * kAsmSites * (3 * 32 + 4))));
+      attr = true;
+    }
+    assemble0_tiled_kernel<<<dim3(g.nblocks, 9), 256, tiled, s>>>((const float2*)V, (const float2*)U,
+                                                                  (const float2*)A, (double2*)M64, g, N);
+  } else {
     return MG_ERR_ARG;
+  }
   count_launches(1);
   SAPMG_CUDA_TRY(cudaGetLastError());
   return MG_OK;

@@ -82,15 +82,23 @@ int launch_gconv_forward(const Geom& g, const void* U, const void* W, const void
 // The same with BF16 links and BF16 weights (inference), FP32 activations and accumulation.
 int launch_gconv_forward_bf16(const Geom& g, const void* U, const void* W, const void* x, void* y, int cin, int cout,
                               cudaStream_t s);
+// work: scratch for gW, best gconv_wgrad_bytes of it (none: one slice of the sites)
+size_t gconv_wgrad_bytes(const Geom& g, int cin, int cout);
 int launch_gconv_backward(const Geom& g, const void* U, const void* W, const void* x, const void* gy, void* gx,
-                          void* gW, int cin, int cout, cudaStream_t s);
+                          void* gW, void* work, size_t work_bytes, int cin, int cout, cudaStream_t s);
 int launch_gate(const Geom& g, const void* x, const void* gy, void* out, int channels, cudaStream_t s);
 int launch_adam(size_t n, float* p, const float* gr, float* m, float* v, double lr, double b1, double b2,
                 double eps, int step, cudaStream_t s);
 
+// orth.cu: N FP32 vectors of n complex entries (contiguous, n even) orthonormalised in
+// vector order by Cholesky QR twice.  work: 1536 double2; *flag != 0 afterwards: a vector
+// is too close to the span of the earlier ones (V then spans what it did).
+int launch_cholqr2(void* V, int N, size_t n, double2* partial, double2* work, int* flag, cudaStream_t s);
+
 // sap.cu
-// pair_shape >= 0: an even number of right-hand sides in FP32 arithmetic
-// goes to the paired kernel with that launch shape; < 0: the one-RHS-per-CTA kernel.
+// b may be null (a zero right-hand side).  pair_shape >= 0: an even number of
+// right-hand sides in FP32 arithmetic goes to the paired kernel with that launch
+// shape; < 0: the one-RHS-per-CTA kernel.
 int launch_sap_colour(int prec, const Geom& g, void* z, const void* b, const void* U, const void* A, int colour,
                       int n_mr, int nrhs, cudaStream_t s, int pair_shape = 0, int* err = nullptr);
 // The paired kernels: two right-hand sides per thread (sap2.cu).  shape 0: two

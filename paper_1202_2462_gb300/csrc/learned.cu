@@ -10,10 +10,10 @@
 // site.  Gradients: G_z = dL/dRe z + i dL/dIm z.
 //
 // Fields are FP32 complex in the blocked layout, channel c at c * 12V; links
-// are the context's FP32 copy.  One thread per (site, output channel) in the
-// forward pass and per (site, input channel) in the input gradient; the weight
-// gradient is one CTA per (a, b, h) reducing over all sites in a fixed order
-// (deterministic).
+// are the context's FP32 copy.  With few output channels one thread per (site,
+// output channel) in the forward pass and per (site, input channel) in the input
+// gradient; with more, and for the weight gradient, blocked products over sites
+// (the tiled forms below), summed in a fixed order (deterministic).
 #include "internal.h"
 #include "stencil.cuh"
 
@@ -174,49 +174,206 @@ __global__ void __launch_bounds__(256) gconv_backward_input_kernel(Geom g, const
   store_spinor<float>(gx + (size_t)b * fs, blk, loc, acc);
 }
 
-// G_W[a][b][h][s][t] = sum_x sum_c G_y_a(x)[s][c] conj((T_h x_b)(x)[t][c]);
-// one CTA per (a, b, h), fixed-order reduction (per-thread sums over a
-// grid-stride of sites, then warps, then the CTA).
-__global__ void __launch_bounds__(256) gconv_backward_weight_kernel(Geom g, const float2* __restrict__ U,
-                                                                    const float2* __restrict__ x,
-                                                                    const float2* __restrict__ gy,
-                                                                    float2* __restrict__ gW, int cin) {
-  const int id = blockIdx.x;
-  const int h = id % 9, b = (id / 9) % cin, a = id / (9 * cin);
+// ------------------------------------------------------------ tiled forms
+// The layer and its input gradient as one blocked product: CTA (32 sites, sixteen
+// output channels).  Per chunk of eight (input channel, hop) pairs every thread
+// transports one pair's spinor at one site into shared memory, and thread
+// (output channel, two sites) accumulates its 4 spins x 2 sites x 3 colours over
+// the chunk's 32 input spins, five 16-byte loads for 24 complex products.  The
+// kernels above transport every input once per output channel (1.7 times the
+// needed flops, at the FP32 peak) or, for the gradient, read every output's
+// gradient from L1 once per hop and input channel: 1.16 and 2.4 ms for 16 -> 16
+// channels at 16^4, 58 Gflop.  Spin matrices and transports commute, so the input
+// gradient is the layer of the adjoint weights, G_x_b = sum_a sum_h
+// W[a][b][adj h]^dagger T_h G_y_a (BWD).  FP32-bound.
+constexpr int kPairs = 8, kTileSites = 32, kTileCh = 16;
+
+template <class TG, class TW, bool BWD>
+__global__ void __launch_bounds__(256, 2) gconv_tile_kernel(Geom g, const TG* __restrict__ U,
+                                                            const TW* __restrict__ W, const float2* __restrict__ x,
+                                                            float2* __restrict__ y, int cin, int cout) {
+  // cin: channels of x; cout: channels of y (BWD: the layer's output and input channels)
+  __shared__ __align__(16) float2 Ts[kPairs * 4][kTileSites * 3];     // [pair, spin][site, colour]
+  __shared__ __align__(16) float2 Ws[kPairs * 4][kTileCh * 4];        // [pair, input spin][channel, spin]
+  const int tid = threadIdx.x, part = blockIdx.x & 7, a0 = blockIdx.y * kTileCh;
+  const int blk = MG_CLAMP(kBlock, blockIdx.x >> 3, g.nblocks);
   const size_t fs = (size_t)g.V * 12;
-  float re[16], im[16];
+  const int ch = tid >> 4, cg = tid & 15;                             // channel a0 + ch, sites 2 cg and 2 cg + 1
+  const bool act = a0 + ch < cout;
+  const int npair = cin * 9;
+  Cplx<float> acc[4][6];
 #pragma unroll
-  for (int k = 0; k < 16; ++k) re[k] = im[k] = 0.f;
-  for (long long i = threadIdx.x; i < g.V; i += blockDim.x) {
-    const int blk = (int)(i >> 8), loc = (int)(i & 255);
-    Cplx<float> v[12], p[12];
-    transport_at(g, U, x + (size_t)b * fs, blk, loc, h, v);
-    load_spinor<float>(gy + (size_t)a * fs, blk, loc, p);
+  for (int s = 0; s < 4; ++s)
 #pragma unroll
-    for (int s = 0; s < 4; ++s)
+    for (int c = 0; c < 6; ++c) acc[s][c] = cmk(0.f, 0.f);
+  for (int p0 = 0; p0 < npair; p0 += kPairs) {
+    __syncthreads();
+    {
+      const int p = tid >> 5, site = tid & 31, q = p0 + p;
+      Cplx<float> v[12];
+      if (q < npair) {
+        transport_at<TG>(g, U, x + (size_t)(q / 9) * fs, blk, part * kTileSites + site, q % 9, v);
+      } else {
+#pragma unroll
+        for (int k = 0; k < 12; ++k) v[k] = cmk(0.f, 0.f);
+      }
 #pragma unroll
       for (int t = 0; t < 4; ++t)
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          // p[s][c] * conj(v[t][c])
-          const Cplx<float> l = p[s * 3 + c], r = v[t * 3 + c];
-          re[s * 4 + t] += l.re * r.re + l.im * r.im;
-          im[s * 4 + t] += l.im * r.re - l.re * r.im;
-        }
-  }
-  __shared__ float red[8][32];
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+        for (int c = 0; c < 3; ++c) Ts[p * 4 + t][site * 3 + c] = make_float2(v[t * 3 + c].re, v[t * 3 + c].im);
+    }
+    for (int e = tid; e < kTileCh * kPairs * 16; e += 256) {
+      const int a = e / (kPairs * 16), p = (e >> 4) & (kPairs - 1), st = e & 15, q = p0 + p;
+      Cplx<float> w = cmk(0.f, 0.f);
+      if (a0 + a < cout && q < npair) {
+        if (BWD)
+          w = conj(Io<float, TW>::ldc(W + (((size_t)(q / 9) * cout + a0 + a) * 9 + adjoint_hop(q % 9)) * 16 +
+                                      (st & 3) * 4 + (st >> 2)));
+        else
+          w = Io<float, TW>::ldc(W + ((size_t)(a0 + a) * npair + q) * 16 + st);
+      }
+      Ws[p * 4 + (st & 3)][a * 4 + (st >> 2)] = make_float2(w.re, w.im);
+    }
+    __syncthreads();
+    if (act) {
+#pragma unroll 4
+      for (int t = 0; t < kPairs * 4; ++t) {
+        const float4* tp = reinterpret_cast<const float4*>(&Ts[t][6 * cg]);
+        const float4* wp = reinterpret_cast<const float4*>(&Ws[t][4 * ch]);
+        const float4 t0 = tp[0], t1 = tp[1], t2 = tp[2], w0 = wp[0], w1 = wp[1];
+        const Cplx<float> tv[6] = {cmk(t0.x, t0.y), cmk(t0.z, t0.w), cmk(t1.x, t1.y),
+                                   cmk(t1.z, t1.w), cmk(t2.x, t2.y), cmk(t2.z, t2.w)};
+        const Cplx<float> wv[4] = {cmk(w0.x, w0.y), cmk(w0.z, w0.w), cmk(w1.x, w1.y), cmk(w1.z, w1.w)};
 #pragma unroll
-  for (int k = 0; k < 16; ++k) {
-    const float sr = warp_sum(re[k]), si = warp_sum(im[k]);
-    if (lane == 0) { red[w][2 * k] = sr; red[w][2 * k + 1] = si; }
+        for (int s = 0; s < 4; ++s)
+#pragma unroll
+          for (int c = 0; c < 6; ++c) cfma(acc[s][c], wv[s], tv[c]);
+      }
+    }
   }
-  __syncthreads();
-  if (threadIdx.x < 16) {
-    float sr = 0.f, si = 0.f;
-    for (int q = 0; q < 8; ++q) { sr += red[q][2 * threadIdx.x]; si += red[q][2 * threadIdx.x + 1]; }
-    gW[(size_t)id * 16 + threadIdx.x] = make_float2(sr, si);
+  if (!act) return;
+  float2* o = y + (size_t)(a0 + ch) * fs + (size_t)blk * 12 * 256 + part * kTileSites + 2 * cg;
+#pragma unroll
+  for (int s = 0; s < 4; ++s)
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+      *reinterpret_cast<float4*>(o + (s * 3 + c) * 256) =
+          make_float4(acc[s][c].re, acc[s][c].im, acc[s][3 + c].re, acc[s][3 + c].im);
+}
+
+// Weight gradient: CTA (sixteen (input channel, hop) pairs, RA output channels,
+// slice of the sites).  Per sixteen sites the output gradients and the transported
+// inputs (one pair and site a thread) are staged in shared memory and each thread
+// accumulates a 4 x 4 tile, (output channel, its 4 spins) x (pair, its 4 spins),
+// over the 48 (site, colour) terms; with RA < 16 the 256 / (16 RA) groups of
+// threads share the terms.  The slices' sums are added in slice order by a second
+// kernel, so the result is deterministic.  One CTA per (a, b, h) over all sites, as
+// before, transported every input once per output channel: 3.4 ms for 16 -> 16
+// channels at 16^4.
+template <int RA>
+__global__ void __launch_bounds__(256, 2) gconv_wgrad_tile_kernel(Geom g, const float2* __restrict__ U,
+                                                                  const float2* __restrict__ x,
+                                                                  const float2* __restrict__ gy,
+                                                                  float2* __restrict__ part, int cin, int cout,
+                                                                  int nslice) {
+  constexpr int kS = 16, G = 16 / RA, LDT = 64 + 2, LDG = RA * 4 + 2;
+  extern __shared__ __align__(16) float2 sm[];
+  float2* Ts = sm;                                                    // [site, colour][pair, spin]
+  float2* Gs = sm + kS * 3 * LDT;                                     // [site, colour][channel, spin]
+  const int tid = threadIdx.x, p0 = blockIdx.x * 16, a0 = blockIdx.y * RA, slice = blockIdx.z;
+  const int npair = cin * 9, tile = tid % (16 * RA), grp = tid / (16 * RA), tp = tile & 15, ta = tile >> 4;
+  const size_t fs = (size_t)g.V * 12;
+  Cplx<float> tot[4][4];
+#pragma unroll
+  for (int s = 0; s < 4; ++s)
+#pragma unroll
+    for (int t = 0; t < 4; ++t) tot[s][t] = cmk(0.f, 0.f);
+  const int nchunk = g.nblocks * 16;
+  for (int ch = slice; ch < nchunk; ch += nslice) {
+    const int blk = ch >> 4, l0 = (ch & 15) * kS;
+    __syncthreads();
+    {
+      const int p = tid >> 4, site = tid & 15, q = p0 + p;
+      Cplx<float> v[12];
+      if (q < npair) {
+        transport_at(g, U, x + (size_t)(q / 9) * fs, blk, l0 + site, q % 9, v);
+      } else {
+#pragma unroll
+        for (int k = 0; k < 12; ++k) v[k] = cmk(0.f, 0.f);
+      }
+#pragma unroll
+      for (int t = 0; t < 4; ++t)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) Ts[(site * 3 + c) * LDT + p * 4 + t] = make_float2(v[t * 3 + c].re, v[t * 3 + c].im);
+    }
+    for (int e = tid; e < RA * 12 * kS; e += 256) {
+      const int site = e & (kS - 1), k = (e / kS) % 12, a = e / (12 * kS);
+      const float2 v = a0 + a < cout ? gy[(size_t)(a0 + a) * fs + ((size_t)blk * 12 + k) * 256 + l0 + site]
+                                     : make_float2(0.f, 0.f);
+      Gs[(site * 3 + k % 3) * LDG + a * 4 + k / 3] = v;
+    }
+    __syncthreads();
+    Cplx<float> acc[4][4];
+#pragma unroll
+    for (int s = 0; s < 4; ++s)
+#pragma unroll
+      for (int t = 0; t < 4; ++t) acc[s][t] = cmk(0.f, 0.f);
+#pragma unroll 2
+    for (int k = grp; k < kS * 3; k += G) {
+      const float4* ga = reinterpret_cast<const float4*>(Gs + k * LDG + 4 * ta);
+      const float4* xa = reinterpret_cast<const float4*>(Ts + k * LDT + 4 * tp);
+      const float4 g0 = ga[0], g1 = ga[1], x0 = xa[0], x1 = xa[1];
+      const Cplx<float> gv[4] = {cmk(g0.x, g0.y), cmk(g0.z, g0.w), cmk(g1.x, g1.y), cmk(g1.z, g1.w)};
+      const Cplx<float> xv[4] = {cmk(x0.x, x0.y), cmk(x0.z, x0.w), cmk(x1.x, x1.y), cmk(x1.z, x1.w)};
+#pragma unroll
+      for (int s = 0; s < 4; ++s)
+#pragma unroll
+        for (int t = 0; t < 4; ++t) cfma_conj(acc[s][t], xv[t], gv[s]);
+    }
+#pragma unroll
+    for (int s = 0; s < 4; ++s)
+#pragma unroll
+      for (int t = 0; t < 4; ++t) tot[s][t] = tot[s][t] + acc[s][t];
   }
+  // the groups' totals, then W's layout: [slice][a][pair][s][t]
+  if (G > 1) {
+    __syncthreads();
+    float2* red = sm;                                                 // [G][16 RA tiles][16]
+#pragma unroll
+    for (int s = 0; s < 4; ++s)
+#pragma unroll
+      for (int t = 0; t < 4; ++t) red[(grp * 16 * RA + tile) * 16 + s * 4 + t] = make_float2(tot[s][t].re, tot[s][t].im);
+    __syncthreads();
+    for (int e = tid; e < 16 * RA * 16; e += 256) {
+      float re = 0.f, im = 0.f;
+      for (int q = 0; q < G; ++q) { re += red[q * 256 * RA + e].x; im += red[q * 256 * RA + e].y; }
+      const int pr = p0 + ((e >> 4) & 15), a = a0 + (e >> 8);
+      if (pr < npair && a < cout)
+        part[(((size_t)slice * cout + a) * npair + pr) * 16 + (e & 15)] = make_float2(re, im);
+    }
+  } else if (p0 + tp < npair && a0 + ta < cout) {
+    float2* o = part + (((size_t)slice * cout + a0 + ta) * npair + p0 + tp) * 16;
+#pragma unroll
+    for (int s = 0; s < 4; ++s)
+#pragma unroll
+      for (int t = 0; t < 4; ++t) o[s * 4 + t] = make_float2(tot[s][t].re, tot[s][t].im);
+  }
+}
+
+__global__ void __launch_bounds__(256) gconv_wgrad_sum_kernel(const float2* __restrict__ part, size_t n, int nslice,
+                                                              float2* __restrict__ gW) {
+  const size_t i = (size_t)blockIdx.x * 256 + threadIdx.x;
+  if (i >= n) return;
+  float re[4] = {0.f, 0.f, 0.f, 0.f}, im[4] = {0.f, 0.f, 0.f, 0.f};   // four chains: loads in flight
+  for (int s = 0; s < nslice; s += 4)
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (s + q < nslice) {
+        const float2 v = part[(size_t)(s + q) * n + i];
+        re[q] += v.x;
+        im[q] += v.y;
+      }
+  gW[i] = make_float2((re[0] + re[1]) + (re[2] + re[3]), (im[0] + im[1]) + (im[2] + im[3]));
 }
 
 // y = x / sqrt(1 + |x(site)|^2) per channel and site
@@ -276,11 +433,22 @@ __global__ void adam_kernel(size_t n, float* __restrict__ p, const float* __rest
   }
 }
 
+// Output channels from which the tiled form runs: below, most of its sixteen
+// channels a CTA would be idle and a thread per site transports little in vain.
+constexpr int kTiledFrom = 4;
+
 template <class TG, class TW>
 static int gconv_forward(const Geom& g, const void* U, const void* W, const void* x, void* y, int cin, int cout,
                          cudaStream_t s) {
   const size_t smem = sizeof(float2) * cin * 9 * 16;
   if (smem > 200 * 1024) return MG_ERR_ARG;
+  if (cout >= kTiledFrom) {
+    gconv_tile_kernel<TG, TW, false><<<dim3(g.nblocks * 8, (cout + kTileCh - 1) / kTileCh), 256, 0, s>>>(
+        g, (const TG*)U, (const TW*)W, (const float2*)x, (float2*)y, cin, cout);
+    count_launches(1);
+    SAPMG_CUDA_TRY(cudaGetLastError());
+    return MG_OK;
+  }
   static bool attr = false;
   if (!attr) {
     cudaFuncSetAttribute(gconv_forward_kernel<TG, TW>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
@@ -303,8 +471,37 @@ int launch_gconv_forward_bf16(const Geom& g, const void* U, const void* W, const
   return gconv_forward<__nv_bfloat162, __nv_bfloat162>(g, U, W, x, y, cin, cout, s);
 }
 
+// Slices of the sites of the weight gradient: two CTAs an SM over all tiles, no more
+// than the sixteen-site chunks, at least four chunks a slice where there are that many.
+static int wgrad_slices(const Geom& g, int cin, int cout) {
+  const int tiles = (cin * 9 + 15) / 16 * (cout >= 16 ? (cout + 15) / 16 : (cout >= 4 ? (cout + 3) / 4 : cout));
+  const int chunks = g.nblocks * 16;
+  return std::max(1, std::min((304 + tiles - 1) / tiles, std::max(1, chunks / 4)));
+}
+size_t gconv_wgrad_bytes(const Geom& g, int cin, int cout) {
+  return (size_t)wgrad_slices(g, cin, cout) * cout * cin * 9 * 16 * sizeof(float2);
+}
+
+template <int RA>
+static int wgrad_run(const Geom& g, const void* U, const void* x, const void* gy, float2* part, int cin, int cout,
+                     int nslice, cudaStream_t s) {
+  constexpr size_t stage = sizeof(float2) * 48 * (66 + RA * 4 + 2);
+  constexpr size_t red = RA < 16 ? sizeof(float2) * 256 * 16 : 0;
+  constexpr size_t smem = stage > red ? stage : red;
+  static bool attr = false;
+  if (!attr) {
+    SAPMG_CUDA_TRY(cudaFuncSetAttribute(gconv_wgrad_tile_kernel<RA>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)smem));
+    attr = true;
+  }
+  gconv_wgrad_tile_kernel<RA><<<dim3((cin * 9 + 15) / 16, (cout + RA - 1) / RA, nslice), 256, smem, s>>>(
+      g, (const float2*)U, (const float2*)x, (const float2*)gy, part, cin, cout, nslice);
+  count_launches(1);
+  return MG_OK;
+}
+
 int launch_gconv_backward(const Geom& g, const void* U, const void* W, const void* x, const void* gy, void* gx,
-                          void* gW, int cin, int cout, cudaStream_t s) {
+                          void* gW, void* work, size_t work_bytes, int cin, int cout, cudaStream_t s) {
   const size_t smem = sizeof(float2) * cout * 9 * 16;
   if (smem > 200 * 1024) return MG_ERR_ARG;
   static bool attr = false;
@@ -313,14 +510,26 @@ int launch_gconv_backward(const Geom& g, const void* U, const void* W, const voi
     attr = true;
   }
   if (gx) {
-    gconv_backward_input_kernel<<<dim3(g.nblocks, cin), 256, smem, s>>>(g, (const float2*)U, (const float2*)W,
-                                                                       (const float2*)gy, (float2*)gx, cin, cout);
+    if (cin >= kTiledFrom)
+      gconv_tile_kernel<float2, float2, true><<<dim3(g.nblocks * 8, (cin + kTileCh - 1) / kTileCh), 256, 0, s>>>(
+          g, (const float2*)U, (const float2*)W, (const float2*)gy, (float2*)gx, cout, cin);
+    else
+      gconv_backward_input_kernel<<<dim3(g.nblocks, cin), 256, smem, s>>>(
+          g, (const float2*)U, (const float2*)W, (const float2*)gy, (float2*)gx, cin, cout);
     count_launches(1);
   }
   if (gW) {
-    gconv_backward_weight_kernel<<<cout * cin * 9, 256, 0, s>>>(g, (const float2*)U, (const float2*)x,
-                                                               (const float2*)gy, (float2*)gW, cin);
-    count_launches(1);
+    const size_t n = (size_t)cout * cin * 9 * 16;
+    const int nslice = std::max(1, std::min(wgrad_slices(g, cin, cout), (int)(work_bytes / (n * sizeof(float2)))));
+    float2* part = nslice > 1 ? (float2*)work : (float2*)gW;         // one slice is gW itself
+    const int rc = cout >= 16 ? wgrad_run<16>(g, U, x, gy, part, cin, cout, nslice, s)
+                 : cout >= 4  ? wgrad_run<4>(g, U, x, gy, part, cin, cout, nslice, s)
+                              : wgrad_run<1>(g, U, x, gy, part, cin, cout, nslice, s);
+    if (rc != MG_OK) return rc;
+    if (nslice > 1) {
+      gconv_wgrad_sum_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(part, n, nslice, (float2*)gW);
+      count_launches(1);
+    }
   }
   SAPMG_CUDA_TRY(cudaGetLastError());
   return MG_OK;

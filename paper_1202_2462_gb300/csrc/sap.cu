@@ -11,7 +11,7 @@
 // memory for the neighbour accesses of D_i, and so does the correction e; the
 // block-wide dots are warp shuffles plus one shared-memory exchange.  The two
 // colours are two launches in stream order.
-#include "async.cuh"
+#include "cluster.cuh"
 #include "internal.h"
 #include "quad.cuh"
 #include "stencil.cuh"
@@ -75,7 +75,7 @@ __global__ void __launch_bounds__(256, (sizeof(R) == 4 ? 2 : 1))
   // right-hand side fastest in the grid (links and clover of a block shared through L2)
   const size_t off = (size_t)(blockIdx.x % nrhs) * g.V * 12;
   z += off;
-  b += off;
+  if (b) b += off;
   const int blk = colour_block(g, blockIdx.x / nrhs, colour);
   const int loc = threadIdx.x;
 
@@ -97,10 +97,10 @@ __global__ void __launch_bounds__(256, (sizeof(R) == 4 ? 2 : 1))
     hops_global_dir<2>(g, z, U, blk, loc, acc);
     asm volatile("" ::: "memory");
     hops_global_dir<3>(g, z, U, blk, loc, acc);
-    const TS* bq = b + (size_t)blk * 12 * 256 + loc;
+    const size_t bq = (size_t)blk * 12 * 256 + loc;
 #pragma unroll
     for (int c = 0; c < 12; ++c) {
-      rs[c * 256 + loc] = Io<R, TS>::ldc(bq + c * 256) + (R)0.5 * acc[c];
+      rs[c * 256 + loc] = (b ? Io<R, TS>::ldc(b + bq + c * 256) : cmk<R>(0, 0)) + (R)0.5 * acc[c];
       es[c * 256 + loc] = cmk<R>(0, 0);
     }
   }
@@ -157,43 +157,18 @@ __global__ void __launch_bounds__(256, (sizeof(R) == 4 ? 2 : 1))
 // clusters of eight warps).  rho stays in the shared memory of the CTA that owns
 // the site, its neighbours read it through distributed shared memory; e, p and
 // the update of a component belong to one thread.
-__device__ __forceinline__ void sap_cluster_barrier() {
-  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
-}
-__device__ __forceinline__ uint32_t sap_cluster_addr(uint32_t addr, int rank) {
-  uint32_t a;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(addr), "r"(rank));
-  return a;
-}
-__device__ __forceinline__ Cplx<double> ld_cluster(uint32_t a, double) {
-  Cplx<double> v;
-  asm volatile("ld.shared::cluster.v2.f64 {%0, %1}, [%2];" : "=d"(v.re), "=d"(v.im) : "r"(a) : "memory");
-  return v;
-}
-__device__ __forceinline__ Cplx<float> ld_cluster(uint32_t a, float) {
-  Cplx<float> v;
-  asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.re), "=f"(v.im) : "r"(a) : "memory");
-  return v;
-}
-__device__ __forceinline__ void st_cluster(uint32_t a, double v) {
-  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
-}
-__device__ __forceinline__ void st_cluster(uint32_t a, float v) {
-  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
-}
-
 // Rows 3 M .. 3 M + 2 of D_i rho at the warp's sites (rsa: the address of the CTAs' rho, [12][32])
 template <int M, class R, class TG>
 __device__ __forceinline__ void quad_block(const Geom& g, const TG* __restrict__ U, const TG* __restrict__ A,
                                            const Cplx<R>* rs, uint32_t rsa, int blk, int loc, Cplx<R>* part,
                                            Cplx<R> (&out)[3]) {
   const int ls = 1 << (2 * M), cm = (loc >> (2 * M)) & 3, lane = loc & 31;
-  auto at = [&](int l) { return sap_cluster_addr(rsa + (uint32_t)((l & 31) * sizeof(Cplx<R>)), l >> 5); };
+  auto at = [&](int l) { return cluster_addr(rsa + (uint32_t)((l & 31) * sizeof(Cplx<R>)), l >> 5); };
   const uint32_t q0 = at(cm < 3 ? loc + ls : loc), q1 = at(cm > 0 ? loc - ls : loc);
   Cplx<R> acc[12];
   quad_hops<M, R, TG, false>(
       g, U, blk, loc,
-      [&](int step, int c) { return ld_cluster((step > 0 ? q0 : q1) + (uint32_t)(c * 32 * sizeof(Cplx<R>)), R(0)); },
+      [&](int step, int c) { return cluster_ld((step > 0 ? q0 : q1) + (uint32_t)(c * 32 * sizeof(Cplx<R>)), R(0)); },
       [&](int step) { return step > 0 ? cm < 3 : cm > 0; }, acc);
   quad_clover<M, R>(A, blk, loc, [&](int c) { return rs[c * 32 + lane]; }, out);
   quad_swap<M>(part, lane, acc, out);
@@ -212,7 +187,7 @@ __global__ void __launch_bounds__(128) sap_cluster_kernel(TS* __restrict__ z, co
   const int id = blockIdx.x >> 3;
   const size_t off = (size_t)(id % nrhs) * g.V * 12;
   z += off;
-  b += off;
+  if (b) b += off;
   const int blk = colour_block(g, id / nrhs, colour);
   const size_t own = ((size_t)blk * 12 + 3 * m) * 256 + loc;   // this thread's components 3 m .. 3 m + 2
   Cplx<R> ro[3], e[3], p[3];
@@ -224,12 +199,12 @@ __global__ void __launch_bounds__(128) sap_cluster_kernel(TS* __restrict__ z, co
   }
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
-    ro[k] = Io<R, TS>::ldc(b + own + k * 256) - p[k];
+    ro[k] = (b ? Io<R, TS>::ldc(b + own + k * 256) : cmk<R>(0, 0)) - p[k];
     rs[(3 * m + k) * 32 + lane] = ro[k];
     e[k] = cmk<R>(0, 0);
   }
   for (int it = 0; it < n_mr; ++it) {
-    sap_cluster_barrier();                               // rho of every site written, part free again
+    cluster_barrier();                               // rho of every site written, part free again
     switch (m) {
       case 0: quad_block<0, R, TG>(g, U, A, rs, rsa, blk, loc, part, p); break;
       case 1: quad_block<1, R, TG>(g, U, A, rs, rsa, blk, loc, part, p); break;
@@ -246,11 +221,11 @@ __global__ void __launch_bounds__(128) sap_cluster_kernel(TS* __restrict__ z, co
 #pragma unroll
     for (int q = 0; q < 3; ++q) v[q] = warp_sum(v[q]);
     if (lane < 8) {                                      // lane q: this warp's sums to CTA q
-      const uint32_t a = sap_cluster_addr(smem_u32(&red[it & 1][rank * 4 + m][0]), lane);
+      const uint32_t a = cluster_addr(smem_u32(&red[it & 1][rank * 4 + m][0]), lane);
 #pragma unroll
-      for (int q = 0; q < 3; ++q) st_cluster(a + (uint32_t)(q * sizeof(R)), v[q]);
+      for (int q = 0; q < 3; ++q) cluster_st(a + (uint32_t)(q * sizeof(R)), v[q]);
     }
-    sap_cluster_barrier();                               // the sums arrived; every neighbour read of rho done
+    cluster_barrier();                               // the sums arrived; every neighbour read of rho done
     // the 32 warps' sums, one a lane
 #pragma unroll
     for (int q = 0; q < 3; ++q) v[q] = warp_sum(red[it & 1][lane][q]);
@@ -263,7 +238,7 @@ __global__ void __launch_bounds__(128) sap_cluster_kernel(TS* __restrict__ z, co
       rs[(3 * m + k) * 32 + lane] = ro[k];
     }
   }
-  sap_cluster_barrier();                                 // n_mr = 0: the residuals' reads of z are over
+  cluster_barrier();                                 // n_mr = 0: the residuals' reads of z are over
 #pragma unroll
   for (int k = 0; k < 3; ++k) Io<R, TS>::st(z + own + k * 256, Io<R, TS>::ldc(z + own + k * 256) + e[k]);
 }
@@ -278,17 +253,8 @@ static bool cluster_wins(const Geom& g, int nrhs) {
 template <class R, class TS, class TG>
 static int run_cluster(const Geom& g, void* z, const void* b, const void* U, const void* A, int colour, int n_mr,
                        int nrhs, cudaStream_t s) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(g.nblocks / 2 * nrhs * 8));
-  cfg.blockDim = dim3(128);
-  cfg.stream = s;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = 8;
-  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  SAPMG_CUDA_TRY(cudaLaunchKernelEx(&cfg, sap_cluster_kernel<R, TS, TG>, (TS*)z, (const TS*)b, (const TG*)U,
+  ClusterLaunch l((unsigned)(g.nblocks / 2 * nrhs * 8), 128, 0, 8, s);
+  SAPMG_CUDA_TRY(cudaLaunchKernelEx(&l.cfg, sap_cluster_kernel<R, TS, TG>, (TS*)z, (const TS*)b, (const TG*)U,
                                     (const TG*)A, g, colour, n_mr, nrhs));
   count_launches(1);
   return MG_OK;

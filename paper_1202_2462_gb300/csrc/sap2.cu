@@ -78,7 +78,7 @@ __global__ void __launch_bounds__(256, MINB)
   const size_t stride = (size_t)g.V * 12;                                // one right-hand side
   const size_t off = (size_t)(blockIdx.x % npairs) * 2 * stride;
   z += off;
-  b += off;
+  if (b) b += off;
   const int blk = colour_block(g, blockIdx.x / npairs, colour);
   const int loc = threadIdx.x;
   const size_t site0 = (size_t)blk * 12 * 256 + loc;
@@ -96,7 +96,7 @@ __global__ void __launch_bounds__(256, MINB)
     global_hops2<3>(g, z, stride, U, blk, loc, acc);
 #pragma unroll
     for (int c = 0; c < 12; ++c) {
-      const P2 bb = ldg2(b, stride, site0 + c * 256);
+      const P2 bb = ldb2(b, stride, site0 + c * 256);
       P2 r;
       r.re = sub2(bb.re, acc[c].re);
       r.im = sub2(bb.im, acc[c].im);
@@ -268,7 +268,7 @@ __device__ __forceinline__ void residual_pair(const Geom& g, const float2* __res
   }
 #pragma unroll
   for (int c = 0; c < 12; ++c) {
-    const P2 bb = ldg2(b, stride, site0 + c * 256);
+    const P2 bb = ldb2(b, stride, site0 + c * 256);
     P2 r;
     r.re = sub2(bb.re, acc[c].re);
     r.im = sub2(bb.im, acc[c].im);
@@ -314,7 +314,7 @@ __global__ void __launch_bounds__(256, 1)
   }
   for (int pr = 0; pr < npairs; ++pr) {
     float2* zp = z + (size_t)pr * 2 * stride;
-    if (pr > 0) residual_pair<true>(g, zp, b + (size_t)pr * 2 * stride, stride, U, A, Us, As, blk, loc, rs);
+    if (pr > 0) residual_pair<true>(g, zp, b ? b + (size_t)pr * 2 * stride : nullptr, stride, U, A, Us, As, blk, loc, rs);
     P2 e[12];
     for (int it = 0; it < n_mr; ++it) {
       __syncthreads();                                 // rho of every site written
@@ -487,7 +487,7 @@ __device__ __forceinline__ void residual_b(const float2* __restrict__ b, size_t 
 #pragma unroll
   for (int k = 0; k < 6; ++k) {
     const int c = 6 * H + k;
-    const P2 bb = ldg2(b, stride, site0 + c * 256);
+    const P2 bb = ldb2(b, stride, site0 + c * 256);
     P2 r;
     r.re = sub2(bb.re, acc[c].re);
     r.im = sub2(bb.im, acc[c].im);
@@ -604,7 +604,7 @@ __global__ void __launch_bounds__(512, 1)
   for (int pr = 0; pr < npairs; ++pr) {
     float2* zp = z + (size_t)pr * 2 * stride;
     if (pr > 0) {
-      const float2* bp = b + (size_t)pr * 2 * stride;
+      const float2* bp = b ? b + (size_t)pr * 2 * stride : nullptr;
       __syncthreads();                      // every read of the previous pair's swap buffer done
       if (h0) residual_a<0, true>(g, zp, stride, U, A, Us, As, blk, loc, xs, acc);
       else residual_a<1, true>(g, zp, stride, U, A, Us, As, blk, loc, xs, acc);

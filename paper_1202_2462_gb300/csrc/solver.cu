@@ -219,6 +219,9 @@ struct mg_ctx {
   int N0 = 0;
   void* V64 = nullptr;                     // locally orthonormal test vectors, FP64 vector-major
   void* Vs64 = nullptr;                    // set-up only: the smoothed vectors before local orthonormalisation
+  void* net_work = nullptr;                // weight gradients of the set-up network (allocated on first use)
+  size_t net_work_bytes = 0;
+  double2* gram = nullptr;                 // set-up only: work of the FP32 orthonormalisation
   void* part2_buf = nullptr;               // set-up only (three levels): part-1 vectors kept for set-up part 2
   const std::vector<double2>* load_v0 = nullptr;  // mg_setup_load: the saved level-0 vectors (host)
   const std::vector<double2>* load_w1 = nullptr;  // mg_setup_load: the saved level-1 vectors (host, three levels)
@@ -1172,14 +1175,22 @@ static int check_finite(mg_ctx* c, const double* x, size_t n_doubles) {
   return h ? fail(MG_ERR_NONFINITE, "non-finite value in input field") : MG_OK;
 }
 
-// Global orthonormalisation of the N set-up vectors (FP64): classical
-// Gram-Schmidt against the previous vectors, applied twice, then normalise.
-// Classical Gram-Schmidt with a second pass of N vectors (type P64, or P32
-// for the mixed form's set-up vectors).
+// Global orthonormalisation of the N set-up vectors (type P64, or P32 for the
+// mixed form's): FP32 by Cholesky QR twice where no vector is nearly in the span of
+// the earlier ones (orth.cu); else classical Gram-Schmidt against the previous
+// vectors, applied twice, then normalise.
 static int orthonormalise(mg_ctx* c, void* V, int N, size_t n, int type = P64) {
   const BVec one = bvec(n, 1, n);
   const size_t eb = type == P64 ? 16 : 8;
   auto Vk = [&](int k) { return (void*)((char*)V + (size_t)k * n * eb); };
+  if (type == P32 && c->gram && N >= 2) {
+    int* flag = (int*)(c->gram + 1536);
+    int bad = 0;
+    TRY(launch_cholqr2(V, N, n, c->partial, c->gram, flag, c->s));
+    SAPMG_CUDA_TRY(cudaMemcpyAsync(&bad, flag, sizeof(int), cudaMemcpyDeviceToHost, c->s));
+    SAPMG_CUDA_TRY(cudaStreamSynchronize(c->s));
+    if (!bad) return MG_OK;
+  }
   std::vector<const void*> vl;
   for (int k = 0; k < N; ++k) {
     for (int pass = 0; pass < 2 && k > 0; ++pass) {
@@ -1217,6 +1228,8 @@ static int build_level0_operators(mg_ctx* c) {
   const bool f32 = c->vt == P32 && c->setup_fp32 && c->U32 && c->A32 && c->Z &&
                    (size_t)c->m * c->p.nrhs_max >= (size_t)N;
   if (f32) {
+    c->gram = (double2*)c->alloc(sizeof(double2) * 1537);
+    if (!c->gram) return fail(MG_ERR_OOM, "set-up workspace");
     TRY(blas_axpby2(P64, scal_all(1.0, N), c->V64, n, P32, scal_all(0.0, N), c->Z, n, n, N, c->s));
     TRY(launch_assemble0(c->g, P32, c->Z, c->U32, c->A32, L.M64, N, c->s));
   } else {
@@ -1460,14 +1473,21 @@ static int setup_level0(mg_ctx* c) {
   // form, or a basis too small for N vectors, keeps them FP64.
   const bool f32 = c->vt == P32 && c->setup_fp32 && p.setup_iters > 0 && (size_t)c->m * p.nrhs_max >= (size_t)N;
   if (f32) {
+    c->gram = (double2*)c->alloc(sizeof(double2) * 1537);
+    if (!c->gram) return fail(MG_ERR_OOM, "set-up workspace");
     TRY(blas_axpby2(P64, scal_all(1.0, N), c->V64, n, P32, scal_all(0.0, N), c->Z, n, n, N, c->s));
     for (int it = 0; it < p.setup_iters; ++it) {
-      for (int k = 0; k < N; ++k) TRY(smoother_sweeps(c, c->zero_f, (char*)c->Z + (size_t)k * n * 8, 1, 1));
+      // in pairs (the paired kernel), an odd last vector on its own
+      if (N > 1) TRY(smoother_sweeps(c, nullptr, c->Z, 1, N & ~1));
+      if (N & 1) TRY(smoother_sweeps(c, nullptr, (char*)c->Z + (size_t)(N - 1) * n * 8, 1, 1));
       t_sweep += clk.lap();
       TRY(orthonormalise(c, c->Z, N, n, P32));
       t_orth += clk.lap();
     }
     TRY(blas_axpby2(P32, scal_all(1.0, N), c->Z, n, P64, scal_all(0.0, N), c->V64, n, n, N, c->s));
+    SAPMG_CUDA_TRY(cudaStreamSynchronize(c->s));
+    c->release(c->gram);
+    c->gram = nullptr;
   }
   for (int it = 0; it < p.setup_iters && !f32; ++it) {
     for (int k = 0; k < N; ++k) {
@@ -2474,7 +2494,23 @@ int mg_net_layer_backward(mg_ctx* c, int cin, int cout, const void* W, const voi
                           void* gW) {
   TRY(net_state(c, cin, cout));
   if (!W || !x || !gy || (!gx && !gW)) return fail(MG_ERR_ARG, "bad argument");
-  return launch_gconv_backward(c->g, c->U32, W, x, gy, gx, gW, cin, cout, c->s);
+  if (gW) {
+    // the slices' sums: grown when a layer needs more and kept by the context; where
+    // that cannot be (stream capture, no memory) the kernel takes fewer slices
+    const size_t bytes = gconv_wgrad_bytes(c->g, cin, cout);
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (bytes > c->net_work_bytes && cudaStreamIsCapturing(c->s, &cap) == cudaSuccess &&
+        cap == cudaStreamCaptureStatusNone) {
+      if (c->net_work) {
+        SAPMG_CUDA_TRY(cudaStreamSynchronize(c->s));         // an earlier layer may still use the old one
+        c->release(c->net_work);
+      }
+      c->net_work = c->alloc(bytes);
+      c->net_work_bytes = c->net_work ? bytes : 0;
+    }
+  }
+  return launch_gconv_backward(c->g, c->U32, W, x, gy, gx, gW, c->net_work, c->net_work_bytes, cin, cout,
+                               c->s);
 }
 
 int mg_net_gate_forward(mg_ctx* c, int channels, const void* x, void* y) {

@@ -1,0 +1,55 @@
+"""The set-up network's tiled layer kernels at channel counts around their tile
+sizes (4 and 16 output channels, 16 (input channel, hop) pairs), against the
+FP64 oracle."""
+
+import numpy as np
+import pytest
+
+import synth
+from oracle import learned as L
+from tests.gpu_util import torch_cuda, dev, host, rel, round_storage
+
+pytestmark = pytest.mark.gpu
+
+DIMS = (8, 8, 8, 16)
+
+
+def _blocked(torch, s, x):
+    from paper_1202_2462_gb300.learned import GaugeNet
+    return torch.cat([GaugeNet.blocked(s, dev(torch, x[c], torch.complex64)) for c in range(x.shape[0])])
+
+
+def _canonical(torch, s, y, c):
+    from paper_1202_2462_gb300.learned import GaugeNet
+    fs = y.numel() // c
+    return np.stack([host(GaugeNet.canonical(s, y[k * fs:(k + 1) * fs].contiguous()))[0] for k in range(c)])
+
+
+# FP32 sums of 36 cin products (forward), of 36 cout (input gradient) and of 3 V
+# (weights): 2e-6 as in the layer's own parity test
+@pytest.mark.parametrize("cin,cout", [(1, 1), (1, 4), (4, 3), (3, 5), (2, 16), (16, 2), (5, 17)])
+def test_layer_tiles(cin, cout):
+    torch = torch_cuda()
+    import paper_1202_2462_gb300 as G
+    u = synth.random_gauge_field(DIMS, 0.4, 321)
+    s = G.Solver(dev(torch, u), 1.0, -0.1, n_levels=1, precision="bf16", fgmres_m=1, antiperiodic_t=0)
+    w = L.init_weights([(cout, cin)], 1)[0] * 3.0
+    x = synth.random_spinor(DIMS, 322, nvec=cin)
+    gy = synth.random_spinor(DIMS, 323, nvec=cout)
+    wd, xd, gyd = dev(torch, w, torch.complex64), _blocked(torch, s, x), _blocked(torch, s, gy)
+    yd = torch.empty(cout * xd.numel() // cin, dtype=torch.complex64, device="cuda")
+    G.mg_net_layer_forward(s.ctx, cin, cout, wd, xd, yd)
+    assert rel(_canonical(torch, s, yd, cout), L.layer(u, w, x)) < 2e-6
+    gxd, gwd = torch.empty_like(xd), torch.empty_like(wd)
+    G.mg_net_layer_backward(s.ctx, cin, cout, wd, xd, gyd, gxd, gwd)
+    gx, gw = L.layer_backward(u, w, x, gy)
+    assert rel(_canonical(torch, s, gxd, cin), gx) < 2e-6
+    assert rel(host(gwd), gw) < 2e-6
+    again = torch.empty_like(wd)
+    G.mg_net_layer_backward(s.ctx, cin, cout, wd, xd, gyd, None, again)
+    assert torch.equal(again, gwd)
+    wb = torch.view_as_real(wd).to(torch.bfloat16).contiguous()
+    G.mg_net_layer_forward_bf16(s.ctx, cin, cout, wb, xd, yd)
+    ref = L.layer(round_storage(u, "bf16"), round_storage(w, "bf16"), x)
+    assert rel(_canonical(torch, s, yd, cout), ref) < 2e-6
+    s.close()
