@@ -6,12 +6,43 @@
 // multiply and FMA is the packed two-wide instruction (pair.cuh), with the -1/2
 // of the hopping term folded into the reconstruction FMAs.  The pairs of one
 // block are adjacent CTAs, so the block's fields are shared through L1/L2.
+#include "async.cuh"
 #include "internal.h"
 #include "pair.cuh"
 
 namespace sapmg {
 namespace {
 using namespace pair;
+
+// Bound by the latency of the neighbours' spinors (L1 holds a quarter of the
+// loads).  So a CTA asks for the spinors and fields of the CTA about one wave later
+// to be brought into L2 (12 right-hand sides, FP32, 737280 sites: 783 -> 733 us; the
+// same in the one-RHS kernel, with three CTAs an SM, made it slower: 203 -> 267 us),
+// and what is used once stays out of L1: clover words by no-allocate loads, the
+// results by streaming stores (733 -> 711 us; the links, each used twice, lose
+// by it: 735 us; the block's spinors staged in shared memory: 794 us).
+constexpr unsigned kAhead = 304;
+
+// a clover entry as a broadcast pair, loaded past L1
+__device__ __forceinline__ B2 once(const float2* p) {
+  float x, y;
+  asm volatile("ld.global.nc.L1::no_allocate.v2.f32 {%0, %1}, [%2];" : "=f"(x), "=f"(y) : "l"(p));
+  B2 b; b.r = f2(x); b.i = f2(y); b.ni = f2(-y); return b;
+}
+__device__ __forceinline__ unsigned once_word(const void* p) {
+  unsigned w;
+  asm volatile("ld.global.nc.L1::no_allocate.b32 %0, [%1];" : "=r"(w) : "l"(p));
+  return w;
+}
+__device__ __forceinline__ B2 once(const __nv_bfloat162* p) {
+  const unsigned w = once_word(p);
+  const float re = __uint_as_float(w << 16), im = __uint_as_float(w & 0xffff0000u);
+  B2 b; b.r = f2(re); b.i = f2(im); b.ni = f2(-im); return b;
+}
+__device__ __forceinline__ B2 once(const __half2* p) {
+  const float2 v = half2_bits_to_float2(once_word(p));
+  B2 b; b.r = f2(v.x); b.i = f2(v.y); b.ni = f2(-v.y); return b;
+}
 
 template <class TG>
 __global__ void __launch_bounds__(256, 2)
@@ -21,12 +52,34 @@ __global__ void __launch_bounds__(256, 2)
   const int loc = threadIdx.x;
   const size_t stride = (size_t)g.V * 12;
   const size_t off = (size_t)(blockIdx.x % npairs) * 2 * stride;
+  if (threadIdx.x == 0) {
+    const unsigned id = blockIdx.x + kAhead;
+    if (id < gridDim.x) {
+      const size_t b2 = id / npairs;
+      const float2* f = in + (id % npairs) * 2 * stride + b2 * 12 * 256;
+      bulk_prefetch_l2(f, 12 * 256 * sizeof(float2));
+      bulk_prefetch_l2(f + stride, 12 * 256 * sizeof(float2));
+      if (id % npairs == 0) {
+        bulk_prefetch_l2(U + b2 * 36 * 256, 36 * 256 * sizeof(TG));
+        bulk_prefetch_l2(A + b2 * 36 * 256, 36 * 256 * sizeof(TG));
+      }
+    }
+  }
   in += off;
   out += off;
   const size_t site0 = (size_t)blk * 12 * 256 + loc;
   // acc = A psi - 1/2 sum(hops) = D psi
   P2 acc[12];
-  clover2<TG>(A, blk, loc, [&](int k) { return ldg2(in, stride, site0 + k * 256); }, acc);
+#pragma unroll
+  for (int chi = 0; chi < 2; ++chi) {
+    P2 p[6], o[6];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) p[k] = ldg2(in, stride, site0 + (chi * 6 + k) * 256);
+    const TG* a = A + ((size_t)(blk * 36 + chi * 18)) * 256 + loc;
+    clover2_chi([&](int q) { return once(a + q * 256); }, p, o);
+#pragma unroll
+    for (int k = 0; k < 6; ++k) acc[chi * 6 + k] = o[k];
+  }
   global_hops2<0>(g, in, stride, U, blk, loc, acc);
   global_hops2<1>(g, in, stride, U, blk, loc, acc);
   global_hops2<2>(g, in, stride, U, blk, loc, acc);
@@ -34,8 +87,8 @@ __global__ void __launch_bounds__(256, 2)
 #pragma unroll
   for (int c = 0; c < 12; ++c) {
     const size_t i = site0 + c * 256;
-    out[i] = make_float2(acc[c].re.x, acc[c].im.x);
-    out[i + stride] = make_float2(acc[c].re.y, acc[c].im.y);
+    __stcs(out + i, make_float2(acc[c].re.x, acc[c].im.x));
+    __stcs(out + i + stride, make_float2(acc[c].re.y, acc[c].im.y));
   }
 }
 
