@@ -15,11 +15,12 @@
 // gradient; with more, and for the weight gradient, blocked products over sites
 // (the tiled forms below), summed in a fixed order (deterministic).
 #include "internal.h"
-#include "stencil.cuh"
+#include "pair.cuh"
 
 namespace sapmg {
 
 namespace {
+using namespace pair;
 
 // T_h psi_b at (blk, loc) into v (4 spins x 3 colours); links in storage type TG
 template <class TG = float2>
@@ -187,25 +188,27 @@ __global__ void __launch_bounds__(256) gconv_backward_input_kernel(Geom g, const
 // gradient is the layer of the adjoint weights, G_x_b = sum_a sum_h
 // W[a][b][adj h]^dagger T_h G_y_a (BWD).  FP32-bound.
 constexpr int kPairs = 8, kTileSites = 32, kTileCh = 16;
+constexpr int kLdW = kTileCh * 4 + 4;              // a row more of 64 bytes: the 16-byte stores of W spread
 
 template <class TG, class TW, bool BWD>
 __global__ void __launch_bounds__(256, 2) gconv_tile_kernel(Geom g, const TG* __restrict__ U,
                                                             const TW* __restrict__ W, const float2* __restrict__ x,
                                                             float2* __restrict__ y, int cin, int cout) {
   // cin: channels of x; cout: channels of y (BWD: the layer's output and input channels)
-  __shared__ __align__(16) float2 Ts[kPairs * 4][kTileSites * 3];     // [pair, spin][site, colour]
-  __shared__ __align__(16) float2 Ws[kPairs * 4][kTileCh * 4];        // [pair, input spin][channel, spin]
+  // [pair, spin][colour][two sites]: (re, re, im, im); [pair, input spin][channel, spin]: (re, re, im, im)
+  __shared__ __align__(16) float4 Ts[kPairs * 4][3][kTileSites / 2];
+  extern __shared__ __align__(16) float4 Ws[];                        // [kPairs * 4][kLdW]
   const int tid = threadIdx.x, part = blockIdx.x & 7, a0 = blockIdx.y * kTileCh;
   const int blk = MG_CLAMP(kBlock, blockIdx.x >> 3, g.nblocks);
   const size_t fs = (size_t)g.V * 12;
   const int ch = tid >> 4, cg = tid & 15;                             // channel a0 + ch, sites 2 cg and 2 cg + 1
   const bool act = a0 + ch < cout;
   const int npair = cin * 9;
-  Cplx<float> acc[4][6];
+  P2 acc[4][3];                                                       // [spin][colour], the two sites packed
 #pragma unroll
   for (int s = 0; s < 4; ++s)
 #pragma unroll
-    for (int c = 0; c < 6; ++c) acc[s][c] = cmk(0.f, 0.f);
+    for (int c = 0; c < 3; ++c) acc[s][c].re = acc[s][c].im = f2(0.f);
   for (int p0 = 0; p0 < npair; p0 += kPairs) {
     __syncthreads();
     {
@@ -220,34 +223,45 @@ __global__ void __launch_bounds__(256, 2) gconv_tile_kernel(Geom g, const TG* __
 #pragma unroll
       for (int t = 0; t < 4; ++t)
 #pragma unroll
-        for (int c = 0; c < 3; ++c) Ts[p * 4 + t][site * 3 + c] = make_float2(v[t * 3 + c].re, v[t * 3 + c].im);
+        for (int c = 0; c < 3; ++c) {
+          float* o = reinterpret_cast<float*>(&Ts[p * 4 + t][c][site >> 1]) + (site & 1);
+          o[0] = v[t * 3 + c].re;
+          o[2] = v[t * 3 + c].im;
+        }
     }
     for (int e = tid; e < kTileCh * kPairs * 16; e += 256) {
-      const int a = e / (kPairs * 16), p = (e >> 4) & (kPairs - 1), st = e & 15, q = p0 + p;
+      const int a = e / (kPairs * 16), p = (e >> 4) & (kPairs - 1), so = e & 3, ti = (e >> 2) & 3, q = p0 + p;
       Cplx<float> w = cmk(0.f, 0.f);
       if (a0 + a < cout && q < npair) {
         if (BWD)
           w = conj(Io<float, TW>::ldc(W + (((size_t)(q / 9) * cout + a0 + a) * 9 + adjoint_hop(q % 9)) * 16 +
-                                      (st & 3) * 4 + (st >> 2)));
+                                      ti * 4 + so));
         else
-          w = Io<float, TW>::ldc(W + ((size_t)(a0 + a) * npair + q) * 16 + st);
+          w = Io<float, TW>::ldc(W + ((size_t)(a0 + a) * npair + q) * 16 + so * 4 + ti);
       }
-      Ws[p * 4 + (st & 3)][a * 4 + (st >> 2)] = make_float2(w.re, w.im);
+      Ws[(p * 4 + ti) * kLdW + a * 4 + so] = make_float4(w.re, w.re, w.im, w.im);
     }
     __syncthreads();
     if (act) {
 #pragma unroll 4
       for (int t = 0; t < kPairs * 4; ++t) {
-        const float4* tp = reinterpret_cast<const float4*>(&Ts[t][6 * cg]);
-        const float4* wp = reinterpret_cast<const float4*>(&Ws[t][4 * ch]);
-        const float4 t0 = tp[0], t1 = tp[1], t2 = tp[2], w0 = wp[0], w1 = wp[1];
-        const Cplx<float> tv[6] = {cmk(t0.x, t0.y), cmk(t0.z, t0.w), cmk(t1.x, t1.y),
-                                   cmk(t1.z, t1.w), cmk(t2.x, t2.y), cmk(t2.z, t2.w)};
-        const Cplx<float> wv[4] = {cmk(w0.x, w0.y), cmk(w0.z, w0.w), cmk(w1.x, w1.y), cmk(w1.z, w1.w)};
+        P2 tv[3];
 #pragma unroll
-        for (int s = 0; s < 4; ++s)
+        for (int c = 0; c < 3; ++c) {
+          const float4 v = Ts[t][c][cg];
+          tv[c].re = make_float2(v.x, v.y);
+          tv[c].im = make_float2(v.z, v.w);
+        }
 #pragma unroll
-          for (int c = 0; c < 6; ++c) cfma(acc[s][c], wv[s], tv[c]);
+        for (int s = 0; s < 4; ++s) {
+          const float4 w = Ws[t * kLdW + ch * 4 + s];
+          B2 u;
+          u.r = make_float2(w.x, w.y);
+          u.i = make_float2(w.z, w.w);
+          u.ni = make_float2(-w.z, -w.w);
+#pragma unroll
+          for (int c = 0; c < 3; ++c) cmac(acc[s][c], u, tv[c]);
+        }
       }
     }
   }
@@ -258,8 +272,10 @@ __global__ void __launch_bounds__(256, 2) gconv_tile_kernel(Geom g, const TG* __
 #pragma unroll
     for (int c = 0; c < 3; ++c)
       *reinterpret_cast<float4*>(o + (s * 3 + c) * 256) =
-          make_float4(acc[s][c].re, acc[s][c].im, acc[s][3 + c].re, acc[s][3 + c].im);
+          make_float4(acc[s][c].re.x, acc[s][c].im.x, acc[s][c].re.y, acc[s][c].im.y);
 }
+
+constexpr size_t kTileSmem = sizeof(float4) * kPairs * 4 * kLdW;
 
 // Weight gradient: CTA (sixteen (input channel, hop) pairs, RA output channels,
 // slice of the sites).  Per sixteen sites the output gradients and the transported
@@ -276,18 +292,18 @@ __global__ void __launch_bounds__(256, 2) gconv_wgrad_tile_kernel(Geom g, const 
                                                                   const float2* __restrict__ gy,
                                                                   float2* __restrict__ part, int cin, int cout,
                                                                   int nslice) {
-  constexpr int kS = 16, G = 16 / RA, LDT = 64 + 2, LDG = RA * 4 + 2;
-  extern __shared__ __align__(16) float2 sm[];
-  float2* Ts = sm;                                                    // [site, colour][pair, spin]
-  float2* Gs = sm + kS * 3 * LDT;                                     // [site, colour][channel, spin]
+  constexpr int kS = 16, G = 16 / RA, LDT = 33, LDG = RA * 4 + 1;   // odd: the sites' 16-byte stores spread
+  extern __shared__ __align__(16) float4 sm[];
+  float4* Ts = sm;                                 // [site, colour][two spins][pair]: (re, re, im, im)
+  float4* Gs = sm + kS * 3 * LDT;                  // [site, colour][channel, spin]: (re, re, im, im)
   const int tid = threadIdx.x, p0 = blockIdx.x * 16, a0 = blockIdx.y * RA, slice = blockIdx.z;
   const int npair = cin * 9, tile = tid % (16 * RA), grp = tid / (16 * RA), tp = tile & 15, ta = tile >> 4;
   const size_t fs = (size_t)g.V * 12;
-  Cplx<float> tot[4][4];
+  P2 tot[4][2];                                    // [spin of the gradient][two input spins, packed]
 #pragma unroll
   for (int s = 0; s < 4; ++s)
 #pragma unroll
-    for (int t = 0; t < 4; ++t) tot[s][t] = cmk(0.f, 0.f);
+    for (int t = 0; t < 2; ++t) tot[s][t].re = tot[s][t].im = f2(0.f);
   const int nchunk = g.nblocks * 16;
   for (int ch = slice; ch < nchunk; ch += nslice) {
     const int blk = ch >> 4, l0 = (ch & 15) * kS;
@@ -302,47 +318,71 @@ __global__ void __launch_bounds__(256, 2) gconv_wgrad_tile_kernel(Geom g, const 
         for (int k = 0; k < 12; ++k) v[k] = cmk(0.f, 0.f);
       }
 #pragma unroll
-      for (int t = 0; t < 4; ++t)
+      for (int t = 0; t < 2; ++t)
 #pragma unroll
-        for (int c = 0; c < 3; ++c) Ts[(site * 3 + c) * LDT + p * 4 + t] = make_float2(v[t * 3 + c].re, v[t * 3 + c].im);
+        for (int c = 0; c < 3; ++c) {
+          const Cplx<float> a = v[2 * t * 3 + c], b = v[(2 * t + 1) * 3 + c];
+          Ts[(site * 3 + c) * LDT + t * 16 + p] = make_float4(a.re, b.re, a.im, b.im);
+        }
     }
     for (int e = tid; e < RA * 12 * kS; e += 256) {
       const int site = e & (kS - 1), k = (e / kS) % 12, a = e / (12 * kS);
       const float2 v = a0 + a < cout ? gy[(size_t)(a0 + a) * fs + ((size_t)blk * 12 + k) * 256 + l0 + site]
                                      : make_float2(0.f, 0.f);
-      Gs[(site * 3 + k % 3) * LDG + a * 4 + k / 3] = v;
+      Gs[(site * 3 + k % 3) * LDG + a * 4 + k / 3] = make_float4(v.x, v.x, v.y, v.y);
     }
     __syncthreads();
-    Cplx<float> acc[4][4];
+    P2 acc[4][2];
 #pragma unroll
     for (int s = 0; s < 4; ++s)
 #pragma unroll
-      for (int t = 0; t < 4; ++t) acc[s][t] = cmk(0.f, 0.f);
+      for (int t = 0; t < 2; ++t) acc[s][t].re = acc[s][t].im = f2(0.f);
 #pragma unroll 2
     for (int k = grp; k < kS * 3; k += G) {
-      const float4* ga = reinterpret_cast<const float4*>(Gs + k * LDG + 4 * ta);
-      const float4* xa = reinterpret_cast<const float4*>(Ts + k * LDT + 4 * tp);
-      const float4 g0 = ga[0], g1 = ga[1], x0 = xa[0], x1 = xa[1];
-      const Cplx<float> gv[4] = {cmk(g0.x, g0.y), cmk(g0.z, g0.w), cmk(g1.x, g1.y), cmk(g1.z, g1.w)};
-      const Cplx<float> xv[4] = {cmk(x0.x, x0.y), cmk(x0.z, x0.w), cmk(x1.x, x1.y), cmk(x1.z, x1.w)};
+      P2 xv[2];
+      float2 nxi[2];
 #pragma unroll
-      for (int s = 0; s < 4; ++s)
+      for (int t = 0; t < 2; ++t) {
+        const float4 v = Ts[k * LDT + t * 16 + tp];
+        xv[t].re = make_float2(v.x, v.y);
+        xv[t].im = make_float2(v.z, v.w);
+        nxi[t] = make_float2(-v.z, -v.w);
+      }
 #pragma unroll
-        for (int t = 0; t < 4; ++t) cfma_conj(acc[s][t], xv[t], gv[s]);
+      for (int s = 0; s < 4; ++s) {
+        const float4 w = Gs[k * LDG + ta * 4 + s];
+        const float2 gr = make_float2(w.x, w.y), gi = make_float2(w.z, w.w);
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {              // G_y conj(T x)
+          acc[s][t].re = fma2(xv[t].re, gr, acc[s][t].re);
+          acc[s][t].re = fma2(xv[t].im, gi, acc[s][t].re);
+          acc[s][t].im = fma2(xv[t].re, gi, acc[s][t].im);
+          acc[s][t].im = fma2(nxi[t], gr, acc[s][t].im);
+        }
+      }
     }
 #pragma unroll
     for (int s = 0; s < 4; ++s)
 #pragma unroll
-      for (int t = 0; t < 4; ++t) tot[s][t] = tot[s][t] + acc[s][t];
+      for (int t = 0; t < 2; ++t) {
+        tot[s][t].re = add2(tot[s][t].re, acc[s][t].re);
+        tot[s][t].im = add2(tot[s][t].im, acc[s][t].im);
+      }
   }
   // the groups' totals, then W's layout: [slice][a][pair][s][t]
-  if (G > 1) {
-    __syncthreads();
-    float2* red = sm;                                                 // [G][16 RA tiles][16]
+  auto put = [&](float2* o) {
 #pragma unroll
     for (int s = 0; s < 4; ++s)
 #pragma unroll
-      for (int t = 0; t < 4; ++t) red[(grp * 16 * RA + tile) * 16 + s * 4 + t] = make_float2(tot[s][t].re, tot[s][t].im);
+      for (int t = 0; t < 2; ++t) {
+        o[s * 4 + 2 * t] = make_float2(tot[s][t].re.x, tot[s][t].im.x);
+        o[s * 4 + 2 * t + 1] = make_float2(tot[s][t].re.y, tot[s][t].im.y);
+      }
+  };
+  if (G > 1) {
+    __syncthreads();
+    float2* red = reinterpret_cast<float2*>(sm);                      // [G][16 RA tiles][16]
+    put(red + (grp * 16 * RA + tile) * 16);
     __syncthreads();
     for (int e = tid; e < 16 * RA * 16; e += 256) {
       float re = 0.f, im = 0.f;
@@ -352,11 +392,7 @@ __global__ void __launch_bounds__(256, 2) gconv_wgrad_tile_kernel(Geom g, const 
         part[(((size_t)slice * cout + a) * npair + pr) * 16 + (e & 15)] = make_float2(re, im);
     }
   } else if (p0 + tp < npair && a0 + ta < cout) {
-    float2* o = part + (((size_t)slice * cout + a0 + ta) * npair + p0 + tp) * 16;
-#pragma unroll
-    for (int s = 0; s < 4; ++s)
-#pragma unroll
-      for (int t = 0; t < 4; ++t) o[s * 4 + t] = make_float2(tot[s][t].re, tot[s][t].im);
+    put(part + (((size_t)slice * cout + a0 + ta) * npair + p0 + tp) * 16);
   }
 }
 
@@ -437,17 +473,29 @@ __global__ void adam_kernel(size_t n, float* __restrict__ p, const float* __rest
 // channels a CTA would be idle and a thread per site transports little in vain.
 constexpr int kTiledFrom = 4;
 
+template <class TG, class TW, bool BWD>
+static int gconv_tiled(const Geom& g, const void* U, const void* W, const void* x, void* y, int cin, int cout,
+                       cudaStream_t s) {
+  static bool attr = false;
+  if (!attr) {
+    SAPMG_CUDA_TRY(cudaFuncSetAttribute(gconv_tile_kernel<TG, TW, BWD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)kTileSmem));
+    attr = true;
+  }
+  gconv_tile_kernel<TG, TW, BWD><<<dim3(g.nblocks * 8, (cout + kTileCh - 1) / kTileCh), 256, kTileSmem, s>>>(
+      g, (const TG*)U, (const TW*)W, (const float2*)x, (float2*)y, cin, cout);
+  count_launches(1);
+  SAPMG_CUDA_TRY(cudaGetLastError());
+  return MG_OK;
+}
+
 template <class TG, class TW>
 static int gconv_forward(const Geom& g, const void* U, const void* W, const void* x, void* y, int cin, int cout,
                          cudaStream_t s) {
   const size_t smem = sizeof(float2) * cin * 9 * 16;
   if (smem > 200 * 1024) return MG_ERR_ARG;
   if (cout >= kTiledFrom) {
-    gconv_tile_kernel<TG, TW, false><<<dim3(g.nblocks * 8, (cout + kTileCh - 1) / kTileCh), 256, 0, s>>>(
-        g, (const TG*)U, (const TW*)W, (const float2*)x, (float2*)y, cin, cout);
-    count_launches(1);
-    SAPMG_CUDA_TRY(cudaGetLastError());
-    return MG_OK;
+    return gconv_tiled<TG, TW, false>(g, U, W, x, y, cin, cout, s);
   }
   static bool attr = false;
   if (!attr) {
@@ -476,7 +524,7 @@ int launch_gconv_forward_bf16(const Geom& g, const void* U, const void* W, const
 static int wgrad_slices(const Geom& g, int cin, int cout) {
   const int tiles = (cin * 9 + 15) / 16 * (cout >= 16 ? (cout + 15) / 16 : (cout >= 4 ? (cout + 3) / 4 : cout));
   const int chunks = g.nblocks * 16;
-  return std::max(1, std::min((304 + tiles - 1) / tiles, std::max(1, chunks / 4)));
+  return std::max(1, std::min(304 / tiles, chunks / 4));       // one wave: a CTA more doubles the time
 }
 size_t gconv_wgrad_bytes(const Geom& g, int cin, int cout) {
   return (size_t)wgrad_slices(g, cin, cout) * cout * cin * 9 * 16 * sizeof(float2);
@@ -485,7 +533,7 @@ size_t gconv_wgrad_bytes(const Geom& g, int cin, int cout) {
 template <int RA>
 static int wgrad_run(const Geom& g, const void* U, const void* x, const void* gy, float2* part, int cin, int cout,
                      int nslice, cudaStream_t s) {
-  constexpr size_t stage = sizeof(float2) * 48 * (66 + RA * 4 + 2);
+  constexpr size_t stage = sizeof(float4) * 48 * (33 + RA * 4 + 1);
   constexpr size_t red = RA < 16 ? sizeof(float2) * 256 * 16 : 0;
   constexpr size_t smem = stage > red ? stage : red;
   static bool attr = false;
@@ -510,13 +558,14 @@ int launch_gconv_backward(const Geom& g, const void* U, const void* W, const voi
     attr = true;
   }
   if (gx) {
-    if (cin >= kTiledFrom)
-      gconv_tile_kernel<float2, float2, true><<<dim3(g.nblocks * 8, (cin + kTileCh - 1) / kTileCh), 256, 0, s>>>(
-          g, (const float2*)U, (const float2*)W, (const float2*)gy, (float2*)gx, cout, cin);
-    else
+    if (cin >= kTiledFrom) {
+      const int rc = gconv_tiled<float2, float2, true>(g, U, W, gy, gx, cout, cin, s);
+      if (rc != MG_OK) return rc;
+    } else {
       gconv_backward_input_kernel<<<dim3(g.nblocks, cin), 256, smem, s>>>(
           g, (const float2*)U, (const float2*)W, (const float2*)gy, (float2*)gx, cin, cout);
-    count_launches(1);
+      count_launches(1);
+    }
   }
   if (gW) {
     const size_t n = (size_t)cout * cin * 9 * 16;
