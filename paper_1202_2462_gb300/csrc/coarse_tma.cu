@@ -331,19 +331,20 @@ __device__ __forceinline__ uint32_t pack16(float2 v) {
   return *reinterpret_cast<const uint32_t*>(&h);
 }
 
-// The depth st_n of the staging ring is a launch parameter.  With more sites
-// than resident CTAs two stages are the fastest (more CTAs an SM); with fewer,
+// ST: depth of the staging ring (0: the launch parameter depth).  With more sites
+// than resident CTAs two or three stages are the fastest (more CTAs an SM); with fewer,
 // the deepest ring that keeps every site resident (up to all nine blocks in
 // flight at once) shortens the serial chain of nine copies a site: 512 sites,
 // one right-hand side, 12.0 us with 2 stages.
 constexpr int kMaxRing = 9;
-template <int RB, int N2, bool XH>
+template <int RB, int N2, int ST, bool XH>
 __global__ void __launch_bounds__(256) coarse_apply_mma16_kernel(const __half2* __restrict__ M,
                                                                  const void* __restrict__ xv,
                                                                  float2* __restrict__ out, CGeom c, int r0, int nr,
-                                                                 int st_n, int* __restrict__ err) {
+                                                                 int depth, int* __restrict__ err) {
   extern __shared__ __align__(128) unsigned char smem[];
   const int spins = wait_spins(err);
+  const int st_n = ST > 0 ? ST : depth;
   __shared__ __align__(8) uint64_t bar[kMaxRing];
   const int n2 = N2 > 0 ? N2 : c.n2;                         // N2 > 0: block size fixed at compile time
   const int xst = n2 + 4;                                     // padded row stride (conflict-free fragment loads)
@@ -466,16 +467,23 @@ __global__ void __launch_bounds__(256) coarse_apply_mma16_kernel(const __half2* 
   }
 }
 
+template <int RB, int N2, int ST, bool XH>
+static void launch_mma16_st(const CGeom& c, const __half2* M, const void* x, float2* out, int r0, int nr, int* err,
+                            int grid, int threads, size_t smem, int st, cudaStream_t s) {
+  static bool attr = false;
+  if (!attr) {
+    cudaFuncSetAttribute(coarse_apply_mma16_kernel<RB, N2, ST, XH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         200 * 1024);
+    attr = true;
+  }
+  coarse_apply_mma16_kernel<RB, N2, ST, XH><<<grid, threads, smem, s>>>(M, x, out, c, r0, nr, st, err);
+  count_launches(1);
+}
+
 template <int RB, int N2, bool XH>
 static void launch_mma16_t(const CGeom& c, const __half2* M, const void* x, float2* out, int r0, int nr, int* err,
                            const CoarseTune& t, cudaStream_t s) {
   const size_t stage = (size_t)c.n2 * c.n2 * sizeof(__half2) + (size_t)(RB <= 8 ? 8 : 16) * (c.n2 + 4) * (XH ? 4 : 8);
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(coarse_apply_mma16_kernel<RB, N2, XH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         200 * 1024);
-    attr = true;
-  }
   const int threads = 32 * (c.n2 / 8);
   auto per_sm = [&](int st) {
     const int k = (int)std::max<size_t>(1, std::min<size_t>(16, (220 * 1024) / (st * stage + 1024)));
@@ -485,8 +493,10 @@ static void launch_mma16_t(const CGeom& c, const __half2* M, const void* x, floa
   for (int d = kMaxRing; d > st; --d)
     if (d * stage <= 200 * 1024 && c.nsites <= 152 * per_sm(d)) { st = d; break; }
   const int grid = std::min(c.nsites, 152 * per_sm(st));
-  coarse_apply_mma16_kernel<RB, N2, XH><<<grid, threads, st * stage, s>>>(M, x, out, c, r0, nr, st, err);
-  count_launches(1);
+  const size_t smem = st * stage;
+  if (st == 2) launch_mma16_st<RB, N2, 2, XH>(c, M, x, out, r0, nr, err, grid, threads, smem, st, s);
+  else if (st == 3 && N2 > 0) launch_mma16_st<RB, N2, 3, XH>(c, M, x, out, r0, nr, err, grid, threads, smem, st, s);
+  else launch_mma16_st<RB, N2, 0, XH>(c, M, x, out, r0, nr, err, grid, threads, smem, st, s);
 }
 
 // 2N = 40 has a specialised instance with the k loop unrolled.
