@@ -203,16 +203,30 @@ __device__ __forceinline__ void mma_m16n8k8_tf32(float (&d)[4], uint32_t a0, uin
 // Operands are staged in shared memory by asynchronous 16-byte copies
 // (cp.async, kRStages-deep ring over K chunks of kRKC complex entries), so
 // every global load is a coalesced 16-byte piece and the fragments come from
-// shared memory.  Rows N..31 of P and R..15 of x stay zero in every stage.
+// shared memory.  The restriction holds N rows of P and a zero row that the
+// fragments' rows N..31 read, and the 4 NT rows of x that its fragments cover, those
+// past nrhs zero: 71 KB for N = 20 and 12 right-hand sides, three CTAs an SM (two
+// with all 32 and 16 rows).
 constexpr int kRKC = 128;
 constexpr int kRStages = 3;
 template <class TV> struct RPad { static constexpr int sp = 132; };           // 4-byte P entries
 template <> struct RPad<float2> { static constexpr int sp = 130; };           // 8-byte P entries
 constexpr int kRSX = 132;                                                      // x row stride (float2)
 
-template <class TV> __device__ __forceinline__ float2 p_ld(const TV* p) {
-  const Cplx<float> v = Io<float, TV>::ldc(p);
-  return make_float2(v.re, v.im);
+// One component (0 re, 1 im) of a stored P entry as a TF32 operand: read alone,
+// and FP16 and BF16 values need no rounding (their 8 and 11 significand bits fit
+// TF32's 11).  Reading whole entries, selecting and rounding each operand took
+// twice the instructions and bound the transfers (issue slots 66% busy):
+// restriction and interpolation of 12 right-hand sides at 32^3 x 64, N = 20, 1.22 and
+// 1.17 ms.
+__device__ __forceinline__ uint32_t p_tf32(const __half2* p, int comp) {
+  return __float_as_uint(__half2float(reinterpret_cast<const __half*>(p)[comp]));
+}
+__device__ __forceinline__ uint32_t p_tf32(const __nv_bfloat162* p, int comp) {
+  return (uint32_t)reinterpret_cast<const unsigned short*>(p)[comp] << 16;
+}
+__device__ __forceinline__ uint32_t p_tf32(const float2* p, int comp) {
+  return f32_to_tf32(reinterpret_cast<const float*>(p)[comp]);
 }
 
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
@@ -223,8 +237,12 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
 template <class TV>
-__host__ __device__ constexpr size_t restrict_stage_bytes() {
-  return (size_t)32 * RPad<TV>::sp * sizeof(TV) + (size_t)16 * kRSX * sizeof(float2);
+__host__ __device__ constexpr size_t restrict_p_bytes(int N) {
+  return ((size_t)(N + 1) * RPad<TV>::sp * sizeof(TV) + 15) / 16 * 16;
+}
+template <class TV>
+__host__ __device__ constexpr size_t restrict_stage_bytes(int N, int NT) {
+  return restrict_p_bytes<TV>(N) + (size_t)4 * NT * kRSX * sizeof(float2);
 }
 
 template <int NT, class TV>
@@ -233,8 +251,8 @@ __global__ void __launch_bounds__(256) restrict0_mma_kernel(const float2* __rest
                                                             int nblocks) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   constexpr int SP = RPad<TV>::sp;
-  constexpr size_t PB = (size_t)32 * SP * sizeof(TV);
-  constexpr size_t STAGE = restrict_stage_bytes<TV>();
+  const size_t PB = restrict_p_bytes<TV>(N);
+  const size_t STAGE = restrict_stage_bytes<TV>(N, NT);
   auto sP = [&](int st) { return reinterpret_cast<TV*>(smem_raw + st * STAGE); };
   auto sX = [&](int st) { return reinterpret_cast<float2*>(smem_raw + st * STAGE + PB); };
   const int blk = MG_CLAMP(kAggregate, blockIdx.x >> 1, nblocks), chi = blockIdx.x & 1;
@@ -242,13 +260,13 @@ __global__ void __launch_bounds__(256) restrict0_mma_kernel(const float2* __rest
   const int g = lane >> 2, tig = lane & 3, p1 = tig & 1;
   const size_t fs = (size_t)nblocks * 12 * 256;
   const size_t off = ((size_t)blk * 12 + 6 * chi) * 256;      // start of the chiral half-block
-  // zero rows of P (>= N) and of x (>= nrhs) in every stage
+  // the zero row of P and the rows of x past nrhs in every stage
   for (int st = 0; st < kRStages; ++st) {
     TV* P = sP(st);
     float2* X = sX(st);
     uint32_t* pz = reinterpret_cast<uint32_t*>(P + N * SP);
-    for (int e = tid; e < (32 - N) * SP * (int)sizeof(TV) / 4; e += 256) pz[e] = 0u;
-    for (int e = tid; e < (16 - nrhs) * kRSX; e += 256) X[nrhs * kRSX + e] = make_float2(0.f, 0.f);
+    for (int e = tid; e < SP * (int)sizeof(TV) / 4; e += 256) pz[e] = 0u;
+    for (int e = tid; e < (4 * NT - nrhs) * kRSX; e += 256) X[nrhs * kRSX + e] = make_float2(0.f, 0.f);
   }
   constexpr int PP = kRKC * (int)sizeof(TV) / 16;             // 16-byte pieces per P row chunk
   constexpr int XP = kRKC * 8 / 16;                           // per x row chunk
@@ -270,6 +288,8 @@ __global__ void __launch_bounds__(256) restrict0_mma_kernel(const float2* __rest
       }
     }
   };
+  const int bcomp = (g ^ p1) & 1;                             // component and sign of this lane's B entries
+  const uint32_t bsign = (g & p1) ? 0x80000000u : 0u;
   constexpr int NC = 1536 / kRKC;
 #pragma unroll
   for (int st = 0; st < kRStages - 1; ++st) {
@@ -294,22 +314,17 @@ __global__ void __launch_bounds__(256) restrict0_mma_kernel(const float2* __rest
       uint32_t a[2][4];
 #pragma unroll
       for (int m = 0; m < 2; ++m) {
-        const int r0 = 16 * m + g, r1 = r0 + 8;
-        const float2 x00 = p_ld(P + r0 * SP + K), x01 = p_ld(P + r0 * SP + K + 2);
-        const float2 x10 = p_ld(P + r1 * SP + K), x11 = p_ld(P + r1 * SP + K + 2);
-        a[m][0] = f32_to_tf32(p1 ? x00.y : x00.x);
-        a[m][1] = f32_to_tf32(p1 ? x10.y : x10.x);
-        a[m][2] = f32_to_tf32(p1 ? x01.y : x01.x);
-        a[m][3] = f32_to_tf32(p1 ? x11.y : x11.x);
+        const int r0 = min(16 * m + g, N), r1 = min(16 * m + g + 8, N);
+        a[m][0] = p_tf32(P + r0 * SP + K, p1);
+        a[m][1] = p_tf32(P + r1 * SP + K, p1);
+        a[m][2] = p_tf32(P + r0 * SP + K + 2, p1);
+        a[m][3] = p_tf32(P + r1 * SP + K + 2, p1);
       }
 #pragma unroll
       for (int q = 0; q < NT; ++q) {
-        const int col = 8 * q + g, r = col >> 1, pc = col & 1;
-        const float2 x = X[r * kRSX + K], y = X[r * kRSX + K + 2];
-        // B[2K+p1][2r+pc]: (pc, p1) = (0,0) re, (0,1) im, (1,0) im, (1,1) -re
-        const float b0 = pc ? (p1 ? -x.x : x.y) : (p1 ? x.y : x.x);
-        const float b1 = pc ? (p1 ? -y.x : y.y) : (p1 ? y.y : y.x);
-        const uint32_t tb0 = f32_to_tf32(b0), tb1 = f32_to_tf32(b1);
+        // B[2K+p1][2r+pc]: (pc, p1) = (0,0) re, (0,1) im, (1,0) im, (1,1) -re; pc = g & 1
+        const float* x = reinterpret_cast<const float*>(X + ((8 * q + g) >> 1) * kRSX + K) + bcomp;
+        const uint32_t tb0 = f32_to_tf32(x[0]) ^ bsign, tb1 = f32_to_tf32(x[4]) ^ bsign;
 #pragma unroll
         for (int m = 0; m < 2; ++m) mma_m16n8k8_tf32(acc[m][q], a[m][0], a[m][1], a[m][2], a[m][3], tb0, tb1);
       }
@@ -355,8 +370,6 @@ __global__ void __launch_bounds__(256) restrict0_mma_kernel(const float2* __rest
 // exactly); P is staged per chunk of kRKC entries by cp.async; B is loaded
 // into registers once.  Neighbouring lanes (real and imaginary rows of one K)
 // swap halves by a shuffle so that each stores whole complex numbers.
-__device__ __forceinline__ float embed_pr(float2 m, int a, int b) { return a == b ? m.x : (a ? m.y : -m.y); }
-
 template <class TV>
 __host__ __device__ constexpr size_t prolong_stage_bytes(int Np) {
   return (size_t)Np * RPad<TV>::sp * sizeof(TV);
@@ -408,6 +421,9 @@ __global__ void __launch_bounds__(256) prolong0_mma_kernel(const float2* __restr
   }
   __syncthreads();                                             // eb written
   const int KS = Np / 4;                                       // k8 steps (<= 8)
+  // component and sign of this lane's A entries (a, b): (0,0) re, (0,1) -im, (1,0) im, (1,1) re
+  const int acomp = (a ^ tig) & 1;
+  const uint32_t asign = (!a && (tig & 1)) ? 0x80000000u : 0u;
   uint32_t bf[8][NT][2];
 #pragma unroll
   for (int ks = 0; ks < 8; ++ks)
@@ -434,11 +450,11 @@ __global__ void __launch_bounds__(256) prolong0_mma_kernel(const float2* __restr
 #pragma unroll
       for (int ks = 0; ks < 8; ++ks) {
         if (ks < KS) {
-          const int k = 4 * ks + (tig >> 1), b = tig & 1;       // columns tig (k) and tig + 4 (k + 2)
-          const uint32_t a0 = f32_to_tf32(embed_pr(p_ld(P + k * SP + Kl), a, b));
-          const uint32_t a1 = f32_to_tf32(embed_pr(p_ld(P + k * SP + Kl + 4), a, b));
-          const uint32_t a2 = f32_to_tf32(embed_pr(p_ld(P + (k + 2) * SP + Kl), a, b));
-          const uint32_t a3 = f32_to_tf32(embed_pr(p_ld(P + (k + 2) * SP + Kl + 4), a, b));
+          const int k = 4 * ks + (tig >> 1);                    // columns tig (k) and tig + 4 (k + 2)
+          const uint32_t a0 = p_tf32(P + k * SP + Kl, acomp) ^ asign;
+          const uint32_t a1 = p_tf32(P + k * SP + Kl + 4, acomp) ^ asign;
+          const uint32_t a2 = p_tf32(P + (k + 2) * SP + Kl, acomp) ^ asign;
+          const uint32_t a3 = p_tf32(P + (k + 2) * SP + Kl + 4, acomp) ^ asign;
 #pragma unroll
           for (int nt = 0; nt < NT; ++nt) mma_m16n8k8_tf32(acc[nt], a0, a1, a2, a3, bf[ks][nt][0], bf[ks][nt][1]);
         }
@@ -466,13 +482,16 @@ static int transfer0_mrhs(bool restrict_, const Geom& g, const void* in, void* o
                           bool tf32, cudaStream_t s) {
   if (restrict_ && tf32 && nrhs <= 16 && N <= 32) {
     const unsigned grid = (unsigned)(g.nblocks * 2);
-    const size_t smem = kRStages * restrict_stage_bytes<TV>();
+    const int nt = (nrhs + 3) / 4;
+    // the ring, which the warps' partial products (8 x 2 NT x 128 floats) reuse at the end
+    const size_t smem = std::max(kRStages * restrict_stage_bytes<TV>(N, nt), (size_t)8 * 2 * nt * 128 * sizeof(float));
     static bool attr = false;
     if (!attr) {
-      cudaFuncSetAttribute(restrict0_mma_kernel<1, TV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      cudaFuncSetAttribute(restrict0_mma_kernel<2, TV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      cudaFuncSetAttribute(restrict0_mma_kernel<3, TV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      cudaFuncSetAttribute(restrict0_mma_kernel<4, TV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      const int mx = (int)(kRStages * restrict_stage_bytes<TV>(32, 4));
+      cudaFuncSetAttribute(restrict0_mma_kernel<1, TV>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+      cudaFuncSetAttribute(restrict0_mma_kernel<2, TV>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+      cudaFuncSetAttribute(restrict0_mma_kernel<3, TV>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+      cudaFuncSetAttribute(restrict0_mma_kernel<4, TV>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
       attr = true;
     }
     const float2* xi = (const float2*)in;
