@@ -401,16 +401,18 @@ int blas_normalize(int type, const BVec& b, const void* x, void* out, const doub
 // Least-squares solve of the (m+1) x m Hessenberg system min ||beta e1 - H y||
 // of fixed-step GMRES, one warp per right-hand side (hessenberg.cuh).  H for
 // RHS r at H + r*ldr, column-major with leading dimension ldh; beta2[r].x =
-// ||b_r||^2; y[r*ldy + j].  scale != nullptr: basis vector j has the norm
-// scale[r*ldr + j].x (j = 0: 1) and y is divided by it.  Columns after a zero
-// subdiagonal entry are unused.  m <= 32.
+// ||b_r||^2; y[r*ldy + j].  norms != nullptr: H holds the raw dots of
+// blas_arnoldi_step (pairs: as sums of two floats) and norms[r*ldr + j] = (||x||^2,
+// 1/beta) of basis vector j >= 1, whose norm is s_j = ||x|| / beta: with the entries
+// h_ij / s_i and ||x_{j+1}|| the solution is in the basis vectors as they are.
+// Columns after a zero subdiagonal entry are unused.  m <= 32.
 // Latency-bound (an FP64 instruction of a warp takes 64 cycles of its
 // sub-partition): 12 steps on one vector 73 us with two square roots and
 // divisions a step and serial loads, 27 us with one reciprocal square root a
 // step and every load and division issued for all columns at once.
 __global__ void __launch_bounds__(32) hessenberg_solve_kernel(const double2* __restrict__ Hall, int ldh, int ldr,
                                                               int m, const double2* __restrict__ beta2,
-                                                              const double2* __restrict__ scale,
+                                                              const double2* __restrict__ norms, int pairs,
                                                               double2* __restrict__ yall, int ldy) {
   __shared__ double hr[33 * 32], hi[33 * 32];
   const int r = blockIdx.x, lane = threadIdx.x;
@@ -421,27 +423,40 @@ __global__ void __launch_bounds__(32) hessenberg_solve_kernel(const double2* __r
     if (lane < m) y[lane] = make_double2(0, 0);
     return;
   }
-  const double sub = lane < m ? Hin[lane + 1 + lane * ldh].x : 1.0;
-  double inv_s = 1.0;
-  if (scale && lane > 0 && lane < m) {
-    const double t = scale[(size_t)r * ldr + lane].x;
-    inv_s = t > 0.0 ? 1.0 / t : 0.0;
+  double sub = 1.0, is = 1.0;                            // H_{lane+1,lane}; 1 / s_lane
+  if (norms) {
+    const double2* nv = norms + (size_t)r * ldr;
+    if (lane > 0 && lane < m) {
+      const double t = sqrt(nv[lane].x) * nv[lane].y;
+      is = t > 0.0 ? 1.0 / t : 0.0;
+    }
+    if (lane < m) sub = sqrt(nv[lane + 1].x);
+  } else if (lane < m) {
+    sub = Hin[lane + 1 + lane * ldh].x;
   }
   const unsigned zero = __ballot_sync(0xffffffffu, sub == 0.0);
   const int mm = zero ? __ffs(zero) : m;                 // columns up to the first zero subdiagonal entry
-  for (int k = 0; k < mm; ++k) {                         // lane = row; the last row by lane 0
-    const double2 v = lane <= k + 1 && lane <= mm ? Hin[lane + k * ldh] : make_double2(0, 0);
+  for (int k = 0; k < mm; ++k) {                         // lane = row
+    double2 v = make_double2(0, 0);
+    if (lane <= k) {
+      v = Hin[lane + k * ldh];
+      if (pairs) {
+        const float4 f = *reinterpret_cast<const float4*>(&v);
+        v = make_double2((double)f.x + (double)f.y, (double)f.z + (double)f.w);
+      }
+      if (norms) { v.x *= is; v.y *= is; }
+    }
     hr[lane + k * 33] = v.x;
     hi[lane + k * 33] = v.y;
+    if (lane == 0) hr[32 + k * 33] = hi[32 + k * 33] = 0.0;
   }
-  if (lane == 0 && mm == 32) {
-    for (int k = 0; k < 31; ++k) hr[32 + k * 33] = hi[32 + k * 33] = 0.0;
-    const double2 v = Hin[32 + 31 * ldh];
-    hr[32 + 31 * 33] = v.x;
-    hi[32 + 31 * 33] = v.y;
+  __syncwarp();
+  if (lane < mm) {
+    hr[lane + 1 + lane * 33] = sub;
+    hi[lane + 1 + lane * 33] = 0.0;
   }
   const Cplx<double> v = hessenberg_warp(hr, hi, mm, beta);
-  if (lane < m) y[lane] = make_double2(v.re * inv_s, v.im * inv_s);
+  if (lane < m) y[lane] = make_double2(v.re, v.im);
 }
 
 // ------------------------------------------------------------ delayed reorthogonalisation
@@ -1025,18 +1040,71 @@ struct DoubleBasis {
 };
 template <class V> struct PtrsK { const V* p[32]; };
 
-// Scalars of a step (per right-hand side, stride ldr): H (33 x 33 column-major);
-// t[0..32] raw dots of earlier chunks, then the coefficients; t[40] = (1/beta, beta);
-// t[64 + i].x = s_i for i >= 1.
+// Scalars of a step (per right-hand side, stride ldr): H (33 x 33 column-major)
+// takes the raw dots; t[i] a coefficient of the update (Cplx<R>; FP64: the raw dots
+// of earlier chunks before), t[40] 1/beta, t[64 + i] = (||x||^2, 1/beta) of basis
+// vector i >= 1 and, as R from t[100] on, 1 / s_i^2.
 struct ArnoldiOut {
   double2 *H, *t;
   int ldr, j, i0, last;    // the step, the chunk's first vector, the chunk that ends the pass
 };
-__device__ __forceinline__ double inv_scale(const double2* t, int i) {
-  if (i == 0) return 1.0;
-  const double s = t[64 + i].x;
-  return s > 0.0 ? 1.0 / s : 0.0;
+template <class R> __device__ __forceinline__ R inv_scale2(const double2* t, int i) {
+  return i == 0 ? (R)1 : reinterpret_cast<const R*>(t + 100)[i];
 }
+
+// A sum across warps and CTAs: FP32 parts as an unevaluated pair of floats with
+// error-free additions (Knuth, TAOCP vol. 2, 4.2.2), about the precision of FP64,
+// an instruction of which takes 64 cycles of an SM's sub-partition and so made
+// these short serial sums the longest part of a kernel on a short vector.
+template <class R> struct Acc;
+template <> struct Acc<float> {
+  float h, l;
+  __device__ __forceinline__ static Acc of(float v) { return Acc{v, 0.f}; }
+  __device__ __forceinline__ void add(Acc b) {
+    const float s = __fadd_rn(h, b.h), t = __fsub_rn(s, h);
+    const float e = __fadd_rn(__fsub_rn(h, __fsub_rn(s, t)), __fsub_rn(b.h, t));
+    h = s;
+    l = __fadd_rn(__fadd_rn(l, b.l), e);
+  }
+  __device__ __forceinline__ Acc from(int mask) const {
+    return Acc{__shfl_xor_sync(0xffffffffu, h, mask), __shfl_xor_sync(0xffffffffu, l, mask)};
+  }
+  __device__ __forceinline__ float value() const { return h + l; }
+  __device__ __forceinline__ double exact() const { return (double)h + (double)l; }
+};
+template <> struct Acc<double> {
+  double v;
+  __device__ __forceinline__ static Acc of(double x) { return Acc{x}; }
+  __device__ __forceinline__ void add(Acc b) { v += b.v; }
+  __device__ __forceinline__ Acc from(int mask) const { return Acc{__shfl_xor_sync(0xffffffffu, v, mask)}; }
+  __device__ __forceinline__ double value() const { return v; }
+  __device__ __forceinline__ double exact() const { return v; }
+};
+template <class R> struct AccC { Acc<R> re, im; };      // sixteen bytes: a slot of the partial sums
+static_assert(sizeof(AccC<float>) == 16 && sizeof(AccC<double>) == 16, "a slot holds one complex sum");
+
+// The calling warp's sum of a slot over the CTAs of right-hand side r.
+template <class R>
+__device__ __forceinline__ AccC<R> sum_slot_acc(const double2* partial, int r, int slots, int j) {
+  AccC<R> a;
+  a.re = a.im = Acc<R>::of((R)0);
+#pragma unroll 4
+  for (int c = threadIdx.x & 31; c < (int)gridDim.x; c += 32) {
+    const double2 q = __ldcg(partial + ((size_t)r * gridDim.x + c) * slots + j);
+    const AccC<R> v = *reinterpret_cast<const AccC<R>*>(&q);
+    a.re.add(v.re);
+    a.im.add(v.im);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    a.re.add(a.re.from(o));
+    a.im.add(a.im.from(o));
+  }
+  return a;
+}
+
+__device__ __forceinline__ float inv_sqrt(float x) { return rsqrtf(x); }
+__device__ __forceinline__ double inv_sqrt(double x) { return rsqrt(x); }
 
 // v[0..N) summed over the warp, N a power of two up to 32: halving the values a
 // lane holds with every exchange, N - 1 + (5 - log2 N) shuffles instead of 5 N.
@@ -1087,53 +1155,57 @@ __global__ void __launch_bounds__(256) arnoldi_dots_kernel(PtrsK<typename B::V> 
     ww += nrm_of(x);
   }
   constexpr int NV = 2 * KM < 32 ? 2 * KM : 32, NG = 2 * KM / NV;
-  __shared__ double red[8][2 * KM + 1];
+  __shared__ R red[8][2 * KM + 1];
 #pragma unroll
   for (int g = 0; g < NG; ++g) {
     R u[NV];
 #pragma unroll
     for (int q = 0; q < NV; ++q) u[q] = acc[(g * NV + q) >> 1][q & 1];
     const R t = warp_sums<NV>(u);
-    if (lane % (32 / NV) == 0) red[wid][g * NV + lane / (32 / NV)] = (double)t;
+    if (lane % (32 / NV) == 0) red[wid][g * NV + lane / (32 / NV)] = t;
   }
   ww = warp_sum(ww);
-  if (lane == 0) red[wid][2 * KM] = (double)ww;
+  if (lane == 0) red[wid][2 * KM] = ww;
   __syncthreads();
-  double* part = reinterpret_cast<double*>(partial + ((size_t)r * gridDim.x + blockIdx.x) * (KM + 1));
+  Acc<R>* part = reinterpret_cast<Acc<R>*>(partial + ((size_t)r * gridDim.x + blockIdx.x) * (KM + 1));
   if ((int)threadIdx.x <= 2 * KM) {
-    double t = 0;
-    for (int q = 0; q < 8; ++q) t += red[q][threadIdx.x];
+    Acc<R> t = Acc<R>::of(red[0][threadIdx.x]);
+#pragma unroll
+    for (int q = 1; q < 8; ++q) t.add(Acc<R>::of(red[q][threadIdx.x]));
     part[threadIdx.x] = t;
-    if ((int)threadIdx.x == 2 * KM) part[2 * KM + 1] = 0.0;
+    if ((int)threadIdx.x == 2 * KM) part[2 * KM + 1] = Acc<R>::of((R)0);
   }
   if (!last_cta(partial, r)) return;
-  __shared__ double2 raw[KM + 1];
+  __shared__ AccC<R> raw[KM + 1];
   for (int q = wid; q <= KM; q += 8) {
     if (q < k || q == KM) {
-      const double2 t = sum_slot(partial, r, KM + 1, q);
+      const AccC<R> t = sum_slot_acc<R>(partial, r, KM + 1, q);
       if (lane == 0) raw[q] = t;
     }
   }
   __syncthreads();
   if (wid > 0) return;
   double2* t = o.t + (size_t)r * o.ldr;
+  AccC<R>* tr = reinterpret_cast<AccC<R>*>(t);
   if (!o.last) {
-    if (lane < k) t[o.i0 + lane] = raw[lane];
+    if (lane < k) tr[o.i0 + lane] = raw[lane];
     return;
   }
   // lane = basis vector i <= j
   const bool on = lane <= o.j;
-  const double2 d = !on ? make_double2(0, 0) : (lane < o.i0 ? t[lane] : raw[lane - o.i0]);
-  const double is = on ? inv_scale(t, lane) : 0.0, isj = inv_scale(t, o.j);
-  double e = (d.x * d.x + d.y * d.y) * is * is;
-  e = warp_sum(e);
+  AccC<R> d;
+  d.re = d.im = Acc<R>::of((R)0);
+  if (on) d = lane < o.i0 ? tr[lane] : raw[lane - o.i0];
+  const R is2 = on ? inv_scale2<R>(t, lane) : (R)0;
+  const R dr = d.re.value(), di = d.im.value();
+  const R e = warp_sum((dr * dr + di * di) * is2);
   if (on) {
-    o.H[(size_t)r * o.ldr + lane + 33 * o.j] = make_double2(d.x * is * isj, d.y * is * isj);
-    t[lane] = make_double2(d.x * is * is, d.y * is * is);
+    reinterpret_cast<AccC<R>*>(o.H + (size_t)r * o.ldr)[lane + 33 * o.j] = d;
+    reinterpret_cast<Cplx<R>*>(t + lane)[0] = cmk(dr * is2, di * is2);
   }
   if (lane == 0) {
-    const double n2 = raw[KM].x, b = sqrt(fmax(n2 - e, B::kFloor * n2));
-    t[40] = make_double2(b > 0.0 ? 1.0 / b : 0.0, b);
+    const R n2 = raw[KM].re.value(), b2 = max(n2 - e, (R)B::kFloor * n2);
+    reinterpret_cast<R*>(t + 40)[0] = b2 > (R)0 ? inv_sqrt(b2) : (R)0;
   }
 }
 
@@ -1147,15 +1219,15 @@ __global__ void __launch_bounds__(256) arnoldi_update_kernel(PtrsK<typename B::V
   typedef typename B::R R;
   typedef typename B::V V;
   __shared__ R cf[2][KM];
-  __shared__ double red[8];
+  __shared__ R red[8];
   const int r = blockIdx.y, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   double2* t = o.t + (size_t)r * o.ldr;
   if ((int)threadIdx.x < k) {
-    const double2 c = t[o.i0 + threadIdx.x];
-    cf[0][threadIdx.x] = (R)-c.x;
-    cf[1][threadIdx.x] = (R)-c.y;
+    const Cplx<R> c = reinterpret_cast<const Cplx<R>*>(t + o.i0 + threadIdx.x)[0];
+    cf[0][threadIdx.x] = -c.re;
+    cf[1][threadIdx.x] = -c.im;
   }
-  const R invb = (R)t[40].x;
+  const R invb = reinterpret_cast<const R*>(t + 40)[0];
   __syncthreads();
   typename B::W* wr = w + r * stride;
   R nn = 0;
@@ -1178,20 +1250,23 @@ __global__ void __launch_bounds__(256) arnoldi_update_kernel(PtrsK<typename B::V
   }
   if (!o.last) return;
   nn = warp_sum(nn);
-  if (lane == 0) red[wid] = (double)nn;
+  if (lane == 0) red[wid] = nn;
   __syncthreads();
   if (threadIdx.x == 0) {
-    double sum = 0;
-    for (int q = 0; q < 8; ++q) sum += red[q];
-    partial[(size_t)r * gridDim.x + blockIdx.x] = make_double2(sum, 0.0);
+    AccC<R> sum;
+    sum.re = Acc<R>::of(red[0]);
+    sum.im = Acc<R>::of((R)0);
+#pragma unroll
+    for (int q = 1; q < 8; ++q) sum.re.add(Acc<R>::of(red[q]));
+    reinterpret_cast<AccC<R>*>(partial)[(size_t)r * gridDim.x + blockIdx.x] = sum;
   }
   if (!last_cta(partial, r)) return;
   if (wid > 0) return;
-  const double2 sum = sum_slot(partial, r, 1, 0);
+  const Acc<R> sum = sum_slot_acc<R>(partial, r, 1, 0).re;
   if (lane == 0) {
-    const double nrm = sqrt(fmax(sum.x, 0.0));
-    o.H[(size_t)r * o.ldr + o.j + 1 + 33 * o.j] = make_double2(nrm * inv_scale(t, o.j), 0.0);
-    t[64 + o.j + 1] = make_double2(nrm * (double)invb, 0.0);
+    const R s2 = max(sum.value(), (R)0) * invb * invb;
+    reinterpret_cast<R*>(t + 100)[o.j + 1] = s2 > (R)0 ? (R)1 / s2 : (R)0;
+    t[64 + o.j + 1] = make_double2(fmax(sum.exact(), 0.0), (double)invb);
   }
 }
 
@@ -1322,9 +1397,9 @@ int blas_combine(int basis, const BVec& b, const void* const* v, int k, const do
 }
 
 int blas_hessenberg_solve(const double2* H, int ldh, int ldr, int m, const double2* beta2, double2* y, int ldy,
-                          int R, cudaStream_t s, const double2* scale) {
+                          int R, cudaStream_t s, const double2* norms, bool pairs) {
   if (m > 32) return MG_ERR_ARG;
-  hessenberg_solve_kernel<<<R, 32, 0, s>>>(H, ldh, ldr, m, beta2, scale, y, ldy); count_launches(1);
+  hessenberg_solve_kernel<<<R, 32, 0, s>>>(H, ldh, ldr, m, beta2, norms, pairs, y, ldy); count_launches(1);
   SAPMG_CUDA_TRY(cudaGetLastError());
   return MG_OK;
 }

@@ -63,14 +63,14 @@ int blas_normalize_h(const BVec& b, const void* x, void* out, const double2* nrm
                      cudaStream_t s);
 // Scalars of fixed-step GMRES on a coarse level, per right-hand side at stride
 // ldr >= 33 * 33: H (column-major, leading dimension 33) and scratch t (33 * 33),
-// whose entries 64 + i hold the norms s_i of the basis vectors.
+// for blas_hessenberg_solve with norms = t + 64 and pairs for FP32 w.
 struct ArnoldiWork {
   double2 *H, *t;
   int ldr;
   double2* partial;
 };
 // Step j < 32 of the Arnoldi process on w = A v_j (contents undefined
-// afterwards): column j of H and, unless vnext is null, v_{j+1}, whose norm s_{j+1} is near 1.
+// afterwards): the dots of column j and, unless vnext is null, v_{j+1}, whose norm is near 1.
 // basis: P16 (FP16 vectors as blas_normalize_h stores them, FP32 w), P32 or P64.
 int blas_arnoldi_step(int basis, const BVec& b, const void* const* v, int j, void* w, void* vnext,
                       const ArnoldiWork& a, cudaStream_t s);
@@ -78,8 +78,8 @@ int blas_arnoldi_step(int basis, const BVec& b, const void* const* v, int j, voi
 int blas_combine(int basis, const BVec& b, const void* const* v, int k, const double2* y, int ldy, void* out,
                  cudaStream_t s);
 // y[r] = argmin || sqrt(beta2[r]) e1 - H_r y || for (m+1) x m Hessenberg H_r (column-major, ldh; H_r at H + r*ldr);
-// scale: divide y_i by the norm scale[r*ldr + i] of basis vector i >= 1.
+// norms, pairs: H and the basis vectors' norms as blas_arnoldi_step leaves them.
 int blas_hessenberg_solve(const double2* H, int ldh, int ldr, int m, const double2* beta2, double2* y, int ldy,
-                          int R, cudaStream_t s, const double2* scale = nullptr);
+                          int R, cudaStream_t s, const double2* norms = nullptr, bool pairs = false);
 
 }  // namespace sapmg

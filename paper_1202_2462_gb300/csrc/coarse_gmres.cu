@@ -12,7 +12,8 @@
 //
 // Per step, as the two-kernel form of the coarse GMRES (blas.cu): h_i = <v_i, w>,
 // beta^2 = <w, w> - sum |h_i|^2 / |v_i|^2 (floored), v_{j+1} = (w - sum h_i v_i /
-// |v_i|^2) / beta, whose exact norm s_{j+1} is kept and divided out of H and y.
+// |v_i|^2) / beta, whose exact norm s_{j+1} is kept: with rows h_ij / s_i and the
+// subdiagonal ||x|| the least squares gives the coefficients of the v_i as they are.
 #include "cluster.cuh"
 #include "coarse.h"
 #include "hessenberg.cuh"
@@ -41,14 +42,25 @@ struct DoubleOp {
 };
 
 // Sum of one value over lanes 0..15 in a fixed order.  FP32 parts are added as
-// unevaluated pairs (error-free sums, Knuth 1969): the precision of an FP64 sum,
-// whose instructions take 64 cycles of the sub-partition each.
-__device__ __forceinline__ double sum16(double v) {
+// unevaluated pairs (error-free sums, Knuth, TAOCP vol. 2, 4.2.2): the precision of
+// an FP64 sum, whose instructions take 64 cycles of the sub-partition each.
+template <class R> struct Sum16;
+template <> struct Sum16<double> {
+  double v;
+  __device__ __forceinline__ double value() const { return v; }
+  __device__ __forceinline__ double exact() const { return v; }
+};
+template <> struct Sum16<float> {
+  float h, l;
+  __device__ __forceinline__ float value() const { return h + l; }
+  __device__ __forceinline__ double exact() const { return (double)h + (double)l; }
+};
+__device__ __forceinline__ Sum16<double> sum16(double v) {
 #pragma unroll
   for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
+  return Sum16<double>{v};
 }
-__device__ __forceinline__ double sum16(float v) {
+__device__ __forceinline__ Sum16<float> sum16(float v) {
   float h = v, l = 0.f;
 #pragma unroll
   for (int o = 8; o > 0; o >>= 1) {
@@ -58,13 +70,13 @@ __device__ __forceinline__ double sum16(float v) {
     h = s;
     l = __fadd_rn(__fadd_rn(l, l2), e);
   }
-  return (double)h + (double)l;
+  return Sum16<float>{h, l};
 }
 __device__ __forceinline__ float rsqrt_of(float x) { return rsqrtf(x); }
 __device__ __forceinline__ double rsqrt_of(double x) { return rsqrt(x); }
 
 struct Layout {          // byte offsets in shared memory
-  int ms, vf, basis, ts, w, pd, pn, hr, hi, coef, sc, tab, flag, bar, total;
+  int ms, vf, basis, ts, w, pd, pn, hr, hi, coef, dots, sc, tab, flag, bar, total;
 };
 template <class OP>
 __host__ __device__ inline Layout layout(int spc, int nsites, int n2, int k) {
@@ -81,8 +93,9 @@ __host__ __device__ inline Layout layout(int spc, int nsites, int n2, int k) {
   l.pn = take(2 * kSolveCluster * (int)sizeof(typename OP::R));   // partial norms, two buffers
   l.hr = take(33 * 32 * 8);
   l.hi = take(33 * 32 * 8);
-  l.coef = take(34 * 16);                                  // dots of the step (FP64)
-  l.sc = take(34 * 8 * 2);                                 // 1/s_i, and 1/s_i^2
+  l.coef = take(34 * 16);                                  // y (FP64)
+  l.dots = take(34 * cb);                                  // the step's dots
+  l.sc = take(34 * 8 * 2);                                 // 1/s_i (FP64), and 1/s_i^2
   l.tab = take(spc * 9 * 4);
   l.flag = take(kSolveCluster * 4);
   l.bar = take(8);
@@ -90,7 +103,10 @@ __host__ __device__ inline Layout layout(int spc, int nsites, int n2, int k) {
   return l;
 }
 
-template <class OP, class TX>
+// N2 > 0: 2N at compile time.  The last warp, beyond those of the products, turns
+// sums into H's column and the norms' reciprocals (FP64, 64 cycles an instruction)
+// while the others are at the next product.
+template <class OP, class TX, int N2>
 __global__ void __launch_bounds__(768) coarse_gmres_cluster_kernel(const typename OP::M* __restrict__ M,
                                                                    const TX* __restrict__ b, TX* __restrict__ x,
                                                                    CGeom c, int spc, int k, int* __restrict__ err) {
@@ -98,7 +114,7 @@ __global__ void __launch_bounds__(768) coarse_gmres_cluster_kernel(const typenam
   typedef typename OP::M TM;
   typedef Cplx<R> C;
   extern __shared__ __align__(128) unsigned char smem[];
-  const int n2 = c.n2, tile = n2 * n2, rank = cluster_rank(), rows = spc * n2, n = c.nsites * n2;
+  const int n2 = N2 > 0 ? N2 : c.n2, tile = n2 * n2, rank = cluster_rank(), rows = spc * n2, n = c.nsites * n2;
   const Layout lo = layout<OP>(spc, c.nsites, n2, k);
   TM* Ms = reinterpret_cast<TM*>(smem + lo.ms);
   C* vf = reinterpret_cast<C*>(smem + lo.vf);
@@ -111,7 +127,8 @@ __global__ void __launch_bounds__(768) coarse_gmres_cluster_kernel(const typenam
   double* hi = reinterpret_cast<double*>(smem + lo.hi);
   double2* coef = reinterpret_cast<double2*>(smem + lo.coef);
   double* is = reinterpret_cast<double*>(smem + lo.sc);       // 1 / s_i
-  double* is2 = is + 34;
+  R* is2 = reinterpret_cast<R*>(is + 34);                     // 1 / s_i^2
+  C* dots = reinterpret_cast<C*>(smem + lo.dots);
   int* tab = reinterpret_cast<int*>(smem + lo.tab);
   int* flag = reinterpret_cast<int*>(smem + lo.flag);
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem + lo.bar);
@@ -190,7 +207,7 @@ __global__ void __launch_bounds__(768) coarse_gmres_cluster_kernel(const typenam
       return;
     }
   }
-  const double bb = sum16(pn[kSolveCluster + (lane & 15)]);
+  const double bb = sum16(pn[kSolveCluster + (lane & 15)]).exact();
   const double beta0 = sqrt(fmax(bb, 0.0));
   {
     const R f = beta0 > 0.0 ? (R)(1.0 / beta0) : (R)0;
@@ -202,7 +219,7 @@ __global__ void __launch_bounds__(768) coarse_gmres_cluster_kernel(const typenam
       for (int q = 0; q < kSolveCluster; ++q) cluster_st(cluster_addr(a, q), v);
     }
   }
-  if (tid == 0) { is[0] = is2[0] = 1.0; }
+  if (tid == 0) { is[0] = 1.0; is2[0] = (R)1; }
   cluster_barrier();
   for (int j = 0; j < k; ++j) {
     // w = A v_j on the CTA's rows
@@ -236,33 +253,30 @@ __global__ void __launch_bounds__(768) coarse_gmres_cluster_kernel(const typenam
     cluster_barrier();
     for (int i = warp; i <= j + 1; i += nw) {
       const C t = pd[(lane & 15) * 33 + i];
-      const double a = sum16(t.re), c2 = sum16(t.im);
-      if (lane == 0) coef[i] = make_double2(a, c2);
-    }
-    __syncthreads();
-    if (warp == nw - 1) {                                    // column j of H, for the unit vectors
-      const double f = is[j];
-      if (lane <= j) {
-        hr[lane + 33 * j] = coef[lane].x * is[lane] * f;
-        hi[lane + 33 * j] = coef[lane].y * is[lane] * f;
+      const Sum16<R> a = sum16(t.re), c2 = sum16(t.im);
+      if (lane == 0) {
+        dots[i] = cmk(a.value(), c2.value());
+        if (i <= j) {                                        // raw; scaled by the last warp
+          hr[i + 33 * j] = a.exact();
+          hi[i + 33 * j] = c2.exact();
+        }
       }
     }
+    __syncthreads();
     // x = w - sum h_i v_i / |v_i|^2, v_{j+1} = x / beta
-    R e2 = 0;
-    for (int i = 0; i <= j; ++i) {
-      const R a = (R)coef[i].x, c2 = (R)coef[i].y;
-      e2 += (a * a + c2 * c2) * (R)is2[i];
+    R invb = 0, nn = 0;
+    if (tid < nr || warp == nw - 1) {
+      R e2 = 0;
+      for (int i = 0; i <= j; ++i) e2 += (dots[i].re * dots[i].re + dots[i].im * dots[i].im) * is2[i];
+      const R ww = dots[j + 1].re;
+      const R d2 = max(ww - e2, OP::kFloor * ww);
+      invb = d2 > (R)0 ? rsqrt_of(d2) : (R)0;
     }
-    const R ww = (R)coef[j + 1].x;
-    const R d2 = max(ww - e2, OP::kFloor * ww);
-    const R invb = d2 > (R)0 ? rsqrt_of(d2) : (R)0;
-    R nn = 0;
     for (int e = tid; e < nr; e += nt) {
       C t = w[e];
       for (int i = 0; i <= j; ++i) {
-        const R f = (R)is2[i];
-        const C a = cmk(-(R)coef[i].x * f, -(R)coef[i].y * f);
-        cfma(t, a, basis[i * rows + e]);
+        const R f = is2[i];
+        cfma(t, cmk(-dots[i].re * f, -dots[i].im * f), basis[i * rows + e]);
       }
       nn += t.re * t.re + t.im * t.im;
       if (j + 1 < k) {
@@ -275,23 +289,30 @@ __global__ void __launch_bounds__(768) coarse_gmres_cluster_kernel(const typenam
     }
     all_norm(nn, j & 1);
     cluster_barrier();
-    if (warp == 0) {
-      const double nrm = sqrt(fmax(sum16(pn[(j & 1) * kSolveCluster + (lane & 15)]), 0.0));
+    if (warp == nw - 1) {                                    // while the others start the next product
+      const Sum16<R> q = sum16(pn[(j & 1) * kSolveCluster + (lane & 15)]);
+      const R s2 = q.value() * invb * invb;
+      if (lane == 0) is2[j + 1] = s2 > (R)0 ? (R)1 / s2 : (R)0;
+      const double nrm = sqrt(fmax(q.exact(), 0.0));
+      if (lane <= j) {
+        hr[lane + 33 * j] *= is[lane];
+        hi[lane + 33 * j] *= is[lane];
+      }
+      __syncwarp();
       if (lane == 0) {
-        hr[j + 1 + 33 * j] = nrm * is[j];
-        const double s = nrm * (double)invb, q = s > 0.0 ? 1.0 / s : 0.0;
-        is[j + 1] = q;
-        is2[j + 1] = q * q;
+        hr[j + 1 + 33 * j] = nrm;
+        const double sc = nrm * (double)invb;
+        is[j + 1] = sc > 0.0 ? 1.0 / sc : 0.0;
       }
     }
-    // is[j + 1] is first read after the barriers of the next step's products
+    // is2[j + 1] is first read after the barriers of the next step's products
   }
   __syncthreads();
   if (warp == 0) {
     const unsigned zero = __ballot_sync(0xffffffffu, lane < k && hr[min(lane, k - 1) + 1 + 33 * min(lane, k - 1)] == 0.0);
     const int mm = zero ? __ffs(zero) : k;                   // columns up to the first zero subdiagonal entry
     const Cplx<double> y = beta0 > 0.0 ? hessenberg_warp(hr, hi, mm, beta0) : cmk(0.0, 0.0);
-    if (lane < k) coef[lane] = lane < mm ? make_double2(y.re * is[lane], y.im * is[lane]) : make_double2(0, 0);
+    if (lane < k) coef[lane] = lane < mm ? make_double2(y.re, y.im) : make_double2(0, 0);
   }
   __syncthreads();
   for (int e = tid; e < nr; e += nt) {
@@ -303,19 +324,19 @@ __global__ void __launch_bounds__(768) coarse_gmres_cluster_kernel(const typenam
 
 // Whether the cluster form holds a system of this size on the current device
 // (sixteen CTAs are more than the portable cluster; asked once per process).
-template <class OP, class TX>
+template <class OP, class TX, int N2>
 bool device_takes_cluster() {
   static const bool ok = [] {
-    if (cudaFuncSetAttribute(coarse_gmres_cluster_kernel<OP, TX>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
-            cudaSuccess ||
-        cudaFuncSetAttribute(coarse_gmres_cluster_kernel<OP, TX>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if (cudaFuncSetAttribute(coarse_gmres_cluster_kernel<OP, TX, N2>, cudaFuncAttributeNonPortableClusterSizeAllowed,
+                             1) != cudaSuccess ||
+        cudaFuncSetAttribute(coarse_gmres_cluster_kernel<OP, TX, N2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              227 * 1024 - 256) != cudaSuccess) {
       cudaGetLastError();
       return false;
     }
     ClusterLaunch l(kSolveCluster, 768, 220 * 1024, kSolveCluster, nullptr);
     int nclusters = 0;
-    if (cudaOccupancyMaxActiveClusters(&nclusters, coarse_gmres_cluster_kernel<OP, TX>, &l.cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&nclusters, coarse_gmres_cluster_kernel<OP, TX, N2>, &l.cfg) != cudaSuccess) {
       cudaGetLastError();
       return false;
     }
@@ -330,13 +351,13 @@ bool fits(const CGeom& c, int k) {
   return c.n2 % 2 == 0 && c.n2 <= 64 && spc <= 4 && k <= 32 && layout<OP>(spc, c.nsites, c.n2, k).total <= 220 * 1024;
 }
 
-template <class OP, class TX>
+template <class OP, class TX, int N2>
 int run(const CGeom& c, const void* M, const void* b, void* x, int k, int R, int* err, cudaStream_t s) {
   const int spc = (c.nsites + kSolveCluster - 1) / kSolveCluster;
-  const int threads = std::min(768, std::max(128, (spc * 9 * c.n2 + 31) / 32 * 32));
+  const int threads = std::min(768, std::max(96, (spc * 9 * c.n2 + 31) / 32 * 32) + 32);
   ClusterLaunch l((unsigned)(R * kSolveCluster), (unsigned)threads, (size_t)layout<OP>(spc, c.nsites, c.n2, k).total,
                   kSolveCluster, s);
-  SAPMG_CUDA_TRY(cudaLaunchKernelEx(&l.cfg, coarse_gmres_cluster_kernel<OP, TX>, (const typename OP::M*)M,
+  SAPMG_CUDA_TRY(cudaLaunchKernelEx(&l.cfg, coarse_gmres_cluster_kernel<OP, TX, N2>, (const typename OP::M*)M,
                                     (const TX*)b, (TX*)x, c, spc, k, err));
   count_launches(1);
   return MG_OK;
@@ -345,15 +366,19 @@ int run(const CGeom& c, const void* M, const void* b, void* x, int k, int R, int
 }  // namespace
 
 bool coarse_gmres_cluster_ok(int store, const CGeom& c, int k) {
-  if (store == P16) return fits<HalfOp>(c, k) && device_takes_cluster<HalfOp, float2>();
-  if (store == P64) return fits<DoubleOp>(c, k) && device_takes_cluster<DoubleOp, double2>();
+  if (store == P16)
+    return fits<HalfOp>(c, k) &&
+           (c.n2 == 40 ? device_takes_cluster<HalfOp, float2, 40>() : device_takes_cluster<HalfOp, float2, 0>());
+  if (store == P64) return fits<DoubleOp>(c, k) && device_takes_cluster<DoubleOp, double2, 0>();
   return false;
 }
 
 int launch_coarse_gmres_cluster(int store, const CGeom& c, const void* M, const void* b, void* x, int k, int R,
                                 int* err, cudaStream_t s) {
-  if (store == P16) return run<HalfOp, float2>(c, M, b, x, k, R, err, s);
-  if (store == P64) return run<DoubleOp, double2>(c, M, b, x, k, R, err, s);
+  if (store == P16)
+    return c.n2 == 40 ? run<HalfOp, float2, 40>(c, M, b, x, k, R, err, s)
+                      : run<HalfOp, float2, 0>(c, M, b, x, k, R, err, s);
+  if (store == P64) return run<DoubleOp, double2, 0>(c, M, b, x, k, R, err, s);
   return MG_ERR_ARG;
 }
 
