@@ -217,12 +217,6 @@ __device__ __forceinline__ P2 ldg2(const float2* __restrict__ f, size_t stride, 
   P2 p; p.re = make_float2(a.x, b.x); p.im = make_float2(a.y, b.y); return p;
 }
 
-// the same of a right-hand side that may be absent (nullptr: zero)
-__device__ __forceinline__ P2 ldb2(const float2* __restrict__ b, size_t stride, size_t idx) {
-  if (b) return ldg2(b, stride, idx);
-  P2 p; p.re = p.im = f2(0.f); return p;
-}
-
 template <int MU, class TG>
 __device__ __forceinline__ void global_hops2(const Geom& g, const float2* __restrict__ z, size_t stride,
                                              const TG* __restrict__ U, int blk, int loc, P2 (&acc)[12]) {

@@ -67,7 +67,9 @@ __device__ __forceinline__ void block_reduce6(float2& a, float2& b, float2& c, f
   c = make_float2(s1.x, s1.y);
 }
 
-template <class TG, bool KEEP_RHO, int MINB>
+// HB false: b is zero and not read (the set-up's sweeps).  A template argument, since a
+// test of the pointer at each load cost 1.4% of a pass.
+template <class TG, bool KEEP_RHO, int MINB, bool HB = true>
 __global__ void __launch_bounds__(256, MINB)
     sap_colour_pair_kernel(float2* __restrict__ z, const float2* __restrict__ b, const TG* __restrict__ U,
                            const TG* __restrict__ A, Geom g, int colour, int n_mr, int npairs) {
@@ -78,7 +80,7 @@ __global__ void __launch_bounds__(256, MINB)
   const size_t stride = (size_t)g.V * 12;                                // one right-hand side
   const size_t off = (size_t)(blockIdx.x % npairs) * 2 * stride;
   z += off;
-  if (b) b += off;
+  if (HB) b += off;
   const int blk = colour_block(g, blockIdx.x / npairs, colour);
   const int loc = threadIdx.x;
   const size_t site0 = (size_t)blk * 12 * 256 + loc;
@@ -96,7 +98,9 @@ __global__ void __launch_bounds__(256, MINB)
     global_hops2<3>(g, z, stride, U, blk, loc, acc);
 #pragma unroll
     for (int c = 0; c < 12; ++c) {
-      const P2 bb = ldb2(b, stride, site0 + c * 256);
+      P2 bb;
+      if (HB) bb = ldg2(b, stride, site0 + c * 256);
+      else bb.re = bb.im = f2(0.f);
       P2 r;
       r.re = sub2(bb.re, acc[c].re);
       r.im = sub2(bb.im, acc[c].im);
@@ -268,7 +272,7 @@ __device__ __forceinline__ void residual_pair(const Geom& g, const float2* __res
   }
 #pragma unroll
   for (int c = 0; c < 12; ++c) {
-    const P2 bb = ldb2(b, stride, site0 + c * 256);
+    const P2 bb = ldg2(b, stride, site0 + c * 256);
     P2 r;
     r.re = sub2(bb.re, acc[c].re);
     r.im = sub2(bb.im, acc[c].im);
@@ -314,7 +318,7 @@ __global__ void __launch_bounds__(256, 1)
   }
   for (int pr = 0; pr < npairs; ++pr) {
     float2* zp = z + (size_t)pr * 2 * stride;
-    if (pr > 0) residual_pair<true>(g, zp, b ? b + (size_t)pr * 2 * stride : nullptr, stride, U, A, Us, As, blk, loc, rs);
+    if (pr > 0) residual_pair<true>(g, zp, b + (size_t)pr * 2 * stride, stride, U, A, Us, As, blk, loc, rs);
     P2 e[12];
     for (int it = 0; it < n_mr; ++it) {
       __syncthreads();                                 // rho of every site written
@@ -487,7 +491,7 @@ __device__ __forceinline__ void residual_b(const float2* __restrict__ b, size_t 
 #pragma unroll
   for (int k = 0; k < 6; ++k) {
     const int c = 6 * H + k;
-    const P2 bb = ldb2(b, stride, site0 + c * 256);
+    const P2 bb = ldg2(b, stride, site0 + c * 256);
     P2 r;
     r.re = sub2(bb.re, acc[c].re);
     r.im = sub2(bb.im, acc[c].im);
@@ -604,7 +608,7 @@ __global__ void __launch_bounds__(512, 1)
   for (int pr = 0; pr < npairs; ++pr) {
     float2* zp = z + (size_t)pr * 2 * stride;
     if (pr > 0) {
-      const float2* bp = b ? b + (size_t)pr * 2 * stride : nullptr;
+      const float2* bp = b + (size_t)pr * 2 * stride;
       __syncthreads();                      // every read of the previous pair's swap buffer done
       if (h0) residual_a<0, true>(g, zp, stride, U, A, Us, As, blk, loc, xs, acc);
       else residual_a<1, true>(g, zp, stride, U, A, Us, As, blk, loc, xs, acc);
@@ -667,18 +671,18 @@ static int run_block(const Geom& g, void* z, const void* b, const void* U, const
   return MG_OK;
 }
 
-template <class TG, bool KEEP_RHO, int MINB>
+template <class TG, bool KEEP_RHO, int MINB, bool HB = true>
 static int run_pair(const Geom& g, void* z, const void* b, const void* U, const void* A, int colour, int n_mr,
                     int nrhs, cudaStream_t s) {
   const size_t smem = sizeof(float4) * (24 * 256 + 16);
   static bool attr = false;
   if (!attr) {
-    SAPMG_CUDA_TRY(cudaFuncSetAttribute(sap_colour_pair_kernel<TG, KEEP_RHO, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    SAPMG_CUDA_TRY(cudaFuncSetAttribute(sap_colour_pair_kernel<TG, KEEP_RHO, MINB, HB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         (int)smem));
     attr = true;
   }
   const int npairs = nrhs / 2;
-  sap_colour_pair_kernel<TG, KEEP_RHO, MINB><<<(unsigned)(g.nblocks / 2 * npairs), 256, smem, s>>>(
+  sap_colour_pair_kernel<TG, KEEP_RHO, MINB, HB><<<(unsigned)(g.nblocks / 2 * npairs), 256, smem, s>>>(
       (float2*)z, (const float2*)b, (const TG*)U, (const TG*)A, g, colour, n_mr, npairs);
   count_launches(1);
   SAPMG_CUDA_TRY(cudaGetLastError());
@@ -692,7 +696,8 @@ int launch_sap_colour_pair(int prec, const Geom& g, void* z, const void* b, cons
   if (shape >= 3 && !err) return MG_ERR_ARG;
   if (nrhs < 2 || nrhs % 2 != 0 || n_mr < 1) return MG_ERR_ARG;
 #define SAPMG_PAIR_CASE(T)                                                                   \
-  return shape == 6 ? run_split<T>(g, z, b, U, A, colour, n_mr, nrhs, err, s)               \
+  return !b ? run_pair<T, false, 2, false>(g, z, b, U, A, colour, n_mr, nrhs, s)              \
+       : shape == 6 ? run_split<T>(g, z, b, U, A, colour, n_mr, nrhs, err, s)               \
        : shape == 5 ? run_block<T, 2>(g, z, b, U, A, colour, n_mr, nrhs, err, s)             \
        : shape == 4 ? run_block<T, 1>(g, z, b, U, A, colour, n_mr, nrhs, err, s)             \
        : shape == 3 ? run_block<T, 0>(g, z, b, U, A, colour, n_mr, nrhs, err, s)             \
