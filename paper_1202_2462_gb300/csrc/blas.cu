@@ -332,13 +332,25 @@ __global__ void axpby_kernel(Scal32 a, const TX* __restrict__ x, Scal32 b, TY* _
   const int r = blockIdx.y;
   const R ar = (R)a.v[r].x, ai = (R)a.v[r].y, br = (R)b.v[r].x, bi = (R)b.v[r].y;
   const bool yz = (b.v[r].x == 0.0 && b.v[r].y == 0.0);
+  // real scalars (every solver update): half the products, which for FP64, where
+  // they were the bound, is 1.72 -> 1.11 ms for x64 += s e32 (12 fields of 7.96 M) and
+  // 1.32 -> 0.72 ms for r = b - r in FP64
+  const bool real = a.v[r].y == 0.0 && b.v[r].y == 0.0;
   const TX* xr = x + r * xs;
   TY* yr = y + r * ys;
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
     const TX u = xr[i];
     const R ux = (R)u.x, uy = (R)u.y;
     TY o;
-    if (yz) {
+    if (real) {
+      o.x = ar * ux;
+      o.y = ar * uy;
+      if (!yz) {
+        const TY v = yr[i];
+        o.x += br * v.x;
+        o.y += br * v.y;
+      }
+    } else if (yz) {
       o.x = ar * ux - ai * uy;
       o.y = ar * uy + ai * ux;
     } else {
@@ -780,10 +792,26 @@ __device__ __forceinline__ uint2 f4_to_h4(float4 v) {
 }
 
 // pass 1 with an FP16 basis: slots as dots2_partial
+// From kRingFrom basis vectors on each thread copies its next element of every vector
+// to shared memory while it works on the current one: the compiler spreads that
+// many loads between the products, which leaves too few bytes in flight (8 vectors,
+// 12 fields of 7.96 M: 1401 us by plain loads, 676 us so, 677 us at the measured HBM
+// rate; 6 vectors by plain loads 581 us, 564 us at that rate).
+constexpr int kRingFrom = 7;
+constexpr size_t dots2h_smem(int K) { return K >= kRingFrom ? (size_t)2 * 256 * (8 * K + 32) : 0; }
+__device__ __forceinline__ void cp_async(void* dst, const uint2* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async(void* dst, const float4* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
 template <int K, bool EXTRA>
 __global__ void __launch_bounds__(256) dots2h_partial(PtrsV<uint2> v, const float4* __restrict__ u,
                                                       const float4* __restrict__ w, size_t nu, size_t stride,
                                                       double2* __restrict__ partial, Dcgs2Out dout) {
+  constexpr bool kRing = K >= kRingFrom;
+  extern __shared__ __align__(16) float4 ring[];       // per stage [2][256] float4, [K][256] uint2
+  constexpr int kStage4 = 256 * (2 + K / 2) + (K % 2) * 128;
   constexpr int NS = 2 * K + (EXTRA ? 3 : 0);
   const int r = blockIdx.y;
   const float4* ur = u + r * stride;
@@ -791,12 +819,38 @@ __global__ void __launch_bounds__(256) dots2h_partial(PtrsV<uint2> v, const floa
   float re[NS > 0 ? NS : 1], im[NS > 0 ? NS : 1];
 #pragma unroll
   for (int q = 0; q < NS; ++q) re[q] = im[q] = 0.f;
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < nu; i += (size_t)gridDim.x * blockDim.x) {
-    uint2 a[K > 0 ? K : 1];
+  const size_t i0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x, step = (size_t)gridDim.x * blockDim.x;
+  auto fetch = [&](size_t i, int st) {                 // a thread reads back its own copies only
+    if (i < nu) {
+      float4* d = ring + st * kStage4 + threadIdx.x;
+      uint2* e = reinterpret_cast<uint2*>(ring + st * kStage4 + 512) + threadIdx.x;
+      cp_async(d, ur + i);
+      cp_async(d + 256, wr + i);
 #pragma unroll
-    for (int q = 0; q < K; ++q) a[q] = __ldg(v.p[q] + r * stride + i);
-    const float4 x = __ldg(ur + i);
-    const float4 y = __ldg(wr + i);
+      for (int q = 0; q < K; ++q) cp_async(e + q * 256, v.p[q] + r * stride + i);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  if (kRing) fetch(i0, 0);
+  int st = 0;
+  for (size_t i = i0; i < nu; i += step, st ^= 1) {
+    uint2 a[K > 0 ? K : 1];
+    float4 x, y;
+    if (kRing) {
+      fetch(i + step, st ^ 1);
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+      const float4* d = ring + st * kStage4 + threadIdx.x;
+      const uint2* e = reinterpret_cast<const uint2*>(ring + st * kStage4 + 512) + threadIdx.x;
+      x = d[0];
+      y = d[256];
+#pragma unroll
+      for (int q = 0; q < K; ++q) a[q] = e[q * 256];
+    } else {
+#pragma unroll
+      for (int q = 0; q < K; ++q) a[q] = __ldg(v.p[q] + r * stride + i);
+      x = __ldg(ur + i);
+      y = __ldg(wr + i);
+    }
 #pragma unroll
     for (int q = 0; q < K; ++q) {
       const float4 av = h4_to_f4(a[q]);
@@ -895,6 +949,23 @@ __global__ void __launch_bounds__(256) axpy2h_kernel(PtrsV<uint2> v, const doubl
   }
 }
 
+template <int K, bool EXTRA>
+static cudaError_t dots2h_run(dim3 grid, const PtrsV<uint2>& p, const float4* u, const float4* w, size_t nu,
+                              size_t stride, double2* partial, const Dcgs2Out& d, cudaStream_t s) {
+  if (dots2h_smem(K) > 0) {
+    static bool attr = false;
+    if (!attr) {
+      const cudaError_t e = cudaFuncSetAttribute(dots2h_partial<K, EXTRA>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 (int)dots2h_smem(K));
+      if (e != cudaSuccess) return e;
+      attr = true;
+    }
+  }
+  dots2h_partial<K, EXTRA><<<grid, 256, dots2h_smem(K), s>>>(p, u, w, nu, stride, partial, d);
+  count_launches(1);
+  return cudaGetLastError();
+}
+
 int blas_dcgs2_step_h(const BVec& b, const void* const* vh, int j, void* u, void* w, void* vout, const DcgsWork& ws,
                       cudaStream_t s) {
   if (b.R <= 0) return MG_OK;
@@ -921,16 +992,17 @@ int blas_dcgs2_step_h(const BVec& b, const void* const* vh, int j, void* u, void
     for (int q = 0; q < 16; ++q) p.p[q] = j > 0 ? (const uint2*)vh[std::max(0, std::min(j0 + q, j - 1))] : (const uint2*)vout;
 #define SAPMG_D2H(K)                                                                                              \
   case K:                                                                                                         \
-    if (extra) { dots2h_partial<K, true><<<g1, 256, 0, s>>>(p, uf, wf, nu, stride, ws.partial, d); }                \
-    else { dots2h_partial<K, false><<<g1, 256, 0, s>>>(p, uf, wf, nu, stride, ws.partial, d); }                     \
-    count_launches(1);                                                                                            \
+    if (extra) rc = dots2h_run<K, true>(g1, p, uf, wf, nu, stride, ws.partial, d, s);                              \
+    else rc = dots2h_run<K, false>(g1, p, uf, wf, nu, stride, ws.partial, d, s);                                   \
     break;
+    cudaError_t rc = cudaSuccess;
     switch (kk) {
       SAPMG_D2H(0) SAPMG_D2H(1) SAPMG_D2H(2) SAPMG_D2H(3) SAPMG_D2H(4) SAPMG_D2H(5) SAPMG_D2H(6)
       SAPMG_D2H(7) SAPMG_D2H(8) SAPMG_D2H(9) SAPMG_D2H(10) SAPMG_D2H(11) SAPMG_D2H(12)
       default: return MG_ERR_ARG;
     }
 #undef SAPMG_D2H
+    SAPMG_CUDA_TRY(rc);
     j0 += kk;
   } while (j0 < j);
   const dim3 g2(reduce_ctas(nu, R), R);
@@ -1136,33 +1208,37 @@ __global__ void __launch_bounds__(256) arnoldi_dots_kernel(PtrsK<typename B::V> 
   typedef typename B::V V;
   const int r = blockIdx.y, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const typename B::W* wr = w + r * stride;
-  R acc[KM][2], ww = 0;
-#pragma unroll
-  for (int q = 0; q < KM; ++q) acc[q][0] = acc[q][1] = 0;
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < nu; i += (size_t)gridDim.x * blockDim.x) {
-    const typename B::W x = wr[i];
-#pragma unroll
-    for (int g = 0; g < KM; g += 8) {                    // up to eight loads in flight
-      constexpr int G = KM < 8 ? KM : 8;
-      V a[G];
-#pragma unroll
-      for (int q = 0; q < G; ++q)
-        if (g + q < k) a[q] = __ldg(v.p[g + q] + r * stride + i);
-#pragma unroll
-      for (int q = 0; q < G; ++q)
-        if (g + q < k) cdot_acc(B::get(a[q]), x, acc[g + q][0], acc[g + q][1]);
-    }
-    ww += nrm_of(x);
-  }
-  constexpr int NV = 2 * KM < 32 ? 2 * KM : 32, NG = 2 * KM / NV;
+  // Sixteen vectors a sweep: with all 32 vectors' sums in registers the compiler spreads
+  // the loads between the products, and a step on 20 vectors (12 fields of 103680) took
+  // 107 us, against 23 us of one on 16 and 44 us so; w is read again, from L2 mostly.
+  constexpr int KS = KM < 16 ? KM : 16, NV = 2 * KS;
   __shared__ R red[8][2 * KM + 1];
+  R ww = 0;
 #pragma unroll
-  for (int g = 0; g < NG; ++g) {
+  for (int h = 0; h < KM; h += KS) {
+    R acc[KS][2];
+#pragma unroll
+    for (int q = 0; q < KS; ++q) acc[q][0] = acc[q][1] = 0;
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < nu; i += (size_t)gridDim.x * blockDim.x) {
+      const typename B::W x = wr[i];
+#pragma unroll
+      for (int g = 0; g < KS; g += 8) {                  // up to eight loads in flight
+        constexpr int G = KS < 8 ? KS : 8;
+        V a[G];
+#pragma unroll
+        for (int q = 0; q < G; ++q)
+          if (h + g + q < k) a[q] = __ldg(v.p[h + g + q] + r * stride + i);
+#pragma unroll
+        for (int q = 0; q < G; ++q)
+          if (h + g + q < k) cdot_acc(B::get(a[q]), x, acc[g + q][0], acc[g + q][1]);
+      }
+      if (h == 0) ww += nrm_of(x);
+    }
     R u[NV];
 #pragma unroll
-    for (int q = 0; q < NV; ++q) u[q] = acc[(g * NV + q) >> 1][q & 1];
+    for (int q = 0; q < NV; ++q) u[q] = acc[q >> 1][q & 1];
     const R t = warp_sums<NV>(u);
-    if (lane % (32 / NV) == 0) red[wid][g * NV + lane / (32 / NV)] = t;
+    if (lane % (32 / NV) == 0) red[wid][2 * h + lane / (32 / NV)] = t;
   }
   ww = warp_sum(ww);
   if (lane == 0) red[wid][2 * KM] = ww;
