@@ -4,8 +4,8 @@
 // three spin-colour components, those whose clover rows it applies.
 //
 // One SM sub-partition issues an FP64 instruction of a warp every 64 cycles, so
-// with a warp per 32 sites the 1176 FP64 instructions of a site take 36 us
-// however few warps there are; four warps of 300 each take a quarter of that
+// with a warp per 32 sites the 1130 FP64 instructions of a site take 36 us
+// however few warps there are; four warps of 280 each take a quarter of that
 // as long as there are sub-partitions for them (608 on the chip).
 #pragma once
 #include "stencil.cuh"
@@ -18,14 +18,15 @@ template <int MU, class R, class TG, bool DAG, class LD, class KEEP>
 __device__ __forceinline__ void quad_hops(const Geom& g, const TG* __restrict__ U, int blk, int loc, LD ld, KEEP keep,
                                           Cplx<R> (&acc)[12]) {
   constexpr int SF = DAG ? 1 : -1;
-#pragma unroll
-  for (int c = 0; c < 12; ++c) acc[c] = cmk<R>(0, 0);
   Cplx<R> h[6], gg[6], u[9];
   if (keep(1)) {
     spin_project_ld<MU, SF, R>([&](int c) { return ld(1, c); }, h);
     load_link<R>(U, blk, MU, loc, u);
     su3_mul(u, h, gg);
-    spin_reconstruct_add<MU, SF>(gg, acc);
+    spin_reconstruct_add<MU, SF, R, kSet>(gg, acc);
+  } else {
+#pragma unroll
+    for (int c = 0; c < 12; ++c) acc[c] = cmk<R>(0, 0);
   }
   if (keep(-1)) {
     int nb, nl;

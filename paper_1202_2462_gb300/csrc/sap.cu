@@ -24,7 +24,7 @@ __device__ __forceinline__ void load_smem_spinor(const Cplx<R>* __restrict__ s, 
   for (int c = 0; c < 12; ++c) p[c] = s[c * 256 + loc];
 }
 
-// Sum of the hops of D_i at loc (neighbours inside the block only, from shared memory).
+// acc - (hops of D_i at loc) / 2 (neighbours inside the block only, from shared memory).
 template <int MU, class R, class TG>
 __device__ __forceinline__ void block_hops_dir(const TG* __restrict__ U, const Cplx<R>* __restrict__ rs, int blk,
                                                int loc, Cplx<R> (&acc)[12]) {
@@ -36,14 +36,14 @@ __device__ __forceinline__ void block_hops_dir(const TG* __restrict__ U, const C
     spin_project_ld<MU, -1, R>([&](int k) { return q[k * 256]; }, h);
     load_link<R>(U, blk, MU, loc, u);
     su3_mul(u, h, gg);
-    spin_reconstruct_add<MU, -1>(gg, acc);
+    spin_reconstruct_add<MU, -1, R, kHalf>(gg, acc);
   }
   if (c > 0) {
     const Cplx<R>* q = rs + loc - ls;
     spin_project_ld<MU, 1, R>([&](int k) { return q[k * 256]; }, h);
     load_link<R>(U, blk, MU, loc - ls, u);
     su3_dag_mul(u, h, gg);
-    spin_reconstruct_add<MU, 1>(gg, acc);
+    spin_reconstruct_add<MU, 1, R, kHalf>(gg, acc);
   }
 }
 
@@ -80,7 +80,7 @@ __global__ void __launch_bounds__(256, (sizeof(R) == 4 ? 2 : 1))
   const int loc = threadIdx.x;
 
   // residual r = b - D z (Algorithm 1: residual update before the colour's block solves);
-  // with acc = -2 A z + sum of hops, D z = -acc/2 and r = b + acc/2
+  // acc = D z = A z - (sum of hops) / 2
   {
     Cplx<R> acc[12];
     {
@@ -88,22 +88,19 @@ __global__ void __launch_bounds__(256, (sizeof(R) == 4 ? 2 : 1))
       load_spinor<R>(z, blk, loc, zz);
       clover_apply<R>(A, blk, loc, zz, acc);
     }
-#pragma unroll
-    for (int c = 0; c < 12; ++c) acc[c] = (R)(-2) * acc[c];
-    hops_global_dir<0>(g, z, U, blk, loc, acc);
+    hops_global_dir<0, R, TS, TG, false, kHalf>(g, z, U, blk, loc, acc);
     asm volatile("" ::: "memory");
-    hops_global_dir<1>(g, z, U, blk, loc, acc);
+    hops_global_dir<1, R, TS, TG, false, kHalf>(g, z, U, blk, loc, acc);
     asm volatile("" ::: "memory");
-    hops_global_dir<2>(g, z, U, blk, loc, acc);
+    hops_global_dir<2, R, TS, TG, false, kHalf>(g, z, U, blk, loc, acc);
     asm volatile("" ::: "memory");
-    hops_global_dir<3>(g, z, U, blk, loc, acc);
+    hops_global_dir<3, R, TS, TG, false, kHalf>(g, z, U, blk, loc, acc);
     const size_t bq = (size_t)blk * 12 * 256 + loc;
 #pragma unroll
-    for (int c = 0; c < 12; ++c) {
-      rs[c * 256 + loc] = (b ? Io<R, TS>::ldc(b + bq + c * 256) : cmk<R>(0, 0)) + (R)0.5 * acc[c];
-      es[c * 256 + loc] = cmk<R>(0, 0);
-    }
+    for (int c = 0; c < 12; ++c)
+      rs[c * 256 + loc] = (b ? Io<R, TS>::ldc(b + bq + c * 256) : cmk<R>(0, 0)) - acc[c];
   }
+  TS* zq = z + (size_t)blk * 12 * 256 + loc;
 
   // n_MR minimal-residual steps on D_i e = r, D_i the block operator (hops leaving the block dropped)
   for (int it = 0; it < n_mr; ++it) {
@@ -114,8 +111,6 @@ __global__ void __launch_bounds__(256, (sizeof(R) == 4 ? 2 : 1))
       load_smem_spinor(rs, loc, ro);
       clover_apply<R>(A, blk, loc, ro, p);
     }
-#pragma unroll
-    for (int c = 0; c < 12; ++c) p[c] = (R)(-2) * p[c];
     // the empty asm statements keep the compiler from hoisting the next
     // direction's loads (which would raise register pressure past the limit)
     block_hops_dir<0>(U, rs, blk, loc, p);
@@ -128,7 +123,6 @@ __global__ void __launch_bounds__(256, (sizeof(R) == 4 ? 2 : 1))
     R pr_re = 0, pr_im = 0, pp = 0;
 #pragma unroll
     for (int c = 0; c < 12; ++c) {
-      p[c] = (R)(-0.5) * p[c];
       const Cplx<R> ro = rs[c * 256 + loc];
       pr_re += p[c].re * ro.re + p[c].im * ro.im;
       pr_im += p[c].re * ro.im - p[c].im * ro.re;
@@ -137,17 +131,20 @@ __global__ void __launch_bounds__(256, (sizeof(R) == 4 ? 2 : 1))
     block_reduce3(pr_re, pr_im, pp, red);            // contains the barrier after all neighbour reads
     Cplx<R> alpha = cmk<R>(0, 0);
     if (pp > (R)0) alpha = cmk(pr_re / pp, pr_im / pp);
+    // the first step starts e, the last adds it to z (own site only: no barrier needed)
 #pragma unroll
     for (int c = 0; c < 12; ++c) {
       const Cplx<R> ro = rs[c * 256 + loc];
-      es[c * 256 + loc] = es[c * 256 + loc] + alpha * ro;
-      rs[c * 256 + loc] = ro - alpha * p[c];
+      Cplx<R> e = alpha * ro;
+      if (it > 0) e = es[c * 256 + loc] + e;
+      if (it == n_mr - 1) {
+        Io<R, TS>::st(zq + c * 256, Io<R, TS>::ldc(zq + c * 256) + e);
+      } else {
+        es[c * 256 + loc] = e;
+        rs[c * 256 + loc] = ro - alpha * p[c];
+      }
     }
   }
-  // z += e on the block (own site only: no barrier needed)
-  TS* zq = z + (size_t)blk * 12 * 256 + loc;
-#pragma unroll
-  for (int c = 0; c < 12; ++c) Io<R, TS>::st(zq + c * 256, Io<R, TS>::ldc(zq + c * 256) + es[c * 256 + loc]);
 }
 
 // The same pass with a block on a cluster of eight CTAs of 32 sites, four threads

@@ -46,20 +46,28 @@ __device__ __forceinline__ void spin_project_ld(LD ld, Cplx<R> (&h)[6]) {
 }
 
 // acc_u += g, acc_l += S * X_MU^dagger g
-template <int MU, int S, class R>
+enum { kAdd, kHalf, kSet };
+template <int MU, int S, class R, int HOW = kAdd>
 __device__ __forceinline__ void spin_reconstruct_add(const Cplx<R> (&g)[6], Cplx<R> (&acc)[12]) {
+  // acc + x, or with HOW = kHalf acc - x / 2 as an exact product in an FMA, or with HOW = kSet x alone
+  auto put = [](Cplx<R>& a, Cplx<R> x) {
+    if constexpr (HOW == kHalf) { a.re = fma((R)-0.5, x.re, a.re); a.im = fma((R)-0.5, x.im, a.im); }
+    else if constexpr (HOW == kSet) a = x;
+    else a = a + x;
+  };
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     const Cplx<R> g0 = g[c], g1 = g[3 + c];
-    acc[c] = acc[c] + g0;
-    acc[3 + c] = acc[3 + c] + g1;
+    put(acc[c], g0);
+    put(acc[3 + c], g1);
     Cplx<R> x0, x1;
     if (MU == 0) { x0 = mul_i(g1); x1 = mul_i(g0); }
     else if (MU == 1) { x0 = g1; x1 = cmk(-g0.re, -g0.im); }
     else if (MU == 2) { x0 = mul_i(g0); x1 = mul_mi(g1); }
     else { x0 = g0; x1 = g1; }
-    if (S > 0) { acc[6 + c] = acc[6 + c] + x0; acc[9 + c] = acc[9 + c] + x1; }
-    else { acc[6 + c] = acc[6 + c] - x0; acc[9 + c] = acc[9 + c] - x1; }
+    if (S < 0) { x0 = cmk(-x0.re, -x0.im); x1 = cmk(-x1.re, -x1.im); }
+    put(acc[6 + c], x0);
+    put(acc[9 + c], x1);
   }
 }
 
@@ -171,7 +179,8 @@ __device__ __forceinline__ void hop_bwd(const TG* __restrict__ U, int nblk, int 
 // gamma5 (1 -+ gamma_mu) gamma5 = (1 +- gamma_mu) (gamma5 anticommutes with
 // gamma_mu; the clover term commutes with gamma5 and is Hermitian, so it is
 // the same in D and D^dagger).
-template <int MU, class R, class TS, class TG, bool DAG = false>
+// HOW = kHalf: acc - hops / 2.
+template <int MU, class R, class TS, class TG, bool DAG = false, int HOW = kAdd>
 __device__ __forceinline__ void hops_global_dir(const Geom& g, const TS* __restrict__ f, const TG* __restrict__ U,
                                                 int blk, int loc, Cplx<R> (&acc)[12]) {
   constexpr int SF = DAG ? 1 : -1;   // projector sign of the forward hop
@@ -184,7 +193,7 @@ __device__ __forceinline__ void hops_global_dir(const Geom& g, const TS* __restr
   }
   load_link<R>(U, blk, MU, loc, u);
   su3_mul(u, h, gg);
-  spin_reconstruct_add<MU, SF>(gg, acc);
+  spin_reconstruct_add<MU, SF, R, HOW>(gg, acc);
   neighbour(g, blk, loc, MU, -1, nb, nl);
   {
     const TS* q = f + (size_t)nb * 12 * 256 + nl;
@@ -192,7 +201,7 @@ __device__ __forceinline__ void hops_global_dir(const Geom& g, const TS* __restr
   }
   load_link<R>(U, nb, MU, nl, u);
   su3_dag_mul(u, h, gg);
-  spin_reconstruct_add<MU, -SF>(gg, acc);
+  spin_reconstruct_add<MU, -SF, R, HOW>(gg, acc);
 }
 
 template <class R, class TS, class TG>
