@@ -74,6 +74,122 @@ __global__ void __launch_bounds__(256) prolong0_kernel(const TC* __restrict__ in
   store_spinor<R>(out + (size_t)rhs * nblocks * 12 * 256, blk, loc, o);
 }
 
+// The same two for FP32 vectors, with 16-byte loads of P (S consecutive sites of a
+// component).  Bound by P's bytes; with a 4-byte load a thread and, in the restriction,
+// 20 shuffles between one vector's loads and the next's, too few were in flight: 512
+// blocks, N = 20, FP16 P (126 MB, 19 us at the measured HBM rate): restriction 47.6 ->
+// 31 us, prolongation 41.3 -> 22 us.
+template <class TV> constexpr int kPack = 16 / (int)sizeof(TV);
+template <class TV>
+__device__ __forceinline__ void unpack_p(const uint4& w, Cplx<float> (&v)[kPack<TV>]) {
+#pragma unroll
+  for (int i = 0; i < kPack<TV>; ++i) v[i] = Io<float, TV>::ldc(reinterpret_cast<const TV*>(&w) + i);
+}
+
+// A warp sums the 256 sites of a vector (two vectors at a time, k and k + 8, against
+// the same words of r in shared memory) for the CTA's chirality.
+template <class TV>
+__global__ void __launch_bounds__(256, 4) restrict0_vec_kernel(const float2* __restrict__ in, float2* __restrict__ out,
+                                                            const TV* __restrict__ Pv, int N, int nrhs, int nblocks) {
+  constexpr int S = kPack<TV>, Q = 256 / S;
+  __shared__ float4 r[6 * 128];                              // [component][pair of S/2][Q] of two sites each
+  const int blk = MG_CLAMP(kAggregate, blockIdx.x / (2 * nrhs), nblocks), chi = blockIdx.x & 1;
+  const int rhs = (blockIdx.x >> 1) % nrhs;
+  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const float2* src = in + ((size_t)rhs * nblocks + blk) * 12 * 256 + chi * 6 * 256 + threadIdx.x;
+  {
+    const int l = threadIdx.x, at = (((l % S) >> 1) * Q + l / S) * 2 + (l & 1);
+#pragma unroll
+    for (int c = 0; c < 6; ++c) reinterpret_cast<float2*>(r)[c * 256 + at] = src[c * 256];
+  }
+  __syncthreads();
+  float2* o = out + ((size_t)rhs * nblocks + blk) * 2 * N + chi * N;
+  for (int k = wid; k < N; k += 16) {
+    const bool two = k + 8 < N;
+    const uint4* p0 = reinterpret_cast<const uint4*>(Pv + ((size_t)(blk * N + k) * 12 + chi * 6) * 256) + lane;
+    const uint4* p1 = two ? p0 + (size_t)8 * 12 * Q : p0;
+    Cplx<float> acc[2][S];
+#pragma unroll
+    for (int i = 0; i < S; ++i) acc[0][i] = acc[1][i] = cmk(0.f, 0.f);
+#pragma unroll
+    for (int c = 0; c < 6; ++c)
+#pragma unroll
+      for (int h = 0; h < Q / 32; ++h) {
+        const uint4 a = __ldg(p0 + c * Q + h * 32), b = __ldg(p1 + c * Q + h * 32);
+        Cplx<float> x[S], va[S], vb[S];
+#pragma unroll
+        for (int i = 0; i < S / 2; ++i) {
+          const float4 t = r[c * 128 + i * Q + h * 32 + lane];
+          x[2 * i] = cmk(t.x, t.y);
+          x[2 * i + 1] = cmk(t.z, t.w);
+        }
+        unpack_p<TV>(a, va);
+        unpack_p<TV>(b, vb);
+#pragma unroll
+        for (int i = 0; i < S; ++i) {
+          cfma_conj(acc[0][i], va[i], x[i]);
+          cfma_conj(acc[1][i], vb[i], x[i]);
+        }
+      }
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+#pragma unroll
+      for (int n = S / 2; n >= 1; n /= 2)
+#pragma unroll
+        for (int i = 0; i < n; ++i) acc[q][i] = acc[q][i] + acc[q][i + n];
+      const float re = warp_sum(acc[q][0].re), im = warp_sum(acc[q][0].im);
+      if (lane == 0 && (q == 0 || two)) o[k + 8 * q] = make_float2(re, im);
+    }
+  }
+}
+
+// A thread forms 12 / S components of S consecutive sites.  al: out starts on 16 bytes.
+template <class TV>
+__global__ void __launch_bounds__(256) prolong0_vec_kernel(const float2* __restrict__ in, float2* __restrict__ out,
+                                                           const TV* __restrict__ Pv, int N, int nrhs, int nblocks,
+                                                           bool al) {
+  constexpr int S = kPack<TV>, Q = 256 / S, C = 12 / S;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float2* e = reinterpret_cast<float2*>(smem_raw);               // [2N]
+  const int blk = MG_CLAMP(kAggregate, blockIdx.x / nrhs, nblocks), rhs = blockIdx.x % nrhs;
+  const int q = threadIdx.x % Q, c0 = threadIdx.x / Q * C;
+  const float2* ein = in + ((size_t)rhs * nblocks + blk) * 2 * N;
+  for (int t = threadIdx.x; t < 2 * N; t += 256) e[t] = ein[t];
+  __syncthreads();
+  const float2* ec = e + c0 / 6 * N;
+  Cplx<float> o[C][S];
+#pragma unroll
+  for (int c = 0; c < C; ++c)
+#pragma unroll
+    for (int i = 0; i < S; ++i) o[c][i] = cmk(0.f, 0.f);
+  const uint4* p = reinterpret_cast<const uint4*>(Pv + ((size_t)blk * N * 12 + c0) * 256) + q;
+#pragma unroll 4
+  for (int k = 0; k < N; ++k) {
+    const Cplx<float> ek = cmk(ec[k].x, ec[k].y);
+#pragma unroll
+    for (int c = 0; c < C; ++c) {
+      Cplx<float> v[S];
+      unpack_p<TV>(__ldg(p + (size_t)(k * 12 + c) * Q), v);
+#pragma unroll
+      for (int i = 0; i < S; ++i) cfma(o[c][i], v[i], ek);
+    }
+  }
+  float2* dst = out + (((size_t)rhs * nblocks + blk) * 12 + c0) * 256 + q * S;
+#pragma unroll
+  for (int c = 0; c < C; ++c)
+#pragma unroll
+    for (int i = 0; i < S; i += 2) {
+      float2* d = dst + c * 256 + i;
+      const Cplx<float> a = o[c][i], b = o[c][i + 1];
+      if (al) {
+        *reinterpret_cast<float4*>(d) = make_float4(a.re, a.im, b.re, b.im);
+      } else {
+        d[0] = make_float2(a.re, a.im);
+        d[1] = make_float2(b.re, b.im);
+      }
+    }
+}
+
 // Multi-RHS forms for the mixed precision (FP32 vectors):
 //
 // K3': CTA (block, chirality, group of RG right-hand sides).  The group's
@@ -538,19 +654,31 @@ static int transfer0_mrhs(bool restrict_, const Geom& g, const void* in, void* o
   return MG_OK;
 }
 
-template <class R, class TS, class TV, class TC>
-static int transfer0_run(bool restrict_, const Geom& g, const void* in, void* out, const void* Pv, int N, int nrhs,
-                         cudaStream_t s) {
+static int transfer0_fp64(bool restrict_, const Geom& g, const void* in, void* out, const void* Pv, int N, int nrhs,
+                          cudaStream_t s) {
   const unsigned grid = (unsigned)(g.nblocks * nrhs);   // right-hand side fastest: P shared through L2
-  if (restrict_) {
-    const size_t smem = sizeof(R) * 4 * 8 * N;
-    restrict0_kernel<R, TS, TV, TC><<<grid, 256, smem, s>>>((const TS*)in, (TC*)out, (const TV*)Pv, N, nrhs,
-                                                            g.nblocks); count_launches(1);
-  } else {
-    const size_t smem = sizeof(Cplx<R>) * 2 * N;
-    prolong0_kernel<R, TS, TV, TC><<<grid, 256, smem, s>>>((const TC*)in, (TS*)out, (const TV*)Pv, N, nrhs,
-                                                           g.nblocks); count_launches(1);
-  }
+  if (restrict_)
+    restrict0_kernel<double, double2, double2, double2><<<grid, 256, sizeof(double) * 4 * 8 * N, s>>>(
+        (const double2*)in, (double2*)out, (const double2*)Pv, N, nrhs, g.nblocks);
+  else
+    prolong0_kernel<double, double2, double2, double2><<<grid, 256, sizeof(double2) * 2 * N, s>>>(
+        (const double2*)in, (double2*)out, (const double2*)Pv, N, nrhs, g.nblocks);
+  count_launches(1);
+  SAPMG_CUDA_TRY(cudaGetLastError());
+  return MG_OK;
+}
+
+template <class TV>
+static int transfer0_vec(bool restrict_, const Geom& g, const void* in, void* out, const void* Pv, int N, int nrhs,
+                         cudaStream_t s) {
+  const unsigned grid = (unsigned)(g.nblocks * nrhs);
+  if (restrict_)
+    restrict0_vec_kernel<TV><<<2 * grid, 256, 0, s>>>((const float2*)in, (float2*)out, (const TV*)Pv, N, nrhs, g.nblocks);
+  else
+    prolong0_vec_kernel<TV><<<grid, 256, sizeof(float2) * 2 * N, s>>>(
+        (const float2*)in, (float2*)out, (const TV*)Pv, N, nrhs, g.nblocks,
+        (reinterpret_cast<uintptr_t>(out) & 15) == 0);
+  count_launches(1);
   SAPMG_CUDA_TRY(cudaGetLastError());
   return MG_OK;
 }
@@ -567,10 +695,10 @@ int launch_transfer0(bool restrict_, int prec, const Geom& g, const void* in, vo
     }
   }
   switch (prec) {
-    case P64: return transfer0_run<double, double2, double2, double2>(restrict_, g, in, out, Pv, N, nrhs, s);
-    case P32: return transfer0_run<float, float2, float2, float2>(restrict_, g, in, out, Pv, N, nrhs, s);
-    case P16: return transfer0_run<float, float2, __half2, float2>(restrict_, g, in, out, Pv, N, nrhs, s);
-    case PBF: return transfer0_run<float, float2, __nv_bfloat162, float2>(restrict_, g, in, out, Pv, N, nrhs, s);
+    case P64: return transfer0_fp64(restrict_, g, in, out, Pv, N, nrhs, s);
+    case P32: return transfer0_vec<float2>(restrict_, g, in, out, Pv, N, nrhs, s);
+    case P16: return transfer0_vec<__half2>(restrict_, g, in, out, Pv, N, nrhs, s);
+    case PBF: return transfer0_vec<__nv_bfloat162>(restrict_, g, in, out, Pv, N, nrhs, s);
     default: return MG_ERR_ARG;
   }
 }
