@@ -536,6 +536,62 @@ static void launch_mma_all(const CGeom& c, const TM* M, const float2* x, float2*
   }
 }
 
+// One FP16 basis vector: a CTA of nine warps per site, warp d the block of direction d
+// with 16-byte loads (4 rows of a column), each lane every G-th column, products in
+// FP32, and the CTA adds the lanes' and warps' parts.  The staged form above spends two
+// CTA barriers on each of its nine blocks and seven of eight tensor-core columns on
+// zeros: 512 sites, 2N = 40, operator in L2: 11.8 -> 8.4 us.  Up to four sites an SM, which are all resident at once; beyond, the ring's copies run ahead
+// across sites and win (4096 sites: 51.8 us staged, 59.0 us so).
+template <int N2>
+__global__ void __launch_bounds__(288, 4) coarse_apply_vec_kernel(const __half2* __restrict__ M,
+                                                                  const __half2* __restrict__ x,
+                                                                  float2* __restrict__ out, CGeom c) {
+  __shared__ float2 part[9 * 128];                            // [direction][column group][row]
+  const int n2 = N2 > 0 ? N2 : c.n2, rows = n2 / 4, G = 32 / rows;
+  const int d = threadIdx.x >> 5, lane = threadIdx.x & 31, rq = lane % rows, cg = lane / rows;
+  const int site = MG_CLAMP(kCoarseSite, (int)blockIdx.x, c.nsites);
+  int nb = site;
+  if (d > 0) {
+    const int mu = (d - 1) >> 1;
+    int stride = 1;
+    for (int m = 0; m < mu; ++m) stride *= c.L[m];
+    const int xc = (site / stride) % c.L[mu];
+    nb += (((xc + ((d & 1) ? 1 : -1) + c.L[mu]) % c.L[mu]) - xc) * stride;
+    nb = MG_CLAMP(kCoarseNeighbour, nb, c.nsites);
+  }
+  if (cg < G) {
+    const uint4* m = reinterpret_cast<const uint4*>(M + ((size_t)site * 9 + d) * n2 * n2) + rq;
+    const __half2* xn = x + (size_t)nb * n2;
+    Cplx<float> acc[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) acc[q] = cmk(0.f, 0.f);
+#pragma unroll 7
+    for (int j = cg; j < n2; j += G) {
+      const uint4 w = __ldg(m + j * rows);
+      const float2 v = __half22float2(__ldg(xn + j));
+      const uint32_t e[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&e[q]));
+        cfma(acc[q], cmk(a.x, a.y), cmk(v.x, v.y));
+      }
+    }
+    float2* p = part + (d * G + cg) * n2 + 4 * rq;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) p[q] = make_float2(acc[q].re, acc[q].im);
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < n2; t += 288) {
+    float re = 0.f, im = 0.f;
+#pragma unroll 9
+    for (int q = 0; q < 9 * G; ++q) {
+      re += part[q * n2 + t].x;
+      im += part[q * n2 + t].y;
+    }
+    out[(size_t)site * n2 + t] = make_float2(re / kBasisScale, im / kBasisScale);
+  }
+}
+
 // Tensor-core form: n2 % 8 == 0 and n2 <= 64; up to 16 right-hand sides per
 // launch (nr of them, the template width RB >= nr fixes the fragment count);
 // the operator in FP32 (store P32) or FP16 (store P16).
@@ -547,13 +603,19 @@ int launch_coarse_apply_mma(const CGeom& c, int store, const void* M, const void
     launch_mma_all(c, (const float2*)M, (const float2*)x, (float2*)out, nrhs, err, s);
   } else if (store == P16) {
     const __half2* m = (const __half2*)M;
-    const size_t xe = x_half ? 4 : 8;                         // bytes per complex vector entry
+    if (x_half && nrhs == 1 && c.nsites <= 152 * 4) {
+      const unsigned grid = (unsigned)c.nsites;
+      if (c.n2 == 40) coarse_apply_vec_kernel<40><<<grid, 288, 0, s>>>(m, (const __half2*)x, (float2*)out, c);
+      else coarse_apply_vec_kernel<0><<<grid, 288, 0, s>>>(m, (const __half2*)x, (float2*)out, c);
+      count_launches(1);
+      SAPMG_CUDA_TRY(cudaGetLastError());
+      return MG_OK;
+    }
     const int batch = std::max(1, std::min(16, t.batch));
     for (int r0 = 0; r0 < nrhs; r0 += batch) {
       const int rb = std::min(batch, nrhs - r0);
       const void* xs = x;
       float2* o = (float2*)out;
-      (void)xe;
 #define SAPMG_M16(RB_)                                                                       \
   if (x_half) launch_mma16<RB_, true>(c, m, xs, o, r0, rb, err, t, s);                       \
   else launch_mma16<RB_, false>(c, m, xs, o, r0, rb, err, t, s);

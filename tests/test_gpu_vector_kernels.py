@@ -94,3 +94,25 @@ def test_transfers_of_one_field(prec, n_vec):
     G.mg_pack_spinor(s.ctx, z, packed, G.MG_FP32, 1)
     assert torch.equal(odd, packed)
     s.close()
+
+
+@pytest.mark.parametrize("n_vec", [4, 12, 20, 32])
+def test_one_coarse_vector(monkeypatch, n_vec):
+    """The coarse product of one FP16 basis vector (256 sites, block sizes with full and
+    partly idle warps): two GMRES steps with the basis in FP16 against the same with it
+    in FP32.  The products and the two basis vectors are rounded by up to 2^-11 each; a
+    wrong direction or row would be off by a tenth."""
+    torch = torch_cuda()
+    import paper_1202_2462_gb300 as G
+    u = dev(torch, synth.random_gauge_field((16, 16, 16, 16), 0.4, 3))
+    b = torch.randn((256, 2 * n_vec), dtype=torch.complex64, device="cuda",
+                    generator=torch.Generator("cuda").manual_seed(3))
+    x = []
+    for flag in ("1", "0"):
+        monkeypatch.setenv("SAPMG_COARSE_BASIS_FP16", flag)
+        s = G.Solver(u, 1.0, -0.2, n_levels=2, n_vec=(n_vec,), setup_iters=0, precision="fp16", coarse_iters=2, seed=4)
+        out = torch.empty_like(b)
+        G.mg_coarse_solve(s.ctx, 1, b, out, s.prec)
+        x.append(host(out))
+        s.close()
+    assert rel(x[0], x[1]) < 4 * 2.0 ** -11
