@@ -341,20 +341,14 @@ __global__ void axpby_kernel(Scal32 a, const TX* __restrict__ x, Scal32 b, TY* _
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
     const TX u = xr[i];
     const R ux = (R)u.x, uy = (R)u.y;
+    TY v;
+    v.x = v.y = 0;
+    if (!yz) v = yr[i];
     TY o;
     if (real) {
-      o.x = ar * ux;
-      o.y = ar * uy;
-      if (!yz) {
-        const TY v = yr[i];
-        o.x += br * v.x;
-        o.y += br * v.y;
-      }
-    } else if (yz) {
-      o.x = ar * ux - ai * uy;
-      o.y = ar * uy + ai * ux;
+      o.x = ar * ux + br * v.x;
+      o.y = ar * uy + br * v.y;
     } else {
-      const TY v = yr[i];
       o.x = ar * ux - ai * uy + br * v.x - bi * v.y;
       o.y = ar * uy + ai * ux + br * v.y + bi * v.x;
     }
