@@ -9,6 +9,7 @@
 #include "internal.h"
 #include "blas.h"
 #include "hessenberg.cuh"
+#include "pdl.cuh"
 
 #include <type_traits>
 
@@ -34,6 +35,11 @@ static int reduce_ctas(size_t n, int R, size_t slots = kChunk) {
   const size_t fill = std::min<size_t>((n + 255) / 256, (152 + r - 1) / r);
   return (int)std::max<size_t>(1, std::min<size_t>(std::max((n + 2047) / 2048, fill), per));
 }
+
+// Dependent launch (pdl.cuh) below one CTA an SM, where the launch is a large part of a
+// kernel: one field's cycle on 512 coarse sites 463 -> 447 us with the coarse product
+// (coarse_tma.cu); the chain of 12 fields did not gain.
+static bool starts_early(dim3 grid) { return grid.x * grid.y <= 152; }
 
 // Reductions end inside the kernel that forms the partial sums: the CTA of a
 // right-hand side that arrives last (a counter per right-hand side behind the
@@ -424,7 +430,8 @@ __global__ void __launch_bounds__(32) hessenberg_solve_kernel(const double2* __r
   const int r = blockIdx.x, lane = threadIdx.x;
   const double2* Hin = Hall + (size_t)r * ldr;
   double2* y = yall + (size_t)r * ldy;
-  const double beta = sqrt(fmax(beta2[r].x, 0.0));
+  pdl_begin();
+  const double beta = sqrt(fmax(__ldcg(beta2 + r).x, 0.0));
   if (beta == 0.0) {
     if (lane < m) y[lane] = make_double2(0, 0);
     return;
@@ -433,19 +440,20 @@ __global__ void __launch_bounds__(32) hessenberg_solve_kernel(const double2* __r
   if (norms) {
     const double2* nv = norms + (size_t)r * ldr;
     if (lane > 0 && lane < m) {
-      const double t = sqrt(nv[lane].x) * nv[lane].y;
+      const double2 q = __ldcg(nv + lane);
+      const double t = sqrt(q.x) * q.y;
       is = t > 0.0 ? 1.0 / t : 0.0;
     }
-    if (lane < m) sub = sqrt(nv[lane + 1].x);
+    if (lane < m) sub = sqrt(__ldcg(nv + lane + 1).x);
   } else if (lane < m) {
-    sub = Hin[lane + 1 + lane * ldh].x;
+    sub = __ldcg(Hin + lane + 1 + lane * ldh).x;
   }
   const unsigned zero = __ballot_sync(0xffffffffu, sub == 0.0);
   const int mm = zero ? __ffs(zero) : m;                 // columns up to the first zero subdiagonal entry
   for (int k = 0; k < mm; ++k) {                         // lane = row
     double2 v = make_double2(0, 0);
     if (lane <= k) {
-      v = Hin[lane + k * ldh];
+      v = __ldcg(Hin + lane + k * ldh);
       if (pairs) {
         const float4 f = *reinterpret_cast<const float4*>(&v);
         v = make_double2((double)f.x + (double)f.y, (double)f.z + (double)f.w);
@@ -1115,7 +1123,7 @@ struct ArnoldiOut {
   int ldr, j, i0, last;    // the step, the chunk's first vector, the chunk that ends the pass
 };
 template <class R> __device__ __forceinline__ R inv_scale2(const double2* t, int i) {
-  return i == 0 ? (R)1 : reinterpret_cast<const R*>(t + 100)[i];
+  return i == 0 ? (R)1 : __ldcg(reinterpret_cast<const R*>(t + 100) + i);
 }
 
 // A sum across warps and CTAs: FP32 parts as an unevaluated pair of floats with
@@ -1206,6 +1214,7 @@ __global__ void __launch_bounds__(256) arnoldi_dots_kernel(PtrsK<typename B::V> 
   // the loads between the products, and a step on 20 vectors (12 fields of 103680) took
   // 107 us, against 23 us of one on 16 and 44 us so; w is read again, from L2 mostly.
   constexpr int KS = KM < 16 ? KM : 16, NV = 2 * KS;
+  pdl_begin();
   __shared__ R red[8][2 * KM + 1];
   R ww = 0;
 #pragma unroll
@@ -1214,14 +1223,14 @@ __global__ void __launch_bounds__(256) arnoldi_dots_kernel(PtrsK<typename B::V> 
 #pragma unroll
     for (int q = 0; q < KS; ++q) acc[q][0] = acc[q][1] = 0;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < nu; i += (size_t)gridDim.x * blockDim.x) {
-      const typename B::W x = wr[i];
+      const typename B::W x = __ldcg(wr + i);
 #pragma unroll
       for (int g = 0; g < KS; g += 8) {                  // up to eight loads in flight
         constexpr int G = KS < 8 ? KS : 8;
         V a[G];
 #pragma unroll
         for (int q = 0; q < G; ++q)
-          if (h + g + q < k) a[q] = __ldg(v.p[h + g + q] + r * stride + i);
+          if (h + g + q < k) a[q] = __ldcg(v.p[h + g + q] + r * stride + i);
 #pragma unroll
         for (int q = 0; q < G; ++q)
           if (h + g + q < k) cdot_acc(B::get(a[q]), x, acc[g + q][0], acc[g + q][1]);
@@ -1265,7 +1274,12 @@ __global__ void __launch_bounds__(256) arnoldi_dots_kernel(PtrsK<typename B::V> 
   const bool on = lane <= o.j;
   AccC<R> d;
   d.re = d.im = Acc<R>::of((R)0);
-  if (on) d = lane < o.i0 ? tr[lane] : raw[lane - o.i0];
+  if (on && lane < o.i0) {
+    const double2 q = __ldcg(t + lane);
+    d = *reinterpret_cast<const AccC<R>*>(&q);
+  } else if (on) {
+    d = raw[lane - o.i0];
+  }
   const R is2 = on ? inv_scale2<R>(t, lane) : (R)0;
   const R dr = d.re.value(), di = d.im.value();
   const R e = warp_sum((dr * dr + di * di) * is2);
@@ -1292,24 +1306,26 @@ __global__ void __launch_bounds__(256) arnoldi_update_kernel(PtrsK<typename B::V
   __shared__ R red[8];
   const int r = blockIdx.y, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   double2* t = o.t + (size_t)r * o.ldr;
+  pdl_begin();
   if ((int)threadIdx.x < k) {
-    const Cplx<R> c = reinterpret_cast<const Cplx<R>*>(t + o.i0 + threadIdx.x)[0];
+    const double2 q = __ldcg(t + o.i0 + threadIdx.x);
+    const Cplx<R> c = reinterpret_cast<const Cplx<R>*>(&q)[0];
     cf[0][threadIdx.x] = -c.re;
     cf[1][threadIdx.x] = -c.im;
   }
-  const R invb = reinterpret_cast<const R*>(t + 40)[0];
+  const R invb = __ldcg(reinterpret_cast<const R*>(t + 40));
   __syncthreads();
   typename B::W* wr = w + r * stride;
   R nn = 0;
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < nu; i += (size_t)gridDim.x * blockDim.x) {
-    typename B::W x = wr[i];
+    typename B::W x = __ldcg(wr + i);
 #pragma unroll
     for (int g = 0; g < KM; g += 8) {
       constexpr int G = KM < 8 ? KM : 8;
       V a[G];
 #pragma unroll
       for (int q = 0; q < G; ++q)
-        if (g + q < k) a[q] = __ldg(v.p[g + q] + r * stride + i);
+        if (g + q < k) a[q] = __ldcg(v.p[g + q] + r * stride + i);
 #pragma unroll
       for (int q = 0; q < G; ++q)
         if (g + q < k) caxpy(cf[0][g + q], cf[1][g + q], B::get(a[q]), x);
@@ -1349,22 +1365,23 @@ __global__ void __launch_bounds__(256) combine_kernel(PtrsK<typename B::V> v, in
   typedef typename B::V V;
   __shared__ R cf[2][KM];
   const int r = blockIdx.y;
+  pdl_begin();
   if ((int)threadIdx.x < k) {
-    const double2 c = y[(size_t)r * ldy + threadIdx.x];
+    const double2 c = __ldcg(y + (size_t)r * ldy + threadIdx.x);
     cf[0][threadIdx.x] = (R)c.x;
     cf[1][threadIdx.x] = (R)c.y;
   }
   __syncthreads();
   typename B::W* o = out + r * stride;
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < nu; i += (size_t)gridDim.x * blockDim.x) {
-    typename B::W x = acc ? o[i] : vzero<typename B::W>();
+    typename B::W x = acc ? __ldcg(o + i) : vzero<typename B::W>();
 #pragma unroll
     for (int g = 0; g < KM; g += 8) {
       constexpr int G = KM < 8 ? KM : 8;
       V a[G];
 #pragma unroll
       for (int q = 0; q < G; ++q)
-        if (g + q < k) a[q] = __ldg(v.p[g + q] + r * stride + i);
+        if (g + q < k) a[q] = __ldcg(v.p[g + q] + r * stride + i);
 #pragma unroll
       for (int q = 0; q < G; ++q)
         if (g + q < k) caxpy(cf[0][g + q], cf[1][g + q], B::get(a[q]), x);
@@ -1376,10 +1393,10 @@ __global__ void __launch_bounds__(256) combine_kernel(PtrsK<typename B::V> v, in
 // Vectors per kernel: the smallest of 4, 8, 16, 32 (FP64: 16, longer lists in
 // chunks of 16) that holds the list.
 #define SAPMG_KM(KERNEL, kk, ...)                                                                          \
-  if ((kk) <= 4) { KERNEL<B, 4><<<grid, 256, 0, s>>>(__VA_ARGS__); }                                       \
-  else if ((kk) <= 8) { KERNEL<B, 8><<<grid, 256, 0, s>>>(__VA_ARGS__); }                                  \
-  else if ((kk) <= 16) { KERNEL<B, 16><<<grid, 256, 0, s>>>(__VA_ARGS__); }                                \
-  else { KERNEL<B, B::CH><<<grid, 256, 0, s>>>(__VA_ARGS__); }                                             \
+  SAPMG_CUDA_TRY((kk) <= 4    ? cudaLaunchKernelEx(&l.cfg, KERNEL<B, 4>, __VA_ARGS__)                      \
+                 : (kk) <= 8  ? cudaLaunchKernelEx(&l.cfg, KERNEL<B, 8>, __VA_ARGS__)                      \
+                 : (kk) <= 16 ? cudaLaunchKernelEx(&l.cfg, KERNEL<B, 16>, __VA_ARGS__)                     \
+                              : cudaLaunchKernelEx(&l.cfg, KERNEL<B, B::CH>, __VA_ARGS__));                \
   count_launches(1);
 
 template <class B>
@@ -1399,12 +1416,14 @@ static int arnoldi_step_t(const BVec& b, const void* const* v, int j, void* w, v
     const int kk = std::min(B::CH, j + 1 - i0);
     const ArnoldiOut o{a.H, a.t, a.ldr, j, i0, i0 + kk > j};
     const dim3 grid(reduce_ctas(nu, b.R, 33), b.R);
+    const PdlLaunch l(grid, 256, 0, s, starts_early(grid));
     SAPMG_KM(arnoldi_dots_kernel, kk, ptrs_k<B>(v, i0, kk), kk, (const W*)w, nu, stride, a.partial, o)
   }
   for (int i0 = 0; i0 <= j; i0 += B::CH) {
     const int kk = std::min(B::CH, j + 1 - i0);
     const ArnoldiOut o{a.H, a.t, a.ldr, j, i0, i0 + kk > j};
     const dim3 grid(reduce_ctas(nu, b.R), b.R);
+    const PdlLaunch l(grid, 256, 0, s, starts_early(grid));
     SAPMG_KM(arnoldi_update_kernel, kk, ptrs_k<B>(v, i0, kk), kk, (W*)w, (V*)vnext, nu, stride, a.partial, o)
   }
   SAPMG_CUDA_TRY(cudaGetLastError());
@@ -1419,6 +1438,7 @@ static int combine_t(const BVec& b, const void* const* v, int k, const double2* 
   const dim3 grid = stream_grid(nu, b.R);
   for (int i0 = 0; i0 < k; i0 += B::CH) {
     const int kk = std::min(B::CH, k - i0);
+    const PdlLaunch l(grid, 256, 0, s, starts_early(grid));
     SAPMG_KM(combine_kernel, kk, ptrs_k<B>(v, i0, kk), kk, y + i0, ldy, (W*)out, nu, stride, i0 > 0)
   }
   SAPMG_CUDA_TRY(cudaGetLastError());
@@ -1469,7 +1489,8 @@ int blas_combine(int basis, const BVec& b, const void* const* v, int k, const do
 int blas_hessenberg_solve(const double2* H, int ldh, int ldr, int m, const double2* beta2, double2* y, int ldy,
                           int R, cudaStream_t s, const double2* norms, bool pairs) {
   if (m > 32) return MG_ERR_ARG;
-  hessenberg_solve_kernel<<<R, 32, 0, s>>>(H, ldh, ldr, m, beta2, norms, pairs, y, ldy); count_launches(1);
+  const PdlLaunch l(dim3((unsigned)R), 32, 0, s, starts_early(dim3((unsigned)R)));
+  SAPMG_CUDA_TRY(cudaLaunchKernelEx(&l.cfg, hessenberg_solve_kernel, H, ldh, ldr, m, beta2, norms, pairs, y, ldy)); count_launches(1);
   SAPMG_CUDA_TRY(cudaGetLastError());
   return MG_OK;
 }

@@ -12,6 +12,7 @@
 // the host turns into MG_ERR_TIMEOUT.
 #include "internal.h"
 #include "coarse.h"
+#include "pdl.cuh"
 #include "async.cuh"
 
 namespace sapmg {
@@ -540,12 +541,15 @@ static void launch_mma_all(const CGeom& c, const TM* M, const float2* x, float2*
 // with 16-byte loads (4 rows of a column), each lane every G-th column, products in
 // FP32, and the CTA adds the lanes' and warps' parts.  The staged form above spends two
 // CTA barriers on each of its nine blocks and seven of eight tensor-core columns on
-// zeros: 512 sites, 2N = 40, operator in L2: 11.8 -> 8.4 us.  Up to four sites an SM, which are all resident at once; beyond, the ring's copies run ahead
+// zeros: 512 sites, 2N = 40, operator in L2: 11.8 -> 8.4 us; a
+// dependent launch (pdl.cuh) issues the first loads of the operator before the
+// predecessor ends.  Up to four sites an SM, which are all resident at once; beyond, the ring's copies run ahead
 // across sites and win (4096 sites: 51.8 us staged, 59.0 us so).
 template <int N2>
 __global__ void __launch_bounds__(288, 4) coarse_apply_vec_kernel(const __half2* __restrict__ M,
                                                                   const __half2* __restrict__ x,
                                                                   float2* __restrict__ out, CGeom c) {
+  constexpr int kAhead = 7;                                   // loads in flight a lane
   __shared__ float2 part[9 * 128];                            // [direction][column group][row]
   const int n2 = N2 > 0 ? N2 : c.n2, rows = n2 / 4, G = 32 / rows;
   const int d = threadIdx.x >> 5, lane = threadIdx.x & 31, rq = lane % rows, cg = lane / rows;
@@ -565,20 +569,34 @@ __global__ void __launch_bounds__(288, 4) coarse_apply_vec_kernel(const __half2*
     Cplx<float> acc[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) acc[q] = cmk(0.f, 0.f);
-#pragma unroll 7
-    for (int j = cg; j < n2; j += G) {
-      const uint4 w = __ldg(m + j * rows);
-      const float2 v = __half22float2(__ldg(xn + j));
-      const uint32_t e[4] = {w.x, w.y, w.z, w.w};
+    uint4 w[kAhead];                                          // the operator does not depend on the predecessor
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&e[q]));
-        cfma(acc[q], cmk(a.x, a.y), cmk(v.x, v.y));
+    for (int u = 0; u < kAhead; ++u)
+      if (cg + u * G < n2) w[u] = __ldg(m + (cg + u * G) * rows);
+    pdl_begin();
+    for (int j0 = cg; j0 < n2; j0 += kAhead * G) {
+      if (j0 > cg) {
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u)
+          if (j0 + u * G < n2) w[u] = __ldg(m + (j0 + u * G) * rows);
+      }
+#pragma unroll
+      for (int u = 0; u < kAhead; ++u) {
+        if (j0 + u * G >= n2) continue;
+        const float2 v = __half22float2(__ldcg(xn + j0 + u * G));
+        const uint32_t e[4] = {w[u].x, w[u].y, w[u].z, w[u].w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&e[q]));
+          cfma(acc[q], cmk(a.x, a.y), cmk(v.x, v.y));
+        }
       }
     }
     float2* p = part + (d * G + cg) * n2 + 4 * rq;
 #pragma unroll
     for (int q = 0; q < 4; ++q) p[q] = make_float2(acc[q].re, acc[q].im);
+  } else {
+    pdl_begin();
   }
   __syncthreads();
   for (int t = threadIdx.x; t < n2; t += 288) {
@@ -605,8 +623,10 @@ int launch_coarse_apply_mma(const CGeom& c, int store, const void* M, const void
     const __half2* m = (const __half2*)M;
     if (x_half && nrhs == 1 && c.nsites <= 152 * 4) {
       const unsigned grid = (unsigned)c.nsites;
-      if (c.n2 == 40) coarse_apply_vec_kernel<40><<<grid, 288, 0, s>>>(m, (const __half2*)x, (float2*)out, c);
-      else coarse_apply_vec_kernel<0><<<grid, 288, 0, s>>>(m, (const __half2*)x, (float2*)out, c);
+      const PdlLaunch l(dim3(grid), 288, 0, s, true);
+      SAPMG_CUDA_TRY(c.n2 == 40
+                         ? cudaLaunchKernelEx(&l.cfg, coarse_apply_vec_kernel<40>, m, (const __half2*)x, (float2*)out, c)
+                         : cudaLaunchKernelEx(&l.cfg, coarse_apply_vec_kernel<0>, m, (const __half2*)x, (float2*)out, c));
       count_launches(1);
       SAPMG_CUDA_TRY(cudaGetLastError());
       return MG_OK;
