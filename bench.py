@@ -81,9 +81,9 @@ FAMILY_KERNELS = {
     "dirac": "dirac_pair_kernel + dirac_kernel", "sap": "sap_colour_pair_kernel + sap_block_kernel + sap_split_kernel",
     "coarse": "coarse_apply_mma16_kernel",
     "restrict": "restrict0_mma_kernel", "prolong": "prolong0_mma_kernel",
-    "blas": "dots2h_partial + dcgs2_coeff_kernel + axpy2h_kernel (outer Arnoldi, FP16 basis)",
-    "coarse_blas": "multidot_h_partial + multiaxpy_h_kernel + normalize_h_kernel + hessenberg_solve_kernel",
-    "sap1": "coarse_sap_mrhs_kernel (level-1 Schwarz of three levels)",
+    "blas": "dots2h_partial + axpy2h_kernel (outer Arnoldi, FP16 basis)",
+    "coarse_blas": "arnoldi_dots_kernel + arnoldi_update_kernel + hessenberg_solve_kernel",
+    "sap1": "coarse_sap_mrhs_kernel + coarse_sap_cluster_kernel (level-1 Schwarz of three levels)",
 }
 
 

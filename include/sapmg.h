@@ -300,8 +300,9 @@ int mg_coarse_solve(mg_ctx* ctx, int level, const void* in, void* out, int prec)
  * fixed-step GMRES); a three-level context gets MG_ERR_STATE.  The Krylov
  * basis is kept in the context's vector precision (FP64, or FP32 in the mixed
  * form): where mg_coarse_solve keeps the mixed form's basis in FP16 (the FP16
- * operator copy exists, 2N a multiple of 8), the two results differ by the
- * FP16 rounding of that basis.  A coarse system whose basis does not fit
+ * operator copy exists, 2N a multiple of 8, and the level is too large for the
+ * one-kernel form, which keeps FP32), the two results differ by the FP16
+ * rounding of that basis.  A coarse system whose basis does not fit
  * (about (coarse_iters + 2) vectors of the level's size) is rejected with
  * MG_ERR_ARG and a message naming the sizes.  Synchronises. */
 int mg_coarse_solve_noalloc(mg_ctx* ctx, int level, const void* in, void* out, int prec);
