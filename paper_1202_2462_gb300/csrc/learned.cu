@@ -183,8 +183,8 @@ __global__ void __launch_bounds__(256) gconv_backward_input_kernel(Geom g, const
 // the chunk's 32 input spins, five 16-byte loads for 24 complex products.  The
 // kernels above transport every input once per output channel (1.7 times the
 // needed flops, at the FP32 peak) or, for the gradient, read every output's
-// gradient from L1 once per hop and input channel: 1.16 and 2.4 ms for 16 -> 16
-// channels at 16^4, 58 Gflop.  Spin matrices and transports commute, so the input
+// gradient from L1 once per hop and input channel: 2.17 and 2.40 ms for 16 -> 16
+// channels at 16^4, 58 Gflop, against 1.20 and 1.23 ms.  Spin matrices and transports commute, so the input
 // gradient is the layer of the adjoint weights, G_x_b = sum_a sum_h
 // W[a][b][adj h]^dagger T_h G_y_a (BWD).  FP32-bound.
 constexpr int kPairs = 8, kTileSites = 32, kTileCh = 16;
@@ -285,7 +285,7 @@ constexpr size_t kTileSmem = sizeof(float4) * kPairs * 4 * kLdW;
 // threads share the terms.  The slices' sums are added in slice order by a second
 // kernel, so the result is deterministic.  One CTA per (a, b, h) over all sites, as
 // before, transported every input once per output channel: 3.4 ms for 16 -> 16
-// channels at 16^4.
+// channels at 16^4, against 1.70 ms.
 template <int RA>
 __global__ void __launch_bounds__(256, 2) gconv_wgrad_tile_kernel(Geom g, const float2* __restrict__ U,
                                                                   const float2* __restrict__ x,
@@ -469,9 +469,12 @@ __global__ void adam_kernel(size_t n, float* __restrict__ p, const float* __rest
   }
 }
 
-// Output channels from which the tiled form runs: below, most of its sixteen
-// channels a CTA would be idle and a thread per site transports little in vain.
-constexpr int kTiledFrom = 4;
+// Output channels (BWD: input channels) from which the tiled form runs: below, most of
+// its sixteen channels a CTA would be idle and a thread per site transports little in
+// vain.  Thread per site against tiled, 16^4 sites, FP32: layer 4 -> 4 155 and 192 us,
+// 5 -> 5 235 and 235, 8 -> 8 572 and 361; input gradient 125 and 194, 185 and 239, 415
+// and 371.
+constexpr int kTiledFrom = 6, kTiledFromBwd = 8;
 
 template <class TG, class TW, bool BWD>
 static int gconv_tiled(const Geom& g, const void* U, const void* W, const void* x, void* y, int cin, int cout,
@@ -558,7 +561,7 @@ int launch_gconv_backward(const Geom& g, const void* U, const void* W, const voi
     attr = true;
   }
   if (gx) {
-    if (cin >= kTiledFrom) {
+    if (cin >= kTiledFromBwd) {
       const int rc = gconv_tiled<float2, float2, true>(g, U, W, gy, gx, cout, cin, s);
       if (rc != MG_OK) return rc;
     } else {
