@@ -27,7 +27,7 @@ def _canonical(torch, s, y, c):
 
 # FP32 sums of 36 cin products (forward), of 36 cout (input gradient) and of 3 V
 # (weights): 2e-6 as in the layer's own parity test
-@pytest.mark.parametrize("cin,cout", [(1, 1), (1, 4), (4, 3), (3, 5), (2, 16), (16, 2), (5, 17)])
+@pytest.mark.parametrize("cin,cout", [(1, 1), (1, 4), (4, 3), (3, 5), (2, 16), (16, 2), (5, 17), (7, 5), (8, 6)])
 def test_layer_tiles(cin, cout):
     torch = torch_cuda()
     import paper_1202_2462_gb300 as G
