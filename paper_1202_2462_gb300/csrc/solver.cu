@@ -423,7 +423,7 @@ static int coarse_gmres(mg_ctx* c, CoarseLevel& L, int k, int R) {
     }
   }
   CBLAS(blas_hessenberg_solve(L.H, 33, 33 * 33, k, L.beta2, L.y, 33, R, c->s,
-                              c->coarse_reorth ? nullptr : L.tmp + 64, vt == P32));
+                              c->coarse_reorth ? nullptr : L.tmp + 64, vt == P32 && !c->coarse_reorth));
   CBLAS(blas_combine(vt, bv, vl.data(), k, L.y, 33, L.x, c->s));
   return MG_OK;
 }
@@ -484,7 +484,7 @@ static int fgmres_fixed1(mg_ctx* c, int k, int R) {
     }
   }
   CBLAS(blas_hessenberg_solve(c->f1H, 33, 33 * 33, k, c->f1beta2, c->f1y, 33, R, c->s,
-                              c->coarse_reorth ? nullptr : c->f1tmp + 64, vt == P32));
+                              c->coarse_reorth ? nullptr : c->f1tmp + 64, vt == P32 && !c->coarse_reorth));
   CBLAS(blas_combine(vt, bv, zl.data(), k, c->f1y, 33, L.x, c->s));
   return MG_OK;
 }
