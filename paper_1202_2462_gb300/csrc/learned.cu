@@ -193,8 +193,8 @@ constexpr int kLdW = kTileCh * 4 + 4;              // a row more of 64 bytes: th
 template <class TG, class TW, bool BWD>
 __global__ void __launch_bounds__(256, 2) gconv_tile_kernel(Geom g, const TG* __restrict__ U,
                                                             const TW* __restrict__ W, const float2* __restrict__ x,
-                                                            float2* __restrict__ y, int cin, int cout) {
-  // cin: channels of x; cout: channels of y (BWD: the layer's output and input channels)
+                                                            float2* __restrict__ y, int cin, int cout, bool al) {
+  // cin: channels of x; cout: channels of y (BWD: the layer's output and input channels); al: y starts on 16 bytes
   // [pair, spin][colour][two sites]: (re, re, im, im); [pair, input spin][channel, spin]: (re, re, im, im)
   __shared__ __align__(16) float4 Ts[kPairs * 4][3][kTileSites / 2];
   extern __shared__ __align__(16) float4 Ws[];                        // [kPairs * 4][kLdW]
@@ -270,9 +270,16 @@ __global__ void __launch_bounds__(256, 2) gconv_tile_kernel(Geom g, const TG* __
 #pragma unroll
   for (int s = 0; s < 4; ++s)
 #pragma unroll
-    for (int c = 0; c < 3; ++c)
-      *reinterpret_cast<float4*>(o + (s * 3 + c) * 256) =
-          make_float4(acc[s][c].re.x, acc[s][c].im.x, acc[s][c].re.y, acc[s][c].im.y);
+    for (int c = 0; c < 3; ++c) {
+      float2* d = o + (s * 3 + c) * 256;
+      const P2 v = acc[s][c];
+      if (al) {
+        *reinterpret_cast<float4*>(d) = make_float4(v.re.x, v.im.x, v.re.y, v.im.y);
+      } else {
+        d[0] = make_float2(v.re.x, v.im.x);
+        d[1] = make_float2(v.re.y, v.im.y);
+      }
+    }
 }
 
 constexpr size_t kTileSmem = sizeof(float4) * kPairs * 4 * kLdW;
@@ -486,7 +493,8 @@ static int gconv_tiled(const Geom& g, const void* U, const void* W, const void* 
     attr = true;
   }
   gconv_tile_kernel<TG, TW, BWD><<<dim3(g.nblocks * 8, (cout + kTileCh - 1) / kTileCh), 256, kTileSmem, s>>>(
-      g, (const TG*)U, (const TW*)W, (const float2*)x, (float2*)y, cin, cout);
+      g, (const TG*)U, (const TW*)W, (const float2*)x, (float2*)y, cin, cout,
+      (reinterpret_cast<uintptr_t>(y) & 15) == 0);
   count_launches(1);
   SAPMG_CUDA_TRY(cudaGetLastError());
   return MG_OK;

@@ -53,3 +53,32 @@ def test_layer_tiles(cin, cout):
     ref = L.layer(round_storage(u, "bf16"), round_storage(w, "bf16"), x)
     assert rel(_canonical(torch, s, yd, cout), ref) < 2e-6
     s.close()
+
+
+@pytest.mark.parametrize("cin,cout", [(4, 4), (8, 16), (16, 6)])
+def test_layer_fields_at_odd_elements(cin, cout):
+    """Fields that start on 8 bytes but not on 16 give the aligned fields' results bit for bit."""
+    torch = torch_cuda()
+    import paper_1202_2462_gb300 as G
+    s = G.Solver(dev(torch, synth.random_gauge_field(DIMS, 0.4, 324)), 1.0, -0.1, n_levels=1, precision="bf16", fgmres_m=1)
+    fs = int(np.prod(DIMS)) * 12
+    gen = torch.Generator("cuda").manual_seed(5)
+
+    def rnd(n):
+        return torch.randn(n, dtype=torch.complex64, device="cuda", generator=gen)
+
+    def odd(t):
+        return torch.cat([t[:1], t])[1:]
+
+    w, x, gy = rnd(cout * cin * 144), rnd(cin * fs), rnd(cout * fs)
+    wb = torch.view_as_real(w).to(torch.bfloat16).contiguous()
+    out = []
+    for f in (lambda t: t, odd):
+        xx, yy, yb, gg, gx, gw = f(x), f(torch.zeros_like(gy)), f(torch.zeros_like(gy)), f(gy), f(torch.zeros_like(x)), f(torch.zeros_like(w))
+        assert all(t.data_ptr() % 16 == (0 if f is not odd else 8) for t in (xx, yy, yb, gg, gx, gw))
+        G.mg_net_layer_forward(s.ctx, cin, cout, f(w), xx, yy)
+        G.mg_net_layer_forward_bf16(s.ctx, cin, cout, wb, xx, yb)
+        G.mg_net_layer_backward(s.ctx, cin, cout, f(w), xx, gg, gx, gw)
+        out.append((yy, yb, gx, gw))
+    assert all(torch.equal(a, b) for a, b in zip(*out))
+    s.close()
