@@ -82,10 +82,11 @@ int launch_gconv_forward(const Geom& g, const void* U, const void* W, const void
 // The same with BF16 links and BF16 weights (inference), FP32 activations and accumulation.
 int launch_gconv_forward_bf16(const Geom& g, const void* U, const void* W, const void* x, void* y, int cin, int cout,
                               cudaStream_t s);
-// work: scratch for gW, best gconv_wgrad_bytes of it (none: one slice of the sites)
-size_t gconv_wgrad_bytes(const Geom& g, int cin, int cout);
+constexpr int kNetChannels = 64;           // most input or output channels of a layer
+// work: scratch for gW, gconv_wgrad_bytes of it for layers of up to max_channels
+size_t gconv_wgrad_bytes(const Geom& g, int max_channels);
 int launch_gconv_backward(const Geom& g, const void* U, const void* W, const void* x, const void* gy, void* gx,
-                          void* gW, void* work, size_t work_bytes, int cin, int cout, cudaStream_t s);
+                          void* gW, void* work, int cin, int cout, cudaStream_t s);
 int launch_gate(const Geom& g, const void* x, const void* gy, void* out, int channels, cudaStream_t s);
 int launch_adam(size_t n, float* p, const float* gr, float* m, float* v, double lr, double b1, double b2,
                 double eps, int step, cudaStream_t s);

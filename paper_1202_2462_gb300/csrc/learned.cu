@@ -537,8 +537,12 @@ static int wgrad_slices(const Geom& g, int cin, int cout) {
   const int chunks = g.nblocks * 16;
   return std::max(1, std::min(304 / tiles, chunks / 4));       // one wave: a CTA more doubles the time
 }
-size_t gconv_wgrad_bytes(const Geom& g, int cin, int cout) {
-  return (size_t)wgrad_slices(g, cin, cout) * cout * cin * 9 * 16 * sizeof(float2);
+size_t gconv_wgrad_bytes(const Geom& g, int max_channels) {
+  size_t most = 0;
+  for (int cin = 1; cin <= max_channels; ++cin)
+    for (int cout = 1; cout <= max_channels; ++cout)
+      if (wgrad_slices(g, cin, cout) > 1) most = std::max(most, (size_t)wgrad_slices(g, cin, cout) * cout * cin * 9 * 16);
+  return most * sizeof(float2);
 }
 
 template <int RA>
@@ -560,7 +564,7 @@ static int wgrad_run(const Geom& g, const void* U, const void* x, const void* gy
 }
 
 int launch_gconv_backward(const Geom& g, const void* U, const void* W, const void* x, const void* gy, void* gx,
-                          void* gW, void* work, size_t work_bytes, int cin, int cout, cudaStream_t s) {
+                          void* gW, void* work, int cin, int cout, cudaStream_t s) {
   const size_t smem = sizeof(float2) * cout * 9 * 16;
   if (smem > 200 * 1024) return MG_ERR_ARG;
   static bool attr = false;
@@ -580,7 +584,7 @@ int launch_gconv_backward(const Geom& g, const void* U, const void* W, const voi
   }
   if (gW) {
     const size_t n = (size_t)cout * cin * 9 * 16;
-    const int nslice = std::max(1, std::min(wgrad_slices(g, cin, cout), (int)(work_bytes / (n * sizeof(float2)))));
+    const int nslice = wgrad_slices(g, cin, cout);
     float2* part = nslice > 1 ? (float2*)work : (float2*)gW;         // one slice is gW itself
     const int rc = cout >= 16 ? wgrad_run<16>(g, U, x, gy, part, cin, cout, nslice, s)
                  : cout >= 4  ? wgrad_run<4>(g, U, x, gy, part, cin, cout, nslice, s)

@@ -219,8 +219,10 @@ struct mg_ctx {
   int N0 = 0;
   void* V64 = nullptr;                     // locally orthonormal test vectors, FP64 vector-major
   void* Vs64 = nullptr;                    // set-up only: the smoothed vectors before local orthonormalisation
-  void* net_work = nullptr;                // weight gradients of the set-up network (allocated on first use)
-  size_t net_work_bytes = 0;
+  // mixed form: the weight gradients' slices of the set-up network, for the widest layer;
+  // allocated with the context, so that a captured call keeps a valid address and
+  // no call allocates (10 MB at most)
+  void* net_work = nullptr;
   double2* gram = nullptr;                 // set-up only: work of the FP32 orthonormalisation
   void* part2_buf = nullptr;               // set-up only (three levels): part-1 vectors kept for set-up part 2
   const std::vector<double2>* load_v0 = nullptr;  // mg_setup_load: the saved level-0 vectors (host)
@@ -1713,6 +1715,8 @@ static int do_setup(mg_ctx* c, const double* U) {
     if (!c->U32 || !c->A32) return fail(MG_ERR_OOM, "gauge field");
     TRY(launch_convert(P64, c->U64, P32, c->U32, ulinks, c->s));
     TRY(launch_convert(P64, c->A64, P32, c->A32, aslots, c->s));
+    c->net_work = c->alloc(gconv_wgrad_bytes(c->g, kNetChannels));
+    if (!c->net_work) return fail(MG_ERR_OOM, "network workspace");
     if (c->prec == P32) {
       c->Us = c->U32;
       c->As = c->A32;
@@ -2473,7 +2477,8 @@ int mg_precondition(mg_ctx* c, const void* v, void* z, int prec) {
 static int net_state(mg_ctx* c, int a, int b) {
   if (!c) return fail(MG_ERR_ARG, "bad argument");
   if (!c->U32) return fail(MG_ERR_STATE, "the network needs a mixed-form context (FP32 links)");
-  if (a < 1 || b < 1 || a > 64 || b > 64) return fail(MG_ERR_ARG, "channel counts must be in 1..64");
+  if (a < 1 || b < 1 || a > kNetChannels || b > kNetChannels)
+    return fail(MG_ERR_ARG, "channel counts must be in 1.." + std::to_string(kNetChannels));
   return MG_OK;
 }
 
@@ -2494,23 +2499,7 @@ int mg_net_layer_backward(mg_ctx* c, int cin, int cout, const void* W, const voi
                           void* gW) {
   TRY(net_state(c, cin, cout));
   if (!W || !x || !gy || (!gx && !gW)) return fail(MG_ERR_ARG, "bad argument");
-  if (gW) {
-    // the slices' sums: grown when a layer needs more and kept by the context; where
-    // that cannot be (stream capture, no memory) the kernel takes fewer slices
-    const size_t bytes = gconv_wgrad_bytes(c->g, cin, cout);
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (bytes > c->net_work_bytes && cudaStreamIsCapturing(c->s, &cap) == cudaSuccess &&
-        cap == cudaStreamCaptureStatusNone) {
-      if (c->net_work) {
-        SAPMG_CUDA_TRY(cudaStreamSynchronize(c->s));         // an earlier layer may still use the old one
-        c->release(c->net_work);
-      }
-      c->net_work = c->alloc(bytes);
-      c->net_work_bytes = c->net_work ? bytes : 0;
-    }
-  }
-  return launch_gconv_backward(c->g, c->U32, W, x, gy, gx, gW, c->net_work, c->net_work_bytes, cin, cout,
-                               c->s);
+  return launch_gconv_backward(c->g, c->U32, W, x, gy, gx, gW, c->net_work, cin, cout, c->s);
 }
 
 int mg_net_gate_forward(mg_ctx* c, int channels, const void* x, void* y) {

@@ -82,3 +82,42 @@ def test_layer_fields_at_odd_elements(cin, cout):
         out.append((yy, yb, gx, gw))
     assert all(torch.equal(a, b) for a, b in zip(*out))
     s.close()
+
+
+def test_captured_weight_gradient():
+    """A weight gradient captured as the first call of its context and replayed after a
+    wider layer's: the eager call's result bit for bit, each time."""
+    torch = torch_cuda()
+    import paper_1202_2462_gb300 as G
+    stream = torch.cuda.Stream()
+    u = dev(torch, synth.random_gauge_field(DIMS, 0.4, 325))
+    fs = int(np.prod(DIMS)) * 12
+    gen = torch.Generator("cuda").manual_seed(6)
+
+    def layer(cin, cout):
+        def rnd(n):
+            return torch.randn(n, dtype=torch.complex64, device="cuda", generator=gen)
+        return cin, cout, rnd(cout * cin * 144), rnd(cin * fs), rnd(cout * fs)
+
+    narrow, wide = layer(6, 6), layer(24, 16)
+    gw = torch.empty_like(narrow[2])
+    gwide = torch.empty_like(wide[2])
+    torch.cuda.synchronize()
+    with torch.cuda.stream(stream):
+        s = G.Solver(u, 1.0, -0.1, n_levels=1, precision="fp32", fgmres_m=1)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        G.mg_net_layer_backward(s.ctx, *narrow, None, gw)
+    got = []
+    for _ in range(2):
+        gw.zero_()
+        torch.cuda.synchronize()
+        graph.replay()
+        torch.cuda.synchronize()
+        got.append(gw.clone())
+        G.mg_net_layer_backward(s.ctx, *wide, None, gwide)
+        torch.cuda.synchronize()
+    G.mg_net_layer_backward(s.ctx, *narrow, None, gw)
+    torch.cuda.synchronize()
+    assert torch.equal(got[0], gw) and torch.equal(got[1], gw)
+    s.close()
