@@ -8,6 +8,7 @@
 // sums use the vector's own precision; CTA-level and final sums use FP64.
 #include "internal.h"
 #include "blas.h"
+#include "accum.cuh"
 #include "hessenberg.cuh"
 #include "pdl.cuh"
 
@@ -1078,8 +1079,9 @@ int blas_normalize_h(const BVec& b, const void* x, void* out, const double2* nrm
 //           itself, which is H_{j+1,j}.
 // beta (formed before x exists) only has to be near ||x||: v_{j+1} has the norm
 // s_{j+1} = ||x|| / beta, which is kept, and H and y are those of the unit
-// vectors v_i / s_i, so a beta that cancellation has made inexact costs no
-// accuracy; a floor under it (kFloor <w, w>) bounds s_{j+1}.  Against a norm pass
+// vectors v_i / s_i, so a beta that cancellation or FP32 has made inexact costs no
+// accuracy (the FP32 value that divided x is the one kept); a floor under it
+// (kFloor <w, w>) bounds s_{j+1}.  Against a norm pass
 // before a separate normalisation this reads and writes w once less and takes
 // two launches a step instead of five.  Bound by L2/HBM bandwidth for 12 right-hand
 // sides, by latency for one.
@@ -1117,42 +1119,10 @@ template <class V> struct PtrsK { const V* p[32]; };
 // Scalars of a step (per right-hand side, stride ldr): H (33 x 33 column-major)
 // takes the raw dots; t[i] a coefficient of the update (Cplx<R>; FP64: the raw dots
 // of earlier chunks before), t[40] 1/beta, t[64 + i] = (||x||^2, 1/beta) of basis
-// vector i >= 1 and, as R from t[100] on, 1 / s_i^2.
+// vector i >= 1 and, as Scale<R> from t[100] on, 1 / s_i^2.
 struct ArnoldiOut {
   double2 *H, *t;
   int ldr, j, i0, last;    // the step, the chunk's first vector, the chunk that ends the pass
-};
-template <class R> __device__ __forceinline__ R inv_scale2(const double2* t, int i) {
-  return i == 0 ? (R)1 : __ldcg(reinterpret_cast<const R*>(t + 100) + i);
-}
-
-// A sum across warps and CTAs: FP32 parts as an unevaluated pair of floats with
-// error-free additions (Knuth, TAOCP vol. 2, 4.2.2), about the precision of FP64,
-// an instruction of which takes 64 cycles of an SM's sub-partition and so made
-// these short serial sums the longest part of a kernel on a short vector.
-template <class R> struct Acc;
-template <> struct Acc<float> {
-  float h, l;
-  __device__ __forceinline__ static Acc of(float v) { return Acc{v, 0.f}; }
-  __device__ __forceinline__ void add(Acc b) {
-    const float s = __fadd_rn(h, b.h), t = __fsub_rn(s, h);
-    const float e = __fadd_rn(__fsub_rn(h, __fsub_rn(s, t)), __fsub_rn(b.h, t));
-    h = s;
-    l = __fadd_rn(__fadd_rn(l, b.l), e);
-  }
-  __device__ __forceinline__ Acc from(int mask) const {
-    return Acc{__shfl_xor_sync(0xffffffffu, h, mask), __shfl_xor_sync(0xffffffffu, l, mask)};
-  }
-  __device__ __forceinline__ float value() const { return h + l; }
-  __device__ __forceinline__ double exact() const { return (double)h + (double)l; }
-};
-template <> struct Acc<double> {
-  double v;
-  __device__ __forceinline__ static Acc of(double x) { return Acc{x}; }
-  __device__ __forceinline__ void add(Acc b) { v += b.v; }
-  __device__ __forceinline__ Acc from(int mask) const { return Acc{__shfl_xor_sync(0xffffffffu, v, mask)}; }
-  __device__ __forceinline__ double value() const { return v; }
-  __device__ __forceinline__ double exact() const { return v; }
 };
 template <class R> struct AccC { Acc<R> re, im; };      // sixteen bytes: a slot of the partial sums
 static_assert(sizeof(AccC<float>) == 16 && sizeof(AccC<double>) == 16, "a slot holds one complex sum");
@@ -1280,12 +1250,16 @@ __global__ void __launch_bounds__(256) arnoldi_dots_kernel(PtrsK<typename B::V> 
   } else if (on) {
     d = raw[lane - o.i0];
   }
-  const R is2 = on ? inv_scale2<R>(t, lane) : (R)0;
-  const R dr = d.re.value(), di = d.im.value();
-  const R e = warp_sum((dr * dr + di * di) * is2);
+  Scale<R> is2 = Scale<R>::one();
+  if (on && lane > 0) {
+    const double q = __ldcg(reinterpret_cast<const double*>(t + 100) + lane);
+    is2 = *reinterpret_cast<const Scale<R>*>(&q);
+  }
+  const R cr = is2.times(d.re), ci = is2.times(d.im);
+  const R e = warp_sum(d.re.value() * cr + d.im.value() * ci);
   if (on) {
     reinterpret_cast<AccC<R>*>(o.H + (size_t)r * o.ldr)[lane + 33 * o.j] = d;
-    reinterpret_cast<Cplx<R>*>(t + lane)[0] = cmk(dr * is2, di * is2);
+    reinterpret_cast<Cplx<R>*>(t + lane)[0] = cmk(cr, ci);
   }
   if (lane == 0) {
     const R n2 = raw[KM].re.value(), b2 = max(n2 - e, (R)B::kFloor * n2);
@@ -1350,8 +1324,7 @@ __global__ void __launch_bounds__(256) arnoldi_update_kernel(PtrsK<typename B::V
   if (wid > 0) return;
   const Acc<R> sum = sum_slot_acc<R>(partial, r, 1, 0).re;
   if (lane == 0) {
-    const R s2 = max(sum.value(), (R)0) * invb * invb;
-    reinterpret_cast<R*>(t + 100)[o.j + 1] = s2 > (R)0 ? (R)1 / s2 : (R)0;
+    reinterpret_cast<Scale<R>*>(t + 100)[o.j + 1] = Scale<R>::of(sum, invb);
     t[64 + o.j + 1] = make_double2(fmax(sum.exact(), 0.0), (double)invb);
   }
 }

@@ -14,6 +14,7 @@
 // beta^2 = <w, w> - sum |h_i|^2 / |v_i|^2 (floored), v_{j+1} = (w - sum h_i v_i /
 // |v_i|^2) / beta, whose exact norm s_{j+1} is kept: with rows h_ij / s_i and the
 // subdiagonal ||x|| the least squares gives the coefficients of the v_i as they are.
+#include "accum.cuh"
 #include "cluster.cuh"
 #include "coarse.h"
 #include "hessenberg.cuh"
@@ -41,37 +42,14 @@ struct DoubleOp {
   static __device__ __forceinline__ Cplx<double> get(double2 m) { return cmk(m.x, m.y); }
 };
 
-// Sum of one value over lanes 0..15 in a fixed order.  FP32 parts are added as
-// unevaluated pairs (error-free sums, Knuth, TAOCP vol. 2, 4.2.2): the precision of
-// an FP64 sum, whose instructions take 64 cycles of the sub-partition each.
-template <class R> struct Sum16;
-template <> struct Sum16<double> {
-  double v;
-  __device__ __forceinline__ double value() const { return v; }
-  __device__ __forceinline__ double exact() const { return v; }
-};
-template <> struct Sum16<float> {
-  float h, l;
-  __device__ __forceinline__ float value() const { return h + l; }
-  __device__ __forceinline__ double exact() const { return (double)h + (double)l; }
-};
-__device__ __forceinline__ Sum16<double> sum16(double v) {
+// Sum of one value over lanes 0..15 in a fixed order.
+template <class R> __device__ __forceinline__ Acc<R> sum16(Acc<R> v) {
 #pragma unroll
-  for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return Sum16<double>{v};
+  for (int o = 8; o > 0; o >>= 1) v.add(v.from(o));
+  return v;
 }
-__device__ __forceinline__ Sum16<float> sum16(float v) {
-  float h = v, l = 0.f;
-#pragma unroll
-  for (int o = 8; o > 0; o >>= 1) {
-    const float h2 = __shfl_xor_sync(0xffffffffu, h, o), l2 = __shfl_xor_sync(0xffffffffu, l, o);
-    const float s = __fadd_rn(h, h2), t = __fsub_rn(s, h);
-    const float e = __fadd_rn(__fsub_rn(h, __fsub_rn(s, t)), __fsub_rn(h2, t));
-    h = s;
-    l = __fadd_rn(__fadd_rn(l, l2), e);
-  }
-  return Sum16<float>{h, l};
-}
+__device__ __forceinline__ void cluster_st_acc(uint32_t a, Acc<float> v) { cluster_st(a, cmk(v.h, v.l)); }
+__device__ __forceinline__ void cluster_st_acc(uint32_t a, Acc<double> v) { cluster_st(a, v.v); }
 __device__ __forceinline__ float rsqrt_of(float x) { return rsqrtf(x); }
 __device__ __forceinline__ double rsqrt_of(double x) { return rsqrt(x); }
 
@@ -90,12 +68,12 @@ __host__ __device__ inline Layout layout(int spc, int nsites, int n2, int k) {
   l.ts = take(spc * 9 * n2 * cb);
   l.w = take(rows * cb);
   l.pd = take(kSolveCluster * 33 * cb);                    // partial dots [rank][33]
-  l.pn = take(2 * kSolveCluster * (int)sizeof(typename OP::R));   // partial norms, two buffers
+  l.pn = take(2 * kSolveCluster * 8);                      // partial norms (Acc), two buffers
   l.hr = take(33 * 32 * 8);
   l.hi = take(33 * 32 * 8);
   l.coef = take(34 * 16);                                  // y (FP64)
-  l.dots = take(34 * cb);                                  // the step's dots
-  l.sc = take(34 * 8 * 2);                                 // 1/s_i (FP64), and 1/s_i^2
+  l.dots = take(34 * cb);                                  // <v_i, w> / |v_i|^2
+  l.sc = take(34 * 8 * 3);                                 // 1/s_i (FP64), 1/s_i^2 (Scale), |<v_i, w>|^2 / |v_i|^2
   l.tab = take(spc * 9 * 4);
   l.flag = take(kSolveCluster * 4);
   l.bar = take(8);
@@ -122,12 +100,13 @@ __global__ void __launch_bounds__(768) coarse_gmres_cluster_kernel(const typenam
   C* ts = reinterpret_cast<C*>(smem + lo.ts);
   C* w = reinterpret_cast<C*>(smem + lo.w);
   C* pd = reinterpret_cast<C*>(smem + lo.pd);
-  R* pn = reinterpret_cast<R*>(smem + lo.pn);
+  Acc<R>* pn = reinterpret_cast<Acc<R>*>(smem + lo.pn);
   double* hr = reinterpret_cast<double*>(smem + lo.hr);
   double* hi = reinterpret_cast<double*>(smem + lo.hi);
   double2* coef = reinterpret_cast<double2*>(smem + lo.coef);
   double* is = reinterpret_cast<double*>(smem + lo.sc);       // 1 / s_i
-  R* is2 = reinterpret_cast<R*>(is + 34);                     // 1 / s_i^2
+  Scale<R>* is2 = reinterpret_cast<Scale<R>*>(is + 34);       // 1 / s_i^2
+  R* part2 = reinterpret_cast<R*>(is + 68);                   // what <w, w> loses to v_i
   C* dots = reinterpret_cast<C*>(smem + lo.dots);
   int* tab = reinterpret_cast<int*>(smem + lo.tab);
   int* flag = reinterpret_cast<int*>(smem + lo.flag);
@@ -174,9 +153,9 @@ __global__ void __launch_bounds__(768) coarse_gmres_cluster_kernel(const typenam
     if (lane == 0) part[warp] = v;
     __syncthreads();
     if (tid < kSolveCluster) {
-      R t = 0;
-      for (int q = 0; q < (nr + 31) / 32 && q < nw; ++q) t += part[q];
-      cluster_st(cluster_addr(smem_u32(pn + buf * kSolveCluster + rank), tid), t);
+      Acc<R> t = Acc<R>::of((R)0);
+      for (int q = 0; q < (nr + 31) / 32 && q < nw; ++q) t.add(Acc<R>::of(part[q]));
+      cluster_st_acc(cluster_addr(smem_u32(pn + buf * kSolveCluster + rank), tid), t);
     }
   };
   const uint32_t vf_a = smem_u32(vf), pd_a = smem_u32(pd);
@@ -207,7 +186,7 @@ __global__ void __launch_bounds__(768) coarse_gmres_cluster_kernel(const typenam
       return;
     }
   }
-  const double bb = sum16(pn[kSolveCluster + (lane & 15)]).exact();
+  const double bb = sum16<R>(pn[kSolveCluster + (lane & 15)]).exact();
   const double beta0 = sqrt(fmax(bb, 0.0));
   {
     const R f = beta0 > 0.0 ? (R)(1.0 / beta0) : (R)0;
@@ -219,7 +198,7 @@ __global__ void __launch_bounds__(768) coarse_gmres_cluster_kernel(const typenam
       for (int q = 0; q < kSolveCluster; ++q) cluster_st(cluster_addr(a, q), v);
     }
   }
-  if (tid == 0) { is[0] = 1.0; is2[0] = (R)1; }
+  if (tid == 0) { is[0] = 1.0; is2[0] = Scale<R>::one(); }
   cluster_barrier();
   for (int j = 0; j < k; ++j) {
     // w = A v_j on the CTA's rows
@@ -253,12 +232,16 @@ __global__ void __launch_bounds__(768) coarse_gmres_cluster_kernel(const typenam
     cluster_barrier();
     for (int i = warp; i <= j + 1; i += nw) {
       const C t = pd[(lane & 15) * 33 + i];
-      const Sum16<R> a = sum16(t.re), c2 = sum16(t.im);
+      const Acc<R> a = sum16(Acc<R>::of(t.re)), c2 = sum16(Acc<R>::of(t.im));
       if (lane == 0) {
-        dots[i] = cmk(a.value(), c2.value());
-        if (i <= j) {                                        // raw; scaled by the last warp
-          hr[i + 33 * j] = a.exact();
+        if (i <= j) {
+          const Scale<R> f = is2[i];
+          dots[i] = cmk(f.times(a), f.times(c2));
+          part2[i] = dots[i].re * a.value() + dots[i].im * c2.value();
+          hr[i + 33 * j] = a.exact();                        // raw; scaled by the last warp
           hi[i + 33 * j] = c2.exact();
+        } else {
+          part2[i] = a.value();                              // <w, w>
         }
       }
     }
@@ -267,17 +250,14 @@ __global__ void __launch_bounds__(768) coarse_gmres_cluster_kernel(const typenam
     R invb = 0, nn = 0;
     if (tid < nr || warp == nw - 1) {
       R e2 = 0;
-      for (int i = 0; i <= j; ++i) e2 += (dots[i].re * dots[i].re + dots[i].im * dots[i].im) * is2[i];
-      const R ww = dots[j + 1].re;
+      for (int i = 0; i <= j; ++i) e2 += part2[i];
+      const R ww = part2[j + 1];
       const R d2 = max(ww - e2, OP::kFloor * ww);
       invb = d2 > (R)0 ? rsqrt_of(d2) : (R)0;
     }
     for (int e = tid; e < nr; e += nt) {
       C t = w[e];
-      for (int i = 0; i <= j; ++i) {
-        const R f = is2[i];
-        cfma(t, cmk(-dots[i].re * f, -dots[i].im * f), basis[i * rows + e]);
-      }
+      for (int i = 0; i <= j; ++i) cfma(t, cmk(-dots[i].re, -dots[i].im), basis[i * rows + e]);
       nn += t.re * t.re + t.im * t.im;
       if (j + 1 < k) {
         const C v = invb * t;
@@ -290,9 +270,8 @@ __global__ void __launch_bounds__(768) coarse_gmres_cluster_kernel(const typenam
     all_norm(nn, j & 1);
     cluster_barrier();
     if (warp == nw - 1) {                                    // while the others start the next product
-      const Sum16<R> q = sum16(pn[(j & 1) * kSolveCluster + (lane & 15)]);
-      const R s2 = q.value() * invb * invb;
-      if (lane == 0) is2[j + 1] = s2 > (R)0 ? (R)1 / s2 : (R)0;
+      const Acc<R> q = sum16<R>(pn[(j & 1) * kSolveCluster + (lane & 15)]);
+      if (lane == 0) is2[j + 1] = Scale<R>::of(q, invb);
       const double nrm = sqrt(fmax(q.exact(), 0.0));
       if (lane <= j) {
         hr[lane + 33 * j] *= is[lane];
