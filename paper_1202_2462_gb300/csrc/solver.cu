@@ -2430,6 +2430,8 @@ int mg_coarse_solve_noalloc(mg_ctx* c, int level, const void* in, void* out, int
   void* w = sb + o_w;
   auto Vj = [&](int j) { return (void*)((char*)V + (size_t)j * n * eb); };
   const BVec bv = bvec(n, 1, n);
+  // the arrival counters, which calls that overlapped may have left in mid-count
+  SAPMG_CUDA_TRY(cudaMemsetAsync(partial + kPartialSums, 0, sizeof(double2) * (kPartialDouble2 - kPartialSums), c->s));
   // the same fixed-step GMRES as the cycle's coarse solve, on the scratch buffers
   {
     const void* v1[1] = {in};

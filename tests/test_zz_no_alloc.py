@@ -122,3 +122,47 @@ def test_noalloc_rejects_oversized_system():
         G.mg_coarse_solve_noalloc(s.ctx, 1, bc, out, G.MG_FP64)
     assert e.value.code == G.MG_ERR_ARG and "no-alloc scratch" in str(e.value)
     s.close()
+
+
+def test_noalloc_after_overlapping_calls():
+    """Overlapping calls spoil each other's results only: two contexts on streams
+    of their own, with coarse lattices whose reductions have different numbers
+    of CTAs, call at the same time; a call on its own afterwards equals, bit
+    for bit, the same call before."""
+    import threading
+    torch = torch_cuda()
+    import paper_1202_2462_gb300 as G
+    ctxs = []
+    for dims, seed in (((8, 8, 8, 8), 103), ((16, 16, 8, 8), 104), ((16, 16, 16, 8), 105)):
+        stream = torch.cuda.Stream()
+        u = dev(torch, synth.random_gauge_field(dims, 0.4, seed))
+        with torch.cuda.stream(stream):
+            s = G.Solver(u, 1.0, -0.2, n_levels=2, n_vec=(6,), setup_iters=1, precision="fp32", seed=9)
+        ns = int(np.prod(dims)) // 256
+        b = torch.randn((ns, 12), dtype=torch.complex64, device="cuda", generator=torch.Generator("cuda").manual_seed(seed))
+        ctxs.append((s, b, torch.empty_like(b)))
+    torch.cuda.synchronize()
+
+    def alone():
+        out = []
+        for s, b, x in ctxs:
+            G.mg_coarse_solve_noalloc(s.ctx, 1, b, x, G.MG_FP32)
+            torch.cuda.synchronize()
+            out.append(x.clone())
+        return out
+
+    def many(s, b, x):
+        for _ in range(200):
+            G.mg_coarse_solve_noalloc(s.ctx, 1, b, x, G.MG_FP32)
+
+    before = alone()
+    threads = [threading.Thread(target=many, args=c) for c in ctxs]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    for a, b in zip(before, alone()):
+        assert torch.equal(a, b)
+    for s, _, _ in ctxs:
+        s.close()
