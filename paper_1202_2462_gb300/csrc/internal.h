@@ -91,8 +91,9 @@ int launch_gate(const Geom& g, const void* x, const void* gy, void* out, int cha
 int launch_adam(size_t n, float* p, const float* gr, float* m, float* v, double lr, double b1, double b2,
                 double eps, int step, cudaStream_t s);
 
+constexpr int kCholWork = 1536;
 // orth.cu: N FP32 vectors of n complex entries (contiguous, n even) orthonormalised in
-// vector order by Cholesky QR twice.  work: 1536 double2; *flag != 0 afterwards: a vector
+// vector order by Cholesky QR twice.  work: kCholWork double2; *flag != 0 afterwards: a vector
 // is too close to the span of the earlier ones (V then spans what it did).
 int launch_cholqr2(void* V, int N, size_t n, double2* partial, double2* work, int* flag, cudaStream_t s);
 

@@ -223,7 +223,6 @@ struct mg_ctx {
   // allocated with the context, so that a captured call keeps a valid address and
   // no call allocates (10 MB at most)
   void* net_work = nullptr;
-  double2* gram = nullptr;                 // set-up only: work of the FP32 orthonormalisation
   void* part2_buf = nullptr;               // set-up only (three levels): part-1 vectors kept for set-up part 2
   const std::vector<double2>* load_v0 = nullptr;  // mg_setup_load: the saved level-0 vectors (host)
   const std::vector<double2>* load_w1 = nullptr;  // mg_setup_load: the saved level-1 vectors (host, three levels)
@@ -1185,10 +1184,11 @@ static int orthonormalise(mg_ctx* c, void* V, int N, size_t n, int type = P64) {
   const BVec one = bvec(n, 1, n);
   const size_t eb = type == P64 ? 16 : 8;
   auto Vk = [&](int k) { return (void*)((char*)V + (size_t)k * n * eb); };
-  if (type == P32 && c->gram && N >= 2) {
-    int* flag = (int*)(c->gram + 1536);
+  if (type == P32 && N >= 2) {
+    double2* work = (double2*)c->io_b;     // staging of calls after the set-up, 49152 numbers at least
+    int* flag = (int*)(work + kCholWork);
     int bad = 0;
-    TRY(launch_cholqr2(V, N, n, c->partial, c->gram, flag, c->s));
+    TRY(launch_cholqr2(V, N, n, c->partial, work, flag, c->s));
     SAPMG_CUDA_TRY(cudaMemcpyAsync(&bad, flag, sizeof(int), cudaMemcpyDeviceToHost, c->s));
     SAPMG_CUDA_TRY(cudaStreamSynchronize(c->s));
     if (!bad) return MG_OK;
@@ -1230,8 +1230,6 @@ static int build_level0_operators(mg_ctx* c) {
   const bool f32 = c->vt == P32 && c->setup_fp32 && c->U32 && c->A32 && c->Z &&
                    (size_t)c->m * c->p.nrhs_max >= (size_t)N;
   if (f32) {
-    c->gram = (double2*)c->alloc(sizeof(double2) * 1537);
-    if (!c->gram) return fail(MG_ERR_OOM, "set-up workspace");
     TRY(blas_axpby2(P64, scal_all(1.0, N), c->V64, n, P32, scal_all(0.0, N), c->Z, n, n, N, c->s));
     TRY(launch_assemble0(c->g, P32, c->Z, c->U32, c->A32, L.M64, N, c->s));
   } else {
@@ -1475,8 +1473,6 @@ static int setup_level0(mg_ctx* c) {
   // form, or a basis too small for N vectors, keeps them FP64.
   const bool f32 = c->vt == P32 && c->setup_fp32 && p.setup_iters > 0 && (size_t)c->m * p.nrhs_max >= (size_t)N;
   if (f32) {
-    c->gram = (double2*)c->alloc(sizeof(double2) * 1537);
-    if (!c->gram) return fail(MG_ERR_OOM, "set-up workspace");
     TRY(blas_axpby2(P64, scal_all(1.0, N), c->V64, n, P32, scal_all(0.0, N), c->Z, n, n, N, c->s));
     for (int it = 0; it < p.setup_iters; ++it) {
       // in pairs (the paired kernel), an odd last vector on its own
@@ -1487,9 +1483,6 @@ static int setup_level0(mg_ctx* c) {
       t_orth += clk.lap();
     }
     TRY(blas_axpby2(P32, scal_all(1.0, N), c->Z, n, P64, scal_all(0.0, N), c->V64, n, n, N, c->s));
-    SAPMG_CUDA_TRY(cudaStreamSynchronize(c->s));
-    c->release(c->gram);
-    c->gram = nullptr;
   }
   for (int it = 0; it < p.setup_iters && !f32; ++it) {
     for (int k = 0; k < N; ++k) {
