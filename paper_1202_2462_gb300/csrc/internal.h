@@ -97,6 +97,9 @@ constexpr int kCholWork = 1536;
 // is too close to the span of the earlier ones (V then spans what it did).
 int launch_cholqr2(void* V, int N, size_t n, double2* partial, double2* work, int* flag, cudaStream_t s);
 
+// SMs without a block in the last wave of n blocks, one an SM.
+inline long long idle_sms(long long n) { return (152 - n % 152) % 152; }
+
 // sap.cu
 // b may be null (a zero right-hand side).  pair_shape >= 0: an even number of
 // right-hand sides in FP32 arithmetic goes to the paired kernel with that launch

@@ -240,11 +240,18 @@ __global__ void __launch_bounds__(128) sap_cluster_kernel(TS* __restrict__ z, co
   for (int k = 0; k < 3; ++k) Io<R, TS>::st(z + own + k * 256, Io<R, TS>::ldc(z + own + k * 256) + e[k]);
 }
 
-// A cluster per block where whole blocks leave SMs idle: FP64, which is bound by
-// the SMs' FP64 units, up to four blocks an SM; FP32 below one block an SM.
+// A cluster per block where whole blocks leave SMs idle.  n blocks of a colour; one
+// sweep (two passes, n_MR = 4) by whole blocks and by clusters, us:
+// FP32 (whole blocks 50 up to 152): 46 at 72, 50 at 88, 84 at 104, where clusters no
+//   longer all fit at once.
+// FP64 (bound by the SMs' FP64 units, one block an SM at a time): whole blocks take
+//   979 a wave of 152, clusters 7.75 a block and 70; so 104: 979 and 919, 120: 979 and
+//   1057, 224: 1962 and 1805, 256: 1962 and 2039, 480: 3916 and 3730, 512: 3916 and 3967.
 template <class R>
 static bool cluster_wins(const Geom& g, int nrhs) {
-  return (long long)(g.nblocks / 2) * nrhs < 152 * (sizeof(R) == 8 ? 4 : 1);
+  const long long n = (long long)(g.nblocks / 2) * nrhs, idle = idle_sms(n);
+  if (sizeof(R) == 4) return n < 96;
+  return n < 608 && 5 * idle > n + 55;       // 6.44 (n + idle) > 7.75 n + 70
 }
 
 template <class R, class TS, class TG>
