@@ -95,10 +95,15 @@ __global__ void __launch_bounds__(128) dirac_quad_kernel(TS* __restrict__ out, c
 // Few blocks: FP64 below eight blocks an SM, where the last wave of whole blocks
 // leaves a tenth or more of the FP64 units' time unused (16 blocks, 8^4: 87 us
 // with a CTA per block on 16 SMs, 46 us with a warp per 32 sites); FP32, which
-// needs the warps of a block to hide latency, below one block an SM.
+// needs the warps of a block to hide latency, below one block an SM.  Double-float
+// arithmetic runs on the FP32 units, where a block alone on an SM loses little:
+// whole blocks 148 us a wave of 152; four threads a site 40 us at 16 blocks, 134 at
+// 96, 192 at 128, 268 at 192, 331 at 240, 438 at 320.
 template <class R>
 static bool few_blocks(const Geom& g, int nrhs) {
-  return (long long)g.nblocks * nrhs < 152 * (sizeof(R) == 8 ? 8 : 1);
+  const long long n = (long long)g.nblocks * nrhs;
+  if (std::is_same<R, DF>::value) return 20 * idle_sms(n) > 9 * n;
+  return n < 152 * (sizeof(R) == 8 ? 8 : 1);
 }
 
 template <class R, class TS, class TG, bool DAG, bool NORM>
