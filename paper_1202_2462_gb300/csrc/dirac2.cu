@@ -21,7 +21,13 @@ using namespace pair;
 // and what is used once stays out of L1: clover words by no-allocate loads, the
 // results by streaming stores (733 -> 711 us; the links, each used twice, lose
 // by it: 735 us; the block's spinors staged in shared memory: 794 us).
+// AHEAD: with few pairs a block the blocks of a wave hold more of the lattice, and what
+// is fetched ahead pushes the neighbours of t out of L2.  FP32, without and with,
+// us: 32^4 two fields 227 and 292, four 403 and 430, six 579 and 577, eight 757 and
+// 730; 16^3 x 32 two 31 and 33, four 60 and 61, six 82 and 85, eight 100 and 99, twelve 145 and
+// 138; 24^4 six 189 and 186.
 constexpr unsigned kAhead = 304;
+static bool ahead_wins(const Geom& g, int npairs) { return npairs >= 4 || (npairs == 3 && g.nblocks >= 1024); }
 
 // a clover entry as a broadcast pair, loaded past L1
 __device__ __forceinline__ B2 once(const float2* p) {
@@ -44,7 +50,7 @@ __device__ __forceinline__ B2 once(const __half2* p) {
   B2 b; b.r = f2(v.x); b.i = f2(v.y); b.ni = f2(-v.y); return b;
 }
 
-template <class TG>
+template <class TG, bool AHEAD>
 __global__ void __launch_bounds__(256, 2)
     dirac_pair_kernel(float2* __restrict__ out, const float2* __restrict__ in, const TG* __restrict__ U,
                       const TG* __restrict__ A, Geom g, int npairs) {
@@ -52,7 +58,7 @@ __global__ void __launch_bounds__(256, 2)
   const int loc = threadIdx.x;
   const size_t stride = (size_t)g.V * 12;
   const size_t off = (size_t)(blockIdx.x % npairs) * 2 * stride;
-  if (threadIdx.x == 0) {
+  if (AHEAD && threadIdx.x == 0) {
     const unsigned id = blockIdx.x + kAhead;
     if (id < gridDim.x) {
       const size_t b2 = id / npairs;
@@ -95,8 +101,13 @@ __global__ void __launch_bounds__(256, 2)
 template <class TG>
 static int run_pair(const Geom& g, void* out, const void* in, const void* U, const void* A, int nrhs, cudaStream_t s) {
   const int npairs = nrhs / 2;
-  dirac_pair_kernel<TG><<<(unsigned)(g.nblocks * npairs), 256, 0, s>>>((float2*)out, (const float2*)in,
-                                                                        (const TG*)U, (const TG*)A, g, npairs);
+  const unsigned grid = (unsigned)(g.nblocks * npairs);
+  if (ahead_wins(g, npairs))
+    dirac_pair_kernel<TG, true><<<grid, 256, 0, s>>>((float2*)out, (const float2*)in, (const TG*)U, (const TG*)A, g,
+                                                     npairs);
+  else
+    dirac_pair_kernel<TG, false><<<grid, 256, 0, s>>>((float2*)out, (const float2*)in, (const TG*)U, (const TG*)A, g,
+                                                      npairs);
   count_launches(1);
   SAPMG_CUDA_TRY(cudaGetLastError());
   return MG_OK;
