@@ -290,8 +290,8 @@ constexpr size_t kTileSmem = sizeof(float4) * kPairs * 4 * kLdW;
 // accumulates a 4 x 4 tile, (output channel, its 4 spins) x (pair, its 4 spins),
 // over the 48 (site, colour) terms; with RA < 16 the 256 / (16 RA) groups of
 // threads share the terms.  The slices' sums are added in slice order by a second
-// kernel, so the result is deterministic.  One CTA per (a, b, h) over all sites, as
-// before, transported every input once per output channel: 3.4 ms for 16 -> 16
+// kernel, so the result is deterministic.  One CTA per (a, b, h) over all sites, the
+// form below, transports every input once per output channel: 3.4 ms for 16 -> 16
 // channels at 16^4, against 1.70 ms.
 template <int RA>
 __global__ void __launch_bounds__(256, 2) gconv_wgrad_tile_kernel(Geom g, const float2* __restrict__ U,
@@ -419,6 +419,51 @@ __global__ void __launch_bounds__(256) gconv_wgrad_sum_kernel(const float2* __re
   gW[i] = make_float2((re[0] + re[1]) + (re[2] + re[3]), (im[0] + im[1]) + (im[2] + im[3]));
 }
 
+// The same for few products: CTA (a, b, h), a thread a site of every block.  The
+// sums of sixteen blocks (48 products a thread) are added to the totals, those over
+// warps and the CTA in a fixed order.
+__global__ void __launch_bounds__(256, 2) gconv_wgrad_site_kernel(Geom g, const float2* __restrict__ U,
+                                                                  const float2* __restrict__ x,
+                                                                  const float2* __restrict__ gy,
+                                                                  float2* __restrict__ gW, int cin) {
+  const int id = blockIdx.x, h = id % 9, b = (id / 9) % cin, a = id / (9 * cin);
+  const size_t fs = (size_t)g.V * 12;
+  Cplx<float> tot[16];
+#pragma unroll
+  for (int k = 0; k < 16; ++k) tot[k] = cmk(0.f, 0.f);
+  for (int b0 = 0; b0 < g.nblocks; b0 += 16) {
+    Cplx<float> acc[16];
+#pragma unroll
+    for (int k = 0; k < 16; ++k) acc[k] = cmk(0.f, 0.f);
+    for (int blk = b0; blk < min(b0 + 16, g.nblocks); ++blk) {
+      Cplx<float> v[12], p[12];
+      transport_at(g, U, x + (size_t)b * fs, blk, threadIdx.x, h, v);
+      load_spinor<float>(gy + (size_t)a * fs, blk, threadIdx.x, p);
+#pragma unroll
+      for (int s = 0; s < 4; ++s)
+#pragma unroll
+        for (int t = 0; t < 4; ++t)
+#pragma unroll
+          for (int c = 0; c < 3; ++c) cfma_conj(acc[s * 4 + t], v[t * 3 + c], p[s * 3 + c]);
+    }
+#pragma unroll
+    for (int k = 0; k < 16; ++k) tot[k] = tot[k] + acc[k];
+  }
+  __shared__ float2 red[8][16];
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll
+  for (int k = 0; k < 16; ++k) {
+    const float re = warp_sum(tot[k].re), im = warp_sum(tot[k].im);
+    if (lane == 0) red[w][k] = make_float2(re, im);
+  }
+  __syncthreads();
+  if (threadIdx.x < 16) {
+    float re = 0.f, im = 0.f;
+    for (int q = 0; q < 8; ++q) { re += red[q][threadIdx.x].x; im += red[q][threadIdx.x].y; }
+    gW[(size_t)id * 16 + threadIdx.x] = make_float2(re, im);
+  }
+}
+
 // y = x / sqrt(1 + |x(site)|^2) per channel and site
 __global__ void gate_forward_kernel(Geom g, const float2* __restrict__ x, float2* __restrict__ y, int channels) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -537,11 +582,24 @@ static int wgrad_slices(const Geom& g, int cin, int cout) {
   const int chunks = g.nblocks * 16;
   return std::max(1, std::min(304 / tiles, chunks / 4));       // one wave: a CTA more doubles the time
 }
+// Whether the tiles beat a CTA per (a, b, h), by the times (us) that describe both within a
+// few percent for 1 to 64 channels on 16, 64 and 256 blocks: chunks of a slice, the
+// slices' sum and what both kernels cost; waves of CTAs, the first one and a half
+// bound by one CTA's own loads.  1 -> 16 channels at 8^4 25 us by sites and 57 by tiles, 1 ->
+// 8 25 and 34, 64 -> 3 at 16^4 2630 and 5490; 16 -> 16 at 8^4 216 and 127.
+static bool wgrad_tiled(const Geom& g, int cin, int cout) {
+  const int ns = wgrad_slices(g, cin, cout);
+  const double chunks = (g.nblocks * 16 + ns - 1) / ns, waves = (9 * cin * cout + 151) / 152;
+  const double tiles = cout >= 16 ? 13.6 * chunks + 0.3 * ns
+                     : cout >= 4 ? 8 + 5.0 * chunks + 0.2 * ns : 10 + 2.5 * chunks + 0.2 * ns;
+  return 0.95 * tiles <= 7 + 0.84 * g.nblocks * std::max(1.43, waves);
+}
+
 size_t gconv_wgrad_bytes(const Geom& g, int max_channels) {
   size_t most = 0;
   for (int cin = 1; cin <= max_channels; ++cin)
     for (int cout = 1; cout <= max_channels; ++cout)
-      if (wgrad_slices(g, cin, cout) > 1) most = std::max(most, (size_t)wgrad_slices(g, cin, cout) * cout * cin * 9 * 16);
+      if (wgrad_tiled(g, cin, cout) && wgrad_slices(g, cin, cout) > 1) most = std::max(most, (size_t)wgrad_slices(g, cin, cout) * cout * cin * 9 * 16);
   return most * sizeof(float2);
 }
 
@@ -582,7 +640,11 @@ int launch_gconv_backward(const Geom& g, const void* U, const void* W, const voi
       count_launches(1);
     }
   }
-  if (gW) {
+  if (gW && !wgrad_tiled(g, cin, cout)) {
+    gconv_wgrad_site_kernel<<<cout * cin * 9, 256, 0, s>>>(g, (const float2*)U, (const float2*)x, (const float2*)gy,
+                                                           (float2*)gW, cin);
+    count_launches(1);
+  } else if (gW) {
     const size_t n = (size_t)cout * cin * 9 * 16;
     const int nslice = wgrad_slices(g, cin, cout);
     float2* part = nslice > 1 ? (float2*)work : (float2*)gW;         // one slice is gW itself
