@@ -528,6 +528,27 @@ __global__ void adam_kernel(size_t n, float* __restrict__ p, const float* __rest
 // and 371.
 constexpr int kTiledFrom = 6, kTiledFromBwd = 8;
 
+// The channels' worth of time that c channels take in tiles of sixteen: nine and more of a
+// last tile keep all its warps' sub-partitions as busy as sixteen, up to eight as ten.
+static int tile_cost(int c) {
+  const int r = c % kTileCh;
+  return c - r + (r == 0 ? 0 : r <= 8 ? 10 : kTileCh);
+}
+// The transports of one or two input channels are cheap to repeat: 16^4, 1 -> 9 92 and 114
+// us, 12 118 and 139, 16 152 and 145, 24 225 and 218, 33 305 and 334; 2 -> 9 172 and 180;
+// 4 -> 9 330 and 299.
+static bool layer_tiled(int cin, int cout) {
+  return cout >= kTiledFrom && (cin > 2 || 10 * tile_cost(cout) <= (cin == 1 ? 11 : 15) * cout);
+}
+// A thread per site reads each output's gradient once per input channel, from L2 while the
+// outputs' gradients fit there (8 channels at 16^4: 9 470 and 539 us, 13 about equal, 16 802 and 628,
+// 17 848 and 874, 24 1186 and 964), from HBM beyond (16 channels: 8 1224 and 733, 9 1374 and
+// 1066, 17 2557 and 1724).
+static bool input_gradient_tiled(const Geom& g, int cin, int cout) {
+  if (cin < kTiledFromBwd) return false;
+  return (size_t)cout * g.V * 96 > (64u << 20) || 10 * tile_cost(cin) <= 13 * cin;
+}
+
 template <class TG, class TW, bool BWD>
 static int gconv_tiled(const Geom& g, const void* U, const void* W, const void* x, void* y, int cin, int cout,
                        cudaStream_t s) {
@@ -550,9 +571,7 @@ static int gconv_forward(const Geom& g, const void* U, const void* W, const void
                          cudaStream_t s) {
   const size_t smem = sizeof(float2) * cin * 9 * 16;
   if (smem > 200 * 1024) return MG_ERR_ARG;
-  if (cout >= kTiledFrom) {
-    return gconv_tiled<TG, TW, false>(g, U, W, x, y, cin, cout, s);
-  }
+  if (layer_tiled(cin, cout)) return gconv_tiled<TG, TW, false>(g, U, W, x, y, cin, cout, s);
   static bool attr = false;
   if (!attr) {
     cudaFuncSetAttribute(gconv_forward_kernel<TG, TW>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
@@ -631,7 +650,7 @@ int launch_gconv_backward(const Geom& g, const void* U, const void* W, const voi
     attr = true;
   }
   if (gx) {
-    if (cin >= kTiledFromBwd) {
+    if (input_gradient_tiled(g, cin, cout)) {
       const int rc = gconv_tiled<float2, float2, true>(g, U, W, gy, gx, cout, cin, s);
       if (rc != MG_OK) return rc;
     } else {
