@@ -14,6 +14,7 @@
 // earlier ones, or zero, or not finite) raises a flag, on which the solves leave
 // V as it was and the caller orthonormalises vector by vector instead; above it
 // the first pass is orthogonal to 1e-2 and the second to rounding.
+#include "accum.cuh"
 #include "internal.h"
 #include "blas.h"
 
@@ -22,7 +23,7 @@ namespace {
 
 constexpr double kPivot = 1e-4;
 constexpr int kChunkE = 64;          // elements per staged chunk
-constexpr int kStagesG = 3;
+constexpr int kRun = 32;             // products in one FP32 sum
 
 __device__ __forceinline__ void cp_async8(void* dst, const void* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
@@ -31,18 +32,22 @@ __device__ __forceinline__ void cp_async8(void* dst, const void* src) {
 
 // Partial Gram matrices: the upper triangle in 4 x 4 tiles of vectors; thread
 // (tile pair, group) takes every G-th element of the staged chunk.  Bound by the FP32
-// units (N^2 / 2 complex products an element).
-__global__ void __launch_bounds__(256) gram_kernel(const float2* __restrict__ V, int N, size_t n, int T,
+// units (N^2 / 2 complex products an element).  Sums of kRun products go to totals of
+// two floats each (accum.cuh) in shared memory: a thread meets 5000 elements at 32^3 x 64.
+template <int STAGES>
+__global__ void __launch_bounds__(256, 2) gram_kernel(const float2* __restrict__ V, int N, size_t n, int T,
                                                    double2* __restrict__ partial) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int P = T * (T + 1) / 2, G = 256 / P, ld = 4 * T + 2;      // row stride of a staged element
   float2* sx = reinterpret_cast<float2*>(smem);
+  float4* tot = reinterpret_cast<float4*>(smem + sizeof(float2) * STAGES * kChunkE * ld);   // [entry][thread]
   const int tid = threadIdx.x, pair = tid % P, grp = tid / P;
   int ti = 0, tj = pair;
   while (tj >= T - ti) { tj -= T - ti; ++ti; }
   tj += ti;
   // vectors N .. 4 T - 1 stay zero in every stage
-  for (int e = tid; e < kStagesG * kChunkE * ld; e += 256) sx[e] = make_float2(0.f, 0.f);
+  for (int e = tid; e < STAGES * kChunkE * ld; e += 256) sx[e] = make_float2(0.f, 0.f);
+  for (int k = 0; k < 16; ++k) tot[k * 256 + tid] = make_float4(0.f, 0.f, 0.f, 0.f);
   __syncthreads();
   const size_t nchunk = (n + kChunkE - 1) / kChunkE;
   auto load = [&](size_t ch, int st) {
@@ -58,16 +63,28 @@ __global__ void __launch_bounds__(256) gram_kernel(const float2* __restrict__ V,
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
   size_t ch = blockIdx.x;
-  for (int s = 0; s < kStagesG - 1; ++s) load(ch + (size_t)s * gridDim.x, s);
+  for (int s = 0; s < STAGES - 1; ++s) load(ch + (size_t)s * gridDim.x, s);
   Cplx<float> acc[4][4];
+  auto flush = [&] {                                               // a thread's own totals: no barrier
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
+    for (int k = 0; k < 16; ++k) {
+      Cplx<float>& a = acc[k >> 2][k & 3];
+      const float4 t = tot[k * 256 + tid];
+      Acc<float> re{t.x, t.y}, im{t.z, t.w};
+      re.add(Acc<float>::of(a.re));
+      im.add(Acc<float>::of(a.im));
+      tot[k * 256 + tid] = make_float4(re.h, re.l, im.h, im.l);
+      a = cmk(0.f, 0.f);
+    }
+  };
 #pragma unroll
-    for (int b = 0; b < 4; ++b) acc[a][b] = cmk(0.f, 0.f);
-  for (int st = 0; ch < nchunk; ch += gridDim.x, st = st + 1 == kStagesG ? 0 : st + 1) {
-    asm volatile("cp.async.wait_group %0;" ::"n"(kStagesG - 2) : "memory");
+  for (int k = 0; k < 16; ++k) acc[k >> 2][k & 3] = cmk(0.f, 0.f);
+  const int run = max(1, kRun * G / kChunkE);                      // chunks a sum
+  int left = run;
+  for (int st = 0; ch < nchunk; ch += gridDim.x, st = st + 1 == STAGES ? 0 : st + 1) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(STAGES - 2) : "memory");
     __syncthreads();
-    load(ch + (size_t)(kStagesG - 1) * gridDim.x, st == 0 ? kStagesG - 1 : st - 1);
+    load(ch + (size_t)(STAGES - 1) * gridDim.x, st == 0 ? STAGES - 1 : st - 1);
     if (grp < G) {
       const float2* x = sx + st * kChunkE * ld;
       for (int e = grp; e < kChunkE; e += G) {
@@ -82,21 +99,34 @@ __global__ void __launch_bounds__(256) gram_kernel(const float2* __restrict__ V,
           for (int q = 0; q < 4; ++q) cfma_conj(acc[p][q], a[p], b[q]);
       }
     }
+    if (--left == 0) {
+      flush();
+      left = run;
+    }
   }
+  flush();
   asm volatile("cp.async.wait_group 0;" ::: "memory");
   __syncthreads();
-  // the groups' sums, added in FP64
-  float2* red = sx;                                                 // [G][P][16]
-  if (grp < G)
-#pragma unroll
-    for (int p = 0; p < 4; ++p)
-#pragma unroll
-      for (int q = 0; q < 4; ++q) red[(grp * P + pair) * 16 + p * 4 + q] = make_float2(acc[p][q].re, acc[p][q].im);
+  // the groups' totals: entry e of the tiles, its groups shared by as many threads as there are
+  const int ne = P * 16, share = max(1, 256 / ne), e0 = tid % ne, part = tid / ne;
+  for (int e = e0; e < ne && part < share; e += 256) {
+    float4* t = tot + (e & 15) * 256 + (e >> 4);
+    Acc<float> re{0.f, 0.f}, im{0.f, 0.f};
+    for (int g = part; g < G; g += share) {
+      re.add(Acc<float>{t[g * P].x, t[g * P].y});
+      im.add(Acc<float>{t[g * P].z, t[g * P].w});
+    }
+    t[part * P] = make_float4(re.h, re.l, im.h, im.l);
+  }
   __syncthreads();
-  for (int e = tid; e < P * 16; e += 256) {
+  for (int e = tid; e < ne; e += 256) {
+    const float4* t = tot + (e & 15) * 256 + (e >> 4);
     double a = 0, b = 0;
-    for (int g = 0; g < G; ++g) { a += red[g * P * 16 + e].x; b += red[g * P * 16 + e].y; }
-    partial[(size_t)blockIdx.x * P * 16 + e] = make_double2(a, b);
+    for (int g = 0; g < share; ++g) {
+      a += (double)t[g * P].x + (double)t[g * P].y;
+      b += (double)t[g * P].z + (double)t[g * P].w;
+    }
+    partial[(size_t)blockIdx.x * ne + e] = make_double2(a, b);
   }
 }
 
@@ -200,18 +230,21 @@ int launch_cholqr2(void* V, int N, size_t n, double2* partial, double2* work, in
   if (N < 1 || N > 32 || n % 2 != 0 || (reinterpret_cast<uintptr_t>(V) & 15) != 0) return MG_ERR_ARG;
   const int T = (N + 3) / 4, P = T * (T + 1) / 2;
   const int ncta = (int)std::min<size_t>({(size_t)304, (n + kChunkE - 1) / kChunkE, kPartialSums / (size_t)(P * 16)});
-  const size_t smem = std::max((size_t)kStagesG * kChunkE * (4 * T + 2), (size_t)(256 / P) * P * 16) * sizeof(float2);
+  const int stages = T < 8 ? 3 : 2;                                // two CTAs' totals and stages on an SM
+  const size_t smem = (size_t)stages * kChunkE * (4 * T + 2) * sizeof(float2) + (size_t)16 * 256 * sizeof(float4);
   double2* Gm = work;                                              // [32][32]
   float2* coef = reinterpret_cast<float2*>(work + 32 * 32);        // [32][32]
   static bool attr = false;
   if (!attr) {
-    SAPMG_CUDA_TRY(cudaFuncSetAttribute(gram_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024));
+    SAPMG_CUDA_TRY(cudaFuncSetAttribute(gram_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, 112 * 1024));
+    SAPMG_CUDA_TRY(cudaFuncSetAttribute(gram_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 112 * 1024));
     attr = true;
   }
   SAPMG_CUDA_TRY(cudaMemsetAsync(flag, 0, sizeof(int), s));
   const unsigned tri = (unsigned)((n / 2 + 255) / 256);
   for (int pass = 0; pass < 2; ++pass) {
-    gram_kernel<<<ncta, 256, smem, s>>>((const float2*)V, N, n, T, partial);
+    if (stages == 3) gram_kernel<3><<<ncta, 256, smem, s>>>((const float2*)V, N, n, T, partial);
+    else gram_kernel<2><<<ncta, 256, smem, s>>>((const float2*)V, N, n, T, partial);
     gram_sum_kernel<<<P, 256, 0, s>>>(partial, ncta, T, Gm);
     gram_chol_kernel<<<1, 256, 0, s>>>(Gm, N, coef, flag);
     if (N <= 8) tri_kernel<8><<<tri, 256, 0, s>>>((float4*)V, N, n / 2, coef, flag);
