@@ -654,23 +654,30 @@ static int transfer0_mrhs(bool restrict_, const Geom& g, const void* in, void* o
   return MG_OK;
 }
 
-static int transfer0_fp64(bool restrict_, const Geom& g, const void* in, void* out, const void* Pv, int N, int nrhs,
-                          cudaStream_t s) {
+template <class R, class TS, class TV>
+static int transfer0_t(bool restrict_, const Geom& g, const void* in, void* out, const void* Pv, int N, int nrhs,
+                       cudaStream_t s) {
   const unsigned grid = (unsigned)(g.nblocks * nrhs);   // right-hand side fastest: P shared through L2
   if (restrict_)
-    restrict0_kernel<double, double2, double2, double2><<<grid, 256, sizeof(double) * 4 * 8 * N, s>>>(
-        (const double2*)in, (double2*)out, (const double2*)Pv, N, nrhs, g.nblocks);
+    restrict0_kernel<R, TS, TV, TS><<<grid, 256, sizeof(R) * 4 * 8 * N, s>>>((const TS*)in, (TS*)out, (const TV*)Pv, N,
+                                                                             nrhs, g.nblocks);
   else
-    prolong0_kernel<double, double2, double2, double2><<<grid, 256, sizeof(double2) * 2 * N, s>>>(
-        (const double2*)in, (double2*)out, (const double2*)Pv, N, nrhs, g.nblocks);
+    prolong0_kernel<R, TS, TV, TS><<<grid, 256, sizeof(TS) * 2 * N, s>>>((const TS*)in, (TS*)out, (const TV*)Pv, N,
+                                                                         nrhs, g.nblocks);
   count_launches(1);
   SAPMG_CUDA_TRY(cudaGetLastError());
   return MG_OK;
 }
 
+// With few vectors a warp a vector leaves most of a CTA idle.  A thread per site and the
+// forms above, FP16 P, us: restriction at 512 blocks N = 1 6.0 and 6.8, 3 6.9 and 8.8, 4
+// 8.6 and 8.8, 8 12.7 and 12.8, at 2048 blocks N = 1 10.7 and 17.1, 4 37.4 and 31.6;
+// interpolation N = 1 6.4 and 8.6, 2 6.8 and 8.6, 4 8.6 and 8.8, at 2048 blocks N = 1 12.7
+// and 16.9, 2 21.3 and 19.0.
 template <class TV>
 static int transfer0_vec(bool restrict_, const Geom& g, const void* in, void* out, const void* Pv, int N, int nrhs,
                          cudaStream_t s) {
+  if (N < (restrict_ ? 4 : 3)) return transfer0_t<float, float2, TV>(restrict_, g, in, out, Pv, N, nrhs, s);
   const unsigned grid = (unsigned)(g.nblocks * nrhs);
   if (restrict_)
     restrict0_vec_kernel<TV><<<2 * grid, 256, 0, s>>>((const float2*)in, (float2*)out, (const TV*)Pv, N, nrhs, g.nblocks);
@@ -695,7 +702,7 @@ int launch_transfer0(bool restrict_, int prec, const Geom& g, const void* in, vo
     }
   }
   switch (prec) {
-    case P64: return transfer0_fp64(restrict_, g, in, out, Pv, N, nrhs, s);
+    case P64: return transfer0_t<double, double2, double2>(restrict_, g, in, out, Pv, N, nrhs, s);
     case P32: return transfer0_vec<float2>(restrict_, g, in, out, Pv, N, nrhs, s);
     case P16: return transfer0_vec<__half2>(restrict_, g, in, out, Pv, N, nrhs, s);
     case PBF: return transfer0_vec<__nv_bfloat162>(restrict_, g, in, out, Pv, N, nrhs, s);
