@@ -841,10 +841,10 @@ __device__ __forceinline__ void assemble_dir(const Geom& g, const T2* U, const T
   }
 }
 
-// FP64 vectors and fields (the plain form, exact to rounding).  The mixed form, whose
-// coarse operator is stored in FP32 and FP16, assembles it from FP32 copies
-// (assemble0_tiled_kernel): FP64 arithmetic is scarce on this GPU.  The entries
-// are written in FP64 either way.
+// FP64 vectors and fields (the plain form, exact to rounding), or FP32 copies of up to three
+// vectors.  The mixed form, whose coarse operator is stored in FP32 and FP16,
+// assembles it from FP32 copies (more vectors: assemble0_tiled_kernel): FP64 arithmetic is
+// scarce on this GPU.  The entries are written in FP64 either way.
 template <class R, class T2>
 __global__ void __launch_bounds__(256) assemble0_kernel(const T2* __restrict__ V, const T2* __restrict__ U,
                                                         const T2* __restrict__ A, double2* __restrict__ M,
@@ -1084,6 +1084,11 @@ int launch_assemble0(const Geom& g, int prec, const void* V, const void* U, cons
   if (prec == P64)
     assemble0_kernel<double, double2><<<grid, 256, smem, s>>>((const double2*)V, (const double2*)U,
                                                               (const double2*)A, (double2*)M64, g, N);
+  else if (prec == P32 && N < 4)
+    // the tiles give sixteen threads a vector: whole set-up at 16^3 x 32, tiles and columns, N = 1
+    // 7.47 and 6.95 ms, 3 7.78 and 7.59, 4 7.93 and 8.00, 6 8.46 and 8.97
+    assemble0_kernel<float, float2><<<grid, 256, smem, s>>>((const float2*)V, (const float2*)U, (const float2*)A,
+                                                            (double2*)M64, g, N);
   else if (prec == P32) {
     const int Np = (N + 3) & ~3;
     const size_t tiled = sizeof(float2) * 12 * kAsmSites * (3 * Np + 4);      // holds the groups' totals too
