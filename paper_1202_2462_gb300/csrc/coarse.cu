@@ -486,16 +486,27 @@ __global__ void __launch_bounds__(256) restrict0_mma_kernel(const float2* __rest
 // exactly); P is staged per chunk of kRKC entries by cp.async; B is loaded
 // into registers once.  Neighbouring lanes (real and imaginary rows of one K)
 // swap halves by a shuffle so that each stores whole complex numbers.
+// Row stride: a fragment's two rows of four neighbouring entries lie on different banks for
+// 4- and 8-byte entries.
+constexpr int kPSP = 132;
 template <class TV>
 __host__ __device__ constexpr size_t prolong_stage_bytes(int Np) {
-  return (size_t)Np * RPad<TV>::sp * sizeof(TV);
+  return (size_t)Np * kPSP * sizeof(TV);
 }
+
+// FP32 entries are read whole and their component is selected: 2 fields, N = 20, 524288
+// sites 218 us, by components 230 (rows of 130 entries 228 and 238).
+template <class TV> __device__ __forceinline__ float2 p_ld(const TV* p) {
+  const Cplx<float> v = Io<float, TV>::ldc(p);
+  return make_float2(v.re, v.im);
+}
+__device__ __forceinline__ float embed_pr(float2 m, int a, int b) { return a == b ? m.x : (a ? m.y : -m.y); }
 
 template <int NT, class TV>
 __global__ void __launch_bounds__(256) prolong0_mma_kernel(const float2* __restrict__ in, float2* __restrict__ out,
                                                            const TV* __restrict__ Pv, int N, int nrhs, int nblocks) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  constexpr int SP = RPad<TV>::sp;
+  constexpr int SP = kPSP;
   const int Np = (N + 3) & ~3;                                 // k padded to whole k8 steps of the embedding
   const size_t PB = prolong_stage_bytes<TV>(Np);
   auto sP = [&](int st) { return reinterpret_cast<TV*>(smem_raw + st * PB); };
@@ -566,11 +577,15 @@ __global__ void __launch_bounds__(256) prolong0_mma_kernel(const float2* __restr
 #pragma unroll
       for (int ks = 0; ks < 8; ++ks) {
         if (ks < KS) {
-          const int k = 4 * ks + (tig >> 1);                    // columns tig (k) and tig + 4 (k + 2)
-          const uint32_t a0 = p_tf32(P + k * SP + Kl, acomp) ^ asign;
-          const uint32_t a1 = p_tf32(P + k * SP + Kl + 4, acomp) ^ asign;
-          const uint32_t a2 = p_tf32(P + (k + 2) * SP + Kl, acomp) ^ asign;
-          const uint32_t a3 = p_tf32(P + (k + 2) * SP + Kl + 4, acomp) ^ asign;
+          const int k = 4 * ks + (tig >> 1), b = tig & 1;       // columns tig (k) and tig + 4 (k + 2)
+          const uint32_t a0 = sizeof(TV) == 8 ? f32_to_tf32(embed_pr(p_ld(P + k * SP + Kl), a, b))
+                                               : p_tf32(P + k * SP + Kl, acomp) ^ asign;
+          const uint32_t a1 = sizeof(TV) == 8 ? f32_to_tf32(embed_pr(p_ld(P + k * SP + Kl + 4), a, b))
+                                               : p_tf32(P + k * SP + Kl + 4, acomp) ^ asign;
+          const uint32_t a2 = sizeof(TV) == 8 ? f32_to_tf32(embed_pr(p_ld(P + (k + 2) * SP + Kl), a, b))
+                                               : p_tf32(P + (k + 2) * SP + Kl, acomp) ^ asign;
+          const uint32_t a3 = sizeof(TV) == 8 ? f32_to_tf32(embed_pr(p_ld(P + (k + 2) * SP + Kl + 4), a, b))
+                                               : p_tf32(P + (k + 2) * SP + Kl + 4, acomp) ^ asign;
 #pragma unroll
           for (int nt = 0; nt < NT; ++nt) mma_m16n8k8_tf32(acc[nt], a0, a1, a2, a3, bf[ks][nt][0], bf[ks][nt][1]);
         }
