@@ -332,21 +332,15 @@ __device__ __forceinline__ uint32_t pack16(float2 v) {
   return *reinterpret_cast<const uint32_t*>(&h);
 }
 
-// ST: depth of the staging ring (0: the launch parameter depth).  With more sites
-// than resident CTAs two or three stages are the fastest (more CTAs an SM); with fewer,
-// the deepest ring that keeps every site resident (up to all nine blocks in
-// flight at once) shortens the serial chain of nine copies a site: 512 sites,
-// one right-hand side, 12.0 us with 2 stages.
-constexpr int kMaxRing = 9;
+// ST: depth of the staging ring.
 template <int RB, int N2, int ST, bool XH>
 __global__ void __launch_bounds__(256) coarse_apply_mma16_kernel(const __half2* __restrict__ M,
                                                                  const void* __restrict__ xv,
                                                                  float2* __restrict__ out, CGeom c, int r0, int nr,
-                                                                 int depth, int* __restrict__ err) {
+                                                                 int* __restrict__ err) {
   extern __shared__ __align__(128) unsigned char smem[];
   const int spins = wait_spins(err);
-  const int st_n = ST > 0 ? ST : depth;
-  __shared__ __align__(8) uint64_t bar[kMaxRing];
+  __shared__ __align__(8) uint64_t bar[ST];
   const int n2 = N2 > 0 ? N2 : c.n2;                         // N2 > 0: block size fixed at compile time
   const int xst = n2 + 4;                                     // padded row stride (conflict-free fragment loads)
   const int tile = n2 * n2;
@@ -367,12 +361,12 @@ __global__ void __launch_bounds__(256) coarse_apply_mma16_kernel(const __half2* 
   const int nsite_cta = (c.nsites - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
   const int T = 9 * nsite_cta;
   if (T <= 0) return;
-  for (int st = 0; st < st_n; ++st) {
+  for (int st = 0; st < ST; ++st) {
     uint32_t* z = reinterpret_cast<uint32_t*>(smem + st * stage_bytes + tile_bytes + (size_t)nr * xst * xb);
     for (int e = tid; e < (kRows - nr) * xst * xb / 4; e += blockDim.x) z[e] = 0u;
   }
   if (tid == 0) {
-    for (int st = 0; st < st_n; ++st) mbar_init(&bar[st], 1);
+    for (int st = 0; st < ST; ++st) mbar_init(&bar[st], 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
@@ -385,7 +379,8 @@ __global__ void __launch_bounds__(256) coarse_apply_mma16_kernel(const __half2* 
     const int xc = (site / stride) % c.L[mu];
     return site + (((xc + step + c.L[mu]) % c.L[mu]) - xc) * stride;
   };
-  auto issue = [&](int t, int st) {
+  auto issue = [&](int t) {
+    const int st = t % ST;
     const int site = MG_CLAMP(kCoarseSite, site_of(t), c.nsites), d = t % 9;
     uint64_t* b = &bar[st];
     mbar_expect_tx(b, tile_bytes + nr * row_bytes);
@@ -397,13 +392,12 @@ __global__ void __launch_bounds__(256) coarse_apply_mma16_kernel(const __half2* 
   };
   if (tid == 0) {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    for (int t = 0; t < st_n - 1 && t < T; ++t) issue(t, t);
+    for (int t = 0; t < ST - 1 && t < T; ++t) issue(t);
   }
   const int m0 = warp * 16;
   const int i0 = (m0 >> 1) + (g >> 1), a = g & 1;            // output rows i0 (fragment row g) and i0 + 4 (g + 8)
   float acc[2][4];
   int tfail = -1;
-  int st = 0, phase = 0;                                      // t % st_n, (t / st_n) & 1
   for (int t = 0; t < T; ++t) {
     const int d = t % 9;
     const int site = MG_CLAMP(kCoarseSite, site_of(t), c.nsites);
@@ -411,11 +405,12 @@ __global__ void __launch_bounds__(256) coarse_apply_mma16_kernel(const __half2* 
 #pragma unroll
       for (int q = 0; q < 2; ++q) acc[q][0] = acc[q][1] = acc[q][2] = acc[q][3] = 0.f;
     }
-    if (tid == 0 && t + st_n - 1 < T) {
+    if (tid == 0 && t + ST - 1 < T) {
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      issue(t + st_n - 1, st == 0 ? st_n - 1 : st - 1);
+      issue(t + ST - 1);
     }
-    const bool waited = mbar_wait(&bar[st], (uint32_t)phase, spins);
+    const int st = t % ST;
+    const bool waited = mbar_wait(&bar[st], (uint32_t)((t / ST) & 1), spins);
     if (__syncthreads_or(!waited)) {
       tfail = t;
       break;
@@ -455,57 +450,52 @@ __global__ void __launch_bounds__(256) coarse_apply_mma16_kernel(const __half2* 
       }
     }
     __syncthreads();
-    if (++st == st_n) { st = 0; phase ^= 1; }
   }
   if (tfail >= 0) {
     if (tid == 0) {
       atomicExch(err, 1);
-      // blocks tfail .. tfail + st_n - 1 were issued (the copy of t + st_n - 1 goes
-      // out before the wait of t): let every one of them land
-      for (int u = tfail; u < T && u < tfail + st_n; ++u) mbar_wait(&bar[u % st_n], (uint32_t)((u / st_n) & 1));
+      // blocks tfail .. tfail + ST - 1 were issued (the copy of t + ST - 1 goes out
+      // before the wait of t): let every one of them land
+      for (int u = tfail; u < T && u < tfail + ST; ++u) mbar_wait(&bar[u % ST], (uint32_t)((u / ST) & 1));
     }
     __syncthreads();
   }
 }
 
 template <int RB, int N2, int ST, bool XH>
-static void launch_mma16_st(const CGeom& c, const __half2* M, const void* x, float2* out, int r0, int nr, int* err,
-                            int grid, int threads, size_t smem, int st, cudaStream_t s) {
+static void launch_mma16_t(const CGeom& c, const __half2* M, const void* x, float2* out, int r0, int nr, int* err,
+                           int ctas, cudaStream_t s) {
+  const size_t stage = (size_t)c.n2 * c.n2 * sizeof(__half2) + (size_t)(RB <= 8 ? 8 : 16) * (c.n2 + 4) * (XH ? 4 : 8);
   static bool attr = false;
   if (!attr) {
     cudaFuncSetAttribute(coarse_apply_mma16_kernel<RB, N2, ST, XH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          200 * 1024);
     attr = true;
   }
-  coarse_apply_mma16_kernel<RB, N2, ST, XH><<<grid, threads, smem, s>>>(M, x, out, c, r0, nr, st, err);
+  // CTAs an SM: what shared memory holds, and with FP32 vectors no more than ten warps a
+  // sub-partition, which 48 registers a thread leave room for; the rest of a larger grid runs
+  // as a second round of few CTAs (4096 sites, one vector: 2N = 40 59 us on 11, 51.8 on 8; 2N = 48
+  // 100 on 8, 84 on 6; 2N = 56 122 on 6, 103 on 5).  With FP16 vectors the larger grid wins:
+  // 2592 sites, 12 systems, 2N = 40 44.9 us on 11, 46.0 on the 9 that are resident.
+  const int warps = c.n2 / 8;
+  int per_sm = (int)std::max<size_t>(1, std::min<size_t>(16, (220 * 1024) / (ST * stage + 1024)));
+  if (!XH) per_sm = std::min(per_sm, 40 / warps);
+  if (ctas > 0) per_sm = std::min(per_sm, ctas);
+  coarse_apply_mma16_kernel<RB, N2, ST, XH><<<std::min(c.nsites, 152 * per_sm), 32 * warps, ST * stage, s>>>(
+      M, x, out, c, r0, nr, err);
   count_launches(1);
 }
 
-template <int RB, int N2, bool XH>
-static void launch_mma16_t(const CGeom& c, const __half2* M, const void* x, float2* out, int r0, int nr, int* err,
-                           const CoarseTune& t, cudaStream_t s) {
-  const size_t stage = (size_t)c.n2 * c.n2 * sizeof(__half2) + (size_t)(RB <= 8 ? 8 : 16) * (c.n2 + 4) * (XH ? 4 : 8);
-  const int threads = 32 * (c.n2 / 8);
-  auto per_sm = [&](int st) {
-    const int k = (int)std::max<size_t>(1, std::min<size_t>(16, (220 * 1024) / (st * stage + 1024)));
-    return t.ctas > 0 ? std::min(k, t.ctas) : k;
-  };
-  int st = c.n2 == 40 && t.stages == 3 ? 3 : 2;
-  for (int d = kMaxRing; d > st; --d)
-    if (d * stage <= 200 * 1024 && c.nsites <= 152 * per_sm(d)) { st = d; break; }
-  const int grid = std::min(c.nsites, 152 * per_sm(st));
-  const size_t smem = st * stage;
-  if (st == 2) launch_mma16_st<RB, N2, 2, XH>(c, M, x, out, r0, nr, err, grid, threads, smem, st, s);
-  else if (st == 3 && N2 > 0) launch_mma16_st<RB, N2, 3, XH>(c, M, x, out, r0, nr, err, grid, threads, smem, st, s);
-  else launch_mma16_st<RB, N2, 0, XH>(c, M, x, out, r0, nr, err, grid, threads, smem, st, s);
-}
-
+// Two stages (one block in flight while the previous is multiplied) unless the autotuner
+// finds three faster; deeper rings, up to all nine blocks of a site, gained nothing at 256 to
+// 4096 sites.
 // 2N = 40 has a specialised instance with the k loop unrolled.
 template <int RB, bool XH>
 static void launch_mma16(const CGeom& c, const __half2* M, const void* x, float2* out, int r0, int nr, int* err,
                          const CoarseTune& t, cudaStream_t s) {
-  if (c.n2 == 40) launch_mma16_t<RB, 40, XH>(c, M, x, out, r0, nr, err, t, s);
-  else launch_mma16_t<RB, 0, XH>(c, M, x, out, r0, nr, err, t, s);
+  if (c.n2 == 40 && t.stages == 3) launch_mma16_t<RB, 40, 3, XH>(c, M, x, out, r0, nr, err, t.ctas, s);
+  else if (c.n2 == 40) launch_mma16_t<RB, 40, 2, XH>(c, M, x, out, r0, nr, err, t.ctas, s);
+  else launch_mma16_t<RB, 0, 2, XH>(c, M, x, out, r0, nr, err, t.ctas, s);
 }
 
 template <int RB, class TM>
