@@ -1,7 +1,7 @@
-"""The launch forms for few blocks (one-warp CTAs of D, a cluster of CTAs per
-Schwarz block, the coarse kernels of a short vector) against the forms that the
-same call takes for many: the same fields once alone and once in a batch that
-is large enough for the other form."""
+"""The launch forms for few blocks (D with four threads a site, a cluster of CTAs
+per Schwarz block) against the forms that the same call takes for many: the same
+fields once alone and once in a batch that is large enough for the other form;
+and the fixed-step coarse GMRES in all its forms against the minimiser."""
 
 import numpy as np
 import pytest
@@ -79,27 +79,40 @@ def test_level1_schwarz_cluster_matches_one_cta_per_box(n_vec, nrhs, monkeypatch
     assert torch.equal(out["0"][0], out["1"][0]) and out["0"][1] == out["1"][1]
 
 
-@pytest.mark.parametrize("prec,tol", [("fp64", 1e-13), ("fp32", 1e-3), ("fp16", 1e-3)])
-@pytest.mark.parametrize("iters", [1, 4, 5, 16, 17, 32])
-def test_coarse_gmres_minimises(prec, tol, iters):
+# 16 coarse sites: the one-kernel form; 128: a kernel for the dots and one for the
+# update a step, with the basis in FP64, FP32 ("fp32") and FP16 ("fp16")
+@pytest.mark.parametrize("dims,prec,tol", [
+    (DIMS, "fp64", 1e-13), (DIMS, "fp32", 1e-3), (DIMS, "fp16", 1e-3),
+    ((16, 8, 16, 16), "fp64", 1e-13), ((16, 8, 16, 16), "fp32", 1e-3), ((16, 8, 16, 16), "fp16", 4e-3)])
+@pytest.mark.parametrize("iters", [1, 4, 5, 8, 9, 16, 17, 32])
+def test_coarse_gmres_minimises(dims, prec, tol, iters, monkeypatch):
     """The fixed-step coarse solve against the least-squares minimiser over the
     Krylov space, at the step counts where its kernels change size: the norms
     of the two residuals, relative to the source's (the mixed form applies an
     FP16 operator, entries rounded by up to 5e-4, so its residual under the FP64
-    operator is off by that much; 1e-13 is FP64 rounding times 256 terms).  The
-    longest runs go on after the Krylov space is exhausted."""
-    torch, G, s = _solver(prec, n_levels=2, n_vec=(8,), setup_iters=2, coarse_iters=iters, seed=3)
-    nb, n2 = 16, 16
+    operator is off by that much; an FP16 basis adds roundings of 2^-11 of up to
+    32 vectors; 1e-13 is FP64 rounding times 256 terms).  On 16 sites the longest
+    runs go on after the Krylov space is exhausted."""
+    torch = torch_cuda()
+    import paper_1202_2462_gb300 as G
+    if prec == "fp32":
+        monkeypatch.setenv("SAPMG_COARSE_BASIS_FP16", "0")
+    u = dev(torch, synth.random_gauge_field(dims, 0.4, 301))
+    s = G.Solver(u, 1.0, -0.1, precision=prec, n_levels=2, n_vec=(8,), setup_iters=2, coarse_iters=iters, seed=3)
+    lat = [d // 4 for d in dims]
+    nb, n2 = int(np.prod(lat)), 16
     m = torch.empty((nb, 9, n2, n2), dtype=torch.complex128, device="cuda")
     G.mg_get_coarse_op(s.ctx, 1, m)
     mh = host(m)
     nbr = np.zeros((nb, 9), dtype=int)
     for a in range(nb):
-        x = [(a >> q) & 1 for q in range(4)]
+        x = list(np.unravel_index(a, lat, order="F"))
         nbr[a, 0] = a
         for mu in range(4):
-            nbr[a, 1 + 2 * mu] = nbr[a, 2 + 2 * mu] = a ^ (1 << mu)
-        assert sum(v << q for q, v in enumerate(x)) == a
+            for step, d in ((1, 1 + 2 * mu), (-1, 2 + 2 * mu)):
+                y = list(x)
+                y[mu] = (y[mu] + step) % lat[mu]
+                nbr[a, d] = np.ravel_multi_index(y, lat, order="F")
     dense = np.zeros((nb * n2, nb * n2), dtype=complex)
     for a in range(nb):
         for d in range(9):

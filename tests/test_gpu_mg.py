@@ -130,19 +130,21 @@ def test_coarse_gmres_parity(fp64_ctx):
     assert rel(host(out), ref) < 1e-11
 
 
-@pytest.mark.parametrize("basis16", ["1", "0"])
-def test_coarse_gmres_mixed_parity(basis16, monkeypatch):
+@pytest.mark.parametrize("basis16,dims", [("1", (8, 8, 8, 16)), ("0", (8, 8, 8, 16)), ("1", (8, 16, 16, 16)),
+                                          ("0", (8, 16, 16, 16))])
+def test_coarse_gmres_mixed_parity(basis16, dims, monkeypatch):
     """Fixed-step GMRES in the mixed form (FP16 operator on the tensor cores),
-    with the Krylov basis in FP16 (default) or FP32 (SAPMG_COARSE_BASIS_FP16=0),
-    against the oracle's GMRES on the FP16-rounded operator (8^3 x 16 lattice,
-    32 coarse sites, m0 = -3.9 so that 12 steps are far from an exact solve):
+    with the Krylov basis in FP16 (default) or FP32 (SAPMG_COARSE_BASIS_FP16=0;
+    on 32 coarse sites one kernel does the whole solve, with its basis in FP32),
+    against the oracle's GMRES on the FP16-rounded operator (32 and 128
+    coarse sites, m0 = -3.9 so that 12 steps are far from an exact solve):
     the same Krylov minimiser up to the rounding of the basis and of the
     vectors fed to the tensor cores (FP16, 2^-11 relative), and a residual
     above the minimal one by no more than that rounding."""
     torch = torch_cuda()
     import paper_1202_2462_gb300 as G
     monkeypatch.setenv("SAPMG_COARSE_BASIS_FP16", basis16)
-    dims = (8, 8, 8, 16)
+    ns = int(np.prod(dims)) // 256
     u = synth.random_gauge_field(dims, 0.4, 59)
     iv = synth.test_vector_draw(dims, 8, 60)
     m0 = -3.9
@@ -151,10 +153,11 @@ def test_coarse_gmres_mixed_parity(basis16, monkeypatch):
     c = CoarseOperator(WilsonClover(u, m0, CSW), Aggregation(dims, (4, 4, 4, 4), (4, 3)).build(iv))
     for name in ("self_", "fwd", "bwd"):
         setattr(c, name, round_storage(getattr(c, name), "fp16"))
-    bc = synth.random_spinor((2, 2, 2, 4), 61).reshape(4, 2, 2, 2, 12)
+    lat = tuple(d // 4 for d in dims)
+    bc = synth.random_spinor(lat, 61).reshape(lat[::-1] + (12,))
     bc = np.concatenate([bc, bc[..., :4]], axis=-1).astype(np.complex64).astype(np.complex128)   # 16 dof
-    out = torch.zeros((32, 16), dtype=torch.complex64, device="cuda")
-    G.mg_coarse_solve(s.ctx, 1, dev(torch, bc.reshape(32, 16), torch.complex64), out, G.MG_FP32)
+    out = torch.zeros((ns, 16), dtype=torch.complex64, device="cuda")
+    G.mg_coarse_solve(s.ctx, 1, dev(torch, bc.reshape(ns, 16), torch.complex64), out, G.MG_FP32)
     torch.cuda.synchronize()
     s.close()
     ref = gmres_fixed(c.apply, bc, 12)
@@ -491,21 +494,25 @@ def test_complex64_initial_vectors_match_complex128():
     assert torch.equal(ops[0], ops[1])
 
 
-@pytest.mark.parametrize("levels", [2, 3])
-def test_coarse_solve_graphs_match_plain_launches(levels, monkeypatch):
+@pytest.mark.parametrize("levels,dims,n_vec,nrhs", [
+    (2, (8, 8, 8, 16), (12,), 4), (3, (16, 8, 8, 16), (12, 8), 4),
+    # coarsest lattices too large for the one-kernel form (128 sites; 32 sites with 2N = 64): these are captured
+    (2, (16, 8, 16, 16), (12,), 4), (2, (16, 8, 16, 16), (20,), 1), (3, (16, 16, 16, 32), (32, 32), 2)])
+def test_coarse_solve_graphs_match_plain_launches(levels, dims, n_vec, nrhs, monkeypatch):
     """The mixed form replays its FP16-basis coarse GMRES as a captured CUDA
     graph (after one run with plain launches): two solves with graphs give
     the solution of the plain launches (SAPMG_GRAPHS=0) bit for bit, and the
     launch counter counts the graphs' kernels as launches."""
     torch = torch_cuda()
     import paper_1202_2462_gb300 as G
-    dims = (8, 8, 8, 16) if levels == 2 else (16, 8, 8, 16)
-    kw = dict(n_levels=levels, n_vec=(12, 8) if levels == 3 else (12,), setup_iters=2, precision="bf16",
-              nrhs_max=4, seed=6, coarse_iters=8, fgmres_m=10)
-    if levels == 3:
+    kw = dict(n_levels=levels, n_vec=n_vec, setup_iters=2, precision="bf16",
+              nrhs_max=nrhs, seed=6, coarse_iters=8, fgmres_m=10)
+    if levels == 3 and dims[1] == 8:
         kw.update(sap_block2=(2, 1, 1, 2), agg2=(2, 2, 2, 2), inner_iters=3)
+    if levels == 3 and dims[1] != 8:
+        kw.update(inner_iters=2)
     u = dev(torch, synth.random_gauge_field(dims, 0.4, 181))
-    b = dev(torch, synth.random_spinor(dims, 182, nvec=4))
+    b = dev(torch, synth.random_spinor(dims, 182, nvec=nrhs))
     out = {}
     for flag in ("0", "1"):
         monkeypatch.setenv("SAPMG_GRAPHS", flag)
@@ -524,6 +531,8 @@ def test_coarse_solve_graphs_match_plain_launches(levels, monkeypatch):
         out[flag] = (zs[1], counts)
     assert torch.equal(out["0"][0], out["1"][0])
     assert out["0"][1] == out["1"][1]
+    if int(np.prod(dims)) > 16384:               # three kernels a step, not one a solve
+        assert out["1"][1][1] > info.iterations // nrhs * 3 * kw["coarse_iters"]
 
 
 @pytest.mark.parametrize("nrhs,m16", [(2, "1"), (3, "1"), (6, "0"), (6, "1"), (12, "0"), (12, "1")])

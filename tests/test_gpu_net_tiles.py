@@ -1,6 +1,7 @@
-"""The set-up network's tiled layer kernels at channel counts around their tile
-sizes (4 and 16 output channels, 16 (input channel, hop) pairs), against the
-FP64 oracle."""
+"""The set-up network's layer kernels at channel counts around their tile sizes (4
+and 16 output channels, 16 (input channel, hop) pairs) and around the lines
+between tiles and threads or CTAs of single channels, against the FP64 oracle;
+fields at odd elements; a captured weight gradient."""
 
 import numpy as np
 import pytest
@@ -27,7 +28,8 @@ def _canonical(torch, s, y, c):
 
 # FP32 sums of 36 cin products (forward), of 36 cout (input gradient) and of 3 V
 # (weights): 2e-6 as in the layer's own parity test
-@pytest.mark.parametrize("cin,cout", [(1, 1), (1, 4), (4, 3), (3, 5), (2, 16), (16, 2), (5, 17), (7, 5), (8, 6)])
+@pytest.mark.parametrize("cin,cout", [(1, 1), (1, 4), (4, 3), (3, 5), (2, 16), (16, 2), (5, 17), (7, 5), (8, 6), (13, 9), (2, 9),
+                                      (1, 16)])
 def test_layer_tiles(cin, cout):
     torch = torch_cuda()
     import paper_1202_2462_gb300 as G

@@ -11,7 +11,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("prec", ["fp64", "fp32"])
-@pytest.mark.parametrize("dims,nrhs", [((8, 16, 8, 24), 1), ((24, 8, 16, 8), 3)])
+@pytest.mark.parametrize("dims,nrhs", [((8, 16, 8, 24), 1), ((24, 8, 16, 8), 3), ((32, 16, 16, 32), 3)])
 def test_layout_moves_every_number(dims, nrhs, prec):
     """Packing against the blocked order written out, unpacking against its inverse:
     numbers are moved, so the results are the same bits."""
@@ -65,10 +65,10 @@ def test_outer_basis_in_half_precision(monkeypatch, nrhs):
 
 
 @pytest.mark.parametrize("prec", ["fp32", "fp16", "bf16"])
-@pytest.mark.parametrize("n_vec", [1, 8, 9, 17, 25])
+@pytest.mark.parametrize("n_vec", [1, 2, 3, 4, 8, 9, 17, 25])
 def test_transfers_of_one_field(prec, n_vec):
-    """One field's restriction and prolongation, at the vector counts where a warp has
-    one, two or three vectors, against the oracle with the same rounded vectors: FP32
+    """One field's restriction and prolongation, at the vector counts where a thread per
+    site gives way to the wide forms and where a warp has one, two or three vectors, against the oracle with the same rounded vectors: FP32
     sums of 1536 and n_vec products.  The prolongation also to an address that is not
     a multiple of 16 bytes."""
     torch = torch_cuda()

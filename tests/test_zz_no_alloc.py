@@ -67,10 +67,11 @@ def test_noalloc_coarse_solve_matches_oracle_fp64():
     s.close()
 
 
-@pytest.mark.parametrize("prec", ["fp32", "bf16"])
-def test_noalloc_against_fp16_basis_solve(prec):
-    """Mixed form with 2N = 16: mg_coarse_solve keeps its Krylov basis in FP16
-    (the FP16 operator copy exists), the no-alloc solve keeps it in FP32.  Both
+@pytest.mark.parametrize("prec,dims", [("fp32", DIMS), ("bf16", DIMS), ("fp32", (16, 8, 16, 16)), ("bf16", (16, 8, 16, 16))])
+def test_noalloc_against_fp16_basis_solve(prec, dims):
+    """Mixed form with 2N = 16: on 128 coarse sites mg_coarse_solve keeps its Krylov
+    basis in FP16 (the FP16 operator copy exists; on 16 sites one kernel does the
+    whole solve, with the basis in FP32), the no-alloc solve keeps it in FP32.  Both
     read the same FP16 operator, so they differ by the basis rounding only:
     FP16 keeps 11 significant bits (relative rounding 2^-11 = 4.9e-4), and a
     12-step GMRES result built on such a basis moves by a small multiple of
@@ -78,12 +79,14 @@ def test_noalloc_against_fp16_basis_solve(prec):
     uses against the oracle."""
     torch = torch_cuda()
     import paper_1202_2462_gb300 as G
-    u = synth.random_gauge_field(DIMS, 0.4, 99)
+    u = synth.random_gauge_field(dims, 0.4, 99)
     s = G.Solver(dev(torch, u), 1.0, -0.2, n_levels=2, n_vec=(8,), setup_iters=1, precision=prec, seed=11,
                  coarse_iters=12)
+    lat = tuple(d // 4 for d in dims)
+    ns = int(np.prod(lat))
     for seed in (100, 101):
-        b = synth.random_spinor((2, 2, 2, 2), seed, nvec=2).reshape(2, 16, 12).transpose(1, 0, 2).reshape(16, 24)
-        b = np.ascontiguousarray(b[:, :16])                 # 16 coarse sites x 2N = 16
+        b = synth.random_spinor(lat, seed, nvec=2).reshape(2, ns, 12).transpose(1, 0, 2).reshape(ns, 24)
+        b = np.ascontiguousarray(b[:, :16])                 # coarse sites x 2N = 16
         bc = dev(torch, b, torch.complex64)
         ref = torch.zeros_like(bc)
         out = torch.full_like(bc, 7.0)
