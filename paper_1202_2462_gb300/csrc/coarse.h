@@ -84,6 +84,7 @@ int launch_coarse_sap_mrhs(const CGeom& c, const Box4& bx, const void* M, bool m
 // nrhs), where the box and its operator rows fit (coarse_sap_cluster_ok: sites a
 // multiple of eight, 2N even; 16 sites up to 2N = 48); the same results bit for bit.
 bool coarse_sap_cluster_ok(const CGeom& c, const Box4& bx);
+bool coarse_sap_cluster_wins(const CGeom& c, const Box4& bx, int nrhs);   // against the forms above
 int launch_coarse_sap_cluster(const CGeom& c, const Box4& bx, const void* M16, void* z, const void* b, int colour,
                               int n_mr, int nrhs, int* err, cudaStream_t s);
 int launch_coarse_sap(int prec, const CGeom& c, const Box4& bx, const void* M, void* z, const void* b, int colour,

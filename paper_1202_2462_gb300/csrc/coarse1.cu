@@ -597,6 +597,22 @@ bool coarse_sap_cluster_ok(const CGeom& c, const Box4& bx) {
          box_cluster_smem(bx, c.n2) <= 227 * 1024;
 }
 
+// Clusters take a box's right-hand sides one after the other, a CTA per box takes them together
+// (its time steps at 3, 5 and 9 of them) until the boxes exceed the CTAs that are
+// resident.  A pass, n_MR = 4, boxes of a colour, right-hand sides: clusters and CTA, us:
+// N = 20: 32, 12 338 and 670; 64, 12 647 and 704; 128, 4 434 and 526, 8 839 and 810, 12 1240 and
+//   821; 256, 4 806 and 1028, 12 2308 and 1612;
+// N = 8: 64, 12 182 and 218; 128, 6 178 and 182, 8 233 and 188; 256, 2 120 and 141, 4 220 and
+//   174, 12 616 and 284.
+// One right-hand side: N = 20 256 242 and 427; N = 8 128 41 and 43, 256 70 and 67.
+bool coarse_sap_cluster_wins(const CGeom& c, const Box4& bx, int nrhs) {
+  const int boxes = bx.nboxes / 2, threads = bx.sites * c.n2;
+  if (nrhs == 1) return threads > 320 || boxes <= 200;
+  if (nrhs > 12) return true;                          // the form for them all ends at twelve
+  const int slots = 152 * (threads <= 512 ? 2 : 1), waves = (boxes + slots - 1) / slots;
+  return (nrhs + 1) * boxes < waves * (nrhs <= 2 ? 500 : nrhs <= 4 ? 667 : nrhs <= 8 ? 1000 : 1094);
+}
+
 template <int MAXT, int MINB>
 static int coarse_sap_cluster_run(const CGeom& c, const Box4& bx, const void* M16, void* z, const void* b, int colour,
                                   int n_mr, int nrhs, int* err, unsigned threads, cudaStream_t s) {

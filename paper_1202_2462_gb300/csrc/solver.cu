@@ -557,14 +557,15 @@ static int coarse_solve(mg_ctx* c, int level, int R) {
 // Schwarz sweeps on level 1 (boxes of coarse sites, red-black as on the fine level).
 // Mixed form: the FP16 copy of the level-1 operator that the level-1 Krylov
 // operator already uses, unless SAPMG_COARSE_SAP_FP16=0, held in the shared
-// memory of a cluster of CTAs per box where it fits; else all right-hand sides in
-// one CTA per box (each operator entry loaded once for all of them).
+// memory of a cluster of CTAs per box where it fits and is the faster; else all
+// right-hand sides in one CTA per box (each operator entry loaded once for all of them).
 // SAPMG_COARSE_SAP_MRHS=0: one right-hand side per CTA.
 static int smoother_sweeps1(mg_ctx* c, const void* b, void* z, int n_sweeps, int R) {
   const bool mrhs = c->coarse_sap_mrhs && c->c1.store == P32 && R >= 2 && R <= 12;
   const bool m16 = c->coarse_sap_fp16 && c->c1.store == P32 && c->c1.Mh != nullptr;
   const void* M = m16 ? c->c1.Mh : c->c1.M;
-  const bool cluster = m16 && c->coarse_sap_mrhs && coarse_sap_cluster_ok(c->c1.cg, c->sap1);
+  const bool cluster = m16 && c->coarse_sap_mrhs && coarse_sap_cluster_ok(c->c1.cg, c->sap1) &&
+                       coarse_sap_cluster_wins(c->c1.cg, c->sap1, R);
   for (int it = 0; it < n_sweeps; ++it)
     for (int col = 0; col < 2; ++col) {
       ProfScope ps(c->prof, FAM_SAP1, c->s);
