@@ -360,10 +360,11 @@ int mg_get_profile(mg_ctx* ctx, int family, long long* launches, double* ms);
  * operand read once and every result written once: fields in storage
  * precision, the right-hand sides' vectors, P, the coarse operator), summed
  * like mg_get_profile's milliseconds; their ratio is the family's achieved
- * bandwidth.  The level-1 Schwarz passes count their operator reads (every
- * MR step reads the box's operator; once for all right-hand sides in the
- * multi-RHS form, once per right-hand side otherwise); the level-1 transfers
- * add no bytes. */
+ * bandwidth.  The level-1 Schwarz passes count their operator reads (the
+ * cluster form, which keeps the box's operator in shared memory, one; the others
+ * one per MR step and one for the residual, once for all right-hand sides in
+ * the multi-RHS form, once per right-hand side otherwise); the level-1
+ * transfers add no bytes. */
 int mg_get_profile_bytes(mg_ctx* ctx, int family, double* bytes);
 int mg_reset_profile(mg_ctx* ctx);
 
@@ -426,7 +427,9 @@ long long mg_debug_failures(void);
 int mg_debug_check(long long value, long long bound);
 
 /* Bound on the main-loop waits of the kernels that stage data with bulk
- * copies (the coarse stencils, the block-resident Schwarz pass): a wait that
+ * copies (the coarse stencils, the block-resident Schwarz pass, the level-1
+ * Schwarz pass and the coarse GMRES that keep their operator in a cluster's
+ * shared memory): a wait that
  * has not completed after `spins` tries gives up, the kernel drains its copies
  * in flight (those waits keep the default bound) and raises the flag that the
  * synchronising calls report as MG_ERR_TIMEOUT.  spins < 0 restores the

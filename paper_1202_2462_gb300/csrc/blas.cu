@@ -267,7 +267,7 @@ __global__ void __launch_bounds__(256) multiaxpy_kernel(T2* __restrict__ w, Ptrs
       for (int q = 0; q < 8; ++q) sum += red[q];
       partial[((size_t)r * gridDim.x + blockIdx.x) * kChunk] = make_double2(sum, 0.0);
     }
-      finish_dots<1>(partial, dout);
+    finish_dots<1>(partial, dout);
   }
 }
 
@@ -687,7 +687,7 @@ __global__ void __launch_bounds__(256) axpy2_kernel(PtrsV<typename Unit<T2>::V> 
       for (int q = 0; q < 8; ++q) sum += red[q][threadIdx.x];
       partial[((size_t)r * gridDim.x + blockIdx.x) * kChunk + threadIdx.x] = make_double2(sum, 0.0);
     }
-      finish_dots<2>(partial, dout);
+    finish_dots<2>(partial, dout);
   }
 }
 
@@ -948,7 +948,7 @@ __global__ void __launch_bounds__(256) axpy2h_kernel(PtrsV<uint2> v, const doubl
       for (int q = 0; q < 8; ++q) sum += red[q][threadIdx.x];
       partial[((size_t)r * gridDim.x + blockIdx.x) * kChunk + threadIdx.x] = make_double2(sum, 0.0);
     }
-      finish_dots<2>(partial, dout);
+    finish_dots<2>(partial, dout);
   }
 }
 
