@@ -190,11 +190,11 @@ __global__ void __launch_bounds__(256) gconv_backward_input_kernel(Geom g, const
 constexpr int kPairs = 8, kTileSites = 32, kTileCh = 16;
 constexpr int kLdW = kTileCh * 4 + 4;              // a row more of 64 bytes: the 16-byte stores of W spread
 
-template <class TG, class TW, bool BWD>
+template <class TG, class TW, bool BWD, bool AL>
 __global__ void __launch_bounds__(256, 2) gconv_tile_kernel(Geom g, const TG* __restrict__ U,
                                                             const TW* __restrict__ W, const float2* __restrict__ x,
-                                                            float2* __restrict__ y, int cin, int cout, bool al) {
-  // cin: channels of x; cout: channels of y (BWD: the layer's output and input channels); al: y starts on 16 bytes
+                                                            float2* __restrict__ y, int cin, int cout) {
+  // cin: channels of x; cout: channels of y (BWD: the layer's output and input channels); AL: y starts on 16 bytes
   // [pair, spin][colour][two sites]: (re, re, im, im); [pair, input spin][channel, spin]: (re, re, im, im)
   __shared__ __align__(16) float4 Ts[kPairs * 4][3][kTileSites / 2];
   extern __shared__ __align__(16) float4 Ws[];                        // [kPairs * 4][kLdW]
@@ -273,7 +273,7 @@ __global__ void __launch_bounds__(256, 2) gconv_tile_kernel(Geom g, const TG* __
     for (int c = 0; c < 3; ++c) {
       float2* d = o + (s * 3 + c) * 256;
       const P2 v = acc[s][c];
-      if (al) {
+      if (AL) {
         *reinterpret_cast<float4*>(d) = make_float4(v.re.x, v.im.x, v.re.y, v.im.y);
       } else {
         d[0] = make_float2(v.re.x, v.im.x);
@@ -549,21 +549,26 @@ static bool input_gradient_tiled(const Geom& g, int cin, int cout) {
   return (size_t)cout * g.V * 96 > (64u << 20) || 10 * tile_cost(cin) <= 13 * cin;
 }
 
-template <class TG, class TW, bool BWD>
-static int gconv_tiled(const Geom& g, const void* U, const void* W, const void* x, void* y, int cin, int cout,
-                       cudaStream_t s) {
+template <class TG, class TW, bool BWD, bool AL>
+static int gconv_tiled_run(const Geom& g, const void* U, const void* W, const void* x, void* y, int cin, int cout,
+                           cudaStream_t s) {
   static bool attr = false;
   if (!attr) {
-    SAPMG_CUDA_TRY(cudaFuncSetAttribute(gconv_tile_kernel<TG, TW, BWD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)kTileSmem));
+    SAPMG_CUDA_TRY(cudaFuncSetAttribute(gconv_tile_kernel<TG, TW, BWD, AL>,
+                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTileSmem));
     attr = true;
   }
-  gconv_tile_kernel<TG, TW, BWD><<<dim3(g.nblocks * 8, (cout + kTileCh - 1) / kTileCh), 256, kTileSmem, s>>>(
-      g, (const TG*)U, (const TW*)W, (const float2*)x, (float2*)y, cin, cout,
-      (reinterpret_cast<uintptr_t>(y) & 15) == 0);
+  gconv_tile_kernel<TG, TW, BWD, AL><<<dim3(g.nblocks * 8, (cout + kTileCh - 1) / kTileCh), 256, kTileSmem, s>>>(
+      g, (const TG*)U, (const TW*)W, (const float2*)x, (float2*)y, cin, cout);
   count_launches(1);
   SAPMG_CUDA_TRY(cudaGetLastError());
   return MG_OK;
+}
+template <class TG, class TW, bool BWD>
+static int gconv_tiled(const Geom& g, const void* U, const void* W, const void* x, void* y, int cin, int cout,
+                       cudaStream_t s) {
+  return (reinterpret_cast<uintptr_t>(y) & 15) == 0 ? gconv_tiled_run<TG, TW, BWD, true>(g, U, W, x, y, cin, cout, s)
+                                                    : gconv_tiled_run<TG, TW, BWD, false>(g, U, W, x, y, cin, cout, s);
 }
 
 template <class TG, class TW>
@@ -617,8 +622,10 @@ static bool wgrad_tiled(const Geom& g, int cin, int cout) {
 size_t gconv_wgrad_bytes(const Geom& g, int max_channels) {
   size_t most = 0;
   for (int cin = 1; cin <= max_channels; ++cin)
-    for (int cout = 1; cout <= max_channels; ++cout)
-      if (wgrad_tiled(g, cin, cout) && wgrad_slices(g, cin, cout) > 1) most = std::max(most, (size_t)wgrad_slices(g, cin, cout) * cout * cin * 9 * 16);
+    for (int cout = 1; cout <= max_channels; ++cout) {
+      const int ns = wgrad_slices(g, cin, cout);
+      if (ns > 1 && wgrad_tiled(g, cin, cout)) most = std::max(most, (size_t)ns * cout * cin * 9 * 16);
+    }
   return most * sizeof(float2);
 }
 
